@@ -1024,7 +1024,8 @@ extern "C" int feplb_set_planner_timing(feplb_ctx* c, int32_t planner_delay_us, 
 extern "C" int feplb_pack_weights(feplb_ctx* c, const void* w1_in, const void* w3_in, const void* w2_in, void* w1, void* w3,
                                   void* w2, void* stream) {
   if (!c) return FEPLB_E_INVALID;
-  if (!w1_in || !w3_in || !w2_in || !w1 || !w3 || !w2) return fail(c, FEPLB_E_INVALID, "pack_weights: null pointer");
+  int rc = check_dev_ptrs(c, {w1_in, w3_in, w2_in, w1, w3, w2});
+  if (rc != FEPLB_OK) return rc;
   // [E,d,f] -> [E,f,d] and [E,f,d] -> [E,d,f]: the transposition of feplb_transpose_weights with d and f exchanged
   CUDA_TRY(c, feplb_launch_transpose_weights(w1_in, w3_in, w2_in, w1, w3, w2, c->cfg.E, c->cfg.f, c->cfg.d,
                                              (cudaStream_t)stream, &c->launches));
@@ -1068,7 +1069,8 @@ extern "C" int feplb_set_preact_buffer(feplb_ctx* c, void* ab) {
 extern "C" int feplb_transpose_weights(feplb_ctx* c, const void* w1, const void* w3, const void* w2, void* w1t, void* w3t,
                                        void* w2t, void* stream) {
   if (!c) return FEPLB_E_INVALID;
-  if (!w1 || !w3 || !w2 || !w1t || !w3t || !w2t) return fail(c, FEPLB_E_INVALID, "transpose_weights: null pointer");
+  int rc = check_dev_ptrs(c, {w1, w3, w2, w1t, w3t, w2t});
+  if (rc != FEPLB_OK) return rc;
   CUDA_TRY(c, feplb_launch_transpose_weights(w1, w3, w2, w1t, w3t, w2t, c->cfg.E, c->cfg.d, c->cfg.f, (cudaStream_t)stream,
                                              &c->launches));
   return FEPLB_OK;
