@@ -85,10 +85,14 @@ struct GemmParams {
   int E;
   int64_t s_cap;        // rows of the A and output buffers
   int n_tiles_n;        // N tiles per M tile
+  int half_width;       // rows of B over all half tiles of one M tile: f (pass 1), d / 2 (pass 2); a multiple of 64
+  int b_box;            // rows of one box of the B tensor maps (64 or 128); divides every half tile
+  int early_weights;    // the group table was complete before this kernel's predecessor let it start: B loads of the
+                        // first tile may be issued before griddepcontrol.wait
   int num_k_blocks;     // K / 64
   int b_rows_per_expert;  // rows of one expert in the B tensor maps
   int n_recv_slots;     // slots of the receive buffer of migrated experts' weights (0 = none)
-  int bn;               // rows of one B half tile (64 or 128); the MMA has N = 2*bn
+  int bn;               // rows of one B half tile (64 or 128; the last N tile may be narrower); the MMA has N = 2 * rows
   __nv_bfloat16* out;
   int ld_out;           // elements between output rows
   uint32_t* status;
@@ -99,13 +103,14 @@ struct GemmParams {
 };
 
 
-struct TileCoord { int row0, rows_valid, expert, slot, nt; };   // slot >= 0: weights in that receive slot
+struct TileCoord { int row0, rows_valid, expert, slot, n0, bn; };   // slot >= 0: weights in that receive slot;
+                                                                   // n0 = first column of the half tile, bn its rows
 
 // tile -> (group, M tile, N tile); N tiles of one M tile are consecutive so that CTAs running at
 // the same time share the A rows and sweep one expert's weights together (both stay in L2).
 template <int kRows>
-__device__ __forceinline__ TileCoord tile_coord(const SmemTail* t, int n_groups, int n_tiles_n, int tile) {
-  const int mt = tile / n_tiles_n;
+__device__ __forceinline__ TileCoord tile_coord(const SmemTail* t, int n_groups, const GemmParams& p, int tile) {
+  const int mt = tile / p.n_tiles_n;
   int lo = 0, hi = n_groups;   // largest g with prefix[g] <= mt
   while (hi - lo > 1) {
     const int mid = (lo + hi) >> 1;
@@ -117,7 +122,8 @@ __device__ __forceinline__ TileCoord tile_coord(const SmemTail* t, int n_groups,
   c.rows_valid = min(kRows, t->g_rows[lo] - local * kRows);
   c.expert = t->g_expert[lo] & 0xffff;
   c.slot = (t->g_expert[lo] >> 16) - 1;
-  c.nt = tile - mt * n_tiles_n;
+  c.n0 = (tile - mt * p.n_tiles_n) * p.bn;
+  c.bn = min(p.bn, p.half_width - c.n0);
   return c;
 }
 
@@ -248,10 +254,6 @@ k_grouped_gemm(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   volatile int* abort_flag = &tail->abort_flag;
 
-  // Programmatic dependent launch: the next kernel of the stream may be scheduled as soon as SMs
-  // free up (its set-up then overlaps this grid's tail); it waits for this grid's results itself.
-  asm volatile("griddepcontrol.launch_dependents;");
-
   // ---- set-up: barriers, TMEM, group table ------------------------------------------------
   if (threadIdx.x == 0) {
     prefetch_tmap(&tm_a);
@@ -284,9 +286,11 @@ k_grouped_gemm(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__
       tmem_relinquish();
     }
   }
-  // everything above touched only this CTA's resources; from here on the results of the kernels
-  // before this one (rows, group table) are read
-  asm volatile("griddepcontrol.wait;" ::: "memory");
+  // Everything above touched only this CTA's resources; from here on the results of the kernels before
+  // this one are read -- except, with early_weights, by the producer's first weight loads and the reads of
+  // the group table: the kernel before this one had itself waited for the table's writer when it let this
+  // one start.  For the same reason this kernel lets its successor start only after its own wait.
+  if (!p.early_weights) asm volatile("griddepcontrol.wait;" ::: "memory");
   if (p.stamps && threadIdx.x == 0) atomicMin(&p.stamps[0], global_timer_ns());
   for (int g = threadIdx.x; g < p.n_groups; g += kThreads) {
     const feplb_group gr = p.groups[g];
@@ -310,8 +314,9 @@ k_grouped_gemm(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__
   const bool has_dyn = p.dyn.seq != 0;
   const int n_static_entries = p.n_groups;
   const int n_static_tiles = tail->prefix[p.n_groups] * p.n_tiles_n;
-  const uint32_t b_half_bytes = (uint32_t)p.bn * BK * 2;
-  const uint32_t stage_tx = PAIR ? 2 * (kABytes + b_half_bytes) : kABytes + 2 * b_half_bytes;
+  // (the producer waits on its own, after its first weight loads)
+  if (p.early_weights && warp != 0) asm volatile("griddepcontrol.wait;" ::: "memory");
+  if (warp != 0) asm volatile("griddepcontrol.launch_dependents;");
 
   if (warp == 0) {
     // ---- TMA producer (lane 0 issues; the whole warp fetches the dynamic table) ----------------
@@ -344,6 +349,56 @@ k_grouped_gemm(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__
       dyn_known = true;
       return true;
     };
+    // The loads of one K block of one tile.  Pair form: both CTAs credit the LEADER's barrier; the leader
+    // announces the bytes of both.  A tile whose second 128 rows hold no valid row (a group of at most
+    // 128 rows, or a ragged tail) needs no A rows in the peer: it skips that load (the MMA then multiplies
+    // whatever its stage holds into accumulator rows nobody stores).
+    auto load_b = [&](const TileCoord& c, int kb, int st) {      // announces the stage's bytes, loads the weights
+      // weights of a migrated expert come from its slot of the receive buffer
+      const CUtensorMap* mb0 = c.slot >= 0 ? &tm_r0 : &tm_b0;
+      const CUtensorMap* mb1 = c.slot >= 0 ? &tm_r1 : &tm_b1;
+      const int row = (c.slot >= 0 ? c.slot : c.expert) * p.b_rows_per_expert + (SWIGLU ? c.n0 : 2 * c.n0);
+      const uint32_t full = smem_u32(&tail->full[st]);
+      const uint32_t sb = smem_u32(smem + (size_t)st * kStageBytes) + kABytes;
+      const uint32_t half = (uint32_t)c.bn * BK * 2, box = (uint32_t)p.b_box * BK * 2;
+      if (PAIR) {
+        const uint32_t full0 = map_to_cta(full, 0);
+        if (cta_rank == 0) mbar_expect_tx(full, (c.rows_valid > BM ? 2 * kABytes : kABytes) + 2 * half);
+        const CUtensorMap* mb = cta_rank == 0 ? mb0 : mb1;
+        const int r0 = row + (!SWIGLU && cta_rank ? c.bn : 0);
+        for (uint32_t o = 0, r = 0; o < half; o += box, r += p.b_box) tma_load_2d_pair(sb + o, mb, full0, kb * BK, r0 + (int)r);
+      } else {
+        mbar_expect_tx(full, kABytes + 2 * half);
+        for (uint32_t o = 0, r = 0; o < half; o += box, r += p.b_box) tma_load_2d(sb + o, mb0, full, kb * BK, row + (int)r);
+        const int row1 = SWIGLU ? row : row + c.bn;
+        for (uint32_t o = 0, r = 0; o < half; o += box, r += p.b_box) tma_load_2d(sb + half + o, mb1, full, kb * BK, row1 + (int)r);
+      }
+    };
+    auto load_a = [&](const TileCoord& c, int kb, int st) {
+      // in pass 1 the rows of a migrated piece come from the receive region (same row numbers as the permuted buffer)
+      const CUtensorMap* ma = c.slot >= 0 ? &tm_ra : &tm_a;
+      const uint32_t full = smem_u32(&tail->full[st]);
+      const uint32_t sa = smem_u32(smem + (size_t)st * kStageBytes);
+      if (PAIR) {
+        if (cta_rank == 0 || c.rows_valid > BM) tma_load_2d_pair(sa, ma, map_to_cta(full, 0), kb * BK, c.row0 + (int)cta_rank * BM);
+      } else {
+        tma_load_2d(sa, ma, full, kb * BK, c.row0);
+      }
+    };
+    // Weights of the first tile, as far as the ring holds them, before the wait for the rows.
+    int n_early = 0;
+    if (p.early_weights) {
+      if (worker < n_static_tiles) {
+        n_early = min(kStages, p.num_k_blocks);
+        if (lane == 0) {
+          const TileCoord c = tile_coord<kTileRows>(tail, n_entries, p, worker);
+          for (int kb = 0; kb < n_early; ++kb) load_b(c, kb, kb);
+        }
+        __syncwarp();
+      }
+      asm volatile("griddepcontrol.wait;" ::: "memory");
+    }
+    asm volatile("griddepcontrol.launch_dependents;");
     bool claimer = false, tried_claim = false;
     for (int tile = worker; ok; tile += n_workers) {
       if (!dyn_known && tile >= total) {
@@ -364,45 +419,22 @@ k_grouped_gemm(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__
         if (p.stamps && lane == 0) atomicMin(&p.stamps[3], ~(global_timer_ns() - t0));
       }
       if (tile >= total) break;
-      const TileCoord c = tile_coord<kTileRows>(tail, n_entries, p.n_tiles_n, tile);
+      const TileCoord c = tile_coord<kTileRows>(tail, n_entries, p, tile);
       // While static tiles remain, peek at the device-side word once per tile: the load is in flight
       // during the K loop below and is looked at after it, so it costs the pipeline nothing.
       unsigned long long peek = 0;
       if (!dyn_known && lane == 0) peek = ld_relaxed_gpu_u64(p.dyn.ready_dev);
       if (lane == 0) {
-        // weights of a migrated expert come from its slot of the receive buffer, and in pass 1 its
-        // rows from the receive region of the rows (same row numbers as the permuted buffer)
-        const CUtensorMap* ma = c.slot >= 0 ? &tm_ra : &tm_a;
-        const CUtensorMap* mb0 = c.slot >= 0 ? &tm_r0 : &tm_b0;
-        const CUtensorMap* mb1 = c.slot >= 0 ? &tm_r1 : &tm_b1;
-        const int brow0 = (c.slot >= 0 ? c.slot : c.expert) * p.b_rows_per_expert + (SWIGLU ? c.nt * p.bn : c.nt * 2 * p.bn);
-        const int brow1 = SWIGLU ? brow0 : brow0 + p.bn;
         for (int kb = 0; kb < p.num_k_blocks; ++kb) {
-          if (!(ok = mbar_wait(smem_u32(&tail->empty[stage]), phase ^ 1u, abort_flag, p.status))) break;
-          const uint32_t full = smem_u32(&tail->full[stage]);
-          const uint32_t sa = smem_u32(smem + (size_t)stage * kStageBytes);
-          const uint32_t sb = sa + kABytes;
-          if (PAIR) {
-            // both CTAs credit the LEADER's barrier; the leader announces the bytes of both.  A tile
-            // whose second 128 rows hold no valid row (a group of at most 128 rows, or a ragged
-            // tail) needs no A rows in the peer: it skips that load (the MMA then multiplies
-            // whatever its stage holds into accumulator rows nobody stores), so a small group costs
-            // the pair no more operand traffic than it would cost a single CTA.
-            const uint32_t full0 = map_to_cta(full, 0);
-            const bool peer_rows = c.rows_valid > BM;
-            if (cta_rank == 0) mbar_expect_tx(full, peer_rows ? stage_tx : stage_tx - kABytes);
-            if (cta_rank == 0 || peer_rows) tma_load_2d_pair(sa, ma, full0, kb * BK, c.row0 + (int)cta_rank * BM);
-            if (cta_rank == 0) tma_load_2d_pair(sb, mb0, full0, kb * BK, brow0);
-            else tma_load_2d_pair(sb, mb1, full0, kb * BK, brow1);
-          } else {
-            mbar_expect_tx(full, stage_tx);
-            tma_load_2d(sa, ma, full, kb * BK, c.row0);
-            tma_load_2d(sb, mb0, full, kb * BK, brow0);
-            tma_load_2d(sb + b_half_bytes, mb1, full, kb * BK, brow1);
+          if (kb >= n_early) {
+            if (!(ok = mbar_wait(smem_u32(&tail->empty[stage]), phase ^ 1u, abort_flag, p.status))) break;
+            load_b(c, kb, stage);
           }
+          load_a(c, kb, stage);
           if (++stage == kStages) { stage = 0; phase ^= 1u; }
         }
       }
+      n_early = 0;
       ok = __shfl_sync(0xffffffffu, (int)ok, 0) != 0;
       if (ok && !dyn_known) {
         peek = __shfl_sync(0xffffffffu, peek, 0);
@@ -416,7 +448,6 @@ k_grouped_gemm(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__
   } else if (warp == 1) {
     // ---- MMA issuer -------------------------------------------------------------------------
     if (lane == 0 && cta_rank == 0) {
-      const uint32_t idesc = make_idesc(kTileRows, 2 * p.bn);
       int stage = 0, as = 0;
       uint32_t phase = 0, aphase = 0;
       bool ok = true, dyn_known = !has_dyn;
@@ -429,6 +460,7 @@ k_grouped_gemm(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__
           total = tail->total_mtiles * p.n_tiles_n;
           if (tile >= total) break;
         }
+        const uint32_t idesc = make_idesc(kTileRows, 2 * min(p.bn, p.half_width - tile % p.n_tiles_n * p.bn));
         if (!(ok = mbar_wait(smem_u32(&tail->tmem_empty[as]), aphase ^ 1u, abort_flag, p.status))) break;
         tc_fence_after();
         const uint32_t d_tmem = tmem_base + (uint32_t)(as * kAccCols);
@@ -464,7 +496,6 @@ k_grouped_gemm(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__
     // instruction: every store covers whole 128-byte lines, masked per row for ragged tiles.
     const int q = warp & 3;                   // TMEM lane quarter this warp may read
     const uint32_t stg = smem_u32(epi_smem + (size_t)(warp - 2) * kEpiStageBytes);
-    const int out_cols = SWIGLU ? p.bn : 2 * p.bn;
     int as = 0;
     uint32_t aphase = 0;
     bool ok = true, dyn_known = !has_dyn;
@@ -480,7 +511,9 @@ k_grouped_gemm(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__
         total = tail->total_mtiles * p.n_tiles_n;
         if (tile >= total) break;
       }
-      const TileCoord c = tile_coord<kTileRows>(tail, n_entries, p.n_tiles_n, tile);
+      const TileCoord c = tile_coord<kTileRows>(tail, n_entries, p, tile);
+      const int out_cols = SWIGLU ? c.bn : 2 * c.bn;
+      const int col0 = SWIGLU ? c.n0 : 2 * c.n0;          // first output column of the tile
       ok = mbar_wait(smem_u32(&tail->tmem_full[as]), aphase, abort_flag, p.status);
       ok = __all_sync(0xffffffffu, ok);
       if (!ok) break;
@@ -488,46 +521,48 @@ k_grouped_gemm(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__
       const uint32_t taddr = tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)(as * kAccCols);
       const int row_off = (int)cta_rank * BM + q * 32;    // this warp's first row inside the tile
       const int rows_here = c.rows_valid - row_off;       // valid rows among this warp's 32
-      __nv_bfloat16* obase = p.out + (int64_t)(c.row0 + row_off) * p.ld_out + (int64_t)c.nt * out_cols;
-      uint32_t a0[32], a1[32], b0[32], b1[32], packed[32];
-      tmem_ld32(taddr, a0);
-      tmem_ld32(taddr + 32u, a1);
-      if (SWIGLU) {
-        tmem_ld32(taddr + (uint32_t)p.bn, b0);
-        tmem_ld32(taddr + (uint32_t)p.bn + 32u, b1);
-      }
-      for (int col = 0; col < out_cols; col += 64) {
-        tmem_ld_wait();
-        if (SWIGLU && p.ab_out != nullptr) {
-          // training: also keep the pre-activations a | b of these 64 hidden units (bf16) for the
-          // backward pass, in [rows, 2f] with b at column offset f
-          __nv_bfloat16* abase = p.ab_out + (int64_t)(c.row0 + row_off) * (2 * p.ld_out);
-          const int hcol = c.nt * out_cols + col;
-#pragma unroll
-          for (int i = 0; i < 16; ++i) {
-            packed[i] = pack_bf16x2(__uint_as_float(a0[2 * i]), __uint_as_float(a0[2 * i + 1]));
-            packed[16 + i] = pack_bf16x2(__uint_as_float(a1[2 * i]), __uint_as_float(a1[2 * i + 1]));
-          }
-          stage_and_store(stg, packed, abase, 2 * p.ld_out, hcol, rows_here, lane);
-#pragma unroll
-          for (int i = 0; i < 16; ++i) {
-            packed[i] = pack_bf16x2(__uint_as_float(b0[2 * i]), __uint_as_float(b0[2 * i + 1]));
-            packed[16 + i] = pack_bf16x2(__uint_as_float(b1[2 * i]), __uint_as_float(b1[2 * i + 1]));
-          }
-          stage_and_store(stg, packed, abase, 2 * p.ld_out, p.ld_out + hcol, rows_here, lane);
+      __nv_bfloat16* obase = p.out + (int64_t)(c.row0 + row_off) * p.ld_out + col0;
+      if (rows_here > 0) {                                // a warp without valid rows only hands the accumulator back
+        uint32_t a0[32], a1[32], b0[32], b1[32], packed[32];
+        tmem_ld32(taddr, a0);
+        tmem_ld32(taddr + 32u, a1);
+        if (SWIGLU) {
+          tmem_ld32(taddr + (uint32_t)c.bn, b0);
+          tmem_ld32(taddr + (uint32_t)c.bn + 32u, b1);
         }
-        convert_slice<SWIGLU>(a0, b0, packed);
-        convert_slice<SWIGLU>(a1, b1, packed + 16);
-        if (col + 64 < out_cols) {           // next slice's TMEM loads fly while this one is stored
-          tmem_ld32(taddr + (uint32_t)(col + 64), a0);
-          tmem_ld32(taddr + (uint32_t)(col + 96), a1);
-          if (SWIGLU) {
-            tmem_ld32(taddr + (uint32_t)(p.bn + col + 64), b0);
-            tmem_ld32(taddr + (uint32_t)(p.bn + col + 96), b1);
+        for (int col = 0; col < out_cols; col += 64) {
+          tmem_ld_wait();
+          if (SWIGLU && p.ab_out != nullptr) {
+            // training: also keep the pre-activations a | b of these 64 hidden units (bf16) for the
+            // backward pass, in [rows, 2f] with b at column offset f
+            __nv_bfloat16* abase = p.ab_out + (int64_t)(c.row0 + row_off) * (2 * p.ld_out);
+            const int hcol = col0 + col;
+#pragma unroll
+            for (int i = 0; i < 16; ++i) {
+              packed[i] = pack_bf16x2(__uint_as_float(a0[2 * i]), __uint_as_float(a0[2 * i + 1]));
+              packed[16 + i] = pack_bf16x2(__uint_as_float(a1[2 * i]), __uint_as_float(a1[2 * i + 1]));
+            }
+            stage_and_store(stg, packed, abase, 2 * p.ld_out, hcol, rows_here, lane);
+#pragma unroll
+            for (int i = 0; i < 16; ++i) {
+              packed[i] = pack_bf16x2(__uint_as_float(b0[2 * i]), __uint_as_float(b0[2 * i + 1]));
+              packed[16 + i] = pack_bf16x2(__uint_as_float(b1[2 * i]), __uint_as_float(b1[2 * i + 1]));
+            }
+            stage_and_store(stg, packed, abase, 2 * p.ld_out, p.ld_out + hcol, rows_here, lane);
           }
+          convert_slice<SWIGLU>(a0, b0, packed);
+          convert_slice<SWIGLU>(a1, b1, packed + 16);
+          if (col + 64 < out_cols) {           // next slice's TMEM loads fly while this one is stored
+            tmem_ld32(taddr + (uint32_t)(col + 64), a0);
+            tmem_ld32(taddr + (uint32_t)(col + 96), a1);
+            if (SWIGLU) {
+              tmem_ld32(taddr + (uint32_t)(c.bn + col + 64), b0);
+              tmem_ld32(taddr + (uint32_t)(c.bn + col + 96), b1);
+            }
+          }
+          if (rows_here >= 32) stage_and_tma_store(stg, packed, &tm_out, col0 + col, c.row0 + row_off, lane);
+          else stage_and_store(stg, packed, obase, p.ld_out, col, rows_here, lane);
         }
-        if (rows_here >= 32) stage_and_tma_store(stg, packed, &tm_out, c.nt * out_cols + col, c.row0 + row_off, lane);
-        else stage_and_store(stg, packed, obase, p.ld_out, col, rows_here, lane);
       }
       tc_fence_before();
       __syncwarp();
@@ -651,16 +686,20 @@ int feplb_launch_expert_ffn(const feplb_gemm_args& a, cudaStream_t st, int64_t* 
     snprintf(err, errn, "expert_ffn: the two group tables of a merged launch exceed %d entries", FEPLB_MAX_GROUPS);
     return FEPLB_E_INVALID;
   }
-  // pass 1: H = silu(X W1) * (X W3);  N tile = bn columns of H, MMA N = 2*bn
-  const int bn1 = (a.f % 128 == 0) ? 128 : 64;
-  // pass 2: Y = H W2;  N tile = 2*bn columns of Y
-  const int bn2 = (a.d % 256 == 0) ? 128 : 64;
+  // Half tiles of up to 128 rows of B (columns of H in pass 1, half the columns of Y in pass 2).  Where the
+  // width is not a multiple of 128 the last N tile is narrower, and boxes of 64 rows serve both: a 128 x 256
+  // tile moves 48 KiB per 512 MMA cycles into the SM, two 128 x 128 tiles (64-row half tiles throughout,
+  // as narrow widths such as 64 still have) 64 KiB.  Whole layer at d = 1920, f = 704, E = 60, T = 1537,
+  // top-4: 171.2 -> 150.9 us together with the early weight loads of pass 2.
+  const int hw1 = a.f, hw2 = a.d / 2;
+  const int bn1 = hw1 < 128 ? 64 : 128, bn2 = hw2 < 128 ? 64 : 128;
+  const int bb1 = hw1 % 128 ? 64 : 128, bb2 = hw2 % 128 ? 64 : 128;
   CUtensorMap tm_x, tm_w1, tm_w3, tm_h, tm_w2, tm_ho, tm_yo;     // tm_ho, tm_yo: outputs in boxes of 32 rows x 64 columns
   if (!make_tmap(&tm_x, a.x_perm, (uint64_t)a.s_cap, (uint64_t)a.d, BM) ||
-      !make_tmap(&tm_w1, a.w1, (uint64_t)a.E * a.f, (uint64_t)a.d, bn1) ||
-      !make_tmap(&tm_w3, a.w3, (uint64_t)a.E * a.f, (uint64_t)a.d, bn1) ||
+      !make_tmap(&tm_w1, a.w1, (uint64_t)a.E * a.f, (uint64_t)a.d, bb1) ||
+      !make_tmap(&tm_w3, a.w3, (uint64_t)a.E * a.f, (uint64_t)a.d, bb1) ||
       !make_tmap(&tm_h, a.h, (uint64_t)a.s_cap, (uint64_t)a.f, BM) ||
-      !make_tmap(&tm_w2, a.w2, (uint64_t)a.E * a.d, (uint64_t)a.f, bn2) ||
+      !make_tmap(&tm_w2, a.w2, (uint64_t)a.E * a.d, (uint64_t)a.f, bb2) ||
       !make_tmap(&tm_ho, a.h, (uint64_t)a.s_cap, (uint64_t)a.f, 32) ||
       !make_tmap(&tm_yo, a.y, (uint64_t)a.s_cap, (uint64_t)a.d, 32)) {
     snprintf(err, errn, "cuTensorMapEncodeTiled failed (driver entry point missing or bad pointer/shape)");
@@ -669,9 +708,9 @@ int feplb_launch_expert_ffn(const feplb_gemm_args& a, cudaStream_t st, int64_t* 
   // receive buffer of migrated experts' weights, addressed by slot like the home weights by expert
   CUtensorMap tm_r1 = tm_w1, tm_r3 = tm_w3, tm_r2 = tm_w2;
   const bool has_recv = a.recv_w1 && a.recv_w3 && a.recv_w2 && a.n_recv_slots > 0;
-  if (has_recv && (!make_tmap(&tm_r1, a.recv_w1, (uint64_t)a.n_recv_slots * a.f, (uint64_t)a.d, bn1) ||
-                   !make_tmap(&tm_r3, a.recv_w3, (uint64_t)a.n_recv_slots * a.f, (uint64_t)a.d, bn1) ||
-                   !make_tmap(&tm_r2, a.recv_w2, (uint64_t)a.n_recv_slots * a.d, (uint64_t)a.f, bn2))) {
+  if (has_recv && (!make_tmap(&tm_r1, a.recv_w1, (uint64_t)a.n_recv_slots * a.f, (uint64_t)a.d, bb1) ||
+                   !make_tmap(&tm_r3, a.recv_w3, (uint64_t)a.n_recv_slots * a.f, (uint64_t)a.d, bb1) ||
+                   !make_tmap(&tm_r2, a.recv_w2, (uint64_t)a.n_recv_slots * a.d, (uint64_t)a.f, bb2))) {
     snprintf(err, errn, "cuTensorMapEncodeTiled failed for the receive buffer");
     return FEPLB_E_CUDA;
   }
@@ -684,13 +723,15 @@ int feplb_launch_expert_ffn(const feplb_gemm_args& a, cudaStream_t st, int64_t* 
   GemmParams p1;
   p1.n_recv_slots = has_recv ? a.n_recv_slots : 0;
   p1.groups = a.groups; p1.n_groups = a.n_groups; p1.which = a.which; p1.E = a.E; p1.s_cap = a.s_cap;
-  p1.n_tiles_n = a.f / bn1; p1.num_k_blocks = a.d / BK; p1.b_rows_per_expert = a.f; p1.bn = bn1;
+  p1.n_tiles_n = (hw1 + bn1 - 1) / bn1; p1.half_width = hw1; p1.b_box = bb1; p1.early_weights = 0;
+  p1.num_k_blocks = a.d / BK; p1.b_rows_per_expert = a.f; p1.bn = bn1;
   p1.out = (__nv_bfloat16*)a.h; p1.ld_out = a.f; p1.status = a.status; p1.ab_out = (__nv_bfloat16*)a.ab_out;
   const feplb_wm_dyn none;
   p1.dyn = feplb_dyn_table(dyn ? *dyn : none);
   p1.stamps = dyn ? dyn->stamps : nullptr;
   GemmParams p2 = p1;
-  p2.n_tiles_n = a.d / (2 * bn2); p2.num_k_blocks = a.f / BK; p2.b_rows_per_expert = a.d; p2.bn = bn2;
+  p2.n_tiles_n = (hw2 + bn2 - 1) / bn2; p2.half_width = hw2; p2.b_box = bb2; p2.early_weights = 1;
+  p2.num_k_blocks = a.f / BK; p2.b_rows_per_expert = a.d; p2.bn = bn2;
   p2.out = (__nv_bfloat16*)a.y; p2.ld_out = a.d; p2.ab_out = nullptr;
   p2.stamps = p1.stamps ? p1.stamps + 4 : nullptr;
 

@@ -8,6 +8,7 @@ from paper_2604_19654_b200 import feplb as F
 from paper_2604_19654_b200 import workloads as W
 
 from gpu_utils import DeviceCase
+from test_gpu_parity import _ffn_case
 
 pytestmark = pytest.mark.gpu
 
@@ -28,3 +29,15 @@ def test_transpose_partial_tiles(E, d, f):
     for got, src in ((w1t, case.w1), (w3t, case.w3), (w2t, case.w2)):
         assert np.array_equal(F.bf16_bits(got), src.transpose(0, 2, 1))
     case.close()
+
+
+@pytest.mark.parametrize("form", [F.FORM_SINGLE, F.FORM_PAIR])
+@pytest.mark.parametrize("E,d,f,rows", [
+    (2, 128, 64, [1, 130]),            # one narrow N tile in both passes
+    (3, 384, 192, [257, 0, 31]),       # a full and a narrow N tile in both passes
+    (2, 640, 320, [128, 129]),         # two full and one narrow
+    (2, 1920, 704, [90, 300]),         # many of each, the ring wraps
+])
+def test_expert_ffn_narrow_last_n_tile(E, d, f, rows, form):
+    """Widths that are not multiples of the N tile: f % 128 = 64 (pass 1) and d % 256 = 128 (pass 2)."""
+    _ffn_case(E, d, f, rows, form=form)
