@@ -777,10 +777,17 @@ extern "C" int feplb_moe_forward(feplb_ctx* c, const void* x, const int32_t* top
   }
   c->flag_seq = c->flag_seq == INT32_MAX ? 1 : c->flag_seq + 1;
   const int32_t seq = c->flag_seq;
-  CUDA_TRY(c, feplb_launch_route_fused(topk_ids, S, g.E, g.R, g.row_align, g.dyn, mask_dev, c->d_block_hist, counts,
-                                       rank_load, c->d_pad_off, c->d_home_groups, nullptr, slot_to_row, row_to_token,
-                                       (int64_t)c->s_cap, c->d_status, c->h_counts_tagged, seq,
-                                       stamps ? stamps + 8 : nullptr, st, &c->launches));
+  const bool small_front = feplb_front_is_small(S, g.E);
+  if (small_front)
+    CUDA_TRY(c, feplb_launch_front_small(x, topk_ids, g.T, g.K, g.E, g.R, g.d, g.row_align, g.dyn, mask_dev, counts, rank_load,
+                                         c->d_pad_off, c->d_home_groups, slot_to_row, row_to_token, x_perm, (int64_t)c->s_cap,
+                                         c->d_status, c->h_counts_tagged, seq, stamps ? stamps + 8 : nullptr, c->num_sms, st,
+                                         &c->launches));
+  else
+    CUDA_TRY(c, feplb_launch_route_fused(topk_ids, S, g.E, g.R, g.row_align, g.dyn, mask_dev, c->d_block_hist, counts,
+                                         rank_load, c->d_pad_off, c->d_home_groups, nullptr, slot_to_row, row_to_token,
+                                         (int64_t)c->s_cap, c->d_status, c->h_counts_tagged, seq,
+                                         stamps ? stamps + 8 : nullptr, st, &c->launches));
   c->job_w1 = w1; c->job_w3 = w3; c->job_w2 = w2;   // read by the planner thread after it is woken
   c->job_x_perm = x_perm;
   if ((rc = plan_kick_flag(c, dyn_mask_host, seq, wm)) != FEPLB_OK) return rc;
@@ -789,9 +796,10 @@ extern "C" int feplb_moe_forward(feplb_ctx* c, const void* x, const int32_t* top
   // step 3: permutation (does not depend on the plan: a migration relabels rows, it does not move
   // them here).  From here on a failure must still join the planner, so errors are carried in rc.
   {
-    cudaError_t e = feplb_launch_gather(x, topk_ids, c->d_block_hist, slot_to_row, counts, c->d_pad_off, x_perm, g.T, g.K,
-                                        g.E, g.d, g.row_align, (int64_t)c->s_cap, c->num_sms, st, &c->launches,
-                                        row_to_token, true);
+    cudaError_t e = cudaSuccess;
+    if (!small_front)
+      e = feplb_launch_gather(x, topk_ids, c->d_block_hist, slot_to_row, counts, c->d_pad_off, x_perm, g.T, g.K, g.E, g.d,
+                              g.row_align, (int64_t)c->s_cap, c->num_sms, st, &c->launches, row_to_token, true);
     if (e == cudaSuccess && g.phase2_copy) {
       // the planner's row copies of Phase 2 wait for the permuted rows
       e = cudaEventRecord(c->ev_gather, st);

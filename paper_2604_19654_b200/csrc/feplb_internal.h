@@ -10,6 +10,7 @@
 #define FEPLB_MAX_EXPERTS 1024
 #define FEPLB_MAX_GROUPS 1024
 #define FEPLB_SLOTS_PER_BLOCK 1024   // slots ranked by one CTA of the permutation kernels
+#define FEPLB_FRONT_SMALL_SLOTS 8192 // most slots of a batch whose routing and gather run as one launch
 #define FEPLB_TILE_M 128             // rows of one GEMM tile
 #ifndef FEPLB_NOALLOC_MAX_HIST_INTS
 #error "feplb.h must define FEPLB_NOALLOC_MAX_HIST_INTS"
@@ -53,6 +54,13 @@ cudaError_t feplb_launch_route_fused(const int32_t* ids, int64_t S, int E, int R
                                      int32_t* slot_to_row, int32_t* row_to_token, int64_t s_cap, uint32_t* status,
                                      unsigned long long* counts_host_tagged, int32_t seq, unsigned long long* t_counts,
                                      cudaStream_t st, int64_t* n_launch);
+// Small batches: feplb_launch_route_fused and feplb_launch_gather in one launch.
+bool feplb_front_is_small(int64_t S, int E);
+cudaError_t feplb_launch_front_small(const void* x, const int32_t* ids, int T, int K, int E, int R, int d, int A, int dyn,
+                                     const uint8_t* mask_in, int32_t* counts, int32_t* rank_load, int32_t* pad_off,
+                                     feplb_group* groups, int32_t* slot_to_row, int32_t* row_to_token, void* x_perm,
+                                     int64_t s_cap, uint32_t* status, unsigned long long* counts_host_tagged, int32_t seq,
+                                     unsigned long long* t_counts, int num_sms, cudaStream_t st, int64_t* n_launch);
 cudaError_t feplb_launch_upload_groups(const feplb_group* src_host_mapped, feplb_group* dst, int n, cudaStream_t st);
 cudaError_t feplb_launch_home_groups(const int32_t* counts, const uint8_t* mask_in, int E, int R, int A, int dyn,
                                      feplb_group* groups, uint8_t* mask_out, cudaStream_t st, int64_t* n_launch);

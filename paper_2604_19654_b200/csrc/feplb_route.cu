@@ -326,6 +326,156 @@ k_gather(const uint4* __restrict__ x, const int32_t* __restrict__ ids, const int
   }
 }
 
+// The whole front of a layer pass for small batches -- histogram, ranks, scan, home group table and row gather --
+// as ONE launch.  Chained, the three kernels it replaces take 11 us of launch and memory latency whatever the
+// size; here every CTA computes the complete routing of the batch for itself (at most kSmallMaxSlots ids, read
+// from L2; the ranks end up in shared memory), so that no CTA needs another one's result, and then copies
+// its share of the rows.  CTA 0 alone publishes the tables.  The redundant part grows with the number of slots
+// and ends the range: see feplb_front_is_small.
+// Whole layer, chained front -> this: 32.3 -> 27.9 us at T = 256, top-2, d = 128, 8 experts; 102.0 -> 97.9 us at
+// T = 64, top-6, d = 2048, 64 experts.
+constexpr int kSmallThreads = 1024;
+constexpr int kSmallWarps = kSmallThreads / 32;
+constexpr int kSmallSlice = 64;              // 16-byte chunks of a row per work unit (2 per lane)
+
+template <int CH>                            // chunks of 32 slots per warp
+__global__ void __launch_bounds__(kSmallThreads, 1)
+k_route_small(const uint4* __restrict__ x, const int32_t* __restrict__ ids, int T, int K, int E, int L, int A, int dyn,
+              const uint8_t* __restrict__ mask_in, int32_t* __restrict__ counts_out, int32_t* __restrict__ rank_load_out,
+              int32_t* __restrict__ pad_off_out, feplb_group* __restrict__ groups, int32_t* __restrict__ slot_to_row,
+              int32_t* __restrict__ row_to_token, uint4* __restrict__ x_perm, int chunks, int64_t s_cap, uint32_t* status,
+              unsigned long long* __restrict__ counts_host_tagged, int32_t seq, unsigned long long* t_counts) {
+  extern __shared__ int sm[];
+  __shared__ int tmp[64];
+  int* wh = sm;                              // [kSmallWarps][E] histograms per warp, then ranks of a warp's first slots
+  int* sc = wh + kSmallWarps * E;            // [E] counts
+  int* pad = sc + E;                         // [E] first row of the segment
+  int* rows = pad + E;                       // [32 * 32 * CH] row of every slot, -1 for an id outside [0, E)
+  const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int S = T * K;
+  for (int i = threadIdx.x; i < kSmallWarps * E; i += kSmallThreads) wh[i] = 0;
+  __syncthreads();
+  pdl_sync();
+  // the first work unit's row piece and this warp's ids, all in flight together
+  const int slices = (chunks + kSmallSlice - 1) / kSmallSlice;
+  const int units = T * slices;
+  int u = blockIdx.x + gridDim.x * w;
+  uint4 v[2];
+  auto load_unit = [&](int unit) {
+    const int t = unit / slices, c0 = (unit - t * slices) * kSmallSlice;
+#pragma unroll
+    for (int i = 0; i < 2; ++i)
+      if (c0 + i * 32 + lane < chunks) v[i] = ld_nc_v4(x + (int64_t)t * chunks + c0 + i * 32 + lane);
+  };
+  int id[CH];
+#pragma unroll
+  for (int c = 0; c < CH; ++c) {
+    const int s = (w * CH + c) * 32 + lane;
+    id[c] = s < S ? ids[s] : -1;
+  }
+  if (u < units) load_unit(u);
+  unsigned mk[CH];
+  bool bad = false;
+#pragma unroll
+  for (int c = 0; c < CH; ++c) {
+    if ((unsigned)id[c] >= (unsigned)E) {
+      bad |= (w * CH + c) * 32 + lane < S;
+      id[c] = -1;
+    }
+    mk[c] = __match_any_sync(0xffffffffu, id[c]);
+    if (id[c] >= 0 && lane == __ffs(mk[c]) - 1) wh[w * E + id[c]] += __popc(mk[c]);
+    __syncwarp();
+  }
+  if (bad && blockIdx.x == 0) atomicOr(status, FEPLB_ST_RANGE);
+  __syncthreads();
+  const int e = threadIdx.x;
+  int cnt = 0;
+  if (e < E) {
+#pragma unroll
+    for (int i = 0; i < kSmallWarps; ++i) {
+      const int n = wh[i * E + e];
+      wh[i * E + e] = cnt;
+      cnt += n;
+    }
+    sc[e] = cnt;
+    if (blockIdx.x == 0) {
+      counts_out[e] = cnt;
+      if (counts_host_tagged)                // see k_scan_fused
+        *reinterpret_cast<volatile unsigned long long*>(counts_host_tagged + e) =
+            ((unsigned long long)(uint32_t)seq << 32) | (uint32_t)cnt;
+    }
+  }
+  if (blockIdx.x == 0 && e == 0 && t_counts) {
+    unsigned long long t;
+    asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
+    *t_counts = t;
+  }
+  int total;
+  const int off = block_exclusive_scan((cnt + A - 1) / A * A, tmp, &total);      // also orders sc[] and wh[] for all threads
+  if (e < E) pad[e] = off;
+  __syncthreads();
+  const unsigned lt = (1u << lane) - 1u;
+#pragma unroll
+  for (int c = 0; c < CH; ++c) {
+    int r = -1;
+    if (id[c] >= 0) r = pad[id[c]] + wh[w * E + id[c]] + __popc(mk[c] & lt);
+    __syncwarp();
+    if (id[c] >= 0 && lane == __ffs(mk[c]) - 1) wh[w * E + id[c]] += __popc(mk[c]);
+    __syncwarp();
+    rows[(w * CH + c) * 32 + lane] = r;
+  }
+  __syncthreads();
+  for (; u < units; u += gridDim.x * kSmallWarps) {
+    const int t = u / slices, c0 = (u - t * slices) * kSmallSlice;
+    if (c0 == 0 && lane < K) {
+      const int row = rows[t * K + lane];
+      slot_to_row[t * K + lane] = row;
+      if (row >= 0) row_to_token[row] = t;
+    }
+    for (int k = 0; k < K; ++k) {
+      const int row = rows[t * K + k];
+      if (row < 0) continue;
+      uint4* dst = x_perm + (int64_t)row * chunks + c0 + lane;
+      if (c0 + lane < chunks) dst[0] = v[0];
+      if (c0 + 32 + lane < chunks) dst[32] = v[1];
+    }
+    if (u + gridDim.x * kSmallWarps < units) load_unit(u + gridDim.x * kSmallWarps);
+  }
+  if (blockIdx.x == 0) {
+    if (e < E) {
+      pad_off_out[e] = off;
+      int is_dyn;
+      if (mask_in) {
+        is_dyn = mask_in[e] != 0;
+      } else {
+        const int b0 = e / L * L;
+        int better = 0;
+        for (int o = b0; o < b0 + L; ++o) better += (sc[o] > cnt) || (sc[o] == cnt && o < e);
+        is_dyn = better < dyn;
+      }
+      groups[e] = feplb_group{e, off, cnt, e / L, is_dyn};
+    }
+    if (e == 0) pad_off_out[E] = total;
+    if (e < E / L) {
+      int sum = 0;
+      for (int o = e * L; o < (e + 1) * L; ++o) sum += sc[o];
+      rank_load_out[e] = sum;
+    }
+  }
+  for (int64_t i = (int64_t)total + (int64_t)blockIdx.x * kSmallThreads + threadIdx.x; i < s_cap;
+       i += (int64_t)gridDim.x * kSmallThreads)
+    row_to_token[i] = -1;
+  if (A > 1) {                               // padding rows at the end of the segments
+    for (int g = blockIdx.x; g < E; g += gridDim.x) {
+      const int r0 = pad[g] + sc[g], r1 = pad[g] + (sc[g] + A - 1) / A * A;
+      for (int r = r0 + (int)threadIdx.x; r < r1; r += kSmallThreads) row_to_token[r] = -1;
+      uint4* p = x_perm + (int64_t)r0 * chunks;
+      const int64_t n = (int64_t)(r1 - r0) * chunks;
+      for (int64_t i = threadIdx.x; i < n; i += kSmallThreads) p[i] = make_uint4(0, 0, 0, 0);
+    }
+  }
+}
+
 // Zero the padding rows at the end of every expert's segment (row_align > 1 only).
 __global__ void __launch_bounds__(kThreads)
 k_zero_pad(const int32_t* __restrict__ counts, const int32_t* __restrict__ pad_off, uint4* __restrict__ x_perm,
@@ -519,6 +669,54 @@ cudaError_t feplb_launch_route_fused(const int32_t* ids, int64_t S, int E, int R
   ++*n_launch;
   return launch(k_scan_fused, 1, 1024, 0, st, true, block_hist, nb, E, E / R, A, dyn, mask_in, counts, rank_load, pad_off,
                 groups, mask_out, row_to_token, s_cap, counts_host_tagged, seq, t_counts);
+}
+
+// The one-launch front pays while the routing that every CTA repeats is short: its eight match rounds at 8192
+// slots take as long as the two launches it saves (T = 1537, top-4, d = 1920: 155.9 us per layer either way).
+constexpr int kSmallMaxSlots = FEPLB_FRONT_SMALL_SLOTS, kSmallMaxExperts = 256;
+bool feplb_front_is_small(int64_t S, int E) { return S > 0 && S <= kSmallMaxSlots && E <= kSmallMaxExperts; }
+
+template <int CH>
+static cudaError_t launch_small(const void* x, const int32_t* ids, int T, int K, int E, int R, int d, int A, int dyn,
+                                const uint8_t* mask_in, int32_t* counts, int32_t* rank_load, int32_t* pad_off, feplb_group* groups,
+                                int32_t* slot_to_row, int32_t* row_to_token, void* x_perm, int64_t s_cap, uint32_t* status,
+                                unsigned long long* counts_host_tagged, int32_t seq, unsigned long long* t_counts, int num_sms,
+                                cudaStream_t st) {
+  static bool ready[64] = {};                // per instantiation and device: the shared-memory attribute
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
+  if (!ready[dev]) {
+    const int most = (int)sizeof(int) * ((kSmallWarps + 2) * kSmallMaxExperts + kSmallThreads * CH);
+    cudaError_t e = cudaFuncSetAttribute(k_route_small<CH>, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
+    if (e != cudaSuccess) return e;
+    ready[dev] = true;
+  }
+  const int chunks = d / 8;
+  const int64_t units = (int64_t)T * ((chunks + kSmallSlice - 1) / kSmallSlice);
+  const int64_t want = A > 1 && units < E ? E : units;       // padding rows are zeroed one expert per CTA
+  const int grid = (int)(want < num_sms ? want : num_sms);
+  const size_t smem = sizeof(int) * ((size_t)(kSmallWarps + 2) * E + (size_t)kSmallThreads * CH);
+  return launch(k_route_small<CH>, grid, kSmallThreads, smem, st, true, (const uint4*)x, ids, T, K, E, E / R, A, dyn, mask_in,
+                counts, rank_load, pad_off, groups, slot_to_row, row_to_token, (uint4*)x_perm, chunks, s_cap, status,
+                counts_host_tagged, seq, t_counts);
+}
+
+cudaError_t feplb_launch_front_small(const void* x, const int32_t* ids, int T, int K, int E, int R, int d, int A, int dyn,
+                                     const uint8_t* mask_in, int32_t* counts, int32_t* rank_load, int32_t* pad_off,
+                                     feplb_group* groups, int32_t* slot_to_row, int32_t* row_to_token, void* x_perm,
+                                     int64_t s_cap, uint32_t* status, unsigned long long* counts_host_tagged, int32_t seq,
+                                     unsigned long long* t_counts, int num_sms, cudaStream_t st, int64_t* n_launch) {
+  const int S = T * K;
+  auto go = [&](auto fn) {
+    return fn(x, ids, T, K, E, R, d, A, dyn, mask_in, counts, rank_load, pad_off, groups, slot_to_row, row_to_token, x_perm,
+              s_cap, status, counts_host_tagged, seq, t_counts, num_sms, st);
+  };
+  ++*n_launch;
+  if (S <= kSmallThreads) return go(launch_small<1>);
+  if (S <= kSmallThreads * 2) return go(launch_small<2>);
+  if (S <= kSmallThreads * 4) return go(launch_small<4>);
+  static_assert(kSmallMaxSlots == kSmallThreads * 8, "slots of the largest instantiation");
+  return go(launch_small<8>);
 }
 
 cudaError_t feplb_launch_route_topk(const float* logits, int T, int E, int K, int32_t* ids, float* gates,
