@@ -47,6 +47,8 @@ struct feplb_ctx {
   bool merged_ok = false;      // both group tables of a forward fit one launch (static, then dynamic groups)
   bool merged = false;         // ... and feplb_moe_forward runs that way: two GEMM launches instead of four
   bool merged_auto = false;
+  bool direct = false;         // no launch of a forward depends on the plan: both passes walk the home table (small batches)
+  bool direct_auto = false;
   bool merged_pair = false;    // form of the merged launches when none is forced
   int32_t planner_delay_us = 0;        // test aid: the planner sleeps before it publishes its table
   int32_t device_wait_limit_us = 0;    // bound of the GEMM's wait for the table (0: default)
@@ -127,6 +129,7 @@ struct feplb_ctx {
   std::vector<feplb_group> groups;
   std::vector<int64_t> load_before, load_after;
   std::vector<uint8_t> mask;
+  std::vector<int64_t> score;
   feplb_plan_out plan;
 };
 
@@ -149,6 +152,52 @@ int fail(feplb_ctx* c, int code, const char* fmt, ...) {
 
 bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; }
 
+// Bounded wait for the counts of job `seq`: either the front of the layer pass writes them straight into pinned
+// host memory, each tagged with the forward's sequence number (whole-layer path), or (seq = 0) a copy was
+// enqueued and its event is polled (stand-alone feplb_plan_async); no blocking driver call either way.
+int await_counts(feplb_ctx* c, int32_t seq) {
+  int rc = FEPLB_OK;
+  const auto w0 = clk::now();
+  for (uint32_t spin = 0;; ++spin) {
+    if (seq) {
+      int e = 0;
+      for (; e < c->cfg.E; ++e) {
+        const unsigned long long v = *(volatile unsigned long long*)(c->h_counts_tagged + e);
+        if ((int32_t)(v >> 32) != seq) break;
+        c->h_counts[e] = (int32_t)(uint32_t)v;
+      }
+      if (e == c->cfg.E) break;
+    } else {
+      cudaError_t q = cudaEventQuery(c->ev_counts);
+      if (q == cudaSuccess) break;
+      if (q != cudaErrorNotReady) { rc = FEPLB_E_CUDA; break; }
+    }
+    if ((spin & 1023u) == 1023u && std::chrono::duration<double>(clk::now() - w0).count() > 1e-3 * c->planner_timeout_ms) { rc = FEPLB_E_TIMEOUT; break; }
+#if defined(__x86_64__) || defined(__i386__)
+    __builtin_ia32_pause();     // a polite spin: the sibling hyper-thread (another rank's host thread) keeps its issue slots
+#endif
+  }
+  std::atomic_thread_fence(std::memory_order_acquire);
+  c->tl.host_counts_ready_us = us_since(c->t0);
+  return rc;
+}
+
+// Mask (given, or derived from the counts) and plan of the counts in h_counts.
+int make_plan(feplb_ctx* c, const uint8_t* mask) {
+  const feplb_config& cfg = c->cfg;
+  if (!mask) {
+    for (int e = 0; e < cfg.E; ++e) c->score[e] = c->h_counts[e];
+    feplb_select_dynamic(c->score.data(), cfg.E, cfg.R, cfg.dyn, c->mask.data());
+  } else {
+    memcpy(c->mask.data(), mask, cfg.E);
+  }
+  const auto p0 = clk::now();
+  const int rc = feplb_plan(&cfg, c->h_counts, c->mask.data(), &c->plan);
+  c->tl.plan_us = us_since(p0);
+  c->tl.host_plan_done_us = us_since(c->t0);
+  return rc;
+}
+
 // The planner thread: waits for the counts, derives mask and plan, uploads the dynamic groups.
 void planner_main(feplb_ctx* c) {
   cudaSetDevice(c->device);
@@ -159,47 +208,10 @@ void planner_main(feplb_ctx* c) {
       if (c->quit) return;
       c->job = JOB_RUNNING;
     }
-    int rc = FEPLB_OK;
-    // bounded wait for the counts: either the scan kernel writes them straight into pinned host
-    // memory, each tagged with the forward's sequence number (whole-layer path), or a copy was enqueued and its event is
-    // polled (stand-alone feplb_plan_async); no blocking driver call either way
-    const auto w0 = clk::now();
-    for (uint32_t spin = 0;; ++spin) {
-      if (c->job_flag_seq) {
-        int e = 0;
-        for (; e < c->cfg.E; ++e) {
-          const unsigned long long v = *(volatile unsigned long long*)(c->h_counts_tagged + e);
-          if ((int32_t)(v >> 32) != c->job_flag_seq) break;
-          c->h_counts[e] = (int32_t)(uint32_t)v;
-        }
-        if (e == c->cfg.E) break;
-      } else {
-        cudaError_t q = cudaEventQuery(c->ev_counts);
-        if (q == cudaSuccess) break;
-        if (q != cudaErrorNotReady) { rc = FEPLB_E_CUDA; break; }
-      }
-      if ((spin & 1023u) == 1023u && std::chrono::duration<double>(clk::now() - w0).count() > 1e-3 * c->planner_timeout_ms) { rc = FEPLB_E_TIMEOUT; break; }
-#if defined(__x86_64__) || defined(__i386__)
-      __builtin_ia32_pause();     // a polite spin: the sibling hyper-thread (another rank's host thread) keeps its issue slots
-#endif
-    }
-    std::atomic_thread_fence(std::memory_order_acquire);
-    c->tl.host_counts_ready_us = us_since(c->t0);
+    int rc = await_counts(c, c->job_flag_seq);
     if (rc == FEPLB_OK) {
       const feplb_config& cfg = c->cfg;
-      const uint8_t* mask = c->job_mask;
-      if (!mask) {
-        std::vector<int64_t> score(cfg.E);
-        for (int e = 0; e < cfg.E; ++e) score[e] = c->h_counts[e];
-        feplb_select_dynamic(score.data(), cfg.E, cfg.R, cfg.dyn, c->mask.data());
-        mask = c->mask.data();
-      } else {
-        memcpy(c->mask.data(), mask, cfg.E);
-      }
-      const auto p0 = clk::now();
-      rc = feplb_plan(&cfg, c->h_counts, mask, &c->plan);
-      c->tl.plan_us = us_since(p0);
-      c->tl.host_plan_done_us = us_since(c->t0);
+      rc = make_plan(c, c->job_mask);
       if (rc == FEPLB_OK) {
         int n = 0;
         for (int i = 0; i < c->plan.n_groups; ++i)
@@ -368,6 +380,17 @@ extern "C" int feplb_create(const feplb_config* cfg, feplb_ctx** out) {
   // do not (from ~1000 rows per expert).
   c->merged_ok = cfg->E + cap_groups <= FEPLB_MAX_GROUPS;
   c->merged_auto = c->merged = c->merged_ok && S < (int64_t)FEPLB_WM_AUTO_ROWS_PER_EXPERT * cfg->E;
+  // Small batches: a migration only relabels the rank that executes rows whose weights are the same everywhere, so
+  // the launches need not wait for the plan at all.  They do where the static groups keep the GPU busy for longer
+  // than the planner takes (its table is then there in time); below that the wait and the table's way to the
+  // device cost up to 10 us per forward, and the plan (returned as ever) is made by the calling thread
+  // instead.  Whole layer, table order -> this: 27.9 -> 19.6 us (T = 256, top-2, d = 128, 8 experts), 30.8 ->
+  // 20.3 (the same at T = 1200), 97.9 -> 88.7 (T = 64, top-6, d = 2048, 64 experts), 156.7 -> 148.9 (102 rows
+  // per expert, d = 1920).  At 384 rows per expert of d = 2048 (325 us by the estimate) the gain would be 3 %,
+  // at 1024 of d = 6144 the order that gives the static groups launches of their own is 4 % ahead.
+  // The time is an estimate: all weights streamed at 6.5 TB/s plus the products at 1 PFLOP/s.
+  const double ffn_us = 6.0 * cfg->d * cfg->f * ((double)cfg->E / 6.5e6 + (double)S / 1e9);
+  c->direct_auto = c->direct = S < (int64_t)FEPLB_DIRECT_ROWS_PER_EXPERT * cfg->E || ffn_us < FEPLB_DIRECT_FFN_US;
   bool ok = true;
   ok = ok && cudaMalloc(&c->d_dyn_ready, 2 * sizeof(unsigned long long)) == cudaSuccess &&     // [0] ready word, [1] claim word
        cudaMemset(c->d_dyn_ready, 0, 2 * sizeof(unsigned long long)) == cudaSuccess;
@@ -426,6 +449,7 @@ extern "C" int feplb_create(const feplb_config* cfg, feplb_ctx** out) {
   c->load_before.resize(cfg->R);
   c->load_after.resize(cfg->R);
   c->mask.resize(cfg->E);
+  c->score.resize(cfg->E);
   c->plan = feplb_plan_out{0, 0, cap_moves, cap_groups, c->moves.data(), c->groups.data(),
                            c->load_before.data(), c->load_after.data()};
   memset(&c->tl, 0, sizeof(c->tl));
@@ -635,6 +659,21 @@ static int plan_kick_flag(feplb_ctx* c, const uint8_t* dyn_mask_host, int32_t se
   return FEPLB_OK;
 }
 
+// The context's plan -> the caller's arrays (NULL: not wanted).
+static int copy_plan(feplb_ctx* c, feplb_plan_out* plan_copy) {
+  if (!plan_copy) return FEPLB_OK;
+  if (plan_copy->cap_moves < c->plan.n_moves || plan_copy->cap_groups < c->plan.n_groups ||
+      !plan_copy->load_before || !plan_copy->load_after)
+    return fail(c, FEPLB_E_NOMEM, "plan_wait: plan_copy too small");
+  plan_copy->n_moves = c->plan.n_moves;
+  plan_copy->n_groups = c->plan.n_groups;
+  if (c->plan.n_moves) memcpy(plan_copy->moves, c->plan.moves, sizeof(feplb_move) * c->plan.n_moves);
+  if (c->plan.n_groups) memcpy(plan_copy->groups, c->plan.groups, sizeof(feplb_group) * c->plan.n_groups);
+  memcpy(plan_copy->load_before, c->plan.load_before, sizeof(int64_t) * c->cfg.R);
+  memcpy(plan_copy->load_after, c->plan.load_after, sizeof(int64_t) * c->cfg.R);
+  return FEPLB_OK;
+}
+
 // Waits for the planner's job and returns the context to idle; copies the plan out.
 static int join_planner(feplb_ctx* c, int32_t timeout_ms, feplb_plan_out* plan_copy) {
   int rc;
@@ -647,17 +686,7 @@ static int join_planner(feplb_ctx* c, int32_t timeout_ms, feplb_plan_out* plan_c
     c->job = JOB_IDLE;
   }
   if (rc != FEPLB_OK) return fail(c, rc, "planner failed: %s", feplb_strerror(rc));
-  if (plan_copy) {
-    if (plan_copy->cap_moves < c->plan.n_moves || plan_copy->cap_groups < c->plan.n_groups ||
-        !plan_copy->load_before || !plan_copy->load_after)
-      return fail(c, FEPLB_E_NOMEM, "plan_wait: plan_copy too small");
-    plan_copy->n_moves = c->plan.n_moves;
-    plan_copy->n_groups = c->plan.n_groups;
-    if (c->plan.n_moves) memcpy(plan_copy->moves, c->plan.moves, sizeof(feplb_move) * c->plan.n_moves);
-    if (c->plan.n_groups) memcpy(plan_copy->groups, c->plan.groups, sizeof(feplb_group) * c->plan.n_groups);
-    memcpy(plan_copy->load_before, c->plan.load_before, sizeof(int64_t) * c->cfg.R);
-    memcpy(plan_copy->load_after, c->plan.load_after, sizeof(int64_t) * c->cfg.R);
-  }
+  if ((rc = copy_plan(c, plan_copy)) != FEPLB_OK) return rc;
   if (c->n_dyn_groups > 0 && !c->job_wm) ++c->launches;     // the planner thread's table upload kernel
   return FEPLB_OK;
 }
@@ -752,7 +781,9 @@ extern "C" int feplb_moe_forward(feplb_ctx* c, const void* x, const int32_t* top
   // Not with Phase-2 weight copies: the dynamic groups would then wait, inside a kernel that holds
   // every SM, for device-to-device copies that the driver may carry out with kernels of its own;
   // that case keeps the four-launch order (the dynamic launches follow the copies in stream order).
-  const bool wm = c->merged && !g.phase2_copy;
+  // (the test aids of feplb_set_planner_timing are about the table a launch waits for: they keep that order)
+  const bool direct = c->direct && !g.phase2_copy && !c->planner_delay_us && !c->device_wait_limit_us;
+  const bool wm = direct || (c->merged && !g.phase2_copy);
   c->tl.ffn_launches = wm ? 2 : 4;
   c->tl.dev_ffn_pass1_us = c->tl.dev_ffn_pass2_us = c->tl.dev_plan_wait_us = 0;
   unsigned long long* stamps = nullptr;
@@ -775,6 +806,10 @@ extern "C" int feplb_moe_forward(feplb_ctx* c, const void* x, const int32_t* top
     CUDA_TRY(c, cudaMemcpyAsync(c->d_mask, c->h_mask, g.E, cudaMemcpyHostToDevice, st));
     mask_dev = c->d_mask;
   }
+  if (direct) {
+    std::lock_guard<std::mutex> lk(c->mu);
+    if (c->job != JOB_IDLE) return fail(c, FEPLB_E_STATE, "moe_forward: a plan is already pending");
+  }
   c->flag_seq = c->flag_seq == INT32_MAX ? 1 : c->flag_seq + 1;
   const int32_t seq = c->flag_seq;
   const bool small_front = feplb_front_is_small(S, g.E);
@@ -790,7 +825,7 @@ extern "C" int feplb_moe_forward(feplb_ctx* c, const void* x, const int32_t* top
                                          stamps ? stamps + 8 : nullptr, st, &c->launches));
   c->job_w1 = w1; c->job_w3 = w3; c->job_w2 = w2;   // read by the planner thread after it is woken
   c->job_x_perm = x_perm;
-  if ((rc = plan_kick_flag(c, dyn_mask_host, seq, wm)) != FEPLB_OK) return rc;
+  if (!direct && (rc = plan_kick_flag(c, dyn_mask_host, seq, wm)) != FEPLB_OK) return rc;
   TL_EVENT(EV_COUNTS);
   TL_EVENT(EV_HIST);
   // step 3: permutation (does not depend on the plan: a migration relabels rows, it does not move
@@ -816,10 +851,10 @@ extern "C" int feplb_moe_forward(feplb_ctx* c, const void* x, const int32_t* top
     dyn.table_dev = c->d_dyn_tab32; dyn.table_host = c->h_dyn_tab32_dev;
     dyn.ready_dev = c->d_dyn_ready; dyn.ready_host = c->h_dyn_ready_dev;
     dyn.claim = reinterpret_cast<uint32_t*>(c->d_dyn_ready + 1);
-    dyn.seq = (uint32_t)seq; dyn.max_groups = c->plan.cap_groups; dyn.stamps = stamps;
+    dyn.seq = direct ? 0u : (uint32_t)seq; dyn.max_groups = direct ? 0 : c->plan.cap_groups; dyn.stamps = stamps;
     dyn.wait_limit_ns = 1000ull * (unsigned long long)c->device_wait_limit_us;
     if (rc == FEPLB_OK)
-      rc = ffn_impl(c, x_perm, w1, w3, w2, c->d_home_groups, g.E, FEPLB_FFN_STATIC, h_scratch, y_perm, st,
+      rc = ffn_impl(c, x_perm, w1, w3, w2, c->d_home_groups, g.E, direct ? FEPLB_FFN_ALL : FEPLB_FFN_STATIC, h_scratch, y_perm, st,
                     c->gemm_pair_forced >= 0 ? c->gemm_pair_forced : (int)c->merged_pair, &dyn);
     TL_EVENT(EV_STATIC1);          // both launches lie between EV_STATIC0 and here; no events of their own for the dynamic part
     c->tl.host_enqueue_static_done_us = us_since(c->t0);
@@ -832,8 +867,18 @@ extern "C" int feplb_moe_forward(feplb_ctx* c, const void* x, const int32_t* top
       if (e == cudaSuccess) e = cudaEventRecord(c->ev[EV_STAMPS], st);
       if (e != cudaSuccess) rc_comb = fail(c, FEPLB_E_CUDA, "timeline records: %s", cudaGetErrorString(e));
     }
-    // join the planner (always, so that the context returns to idle): everything is already enqueued
-    int rc_join = join_planner(c, c->planner_timeout_ms + 500, plan_copy);
+    // Everything is enqueued.  Join the planner (always, so that the context returns to idle); where no launch needs
+    // the plan it is made right here, which spares waking the planner thread and being woken by it.
+    int rc_join;
+    if (direct) {
+      rc_join = await_counts(c, seq);
+      if (rc_join == FEPLB_OK) rc_join = make_plan(c, dyn_mask_host);
+      if (rc_join != FEPLB_OK) rc_join = fail(c, rc_join, "planner failed: %s", feplb_strerror(rc_join));
+      else rc_join = copy_plan(c, plan_copy);
+      c->tl.host_upload_enqueued_us = us_since(c->t0);
+    } else {
+      rc_join = join_planner(c, c->planner_timeout_ms + 500, plan_copy);
+    }
     c->tl.host_join_us = us_since(c->t0);
     if (rc != FEPLB_OK) return rc;
     if (rc_comb != FEPLB_OK) return rc_comb;
@@ -1017,6 +1062,7 @@ extern "C" int feplb_set_launch_merging(feplb_ctx* c, int32_t merged) {
   std::lock_guard<std::mutex> lk(c->mu);
   if (c->job != JOB_IDLE) return fail(c, FEPLB_E_STATE, "set_launch_merging: a plan is pending");
   c->merged = merged < 0 ? c->merged_auto : merged != 0;
+  c->direct = merged < 0 && c->direct_auto;
   return FEPLB_OK;
 }
 

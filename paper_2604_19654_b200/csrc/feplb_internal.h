@@ -23,6 +23,9 @@
 #define FEPLB_ST_GROUP 8u      // a group entry was malformed (expert or rows out of range)
 #define FEPLB_ST_PLAN 16u      // the GEMM's bounded wait for the planner's dynamic group table gave up
 #define FEPLB_WM_AUTO_ROWS_PER_EXPERT 768   // the weights-on-M form is the default below this many rows per expert
+// No launch of a forward waits for the plan below this many rows per expert, or where the expert FFN takes less than this long
+#define FEPLB_DIRECT_ROWS_PER_EXPERT 128
+#define FEPLB_DIRECT_FFN_US 150
 #define FEPLB_WM_MAX_ENTRIES 1024    // group entries (static + dynamic table) one weights-on-M launch can hold
 
 int feplb_validate_config(const feplb_config* c);
