@@ -1,4 +1,5 @@
-"""Builds libfeplb.so (C ABI + sm_100a kernels) in-tree with nvcc.
+"""Builds libfeplb.so (C ABI + sm_100a kernels) in-tree with nvcc, and with g++ the CPython module the binding
+makes its per-micro-batch calls through.
 
 ``python -m paper_2604_19654_b200.build [--force] [-v] [--nvcc-flag=FLAG ...]`` or ``build()``;
 nvcc cross-compiles without a GPU.  ``-v`` prints ptxas resource usage; ``--nvcc-flag`` appends one
@@ -11,11 +12,13 @@ import os
 import shutil
 import subprocess
 import sys
+import sysconfig
 
 HERE = os.path.dirname(os.path.abspath(__file__))
 ROOT = os.path.dirname(HERE)
 CSRC = os.path.join(HERE, "csrc")
 LIB = os.path.join(HERE, "libfeplb.so")
+PY_LIB = os.path.join(HERE, "_feplb_py.so")
 SOURCES = ["feplb_plan.cpp", "feplb_api.cu", "feplb_route.cu", "feplb_combine.cu", "feplb_gemm.cu",
            "feplb_noalloc.cu", "feplb_gemm_bwd.cu", "feplb_gemm_wm.cu"]
 
@@ -28,11 +31,24 @@ def _nvcc() -> str:
 
 
 def needs_build() -> bool:
-    if not os.path.exists(LIB):
+    if not os.path.exists(LIB) or not os.path.exists(PY_LIB):
         return True
-    t = os.path.getmtime(LIB)
+    t = min(os.path.getmtime(LIB), os.path.getmtime(PY_LIB))
     deps = [os.path.join(CSRC, f) for f in os.listdir(CSRC)] + [os.path.join(ROOT, "include", "feplb.h")]
     return any(os.path.getmtime(p) > t for p in deps)
+
+
+def _run(cmd, target: str, verbose: bool):
+    """Runs a compiler that writes `target`.<pid>.tmp and renames the result into place."""
+    tmp = f"{target}.{os.getpid()}.tmp"
+    r = subprocess.run(cmd, capture_output=True, text=True)
+    if verbose or r.returncode:
+        sys.stderr.write(r.stdout + r.stderr)
+    if r.returncode:
+        if os.path.exists(tmp):
+            os.remove(tmp)
+        raise RuntimeError(f"building {os.path.basename(target)} failed")
+    os.replace(tmp, target)
 
 
 def build(force: bool = False, verbose: bool = False, extra_flags=()) -> str:
@@ -46,6 +62,9 @@ def build(force: bool = False, verbose: bool = False, extra_flags=()) -> str:
         try:
             if not force and not needs_build():
                 return LIB
+            _run([shutil.which("g++") or "g++", "-shared", "-fPIC", "-O2", "-std=c++17", "-I", sysconfig.get_paths()["include"],
+                  "-I", os.path.join(ROOT, "include"), "-o", f"{PY_LIB}.{os.getpid()}.tmp", os.path.join(CSRC, "feplb_py.cpp"),
+                  "-ldl"], PY_LIB, verbose)
             tmp = f"{LIB}.{os.getpid()}.tmp"
             cmd = [_nvcc(), "-shared", "-O3", "-std=c++17", "-lineinfo",
                    "-gencode", "arch=compute_100a,code=sm_100a",
@@ -55,14 +74,7 @@ def build(force: bool = False, verbose: bool = False, extra_flags=()) -> str:
             cmd[1:1] = list(extra_flags)
             if verbose:
                 cmd.insert(1, "-Xptxas=-v")
-            r = subprocess.run(cmd, capture_output=True, text=True)
-            if verbose or r.returncode:
-                sys.stderr.write(r.stdout + r.stderr)
-            if r.returncode:
-                if os.path.exists(tmp):
-                    os.remove(tmp)
-                raise RuntimeError("nvcc failed building libfeplb.so")
-            os.replace(tmp, LIB)
+            _run(cmd, LIB, verbose)
             return LIB
         finally:
             fcntl.flock(lock, fcntl.LOCK_UN)

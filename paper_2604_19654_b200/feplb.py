@@ -1,4 +1,5 @@
-"""Thin ctypes binding over the C ABI of ``libfeplb.so`` (see ``include/feplb.h``).
+"""Thin binding over the C ABI of ``libfeplb.so`` (see ``include/feplb.h``): ctypes, and for the calls a program
+makes per micro-batch a small CPython module (``csrc/feplb_py.cpp``).
 
 Argument marshalling only: every step of the path runs in the library's CUDA kernels (or, for
 the plan, in its C++ host code).  PyTorch supplies device memory and streams.  If the library is
@@ -7,6 +8,7 @@ missing the import of a symbol fails loudly -- there is no fallback.
 from __future__ import annotations
 
 import ctypes as C
+import importlib.util
 import os
 from typing import Optional, Sequence
 
@@ -14,6 +16,7 @@ import numpy as np
 
 _HERE = os.path.dirname(os.path.abspath(__file__))
 LIB_PATH = os.path.join(_HERE, "libfeplb.so")
+PY_LIB_PATH = os.path.join(_HERE, "_feplb_py.so")
 
 OK, E_INVALID, E_RANGE, E_CUDA, E_NOMEM, E_TIMEOUT, E_STATE, E_DEVICE = 0, -1, -2, -3, -4, -5, -6, -7
 POLICY_LITERAL, POLICY_FIRST_FIT = 0, 1
@@ -126,6 +129,22 @@ def lib() -> C.CDLL:
             fn.restype, fn.argtypes = res, args
         _lib = L
     return _lib
+
+
+_fast_mod = None
+
+
+def _fast():
+    """The CPython module of the per-micro-batch calls, bound to the same library as lib() (once)."""
+    global _fast_mod
+    if _fast_mod is None:
+        lib()
+        spec = importlib.util.spec_from_file_location("_feplb_py", PY_LIB_PATH)
+        mod = importlib.util.module_from_spec(spec)
+        spec.loader.exec_module(mod)
+        mod.load(LIB_PATH)
+        _fast_mod = mod
+    return _fast_mod
 
 
 def make_config(T, K, E, R, d, f, dyn=4, max_num_dyn=8, tau=0, ranks_per_domain=0,
@@ -278,6 +297,13 @@ def groups_to_numpy(groups) -> np.ndarray:
     return np.ascontiguousarray(a)
 
 
+def _current_stream() -> Optional[int]:
+    """Handle of torch's current stream on the current device (the raw getter takes a tenth of the time of a Stream object)."""
+    import torch
+    raw = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+    return (raw(torch.cuda.current_device()) if raw else torch.cuda.current_stream().cuda_stream) or None
+
+
 class Context:
     """One layer geometry on the current CUDA device.  Calls on one context must not overlap."""
 
@@ -287,6 +313,7 @@ class Context:
         rc = lib().feplb_create(C.byref(cfg), C.byref(self._h))
         if rc:
             raise FeplbError(rc, "feplb_create")
+        self._fast = _fast()
         self.s_cap = s_pad(cfg)
 
     def close(self):
@@ -307,24 +334,21 @@ class Context:
     @staticmethod
     def _stream(stream) -> Optional[int]:
         if stream is None:
-            import torch
-            return torch.cuda.current_stream().cuda_stream or None
+            return _current_stream()
         return getattr(stream, "cuda_stream", stream) or None
 
     def check_status(self, stream=None):
         self._chk(lib().feplb_check_status(self._h, self._stream(stream)), "feplb_check_status")
 
     def route_topk(self, logits, topk_ids, gates, stream=None):
-        self._chk(lib().feplb_route_topk(self._h, _ptr(logits), _ptr(topk_ids), _ptr(gates), self._stream(stream)),
-                  "feplb_route_topk")
+        self._chk(self._fast.route_topk(self._h.value, logits, topk_ids, gates, self._stream(stream)), "feplb_route_topk")
 
     def route_hist(self, topk_ids, counts, rank_load, stream=None):
-        self._chk(lib().feplb_route_hist(self._h, _ptr(topk_ids), _ptr(counts), _ptr(rank_load),
-                                         self._stream(stream)), "feplb_route_hist")
+        self._chk(self._fast.route_hist(self._h.value, topk_ids, counts, rank_load, self._stream(stream)), "feplb_route_hist")
 
     def dispatch(self, x, topk_ids, counts, x_perm, slot_to_row, row_to_token, stream=None):
-        self._chk(lib().feplb_dispatch(self._h, _ptr(x), _ptr(topk_ids), _ptr(counts), _ptr(x_perm),
-                                       _ptr(slot_to_row), _ptr(row_to_token), self._stream(stream)), "feplb_dispatch")
+        self._chk(self._fast.dispatch(self._h.value, x, topk_ids, counts, x_perm, slot_to_row, row_to_token,
+                                      self._stream(stream)), "feplb_dispatch")
 
     def home_groups(self, counts, dyn_mask, groups_out, dyn_mask_out=None, stream=None):
         self._chk(lib().feplb_home_groups(self._h, _ptr(counts), _ptr(dyn_mask), _ptr(groups_out),
@@ -336,8 +360,7 @@ class Context:
                                          self._stream(stream)), "feplb_expert_ffn")
 
     def combine(self, y_perm, slot_to_row, gates, out, stream=None):
-        self._chk(lib().feplb_combine(self._h, _ptr(y_perm), _ptr(slot_to_row), _ptr(gates), _ptr(out),
-                                      self._stream(stream)), "feplb_combine")
+        self._chk(self._fast.combine(self._h.value, y_perm, slot_to_row, gates, out, self._stream(stream)), "feplb_combine")
 
     def plan_async(self, counts, dyn_mask_host=None, stream=None):
         self._mask_keepalive = None if dyn_mask_host is None else np.ascontiguousarray(dyn_mask_host, np.uint8)
@@ -357,11 +380,9 @@ class Context:
         """``buf``: object with counts, rank_load, x_perm, h_scratch, y_perm, slot_to_row, row_to_token, out."""
         p = Plan(self.cfg) if want_plan else None
         mask = None if dyn_mask_host is None else np.ascontiguousarray(dyn_mask_host, np.uint8)
-        self._chk(lib().feplb_moe_forward(
-            self._h, _ptr(x), _ptr(topk_ids), _ptr(gates), _ptr(w1), _ptr(w3), _ptr(w2), _ptr(mask),
-            _ptr(buf.counts), _ptr(buf.rank_load), _ptr(buf.x_perm), _ptr(buf.h_scratch), _ptr(buf.y_perm),
-            _ptr(buf.slot_to_row), _ptr(buf.row_to_token), _ptr(buf.out),
-            C.byref(p.c) if p is not None else None, self._stream(stream)), "feplb_moe_forward")
+        self._chk(self._fast.moe_forward(
+            self._h.value, x, topk_ids, gates, w1, w3, w2, _ptr(mask), buf, C.addressof(p.c) if p is not None else None,
+            self._stream(stream)), "feplb_moe_forward")
         return p
 
     def moe_forward_host(self, x_host, ids_host, gates_host, x_dev, ids_dev, gates_dev, w1, w3, w2, buf, out_host,
@@ -435,11 +456,8 @@ class Context:
     def moe_backward(self, d_out, gates, w1t, w3t, w2t, buf, bwd, dw1=None, dw3=None, dw2=None, accumulate=False,
                      stream=None):
         """``buf``: the forward's Buffers; ``bwd``: a BackwardBuffers (ab, d_y_perm, d_ab, d_x_perm, d_x, d_gates)."""
-        self._chk(lib().feplb_moe_backward(
-            self._h, _ptr(d_out), _ptr(gates), _ptr(w1t), _ptr(w3t), _ptr(w2t), _ptr(buf.x_perm), _ptr(bwd.ab),
-            _ptr(buf.h_scratch), _ptr(buf.y_perm), _ptr(buf.slot_to_row), _ptr(bwd.d_y_perm),
-            _ptr(bwd.d_ab), _ptr(bwd.d_x_perm), _ptr(bwd.d_x), _ptr(bwd.d_gates), _ptr(dw1),
-            _ptr(dw3), _ptr(dw2), int(bool(accumulate)), self._stream(stream)), "feplb_moe_backward")
+        self._chk(self._fast.moe_backward(self._h.value, d_out, gates, w1t, w3t, w2t, buf, bwd, dw1, dw3, dw2,
+                                          int(bool(accumulate)), self._stream(stream)), "feplb_moe_backward")
 
     def set_gemm_form(self, forward_form: int = FORM_AUTO, backward_pair: int = -1):
         """Forces the grouped-GEMM form (FORM_*) of the forward launches and the pair mask of the backward GEMMs."""

@@ -8,7 +8,7 @@ from paper_2604_19654_b200 import feplb as F
 from paper_2604_19654_b200 import workloads as W
 
 from gpu_utils import DeviceCase
-from test_gpu_parity import _ffn_case
+from test_gpu_parity import _check_forward, _ffn_case
 
 pytestmark = pytest.mark.gpu
 
@@ -41,3 +41,58 @@ def test_transpose_partial_tiles(E, d, f):
 def test_expert_ffn_narrow_last_n_tile(E, d, f, rows, form):
     """Widths that are not multiples of the N tile: f % 128 = 64 (pass 1) and d % 256 = 128 (pass 2)."""
     _ffn_case(E, d, f, rows, form=form)
+
+
+@pytest.mark.parametrize("T,K,E,R,A", [
+    (1, 1, 2, 1, 1),              # one slot
+    (13, 7, 24, 3, 128),          # padding rows written by CTAs without rows of their own
+    (1024, 1, 8, 2, 1),           # one chunk of 32 slots per warp, full
+    (1025, 1, 256, 4, 1),         # two chunks; the most experts
+    (2731, 3, 16, 2, 128),        # 8193 slots: the three-launch front
+    (2730, 3, 16, 2, 128),        # 8190: the last one-launch front
+    (300, 32, 64, 4, 1),          # largest top-k, 9600 slots
+    (250, 32, 64, 4, 1),          # ... and 8000
+    (100, 2, 257, 1, 1),          # more experts than the one-launch front takes
+])
+def test_forward_front_range(T, K, E, R, A):
+    """Routing and gather of small batches in one launch, and the sizes next to its range."""
+    w = W.get_workload("cfg1").with_(T=T, K=K, E=E, R=R, d=128, f=64, tau=1, max_num_dyn=2)
+    case = DeviceCase(w, row_align=A)
+    _check_forward(case, sample=None if T < 300 else 100)
+    case.close()
+
+
+def test_forward_front_skips_ids_out_of_range():
+    """A slot with an expert id outside [0, E) gets row -1 and contributes nothing; the rest is routed as without it."""
+    import torch
+    w = W.get_workload("cfg1").with_(T=70, d=128, f=64)
+    case = DeviceCase(w)
+    ids = case.ids.copy()
+    ids[3, 0], ids[69, 1] = w.E, -5
+    case.ctx.moe_forward(case.d_x, torch.from_numpy(ids).cuda(), case.d_gates, case.d_w1, case.d_w3, case.d_w2, case.buf)
+    with pytest.raises(F.FeplbError) as ei:
+        case.ctx.check_status()
+    assert ei.value.code == F.E_RANGE
+    flat = ids.ravel()
+    valid = (flat >= 0) & (flat < w.E)
+    rows = np.full(flat.size, -1)
+    rows[np.flatnonzero(valid)[np.argsort(flat[valid], kind="stable")]] = np.arange(valid.sum())
+    assert np.array_equal(case.buf.slot_to_row.cpu().numpy().ravel(), rows)
+    assert np.array_equal(case.buf.counts.cpu().numpy(), np.bincount(flat[valid], minlength=w.E))
+    assert np.all(case.buf.row_to_token.cpu().numpy()[valid.sum():] == -1)
+    case.close()
+
+
+def test_forward_orders_agree():
+    """The order without a wait for the plan and the two orders that run the planner's table: the same integers and,
+    row for row, the same products."""
+    w = W.get_workload("cfg2").with_(T=300, d=256, f=128)
+    case = DeviceCase(w)
+    got = []
+    for merged in (-1, 1, 0):
+        case.ctx.set_launch_merging(merged)
+        p, _ = _check_forward(case)
+        got.append((p.moves, F.bf16_bits(case.buf.out).copy()))
+    assert got[0][0] == got[1][0] == got[2][0] and len(got[0][0]) > 0
+    assert np.array_equal(got[0][1], got[1][1]) and np.array_equal(got[0][1], got[2][1])
+    case.close()
