@@ -10,7 +10,6 @@
 namespace {
 
 constexpr int kThreads = 256;
-constexpr int kBatch = 8;   // rows loaded before they are accumulated
 
 __device__ __forceinline__ uint4 ld_nc_v4(const uint4* p) {
   uint4 v;
@@ -30,9 +29,16 @@ __device__ __forceinline__ uint32_t pack_bf16x2(float lo, float hi) {
   return *reinterpret_cast<uint32_t*>(&h);
 }
 
-// Work unit = (token, 32-chunk slice of its row) = 512 output bytes; the units are dealt out in
-// equal contiguous ranges to all warps of a grid sized to the machine, so that no tail wave forms.
-__global__ void __launch_bounds__(kThreads, 3)
+// Work unit = (token, 32-chunk slice of its row) = 512 output bytes.  Unit u goes to warp u mod #warps of a grid sized
+// to the machine: the warps work on neighbouring tokens at any time, whose rows in an expert's segment follow
+// one another, so that DRAM pages are read while they are open (see k_gather for the measurement).
+// kBatch rows are loaded before they are accumulated: the smallest even number that takes all K, at most 8 (more
+// rows go through in several batches); what it leaves of the registers goes into further CTAs.  Always 8 rows
+// and 3 CTAs: route + gather + combine at T = 9000, top-4, d = 1920 97.1 us, this way 88.7; at T = 60000,
+// top-2, d = 128 93.7 and 84.1.
+constexpr int ctas_per_sm(int batch) { return batch <= 2 ? 6 : batch <= 4 ? 5 : 3; }
+template <int kBatch>
+__global__ void __launch_bounds__(kThreads, ctas_per_sm(kBatch))
 k_combine(const uint4* __restrict__ y_perm, const int32_t* __restrict__ slot_to_row,
           const float* __restrict__ gates, uint4* __restrict__ out, int T, int K, int chunks, int next_may_start) {
   // launched with programmatic stream serialization: CTAs may become resident while the expert
@@ -47,20 +53,14 @@ k_combine(const uint4* __restrict__ y_perm, const int32_t* __restrict__ slot_to_
   const int64_t nwarps = ((int64_t)gridDim.x * kThreads) >> 5;
   const int slices = (chunks + 31) / 32;
   const int64_t units = (int64_t)T * slices;
-  const int64_t u0 = units * warp / nwarps, u1 = units * (warp + 1) / nwarps;
-  int cur_t = -1, myrow = -1;
-  float myg = 0.f;
-  for (int64_t u = u0; u < u1; ++u) {
-    const int t = (int)(u / slices);
-    const int c = (int)(u - (int64_t)t * slices) * 32 + lane;
-    if (t != cur_t) {            // warp-uniform
-      cur_t = t;
-      myrow = -1;
-      myg = 0.f;
-      if (lane < K) {
-        myrow = slot_to_row[(int64_t)t * K + lane];
-        myg = gates ? gates[(int64_t)t * K + lane] : 1.f;   // no gates: plain sum (backward of the dispatch)
-      }
+  for (int64_t u = warp; u < units; u += nwarps) {
+    const int64_t t = u / slices;
+    const int c = (int)(u - t * slices) * 32 + lane;
+    int myrow = -1;
+    float myg = 0.f;
+    if (lane < K) {
+      myrow = slot_to_row[t * K + lane];
+      myg = gates ? gates[t * K + lane] : 1.f;   // no gates: plain sum (backward of the dispatch)
     }
     const bool on = c < chunks;
     float acc[8];
@@ -94,7 +94,7 @@ k_combine(const uint4* __restrict__ y_perm, const int32_t* __restrict__ slot_to_
       o.y = pack_bf16x2(acc[2], acc[3]);
       o.z = pack_bf16x2(acc[4], acc[5]);
       o.w = pack_bf16x2(acc[6], acc[7]);
-      out[(int64_t)t * chunks + c] = o;
+      out[t * chunks + c] = o;
     }
   }
 }
@@ -104,9 +104,9 @@ k_combine(const uint4* __restrict__ y_perm, const int32_t* __restrict__ slot_to_
 cudaError_t feplb_launch_combine(const void* y_perm, const int32_t* slot_to_row, const float* gates, void* out,
                                  int T, int K, int d, int num_sms, cudaStream_t st, int64_t* n_launch) {
   if (T == 0) return cudaSuccess;
-  // a grid that fills every SM exactly once at 3 CTAs per SM (fewer CTAs if there is less work)
   const int64_t units = (int64_t)T * ((d / 8 + 31) / 32);
-  int blocks = num_sms * 3;
+  const int batch = K <= 2 ? 2 : K <= 4 ? 4 : K <= 6 ? 6 : 8;
+  int blocks = num_sms * ctas_per_sm(batch);   // every SM filled once (fewer CTAs if there is less work)
   const int64_t need = (units + kThreads / 32 - 1) / (kThreads / 32);
   if (need < blocks) blocks = (int)need;
   cudaLaunchConfig_t cfg = {};
@@ -119,6 +119,7 @@ cudaError_t feplb_launch_combine(const void* y_perm, const int32_t* slot_to_row,
   cfg.attrs = at;
   cfg.numAttrs = 1;
   ++*n_launch;
-  return cudaLaunchKernelEx(&cfg, k_combine, (const uint4*)y_perm, slot_to_row, gates, (uint4*)out, T, K, d / 8,
+  auto kernel = batch == 2 ? k_combine<2> : batch == 4 ? k_combine<4> : batch == 6 ? k_combine<6> : k_combine<8>;
+  return cudaLaunchKernelEx(&cfg, kernel, (const uint4*)y_perm, slot_to_row, gates, (uint4*)out, T, K, d / 8,
                             (int)((int64_t)T * K <= FEPLB_FRONT_SMALL_SLOTS));
 }

@@ -269,8 +269,12 @@ __device__ __forceinline__ uint4 ld_nc_v4(const uint4* p) {
 // slot_to_row and row_to_token entries.  Another warp working on a later slice of the same token may
 // read either form of the entry, and gets the same row from both.
 constexpr int kGatherUnroll = 4;
-// Work unit = (token, slice of 4 x 32 chunks = 2 KiB of its row); equal contiguous ranges of units
-// per warp over a grid sized to the machine, so that no tail wave forms.
+// Work unit = (token, slice of 4 x 32 chunks = 2 KiB of its row).  Unit u goes to warp u mod #warps of a grid
+// sized to the machine: all warps work on neighbouring tokens at any time, and the rows of an expert, which
+// follow the token order, are written in one moving window per expert, so that DRAM pages are written while
+// they are open.  With a contiguous range of units per warp (every warp in a place of its own) the gather and
+// the combine together, T = 8192, top-8, d = 6144, ran at 5.5 TB/s; this way at 6.0 (route + gather +
+// combine 353 -> 330 us).  Slices of 1 KiB: 347 us, of 4 KiB: the same.
 __global__ void __launch_bounds__(kThreads)
 k_gather(const uint4* __restrict__ x, const int32_t* __restrict__ ids, const int32_t* __restrict__ pad_off,
          const int32_t* __restrict__ block_base, int32_t* slot_to_row, int32_t* __restrict__ row_to_token,
@@ -281,9 +285,7 @@ k_gather(const uint4* __restrict__ x, const int32_t* __restrict__ ids, const int
   const int64_t nwarps = ((int64_t)gridDim.x * kThreads) >> 5;
   const int slices = (chunks + 32 * kGatherUnroll - 1) / (32 * kGatherUnroll);
   const int64_t units = (int64_t)T * slices;
-  const int64_t u0 = units * warp / nwarps, u1 = units * (warp + 1) / nwarps;
-  int cur_t = -1, myrow = -1;
-  for (int64_t u = u0; u < u1; ++u) {
+  for (int64_t u = warp; u < units; u += nwarps) {
     const int t = (int)(u / slices);
     const int c0 = (int)(u - (int64_t)t * slices) * 32 * kGatherUnroll;
     const uint4* src = x + (int64_t)t * chunks;
@@ -293,24 +295,21 @@ k_gather(const uint4* __restrict__ x, const int32_t* __restrict__ ids, const int
       const int c = c0 + i * 32 + lane;
       if (c < chunks) v[i] = ld_nc_v4(src + c);
     }
-    if (t != cur_t) {            // warp-uniform
-      cur_t = t;
-      myrow = -1;
-      if (lane < K) {
-        const int64_t s = (int64_t)t * K + lane;
-        const int r = __ldcg(slot_to_row + s);
-        const int e = ids[s];    // in flight together with r; its offsets follow in one more round trip
-        if (r >= 0) {
-          myrow = r;             // already final
-        } else if (r <= -2) {    // implies 0 <= e < E (checked by k_block_hist)
-          const int64_t row = (int64_t)pad_off[e] + block_base[s / FEPLB_SLOTS_PER_BLOCK * E + e] + (-2 - r);
-          // rows beyond the buffer: only with counts that disagree with the ids (reported by the scan)
-          myrow = row < s_cap ? (int)row : -1;
-        }
-        if (c0 == 0) {           // the token's first slice: this warp publishes the rows
-          slot_to_row[s] = myrow;
-          if (myrow >= 0) row_to_token[myrow] = t;
-        }
+    int myrow = -1;
+    if (lane < K) {
+      const int64_t s = (int64_t)t * K + lane;
+      const int r = __ldcg(slot_to_row + s);
+      const int e = ids[s];      // in flight together with r; its offsets follow in one more round trip
+      if (r >= 0) {
+        myrow = r;               // already final
+      } else if (r <= -2) {      // implies 0 <= e < E (checked by k_block_hist)
+        const int64_t row = (int64_t)pad_off[e] + block_base[s / FEPLB_SLOTS_PER_BLOCK * E + e] + (-2 - r);
+        // rows beyond the buffer: only with counts that disagree with the ids (reported by the scan)
+        myrow = row < s_cap ? (int)row : -1;
+      }
+      if (c0 == 0) {             // the token's first slice: this warp publishes the rows
+        slot_to_row[s] = myrow;
+        if (myrow >= 0) row_to_token[myrow] = t;
       }
     }
     for (int k = 0; k < K; ++k) {

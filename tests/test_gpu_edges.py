@@ -3,6 +3,7 @@ range, each against the oracle or an exact reordering of the input."""
 import numpy as np
 import pytest
 
+from oracle import feplb_oracle as O
 from paper_2604_19654_b200 import build as B
 from paper_2604_19654_b200 import feplb as F
 from paper_2604_19654_b200 import workloads as W
@@ -96,3 +97,23 @@ def test_forward_orders_agree():
     assert got[0][0] == got[1][0] == got[2][0] and len(got[0][0]) > 0
     assert np.array_equal(got[0][1], got[1][1]) and np.array_equal(got[0][1], got[2][1])
     case.close()
+
+
+@pytest.mark.parametrize("K", [1, 2, 3, 4, 5, 6, 7, 8, 9, 17])
+def test_combine_every_batch_size(K):
+    """Top-k around the row batches of the combine (2, 4, 6, 8 rows, then several batches of 8), a ragged last slice."""
+    import torch
+    T, d = 77, 640
+    rng = np.random.default_rng(K)
+    ctx = F.Context(F.make_config(T, K, 32, 1, d, 64))
+    y = W.f32_to_bf16_bits(rng.standard_normal((T * K, d)).astype(np.float32))
+    s2r = rng.permutation(T * K).astype(np.int32).reshape(T, K)
+    gates = rng.random((T, K)).astype(np.float32)
+    out = torch.zeros(T, d, dtype=torch.bfloat16, device="cuda")
+    ctx.combine(F.bf16_tensor(y), torch.from_numpy(s2r).cuda(), torch.from_numpy(gates).cuda(), out)
+    ref = O.combine(W.bf16_bits_to_f64(y), s2r, gates)
+    mag = O.combine(np.abs(W.bf16_bits_to_f64(y)), s2r, gates)
+    got = W.bf16_bits_to_f64(F.bf16_bits(out))
+    # one bf16 rounding (2^-9 relative) and K fp32 additions (K * 2^-24 of the sum of magnitudes)
+    assert np.all(np.abs(got - ref) <= 2.0 ** -8 * np.abs(ref) + 2.0 ** -19 * mag)
+    ctx.close()
