@@ -117,3 +117,8 @@ def test_combine_every_batch_size(K):
     # one bf16 rounding (2^-9 relative) and K fp32 additions (K * 2^-24 of the sum of magnitudes)
     assert np.all(np.abs(got - ref) <= 2.0 ** -8 * np.abs(ref) + 2.0 ** -19 * mag)
     ctx.close()
+
+
+def test_expert_ffn_few_rows():
+    """Groups around the 32 rows below which a tile loads a smaller box of A."""
+    _ffn_case(6, 256, 128, [31, 32, 33, 1, 160, 161], form=F.FORM_SINGLE)      # 160 = 128 + 32, 161 = 128 + 33
