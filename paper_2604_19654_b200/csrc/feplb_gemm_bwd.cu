@@ -713,6 +713,13 @@ bool make_tmap_out(CUtensorMap* m, float* base, uint64_t E, uint64_t M, uint64_t
             CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_NONE, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
+// Rows of a B half tile for an output n columns wide: the N tile of 2 * 128 or 2 * 64 columns that brings fewer operand
+// bytes into the SMs; the last tile may overhang (its surplus columns are computed and not stored).  A row of
+// 256-column tiles moves 128 + 256 operand rows per tile, one of 128-column tiles 128 + 128.  Forward and backward
+// at d = 1920, f = 704, 60 experts, T = 4096, top-4: 1033 us with 128 columns unless 256 divides the width, 917
+// with this rule.
+int half_tile_rows(int n) { return (n + 255) / 256 * 384 < (n + 127) / 128 * 256 ? 128 : 64; }
+
 template <int KIND, bool PAIR>
 cudaError_t launch_kind(const Maps<KIND>& maps, const BwdParams& p, int num_sms, cudaStream_t st) {
   // per instantiation and device: the shared-memory attribute and the resident grid are set on first use
@@ -796,8 +803,7 @@ int feplb_launch_expert_ffn_bwd(const feplb_bwd_args& a, cudaStream_t st, int64_
     return FEPLB_E_CUDA;
   };
   // ---- dH and the SwiGLU derivative: dAB = SwiGLU'(a, b; dY W2) ----------------------------------
-  const int bn_h = (f % 256 == 0) ? 128 : 64;      // N = f in tiles of 2*bn columns (the last may overhang)
-  const int bn_x = (d % 256 == 0) ? 128 : 64;
+  const int bn_h = half_tile_rows(f), bn_x = half_tile_rows(d);
   CUtensorMap tm_dy, tm_w2t, tm_dab, tm_w1t, tm_w3t;
   if (!make_tmap(&tm_dy, a.d_y_perm, (uint64_t)a.s_cap, (uint64_t)d, (uint64_t)d, BM) ||
       !make_tmap(&tm_w2t, a.w2t, (uint64_t)a.E * f, (uint64_t)d, (uint64_t)d, bn_h) ||
@@ -854,7 +860,7 @@ int feplb_launch_expert_ffn_bwd(const feplb_bwd_args& a, cudaStream_t st, int64_
   const int tile_m = a.pair_wgrad ? 2 * BM : BM;
   for (int i = 0; i < 3; ++i) {
     const WG& j = jobs[i];
-    const int bn = (j.n_total % 256 == 0) ? 128 : 64;
+    const int bn = half_tile_rows(j.n_total);
     if (!make_tmap_mn(&mw.a[i], j.p, (uint64_t)a.s_cap, (uint64_t)j.m_total, (uint64_t)j.ld_p, BM / 64) ||
         !make_tmap_mn(&mw.b[i], j.q, (uint64_t)a.s_cap, (uint64_t)j.n_total, (uint64_t)j.n_total, (a.pair_wgrad ? bn : 2 * bn) / 64) ||
         !make_tmap_out(&mw.out[i], j.out, (uint64_t)a.E, (uint64_t)j.m_total, (uint64_t)j.n_total)) {

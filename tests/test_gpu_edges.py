@@ -9,6 +9,7 @@ from paper_2604_19654_b200 import feplb as F
 from paper_2604_19654_b200 import workloads as W
 
 from gpu_utils import DeviceCase
+from test_gpu_backward import _close, _run_backward
 from test_gpu_parity import _check_forward, _ffn_case
 
 pytestmark = pytest.mark.gpu
@@ -122,3 +123,16 @@ def test_combine_every_batch_size(K):
 def test_expert_ffn_few_rows():
     """Groups around the 32 rows below which a tile loads a smaller box of A."""
     _ffn_case(6, 256, 128, [31, 32, 33, 1, 160, 161], form=F.FORM_SINGLE)      # 160 = 128 + 32, 161 = 128 + 33
+
+
+@pytest.mark.parametrize("pair", [0, 3])
+@pytest.mark.parametrize("d,f", [(640, 192), (384, 320), (1152, 704)])
+def test_backward_overhanging_n_tile(d, f, pair):
+    """Widths whose last 256-column tile of the backward GEMMs overhangs (192, 640, 704, 1152), and ones that keep
+    128-column tiles (320, 384)."""
+    w = W.get_workload("cfg2").with_(T=150, E=6, R=2, K=3, d=d, f=f, dyn=2, max_num_dyn=2, tau=8)
+    case, bwd, dw, ref, _, _ = _run_backward(w, pair=pair)
+    for got, want, what in zip((*dw, bwd.d_gates), (ref[2], ref[3], ref[4], ref[1]), ("dw1", "dw3", "dw2", "dgates")):
+        _close(got.cpu().numpy().astype(np.float64)[: len(want)], want, what)
+    _close(W.bf16_bits_to_f64(F.bf16_bits(bwd.d_x)), ref[0], "dx")
+    case.close()
