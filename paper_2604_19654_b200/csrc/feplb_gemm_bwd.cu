@@ -716,7 +716,7 @@ bool make_tmap_out(CUtensorMap* m, float* base, uint64_t E, uint64_t M, uint64_t
 // Rows of a B half tile for an output n columns wide: the N tile of 2 * 128 or 2 * 64 columns that brings fewer operand
 // bytes into the SMs; the last tile may overhang (its surplus columns are computed and not stored).  A row of
 // 256-column tiles moves 128 + 256 operand rows per tile, one of 128-column tiles 128 + 128.  Forward and backward
-// at d = 1920, f = 704, 60 experts, T = 4096, top-4: 1033 us with 128 columns unless 256 divides the width, 917
+// at d = 1920, f = 704, 60 experts, T = 4096, top-4: 1033 us with 128 columns unless 256 divides the width, 923
 // with this rule.
 int half_tile_rows(int n) { return (n + 255) / 256 * 384 < (n + 127) / 128 * 256 ? 128 : 64; }
 
@@ -824,7 +824,7 @@ int feplb_launch_expert_ffn_bwd(const feplb_bwd_args& a, cudaStream_t st, int64_
   if (e != cudaSuccess) return fail_cuda("k_ffn_bwd_gemm<DH>");
   // ---- dX = [dA | dB] [W1^T ; W3^T] ------------------------------------------------------------------
   BwdParams px = p;
-  px.n_tiles_n = d / (2 * bn_x); px.n_limit = d; px.num_k_blocks = 2 * f / BK; px.k_switch = f / BK; px.b_rows_per_expert = d; px.bn = bn_x;
+  px.n_tiles_n = (d + 2 * bn_x - 1) / (2 * bn_x); px.n_limit = d; px.num_k_blocks = 2 * f / BK; px.k_switch = f / BK; px.b_rows_per_expert = d; px.bn = bn_x;
   px.out = (__nv_bfloat16*)a.d_x_perm; px.ld_out = d;
   const Maps<KIND_DX> mx = {{tm_dab}, {tm_w1t, tm_w3t}};
   e = a.pair_dgrad ? launch_kind<KIND_DX, true>(mx, px, a.num_sms, st) : launch_kind<KIND_DX, false>(mx, px, a.num_sms, st);
