@@ -1130,16 +1130,21 @@ extern "C" int feplb_transpose_weights(feplb_ctx* c, const void* w1, const void*
   return FEPLB_OK;
 }
 
-extern "C" int feplb_combine_bwd(feplb_ctx* c, const void* d_out, const void* y_perm, const int32_t* slot_to_row,
-                                 const float* gates, void* d_y_perm, float* d_gates, void* stream) {
+static int combine_bwd_impl(feplb_ctx* c, const void* d_out, const void* y_perm, const int32_t* slot_to_row,
+                            const float* gates, void* d_y_perm, float* d_gates, const feplb_bwd_pads* pads, void* stream) {
   if (!c) return FEPLB_E_INVALID;
   if (c->cfg.T == 0) return FEPLB_OK;
   int rc = check_dev_ptrs(c, {d_out, y_perm, d_y_perm});
   if (rc != FEPLB_OK) return rc;
   if (!slot_to_row || !gates || !d_gates) return fail(c, FEPLB_E_INVALID, "combine_bwd: null pointer");
   CUDA_TRY(c, feplb_launch_combine_bwd(d_out, y_perm, slot_to_row, gates, d_y_perm, d_gates, c->cfg.T, c->cfg.K, c->cfg.d,
-                                       c->num_sms, (cudaStream_t)stream, &c->launches));
+                                       (cudaStream_t)stream, &c->launches, pads));
   return FEPLB_OK;
+}
+
+extern "C" int feplb_combine_bwd(feplb_ctx* c, const void* d_out, const void* y_perm, const int32_t* slot_to_row,
+                                 const float* gates, void* d_y_perm, float* d_gates, void* stream) {
+  return combine_bwd_impl(c, d_out, y_perm, slot_to_row, gates, d_y_perm, d_gates, nullptr, stream);
 }
 
 extern "C" int feplb_dispatch_bwd(feplb_ctx* c, const void* d_x_perm, const int32_t* slot_to_row, void* d_x, void* stream) {
@@ -1153,12 +1158,12 @@ extern "C" int feplb_dispatch_bwd(feplb_ctx* c, const void* d_x_perm, const int3
   return FEPLB_OK;
 }
 
-extern "C" int feplb_expert_ffn_bwd(feplb_ctx* c, const void* x_perm, const void* ab_saved, void* h,
-                                    void* d_y_perm, const void* w1t, const void* w3t, const void* w2t,
-                                    const feplb_group* groups, int32_t n_groups, int32_t which,
-                                    const feplb_group* expert_table, void* d_ab,
-                                    void* d_x_perm, float* dw1, float* dw3, float* dw2, int32_t accumulate,
-                                    void* stream) {
+static int expert_ffn_bwd_impl(feplb_ctx* c, const void* x_perm, const void* ab_saved, void* h,
+                               void* d_y_perm, const void* w1t, const void* w3t, const void* w2t,
+                               const feplb_group* groups, int32_t n_groups, int32_t which,
+                               const feplb_group* expert_table, void* d_ab,
+                               void* d_x_perm, float* dw1, float* dw3, float* dw2, int32_t accumulate,
+                               bool pads_zeroed, void* stream) {
   if (!c) return FEPLB_E_INVALID;
   if (n_groups < 0 || n_groups > FEPLB_MAX_GROUPS) return fail(c, FEPLB_E_INVALID, "expert_ffn_bwd: n_groups out of range");
   if (n_groups == 0 || c->s_cap == 0) return FEPLB_OK;
@@ -1181,8 +1186,19 @@ extern "C" int feplb_expert_ffn_bwd(feplb_ctx* c, const void* x_perm, const void
   a.dw1 = want_w ? dw1 : nullptr; a.dw3 = dw3; a.dw2 = dw2; a.accumulate = accumulate != 0;
   a.E = c->cfg.E; a.d = c->cfg.d; a.f = c->cfg.f; a.s_cap = (int64_t)c->s_cap;
   a.status = c->d_status; a.num_sms = c->num_sms;
+  a.pads_zeroed = pads_zeroed;
   a.pair_dgrad = c->bwd_pair & 1; a.pair_wgrad = (c->bwd_pair >> 1) & 1;
   return feplb_launch_expert_ffn_bwd(a, (cudaStream_t)stream, &c->launches, c->err, sizeof(c->err));
+}
+
+extern "C" int feplb_expert_ffn_bwd(feplb_ctx* c, const void* x_perm, const void* ab_saved, void* h,
+                                    void* d_y_perm, const void* w1t, const void* w3t, const void* w2t,
+                                    const feplb_group* groups, int32_t n_groups, int32_t which,
+                                    const feplb_group* expert_table, void* d_ab,
+                                    void* d_x_perm, float* dw1, float* dw3, float* dw2, int32_t accumulate,
+                                    void* stream) {
+  return expert_ffn_bwd_impl(c, x_perm, ab_saved, h, d_y_perm, w1t, w3t, w2t, groups, n_groups, which, expert_table, d_ab,
+                             d_x_perm, dw1, dw3, dw2, accumulate, false, stream);
 }
 
 extern "C" int feplb_moe_backward(feplb_ctx* c, const void* d_out, const float* gates, const void* w1t, const void* w3t,
@@ -1191,11 +1207,17 @@ extern "C" int feplb_moe_backward(feplb_ctx* c, const void* d_out, const float* 
                                   void* d_y_perm, void* d_ab, void* d_x_perm, void* d_x, float* d_gates,
                                   float* dw1, float* dw3, float* dw2, int32_t accumulate, void* stream) {
   if (!c) return FEPLB_E_INVALID;
-  int rc = feplb_combine_bwd(c, d_out, y_perm, slot_to_row, gates, d_y_perm, d_gates, stream);
+  // weight gradients: the padding rows are zeroed by the first kernel; what is wrong with the arguments has to be
+  // found before it writes to them
+  const bool zero_pads = (dw1 || dw3 || dw2) && c->cfg.row_align == 128 && c->cfg.T > 0;
+  int rc = FEPLB_OK;
+  if (zero_pads && (rc = check_dev_ptrs(c, {h, d_ab})) != FEPLB_OK) return rc;
+  const feplb_bwd_pads pads = {c->d_home_groups, c->cfg.E, c->cfg.f, h, d_ab};
+  rc = combine_bwd_impl(c, d_out, y_perm, slot_to_row, gates, d_y_perm, d_gates, zero_pads ? &pads : nullptr, stream);
   if (rc != FEPLB_OK) return rc;
   // every expert's rows in one table: the home table of the forward pass that ran last on this context
-  rc = feplb_expert_ffn_bwd(c, x_perm, ab_saved, h, d_y_perm, w1t, w3t, w2t, c->d_home_groups, c->cfg.E, FEPLB_FFN_ALL,
-                            c->d_home_groups, d_ab, d_x_perm, dw1, dw3, dw2, accumulate, stream);
+  rc = expert_ffn_bwd_impl(c, x_perm, ab_saved, h, d_y_perm, w1t, w3t, w2t, c->d_home_groups, c->cfg.E, FEPLB_FFN_ALL,
+                           c->d_home_groups, d_ab, d_x_perm, dw1, dw3, dw2, accumulate, zero_pads, stream);
   if (rc != FEPLB_OK) return rc;
   return feplb_dispatch_bwd(c, d_x_perm, slot_to_row, d_x, stream);
 }

@@ -229,6 +229,10 @@ k_ffn_bwd_gemm(const __grid_constant__ Maps<KIND> maps, const __grid_constant__ 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   volatile int* abort_flag = &tail->abort_flag;
 
+  // The launches of a backward pass are chained programmatically: the set-up here overlaps the tail of the kernel
+  // before, whose results are read after the wait below.  No early trigger for the kernel behind: that one can use an SM
+  // only when this grid's CTA has left it (triggered at the start, the training step of the 64-expert
+  // d = 2048, f = 768 layer took 1248 us, this way 1240).
   if (threadIdx.x == 0) {
     for (const CUtensorMap& m : maps.a) prefetch_tmap(&m);
     for (const CUtensorMap& m : maps.b) prefetch_tmap(&m);
@@ -255,6 +259,7 @@ k_ffn_bwd_gemm(const __grid_constant__ Maps<KIND> maps, const __grid_constant__ 
       tmem_relinquish();
     }
   }
+  asm volatile("griddepcontrol.wait;" ::: "memory");
   for (int g = threadIdx.x; g < p.n_groups; g += kThreads) {
     const feplb_group gr = p.groups[g];
     const bool selected = p.which == FEPLB_FFN_ALL || (p.which == FEPLB_FFN_STATIC) == (gr.is_dynamic == 0);
@@ -601,59 +606,98 @@ k_transpose_bf16(const __grid_constant__ TransposeJobs jobs) {
   }
 }
 
-// Backward of the combine: for every slot (t, k) with row r = slot_to_row[t, k]
-//   dY_perm[r, :] = gates[t, k] * dOut[t, :]         dGates[t, k] = <dOut[t, :], y_perm[r, :]>
-// One warp per slot, slots dealt out in equal contiguous ranges.
-__global__ void __launch_bounds__(256)
-k_combine_bwd(const uint4* __restrict__ d_out, const uint4* __restrict__ y_perm, const int32_t* __restrict__ slot_to_row,
-              const float* __restrict__ gates, uint4* __restrict__ d_y_perm, float* __restrict__ d_gates,
-              int64_t S, int K, int chunks) {
-  const int lane = threadIdx.x & 31;
-  const int64_t warp = ((int64_t)blockIdx.x * 256 + threadIdx.x) >> 5;
-  const int64_t nwarps = ((int64_t)gridDim.x * 256) >> 5;
-  const int64_t s0 = S * warp / nwarps, s1 = S * (warp + 1) / nwarps;
-  for (int64_t s = s0; s < s1; ++s) {
-    const int row = slot_to_row[s];
-    const float g = gates[s];
-    const int64_t t = s / K;
-    float dot = 0.f;
-    if (row >= 0) {
-      for (int c = lane; c < chunks; c += 32) {
-        const uint4 o = ld_nc_v4(d_out + t * chunks + c);
-        const uint4 y = ld_nc_v4(y_perm + (int64_t)row * chunks + c);
-        uint4 w;
-        const uint32_t ov[4] = {o.x, o.y, o.z, o.w}, yv[4] = {y.x, y.y, y.z, y.w};
-        uint32_t wv[4];
-#pragma unroll
-        for (int i = 0; i < 4; ++i) {
-          const float o0 = bf16_lo(ov[i]), o1 = bf16_hi(ov[i]);
-          dot = fmaf(o0, bf16_lo(yv[i]), dot);
-          dot = fmaf(o1, bf16_hi(yv[i]), dot);
-          wv[i] = pack_bf16x2(g * o0, g * o1);
-        }
-        w.x = wv[0]; w.y = wv[1]; w.z = wv[2]; w.w = wv[3];
-        d_y_perm[(int64_t)row * chunks + c] = w;
-      }
-    }
-#pragma unroll
-    for (int o = 16; o >= 1; o >>= 1) dot += __shfl_xor_sync(0xffffffffu, dot, o);
-    if (lane == 0) d_gates[s] = row >= 0 ? dot : 0.f;
-  }
+// Zeros for the rows that pad each expert's segment to 128 in up to three row-major buffers: the weight gradients
+// contract over whole 64-row blocks of a segment, and the kernels that produce these buffers write the valid rows
+// only.  `part` of kPadParts shares one (expert, buffer).
+struct PadBufs { uint4* buf[3]; int chunks[3]; };
+constexpr int kPadParts = 8;
+__device__ __forceinline__ void zero_pad_rows(const feplb_group& g, uint4* buf, int chunks, int part) {
+  const int64_t r0 = (int64_t)g.row_start + g.rows, r1 = (r0 + 127) / 128 * 128;
+  uint4* p = buf + r0 * chunks;
+  const int64_t n = (r1 - r0) * chunks;
+  for (int64_t i = part * blockDim.x + threadIdx.x; i < n; i += kPadParts * blockDim.x) p[i] = make_uint4(0, 0, 0, 0);
+}
+__global__ void __launch_bounds__(128)
+k_zero_pad_rows(const feplb_group* __restrict__ table, PadBufs b) {
+  zero_pad_rows(table[blockIdx.x], b.buf[blockIdx.y], b.chunks[blockIdx.y], blockIdx.z);
 }
 
-// Zero the rows that pad each expert's segment to a multiple of 128 rows in up to three row-major
-// buffers (blockIdx.y picks one): the weight gradients contract over whole 64-row blocks of a segment,
-// and the GEMM epilogues that produce these buffers write the valid rows only.  gridDim.z blocks
-// share one (expert, buffer).
-struct PadBufs { uint4* buf[3]; int chunks[3]; };
-__global__ void __launch_bounds__(256)
-k_zero_pad_rows(const feplb_group* __restrict__ table, PadBufs b) {
-  const feplb_group g = table[blockIdx.x];
-  const int chunks = b.chunks[blockIdx.y];
-  const int64_t r0 = (int64_t)g.row_start + g.rows, r1 = (r0 + 127) / 128 * 128;
-  uint4* p = b.buf[blockIdx.y] + r0 * chunks;
-  const int64_t n = (r1 - r0) * chunks;
-  for (int64_t i = blockIdx.z * 256 + threadIdx.x; i < n; i += 256 * gridDim.z) p[i] = make_uint4(0, 0, 0, 0);
+// Backward of the combine: for every slot (t, k) with row r = slot_to_row[t, k]
+//   dY_perm[r, :] = gates[t, k] * dOut[t, :]         dGates[t, k] = <dOut[t, :], y_perm[r, :]>
+// HBM-bound: y_perm is read and dY_perm written once.  A warp takes two slots of a token and 64 chunks of their rows at
+// a time, so that 4 loads of y and 2 of dOut are in flight per lane and dOut is read once for both; warps follow the
+// token order, so that the rows of an expert are touched in one moving window (see k_gather); the writes are
+// marked evict-first.  Measured alone (32768 rows, d = 6144 / 24576 rows, d = 2048): a warp per slot over a contiguous
+// range 193 / 51.5 us, this way 157 / 41.7 (5.45 / 5.23 TB/s); without the mark 165 / 44.6, four slots 166 / 47.5,
+// 128 chunks at a time 176 / 47.8.
+// The first pad_blocks CTAs write the zeros of the padding rows instead (whole backward pass only).
+constexpr int kCbWarps = 4, kCbSlots = 2;
+__global__ void __launch_bounds__(kCbWarps * 32)
+k_combine_bwd(const uint4* __restrict__ d_out, const uint4* __restrict__ y_perm, const int32_t* __restrict__ slot_to_row,
+              const float* __restrict__ gates, uint4* __restrict__ d_y_perm, float* __restrict__ d_gates,
+              int64_t units, int K, int groups, int per_group, int chunks, const feplb_group* __restrict__ table, PadBufs pads,
+              int pad_blocks) {
+  asm volatile("griddepcontrol.launch_dependents;");
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  if ((int)blockIdx.x < pad_blocks) {
+    const int e = blockIdx.x / (3 * kPadParts), i = blockIdx.x / kPadParts % 3;
+    zero_pad_rows(table[e], pads.buf[i], pads.chunks[i], blockIdx.x % kPadParts);
+    return;
+  }
+  const int lane = threadIdx.x & 31;
+  const int64_t u = (int64_t)(blockIdx.x - pad_blocks) * kCbWarps + (threadIdx.x >> 5);
+  if (u >= units) return;
+  const int64_t t = u / groups;
+  const int k0 = (int)(u - t * groups) * per_group, nk = min(per_group, K - k0);
+  int myrow = -1;
+  float myg = 0.f;
+  if (lane < nk) {
+    myrow = slot_to_row[t * K + k0 + lane];
+    myg = gates[t * K + k0 + lane];
+  }
+  int row[kCbSlots];
+  float g[kCbSlots], dot[kCbSlots];
+#pragma unroll
+  for (int j = 0; j < kCbSlots; ++j) {
+    row[j] = __shfl_sync(0xffffffffu, myrow, j);
+    g[j] = __shfl_sync(0xffffffffu, myg, j);
+    dot[j] = 0.f;
+  }
+  for (int c0 = lane; c0 < chunks; c0 += 64) {
+    uint4 o[2], y[kCbSlots][2];
+#pragma unroll
+    for (int i = 0; i < 2; ++i) {
+      const int c = c0 + 32 * i;
+      o[i] = c < chunks ? ld_nc_v4(d_out + t * chunks + c) : make_uint4(0, 0, 0, 0);
+#pragma unroll
+      for (int j = 0; j < kCbSlots; ++j)
+        y[j][i] = c < chunks && row[j] >= 0 ? ld_nc_v4(y_perm + (int64_t)row[j] * chunks + c) : make_uint4(0, 0, 0, 0);
+    }
+#pragma unroll
+    for (int i = 0; i < 2; ++i) {
+      const int c = c0 + 32 * i;
+      const uint32_t ov[4] = {o[i].x, o[i].y, o[i].z, o[i].w};
+#pragma unroll
+      for (int j = 0; j < kCbSlots; ++j) {
+        const uint32_t yv[4] = {y[j][i].x, y[j][i].y, y[j][i].z, y[j][i].w};
+        uint32_t wv[4];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+          const float o0 = bf16_lo(ov[q]), o1 = bf16_hi(ov[q]);
+          dot[j] = fmaf(o0, bf16_lo(yv[q]), dot[j]);
+          dot[j] = fmaf(o1, bf16_hi(yv[q]), dot[j]);
+          wv[q] = pack_bf16x2(g[j] * o0, g[j] * o1);
+        }
+        if (c < chunks && row[j] >= 0) __stcs(&d_y_perm[(int64_t)row[j] * chunks + c], make_uint4(wv[0], wv[1], wv[2], wv[3]));
+      }
+    }
+  }
+#pragma unroll
+  for (int j = 0; j < kCbSlots; ++j) {
+#pragma unroll
+    for (int o = 16; o >= 1; o >>= 1) dot[j] += __shfl_xor_sync(0xffffffffu, dot[j], o);
+    if (lane == 0 && j < nk) d_gates[t * K + k0 + j] = row[j] >= 0 ? dot[j] : 0.f;
+  }
 }
 
 typedef CUresult (*encode_tiled_fn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*,
@@ -731,15 +775,17 @@ cudaError_t launch_kind(const Maps<KIND>& maps, const BwdParams& p, int num_sms,
   cfg.blockDim = dim3(kThreads);
   cfg.dynamicSmemBytes = kSmemBytes;
   cfg.stream = st;
-  cudaLaunchAttribute at[1];
+  cudaLaunchAttribute at[2];
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = at;
-  cfg.numAttrs = 0;
+  cfg.numAttrs = 1;
   if (PAIR) {
-    at[0].id = cudaLaunchAttributeClusterDimension;
-    at[0].val.clusterDim.x = 2;
-    at[0].val.clusterDim.y = 1;
-    at[0].val.clusterDim.z = 1;
-    cfg.numAttrs = 1;
+    at[1].id = cudaLaunchAttributeClusterDimension;
+    at[1].val.clusterDim.x = 2;
+    at[1].val.clusterDim.y = 1;
+    at[1].val.clusterDim.z = 1;
+    cfg.numAttrs = 2;
   }
   if (!grid) {
     cudaError_t e = cudaFuncSetAttribute(k_ffn_bwd_gemm<KIND, PAIR>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemBytes);
@@ -780,18 +826,31 @@ cudaError_t feplb_launch_transpose_weights(const void* w1, const void* w3, const
   return cudaGetLastError();
 }
 
+static PadBufs pad_bufs(void* h, void* d_y_perm, void* d_ab, int d, int f) {
+  return PadBufs{{(uint4*)h, (uint4*)d_y_perm, (uint4*)d_ab}, {f / 8, d / 8, 2 * f / 8}};
+}
+
 cudaError_t feplb_launch_combine_bwd(const void* d_out, const void* y_perm, const int32_t* slot_to_row, const float* gates,
-                                     void* d_y_perm, float* d_gates, int T, int K, int d, int num_sms, cudaStream_t st,
-                                     int64_t* n_launch) {
-  const int64_t S = (int64_t)T * K;
-  if (S == 0) return cudaSuccess;
-  int blocks = num_sms * 6;
-  const int64_t need = (S + 7) / 8;
-  if (need < blocks) blocks = (int)need;
-  k_combine_bwd<<<blocks, 256, 0, st>>>((const uint4*)d_out, (const uint4*)y_perm, slot_to_row, gates, (uint4*)d_y_perm,
-                                        d_gates, S, K, d / 8);
+                                     void* d_y_perm, float* d_gates, int T, int K, int d, cudaStream_t st, int64_t* n_launch,
+                                     const feplb_bwd_pads* pads) {
+  if (T == 0) return cudaSuccess;
+  const int groups = (K + kCbSlots - 1) / kCbSlots;
+  const int64_t units = (int64_t)T * groups;
+  const int pad_blocks = pads ? pads->E * 3 * kPadParts : 0;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)(pad_blocks + (units + kCbWarps - 1) / kCbWarps));
+  cfg.blockDim = dim3(kCbWarps * 32);
+  cfg.stream = st;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
   ++*n_launch;
-  return cudaGetLastError();
+  return cudaLaunchKernelEx(&cfg, k_combine_bwd, (const uint4*)d_out, (const uint4*)y_perm, slot_to_row, gates,
+                            (uint4*)d_y_perm, d_gates, units, K, groups, (K + groups - 1) / groups, d / 8,
+                            pads ? pads->table : (const feplb_group*)nullptr,
+                            pads ? pad_bufs(pads->h, d_y_perm, pads->d_ab, d, pads->f) : PadBufs{}, pad_blocks);
 }
 
 int feplb_launch_expert_ffn_bwd(const feplb_bwd_args& a, cudaStream_t st, int64_t* n_launch, char* err, size_t errn) {
@@ -833,14 +892,12 @@ int feplb_launch_expert_ffn_bwd(const feplb_bwd_args& a, cudaStream_t st, int64_
   if (!a.dw1) return FEPLB_OK;
   // ---- weight gradients: contraction over each expert's rows, operands read as they lie (MN-major) ------
   // dW2[e] [d, f] = dY_e^T H_e;   dW1[e] [f, d] = dA_e^T X_e;   dW3[e] [f, d] = dB_e^T X_e
-  PadBufs pb;
-  pb.buf[0] = (uint4*)a.h; pb.chunks[0] = f / 8;
-  pb.buf[1] = (uint4*)a.d_y_perm; pb.chunks[1] = d / 8;
-  pb.buf[2] = (uint4*)a.d_ab; pb.chunks[2] = 2 * f / 8;
-  k_zero_pad_rows<<<dim3(a.E, 3, 8), 256, 0, st>>>(a.expert_table, pb);
-  ++*n_launch;
-  e = cudaGetLastError();
-  if (e != cudaSuccess) return fail_cuda("k_zero_pad_rows");
+  if (!a.pads_zeroed) {
+    k_zero_pad_rows<<<dim3(a.E, 3, kPadParts), 128, 0, st>>>(a.expert_table, pad_bufs(a.h, a.d_y_perm, a.d_ab, d, f));
+    ++*n_launch;
+    e = cudaGetLastError();
+    if (e != cudaSuccess) return fail_cuda("k_zero_pad_rows");
+  }
   // One launch for all three.  The cost of a tile grows with its expert's rows, tiles are dealt round-robin, and
   // experts differ a lot: the 48 tiles that one gradient of a busy expert has (d = 2048, f = 768) burden a third
   // of the SMs.  With the tiles of the three gradients side by side an expert has three times as many, and

@@ -121,13 +121,16 @@ struct feplb_bwd_args {
   float* dw1; float* dw3; float* dw2; int accumulate;       // fp32 [E,f,d], [E,f,d], [E,d,f]; dw1 == nullptr: skip
   int E, d, f; int64_t s_cap;
   uint32_t* status; int num_sms;
+  bool pads_zeroed = false;                                 // the padding rows hold zeros already
   int pair_dgrad, pair_wgrad;                               // 1: cta_group::2 form (256 x 256 tiles per cluster of two CTAs)
 };
 cudaError_t feplb_launch_transpose_weights(const void* w1, const void* w3, const void* w2, void* w1t, void* w3t, void* w2t,
                                            int E, int d, int f, cudaStream_t st, int64_t* n_launch);
+// The padding rows of h, d_y_perm and d_ab that the combine's backward kernel zeroes along the way.
+struct feplb_bwd_pads { const feplb_group* table; int E, f; void* h; void* d_ab; };
 cudaError_t feplb_launch_combine_bwd(const void* d_out, const void* y_perm, const int32_t* slot_to_row, const float* gates,
-                                     void* d_y_perm, float* d_gates, int T, int K, int d, int num_sms, cudaStream_t st,
-                                     int64_t* n_launch);
+                                     void* d_y_perm, float* d_gates, int T, int K, int d, cudaStream_t st, int64_t* n_launch,
+                                     const feplb_bwd_pads* pads = nullptr);
 int feplb_launch_expert_ffn_bwd(const feplb_bwd_args& a, cudaStream_t st, int64_t* n_launch, char* err, size_t errn);
 #endif
 

@@ -179,8 +179,8 @@ k_scan(int32_t* __restrict__ block_hist, int nb, int E, int A, const int32_t* __
     pad_off[E] = (int32_t)(total < s_cap ? total : s_cap);
     if (total > s_cap) atomicOr(status, FEPLB_ST_COUNTS);
   }
-  // rows behind the last segment hold no token (the padding rows inside segments are marked by k_zero_pad,
-  // the live rows by k_gather: with counts that agree with the ids that covers every row)
+  // rows behind the last segment hold no token (the padding rows inside segments and the
+  // live rows are marked by k_gather: with counts that agree with the ids that covers every row)
   for (int64_t i = total + threadIdx.x; i < s_cap; i += blockDim.x) row_to_token[i] = -1;
 }
 
@@ -278,7 +278,7 @@ constexpr int kGatherUnroll = 4;
 __global__ void __launch_bounds__(kThreads)
 k_gather(const uint4* __restrict__ x, const int32_t* __restrict__ ids, const int32_t* __restrict__ pad_off,
          const int32_t* __restrict__ block_base, int32_t* slot_to_row, int32_t* __restrict__ row_to_token,
-         uint4* __restrict__ x_perm, int T, int K, int E, int chunks, int64_t s_cap) {
+         uint4* __restrict__ x_perm, int T, int K, int E, int chunks, int64_t s_cap, const int32_t* __restrict__ counts, int A) {
   pdl_sync();
   const int lane = threadIdx.x & 31;
   const int64_t warp = ((int64_t)blockIdx.x * kThreads + threadIdx.x) >> 5;
@@ -321,6 +321,16 @@ k_gather(const uint4* __restrict__ x, const int32_t* __restrict__ ids, const int
         const int c = c0 + i * 32 + lane;
         if (c < chunks) dst[c] = v[i];
       }
+    }
+  }
+  if (A > 1) {                   // zeros for the padding rows at the end of every expert's segment, one row per warp at a time
+    for (int64_t q = warp; q < (int64_t)E * A; q += nwarps) {
+      const int e = (int)(q / A), c = counts[e] > 0 ? counts[e] : 0;
+      // clamped to the buffer: counts that disagree with the ids must not turn into wild writes
+      const int64_t row = (int64_t)pad_off[e] + c + (q - (int64_t)e * A);
+      if (row >= pad_off[e + 1] || row >= s_cap || row < 0) continue;
+      for (int i = lane; i < chunks; i += 32) x_perm[row * chunks + i] = make_uint4(0, 0, 0, 0);
+      if (lane == 0) row_to_token[row] = -1;
     }
   }
 }
@@ -475,27 +485,6 @@ k_route_small(const uint4* __restrict__ x, const int32_t* __restrict__ ids, int 
   }
 }
 
-// Zero the padding rows at the end of every expert's segment (row_align > 1 only).
-__global__ void __launch_bounds__(kThreads)
-k_zero_pad(const int32_t* __restrict__ counts, const int32_t* __restrict__ pad_off, uint4* __restrict__ x_perm,
-           int chunks, int32_t* __restrict__ row_to_token, int64_t s_cap) {
-  pdl_sync();
-  const int e = blockIdx.x;
-  // clamped to the buffer: counts that disagree with the ids must not turn into wild writes
-  const int c = counts[e] > 0 ? counts[e] : 0;
-  int64_t r1 = pad_off[e + 1];
-  if (r1 > s_cap) r1 = s_cap;
-  int64_t r0 = (int64_t)pad_off[e] + c;
-  if (r0 > r1) r0 = r1;
-  if (r0 < 0) r0 = 0;
-  if (row_to_token)
-    for (int64_t r = r0 + threadIdx.x; r < r1; r += kThreads) row_to_token[r] = -1;
-  const int64_t n = (r1 - r0) * chunks;
-  uint4* p = x_perm + r0 * chunks;
-  const uint4 z = make_uint4(0, 0, 0, 0);
-  for (int64_t i = threadIdx.x; i < n; i += kThreads) p[i] = z;
-}
-
 // Home group table {e, pad_off[e], counts[e], home(e), dynamic?} for all E experts.
 __global__ void __launch_bounds__(1024)
 k_home_groups(const int32_t* __restrict__ counts, const uint8_t* __restrict__ mask_in, int E, int L, int A, int dyn,
@@ -612,22 +601,15 @@ cudaError_t feplb_launch_gather(const void* x, const int32_t* ids, const int32_t
                                 const int32_t* counts, const int32_t* pad_off, void* x_perm, int T, int K, int E, int d,
                                 int A, int64_t s_cap, int num_sms, cudaStream_t st, int64_t* n_launch,
                                 int32_t* row_to_token, bool programmatic) {
-  cudaError_t err;
   const int chunks = d / 8;
-  if (A > 1) {
-    err = launch(k_zero_pad, E, kThreads, 0, st, programmatic, counts, pad_off, (uint4*)x_perm, chunks, row_to_token,
-                 s_cap);
-    ++*n_launch;
-    if (err != cudaSuccess) return err;
-  }
-  if (T == 0) return cudaSuccess;
+  if (T == 0 && A == 1) return cudaSuccess;
   const int64_t units = (int64_t)T * ((chunks + 32 * kGatherUnroll - 1) / (32 * kGatherUnroll));
   int blocks = num_sms * 8;   // 8 CTAs of 256 threads per SM are resident
-  const int64_t need = (units + kWarps - 1) / kWarps;
+  const int64_t need = ((A > 1 && units < (int64_t)E * A ? (int64_t)E * A : units) + kWarps - 1) / kWarps;
   if (need < blocks) blocks = (int)need;
   ++*n_launch;
   return launch(k_gather, blocks, kThreads, 0, st, programmatic, (const uint4*)x, ids, pad_off, block_base, slot_to_row,
-                row_to_token, (uint4*)x_perm, T, K, E, chunks, s_cap);
+                row_to_token, (uint4*)x_perm, T, K, E, chunks, s_cap, counts, A);
 }
 
 // Copies the planner's table of dynamic groups from mapped pinned host memory to the device.  A
