@@ -66,6 +66,7 @@ struct feplb_ctx {
   // device scratch
   int32_t* d_block_hist = nullptr;
   int32_t* d_pad_off = nullptr;
+  int32_t* d_totals = nullptr;       // [E + 1] accumulators and ticket of feplb_route_hist, zero between calls
   uint32_t* d_status = nullptr;
   feplb_group* d_home_groups = nullptr;
   feplb_group* d_dyn_groups = nullptr;
@@ -406,6 +407,8 @@ extern "C" int feplb_create(const feplb_config* cfg, feplb_ctx** out) {
   ok = ok && cudaMallocHost(&c->h_stamps, sizeof(unsigned long long) * kEvRing * kStampWords) == cudaSuccess;
   ok = ok && cudaMalloc(&c->d_block_hist, sizeof(int32_t) * (size_t)(c->nb > 0 ? c->nb : 1) * cfg->E) == cudaSuccess;
   ok = ok && cudaMalloc(&c->d_pad_off, sizeof(int32_t) * (cfg->E + 1)) == cudaSuccess;
+  ok = ok && cudaMalloc(&c->d_totals, sizeof(int32_t) * (cfg->E + 1)) == cudaSuccess &&
+       cudaMemset(c->d_totals, 0, sizeof(int32_t) * (cfg->E + 1)) == cudaSuccess;
   ok = ok && cudaMalloc(&c->d_status, sizeof(uint32_t)) == cudaSuccess;
   ok = ok && cudaMalloc(&c->d_home_groups, sizeof(feplb_group) * cfg->E) == cudaSuccess;
   ok = ok && cudaMalloc(&c->d_dyn_groups, (sizeof(feplb_group) * cap_groups + 15) / 16 * 16) == cudaSuccess;
@@ -474,6 +477,7 @@ extern "C" int feplb_destroy(feplb_ctx* c) {
   cudaDeviceSynchronize();
   cudaFree(c->d_block_hist);
   cudaFree(c->d_pad_off);
+  cudaFree(c->d_totals);
   cudaFree(c->d_status);
   cudaFree(c->d_home_groups);
   cudaFree(c->d_dyn_groups);
@@ -536,8 +540,8 @@ extern "C" int feplb_route_hist(feplb_ctx* c, const int32_t* topk_ids, int32_t* 
   if (!c) return FEPLB_E_INVALID;
   if (!counts || !rank_load || (!topk_ids && c->cfg.T > 0)) return fail(c, FEPLB_E_INVALID, "route_hist: null pointer");
   const int64_t S = (int64_t)c->cfg.T * c->cfg.K;
-  CUDA_TRY(c, feplb_launch_block_hist(topk_ids, S, c->cfg.E, c->cfg.R, c->d_block_hist, counts, rank_load,
-                                      c->d_status, (cudaStream_t)stream, &c->launches));
+  CUDA_TRY(c, feplb_launch_route_hist(topk_ids, S, c->cfg.E, c->cfg.R, c->d_totals, counts, rank_load, c->d_status,
+                                      (cudaStream_t)stream, &c->launches));
   return FEPLB_OK;
 }
 
@@ -550,6 +554,12 @@ static int dispatch_impl(feplb_ctx* c, const void* x, const int32_t* topk_ids, c
     int rc = check_dev_ptrs(c, {x, x_perm});
     if (rc != FEPLB_OK) return rc;
     if (!topk_ids || !slot_to_row) return fail(c, FEPLB_E_INVALID, "dispatch: null pointer");
+  }
+  if (feplb_front_is_small(S, g.E)) {
+    CUDA_TRY(c, feplb_launch_front_small(x, topk_ids, g.T, g.K, g.E, g.R, g.d, g.row_align, 0, nullptr, counts, nullptr, nullptr,
+                                         nullptr, nullptr, slot_to_row, row_to_token, x_perm, (int64_t)c->s_cap, c->d_status,
+                                         nullptr, 0, nullptr, c->num_sms, st, &c->launches));
+    return FEPLB_OK;
   }
   CUDA_TRY(c, feplb_launch_permute(topk_ids, S, g.K, g.E, g.row_align, counts, c->d_block_hist, c->d_pad_off,
                                    slot_to_row, row_to_token, (int64_t)c->s_cap, c->d_status, st, &c->launches));
@@ -814,7 +824,7 @@ extern "C" int feplb_moe_forward(feplb_ctx* c, const void* x, const int32_t* top
   const int32_t seq = c->flag_seq;
   const bool small_front = feplb_front_is_small(S, g.E);
   if (small_front)
-    CUDA_TRY(c, feplb_launch_front_small(x, topk_ids, g.T, g.K, g.E, g.R, g.d, g.row_align, g.dyn, mask_dev, counts, rank_load,
+    CUDA_TRY(c, feplb_launch_front_small(x, topk_ids, g.T, g.K, g.E, g.R, g.d, g.row_align, g.dyn, mask_dev, nullptr, counts, rank_load,
                                          c->d_pad_off, c->d_home_groups, slot_to_row, row_to_token, x_perm, (int64_t)c->s_cap,
                                          c->d_status, c->h_counts_tagged, seq, stamps ? stamps + 8 : nullptr, c->num_sms, st,
                                          &c->launches));

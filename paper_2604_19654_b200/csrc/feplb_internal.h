@@ -35,9 +35,9 @@ int feplb_validate_config(const feplb_config* c);
 
 // Kernel launchers (each enqueues on `st` and returns the cudaError_t of the launch).
 // n_launch is incremented by the number of kernels enqueued.
-cudaError_t feplb_launch_block_hist(const int32_t* ids, int64_t S, int E, int R, int32_t* block_hist,
-                                    int32_t* counts, int32_t* rank_load, uint32_t* status,
-                                    cudaStream_t st, int64_t* n_launch);
+// totals: E + 1 ints of scratch, zero between calls.
+cudaError_t feplb_launch_route_hist(const int32_t* ids, int64_t S, int E, int R, int32_t* totals, int32_t* counts,
+                                    int32_t* rank_load, uint32_t* status, cudaStream_t st, int64_t* n_launch);
 cudaError_t feplb_launch_permute(const int32_t* ids, int64_t S, int K, int E, int A, const int32_t* counts,
                                  int32_t* block_hist, int32_t* pad_off, int32_t* slot_to_row,
                                  int32_t* row_to_token, int64_t s_cap, uint32_t* status,
@@ -57,11 +57,12 @@ cudaError_t feplb_launch_route_fused(const int32_t* ids, int64_t S, int E, int R
                                      int32_t* slot_to_row, int32_t* row_to_token, int64_t s_cap, uint32_t* status,
                                      unsigned long long* counts_host_tagged, int32_t seq, unsigned long long* t_counts,
                                      cudaStream_t st, int64_t* n_launch);
-// Small batches: feplb_launch_route_fused and feplb_launch_gather in one launch.
+// Small batches: feplb_launch_route_fused and feplb_launch_gather in one launch; with groups == nullptr (and no mask,
+// counts, rank_load, pad_off) feplb_launch_permute and feplb_launch_gather, counts_in being the caller's counts.
 bool feplb_front_is_small(int64_t S, int E);
 cudaError_t feplb_launch_front_small(const void* x, const int32_t* ids, int T, int K, int E, int R, int d, int A, int dyn,
-                                     const uint8_t* mask_in, int32_t* counts, int32_t* rank_load, int32_t* pad_off,
-                                     feplb_group* groups, int32_t* slot_to_row, int32_t* row_to_token, void* x_perm,
+                                     const uint8_t* mask_in, const int32_t* counts_in, int32_t* counts, int32_t* rank_load,
+                                     int32_t* pad_off, feplb_group* groups, int32_t* slot_to_row, int32_t* row_to_token, void* x_perm,
                                      int64_t s_cap, uint32_t* status, unsigned long long* counts_host_tagged, int32_t seq,
                                      unsigned long long* t_counts, int num_sms, cudaStream_t st, int64_t* n_launch);
 cudaError_t feplb_launch_upload_groups(const feplb_group* src_host_mapped, feplb_group* dst, int n, cudaStream_t st);

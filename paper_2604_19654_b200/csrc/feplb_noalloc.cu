@@ -82,6 +82,10 @@ extern "C" int feplb_dispatch_noalloc(const feplb_config* cfg, const void* x, co
   const int64_t s_cap = S + (int64_t)cfg->E * (cfg->row_align - 1);
   int64_t launches = 0;
   if (!status && cudaMemsetAsync(st_word, 0, sizeof(uint32_t), st) != cudaSuccess) return FEPLB_E_CUDA;
+  if (feplb_front_is_small(S, cfg->E))
+    return feplb_launch_front_small(x, topk_ids, cfg->T, cfg->K, cfg->E, cfg->R, cfg->d, cfg->row_align, 0, nullptr, counts, nullptr,
+                                    nullptr, nullptr, nullptr, slot_to_row, row_to_token, x_perm, s_cap, st_word, nullptr, 0,
+                                    nullptr, num_sms, st, &launches) == cudaSuccess ? FEPLB_OK : FEPLB_E_CUDA;
   if (feplb_launch_permute(topk_ids, S, cfg->K, cfg->E, cfg->row_align, counts, block_hist, pad_off, slot_to_row,
                            row_to_token, s_cap, st_word, st, &launches) != cudaSuccess)
     return FEPLB_E_CUDA;

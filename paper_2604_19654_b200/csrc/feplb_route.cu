@@ -76,11 +76,12 @@ __device__ __forceinline__ bool warp_histograms(const int32_t* __restrict__ ids,
 // slot_to_row for the gather kernel: -2 - rank (final rows are >= 0, -1 marks an id outside [0, E)).
 __device__ __forceinline__ int encode_local_rank(int r) { return -2 - r; }
 
-// Step 1: per-CTA histograms; with counts != nullptr also the totals (one atomic per CTA and expert);
+// Step 1: per-CTA histograms; with totals != nullptr (E accumulators and a ticket, all zero between calls) also counts
+// and rank_load, by one atomic per CTA and expert and a last CTA, so that no memset has to precede the kernel;
 // with local_rank != nullptr also every slot's encoded rank inside this CTA's slots.
 __global__ void __launch_bounds__(kThreads)
 k_block_hist(const int32_t* __restrict__ ids, int64_t S, int E, int L, int32_t* __restrict__ block_hist,
-             int32_t* __restrict__ counts, int32_t* __restrict__ rank_load, uint32_t* status,
+             int32_t* __restrict__ counts, int32_t* __restrict__ rank_load, int32_t* totals, uint32_t* status,
              int32_t* __restrict__ local_rank) {
   extern __shared__ int wh[];
   int id[kChunks];
@@ -98,9 +99,30 @@ k_block_hist(const int32_t* __restrict__ ids, int64_t S, int E, int L, int32_t* 
       sum += t;
     }
     if (block_hist) block_hist[(int64_t)blockIdx.x * E + e] = sum;
-    if (counts && sum) {
-      atomicAdd(&counts[e], sum);
-      atomicAdd(&rank_load[e / L], sum);
+    if (totals && sum) atomicAdd(&totals[e], sum);
+  }
+  if (totals) {
+    // The CTA that arrives last writes the result and leaves the accumulators zero for the next call; the ticket
+    // wraps to zero by itself.
+    __shared__ int last;
+    __threadfence();
+    __syncthreads();
+    if (threadIdx.x == 0) last = atomicInc(reinterpret_cast<unsigned*>(totals + E), gridDim.x - 1) == gridDim.x - 1;
+    __syncthreads();
+    if (last) {
+      __threadfence();
+      for (int e = threadIdx.x; e < E; e += kThreads) {
+        const int n = __ldcg(totals + e);
+        wh[e] = n;
+        counts[e] = n;
+        totals[e] = 0;
+      }
+      __syncthreads();
+      for (int r = threadIdx.x; r < E / L; r += kThreads) {
+        int n = 0;
+        for (int e = r * L; e < (r + 1) * L; ++e) n += wh[e];
+        rank_load[r] = n;
+      }
     }
   }
   if (!local_rank) return;
@@ -148,6 +170,60 @@ __device__ __forceinline__ V block_exclusive_scan(V v, V* tmp, V* total) {
   return warp_off + x - v;
 }
 
+// Exclusive scan over CTAs of the per-CTA histograms by one block of 1024 threads, in three steps: who takes which part
+// of which expert's column (before the histograms are there), the sums, the prefixes in place.  Several threads
+// share an expert, each taking at least four CTAs, so that the loads of a column are a few round trips.
+// From the end of the histogram to the end of the scan, 64 CTAs, 128 experts: 9.9 us with one thread per expert, 5.6
+// this way.  More parts cost more in the sums over the parts than they save (118 CTAs, 8 experts, route + gather +
+// combine: up to 128 parts 65.9 us, up to 16 57.3).
+struct ScanRows { int p, parts, e, r0, r1, base; int v[8]; };
+__device__ __forceinline__ ScanRows scan_rows(int nb, int E) {
+  ScanRows q;
+  q.parts = max(1, min(min(1024 / E, 16), (nb + 3) / 4));
+  q.p = threadIdx.x / E;
+  q.e = threadIdx.x - q.p * E;
+  const int per = (nb + q.parts - 1) / q.parts;
+  q.r0 = q.p < q.parts ? min(nb, per * q.p) : 0;
+  q.r1 = q.p < q.parts ? min(nb, q.r0 + per) : 0;
+  return q;
+}
+// Returns the expert's total (threads < E).  part: 1024 ints of shared memory.
+__device__ __forceinline__ int sum_rows(const int32_t* __restrict__ block_hist, int E, int* part, ScanRows& q) {
+  int sum = 0;
+  for (int b0 = q.r0; b0 < q.r1; b0 += 8) {          // eight independent loads in flight per round
+#pragma unroll
+    for (int j = 0; j < 8; ++j) q.v[j] = b0 + j < q.r1 ? block_hist[(int64_t)(b0 + j) * E + q.e] : 0;
+#pragma unroll
+    for (int j = 0; j < 8; ++j) sum += q.v[j];
+  }
+  part[threadIdx.x] = sum;
+  __syncthreads();
+  q.base = 0;
+  int total = 0;
+  if (q.p < q.parts)
+    for (int o = 0; o < q.parts; ++o) {
+      const int t = part[o * E + q.e];
+      if (o < q.p) q.base += t;
+      total += t;
+    }
+  return total;
+}
+__device__ __forceinline__ void store_scan(int32_t* __restrict__ block_hist, int E, ScanRows& q) {
+  int run = q.base;
+  const bool kept = q.r1 - q.r0 <= 8;
+  for (int b0 = q.r0; b0 < q.r1; b0 += 8) {
+    if (!kept) {
+#pragma unroll
+      for (int j = 0; j < 8; ++j) q.v[j] = b0 + j < q.r1 ? block_hist[(int64_t)(b0 + j) * E + q.e] : 0;
+    }
+#pragma unroll
+    for (int j = 0; j < 8; ++j) {
+      if (b0 + j < q.r1) block_hist[(int64_t)(b0 + j) * E + q.e] = run;
+      run += q.v[j];
+    }
+  }
+}
+
 // Exclusive scan of the per-CTA histograms over CTAs (in place), check against counts, and
 // pad_off[e] = sum_{e'<e} round_up(counts[e'], A); pad_off[E] = padded total.
 // The counts are the caller's: when they disagree with the ids (FEPLB_ST_COUNTS) the result is
@@ -158,16 +234,14 @@ __global__ void __launch_bounds__(1024)
 k_scan(int32_t* __restrict__ block_hist, int nb, int E, int A, const int32_t* __restrict__ counts,
        int32_t* __restrict__ pad_off, int64_t s_cap, uint32_t* status, int32_t* __restrict__ row_to_token) {
   __shared__ long long tmp[64];
+  __shared__ int part[1024];
   const int e = threadIdx.x;
   int c = 0;
+  ScanRows q = scan_rows(nb, E);
   pdl_sync();
+  const int run = sum_rows(block_hist, E, part, q);
+  store_scan(block_hist, E, q);
   if (e < E) {
-    int run = 0;
-    for (int b = 0; b < nb; ++b) {
-      const int v = block_hist[(int64_t)b * E + e];
-      block_hist[(int64_t)b * E + e] = run;
-      run += v;
-    }
     c = counts[e];
     if (run != c) atomicOr(status, FEPLB_ST_COUNTS);
     if (c < 0) c = 0;
@@ -196,24 +270,14 @@ k_scan_fused(int32_t* __restrict__ block_hist, int nb, int E, int L, int A, int 
              int32_t* __restrict__ row_to_token, int64_t s_cap,
              unsigned long long* __restrict__ counts_host_tagged, int32_t seq, unsigned long long* t_counts) {
   __shared__ int tmp[64];
+  __shared__ int part[1024];
   __shared__ int sc[FEPLB_MAX_EXPERTS];
   const int e = threadIdx.x;
   int c = 0;
+  ScanRows q = scan_rows(nb, E);
   pdl_sync();
+  const int run = sum_rows(block_hist, E, part, q);
   if (e < E) {
-    // exclusive scan over CTAs, eight independent loads in flight per round (the in-place stores
-    // would otherwise serialise every load behind the previous store)
-    int run = 0;
-    for (int b0 = 0; b0 < nb; b0 += 8) {
-      int v[8];
-#pragma unroll
-      for (int j = 0; j < 8; ++j) v[j] = b0 + j < nb ? block_hist[(int64_t)(b0 + j) * E + e] : 0;
-#pragma unroll
-      for (int j = 0; j < 8; ++j) {
-        if (b0 + j < nb) block_hist[(int64_t)(b0 + j) * E + e] = run;
-        run += v[j];
-      }
-    }
     c = run;
     counts_out[e] = c;
     sc[e] = c;
@@ -225,6 +289,7 @@ k_scan_fused(int32_t* __restrict__ block_hist, int nb, int E, int L, int A, int 
       *reinterpret_cast<volatile unsigned long long*>(counts_host_tagged + e) =
           ((unsigned long long)(uint32_t)seq << 32) | (uint32_t)c;
   }
+  store_scan(block_hist, E, q);
   if (t_counts && e == 0) {            // timeline: when the counts left for the host (globaltimer, ns)
     unsigned long long t;
     asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
@@ -339,7 +404,8 @@ k_gather(const uint4* __restrict__ x, const int32_t* __restrict__ ids, const int
 // as ONE launch.  Chained, the three kernels it replaces take 11 us of launch and memory latency whatever the
 // size; here every CTA computes the complete routing of the batch for itself (at most kSmallMaxSlots ids, read
 // from L2; the ranks end up in shared memory), so that no CTA needs another one's result, and then copies
-// its share of the rows.  CTA 0 alone publishes the tables.  The redundant part grows with the number of slots
+// its share of the rows.  CTA 0 alone publishes the tables (groups != nullptr) or compares the counts with the
+// caller's (counts_in, stand-alone dispatch: its offsets come from the ids, so wrong counts only raise the status).  The redundant part grows with the number of slots
 // and ends the range: see feplb_front_is_small.
 // Whole layer, chained front -> this: 32.3 -> 27.9 us at T = 256, top-2, d = 128, 8 experts; 102.0 -> 97.9 us at
 // T = 64, top-6, d = 2048, 64 experts.
@@ -350,8 +416,8 @@ constexpr int kSmallSlice = 64;              // 16-byte chunks of a row per work
 template <int CH>                            // chunks of 32 slots per warp
 __global__ void __launch_bounds__(kSmallThreads, 1)
 k_route_small(const uint4* __restrict__ x, const int32_t* __restrict__ ids, int T, int K, int E, int L, int A, int dyn,
-              const uint8_t* __restrict__ mask_in, int32_t* __restrict__ counts_out, int32_t* __restrict__ rank_load_out,
-              int32_t* __restrict__ pad_off_out, feplb_group* __restrict__ groups, int32_t* __restrict__ slot_to_row,
+              const uint8_t* __restrict__ mask_in, const int32_t* __restrict__ counts_in, int32_t* __restrict__ counts_out,
+              int32_t* __restrict__ rank_load_out, int32_t* __restrict__ pad_off_out, feplb_group* __restrict__ groups, int32_t* __restrict__ slot_to_row,
               int32_t* __restrict__ row_to_token, uint4* __restrict__ x_perm, int chunks, int64_t s_cap, uint32_t* status,
               unsigned long long* __restrict__ counts_host_tagged, int32_t seq, unsigned long long* t_counts) {
   extern __shared__ int sm[];
@@ -408,7 +474,8 @@ k_route_small(const uint4* __restrict__ x, const int32_t* __restrict__ ids, int 
     }
     sc[e] = cnt;
     if (blockIdx.x == 0) {
-      counts_out[e] = cnt;
+      if (counts_in && counts_in[e] != cnt) atomicOr(status, FEPLB_ST_COUNTS);
+      if (counts_out) counts_out[e] = cnt;
       if (counts_host_tagged)                // see k_scan_fused
         *reinterpret_cast<volatile unsigned long long*>(counts_host_tagged + e) =
             ((unsigned long long)(uint32_t)seq << 32) | (uint32_t)cnt;
@@ -450,7 +517,7 @@ k_route_small(const uint4* __restrict__ x, const int32_t* __restrict__ ids, int 
     }
     if (u + gridDim.x * kSmallWarps < units) load_unit(u + gridDim.x * kSmallWarps);
   }
-  if (blockIdx.x == 0) {
+  if (groups && blockIdx.x == 0) {       // whole-layer path
     if (e < E) {
       pad_off_out[e] = off;
       int is_dyn;
@@ -510,42 +577,50 @@ k_home_groups(const int32_t* __restrict__ counts, const uint8_t* __restrict__ ma
   if (mask_out) mask_out[e] = (uint8_t)is_dyn;
 }
 
+// Order-preserving map of finite floats to unsigned integers > 0; -0 and +0 map to the same value.
+__device__ __forceinline__ unsigned sortable(float f) {
+  const unsigned u = __float_as_uint(f + 0.f);
+  return u & 0x80000000u ? ~u : u | 0x80000000u;
+}
+__device__ __forceinline__ float unsortable(unsigned u) { return __uint_as_float(u & 0x80000000u ? u & 0x7fffffffu : ~u); }
+
 // Router top-k gating (paper Sections 2.3 and 3.1: top-k routing, no auxiliary loss): one warp per
-// token.  Lane l holds logits l, l+32, ...; K rounds of a warp arg-max (larger value, then lower
-// expert id) pick the experts in descending order; gates = softmax over the K selected logits.
+// token.  Lane l holds logits l, l+32, ... as sortable integers (0 = none or taken); each of the K rounds finds the
+// largest by one warp reduction and the lowest expert id that has it by a second one; gates = softmax over the K
+// selected logits.  Bound by the instructions of the rounds, not by memory: with five shuffles of value and id
+// per round in place of the two reductions 13.1 us
+// at T = 8192, E = 128, top-8, this way 6.9.
 template <int NPER>
 __global__ void __launch_bounds__(kThreads)
 k_route_topk(const float* __restrict__ logits, int T, int E, int K, int32_t* __restrict__ ids,
              float* __restrict__ gates) {
+  pdl_sync();
   const int lane = threadIdx.x & 31;
   const int warp = (blockIdx.x * kThreads + threadIdx.x) >> 5;
   const int nwarps = (gridDim.x * kThreads) >> 5;
   for (int t = warp; t < T; t += nwarps) {
-    float v[NPER];
+    unsigned v[NPER];
 #pragma unroll
     for (int i = 0; i < NPER; ++i) {
       const int e = i * 32 + lane;
-      v[i] = e < E ? logits[(int64_t)t * E + e] : -INFINITY;
+      v[i] = e < E ? sortable(logits[(int64_t)t * E + e]) : 0u;
     }
-    unsigned taken = 0;
     float sel_val = 0.f;
     int sel_idx = 0;
     for (int k = 0; k < K; ++k) {
-      float best = -INFINITY;
-      int bidx = 0x7fffffff;
+      unsigned best = 0;
 #pragma unroll
-      for (int i = 0; i < NPER; ++i) {
-        const int e = i * 32 + lane;
-        if (e < E && !((taken >> i) & 1u) && (v[i] > best || bidx == 0x7fffffff)) { best = v[i]; bidx = e; }
-      }
+      for (int i = 0; i < NPER; ++i) best = max(best, v[i]);
+      best = __reduce_max_sync(0xffffffffu, best);
+      unsigned idx = 0xffffffffu;
 #pragma unroll
-      for (int o = 16; o >= 1; o >>= 1) {
-        const float ov = __shfl_xor_sync(0xffffffffu, best, o);
-        const int oi = __shfl_xor_sync(0xffffffffu, bidx, o);
-        if (oi != 0x7fffffff && (bidx == 0x7fffffff || ov > best || (ov == best && oi < bidx))) { best = ov; bidx = oi; }
-      }
-      if ((bidx & 31) == lane) taken |= 1u << (bidx >> 5);
-      if (lane == k) { sel_val = best; sel_idx = bidx; }
+      for (int i = NPER - 1; i >= 0; --i)
+        if (v[i] == best) idx = i * 32 + lane;
+      idx = __reduce_min_sync(0xffffffffu, idx);
+#pragma unroll
+      for (int i = 0; i < NPER; ++i)
+        if (i * 32 + lane == idx) v[i] = 0u;
+      if (lane == k) { sel_val = unsortable(best); sel_idx = (int)idx; }
     }
     const float m = __shfl_sync(0xffffffffu, sel_val, 0);       // the first pick is the maximum
     float ex = lane < K ? expf(sel_val - m) : 0.f;
@@ -561,20 +636,17 @@ k_route_topk(const float* __restrict__ logits, int T, int E, int K, int32_t* __r
 
 }  // namespace
 
-cudaError_t feplb_launch_block_hist(const int32_t* ids, int64_t S, int E, int R, int32_t* block_hist,
-                                    int32_t* counts, int32_t* rank_load, uint32_t* status,
-                                    cudaStream_t st, int64_t* n_launch) {
+cudaError_t feplb_launch_route_hist(const int32_t* ids, int64_t S, int E, int R, int32_t* totals, int32_t* counts,
+                                    int32_t* rank_load, uint32_t* status, cudaStream_t st, int64_t* n_launch) {
   cudaError_t err;
-  if (counts) {
-    if ((err = cudaMemsetAsync(counts, 0, sizeof(int32_t) * E, st)) != cudaSuccess) return err;
-    if ((err = cudaMemsetAsync(rank_load, 0, sizeof(int32_t) * R, st)) != cudaSuccess) return err;
-  }
   const int nb = (int)((S + FEPLB_SLOTS_PER_BLOCK - 1) / FEPLB_SLOTS_PER_BLOCK);
-  if (nb == 0) return cudaSuccess;
-  k_block_hist<<<nb, kThreads, sizeof(int) * kWarps * E, st>>>(ids, S, E, E / R, block_hist, counts, rank_load, status,
-                                                                (int32_t*)nullptr);
+  if (nb == 0) {
+    if ((err = cudaMemsetAsync(counts, 0, sizeof(int32_t) * E, st)) != cudaSuccess) return err;
+    return cudaMemsetAsync(rank_load, 0, sizeof(int32_t) * R, st);
+  }
   ++*n_launch;
-  return cudaGetLastError();
+  return launch(k_block_hist, nb, kThreads, sizeof(int) * kWarps * E, st, true, ids, S, E, E / R, (int32_t*)nullptr, counts,
+                rank_load, totals, status, (int32_t*)nullptr);
 }
 
 cudaError_t feplb_launch_permute(const int32_t* ids, int64_t S, int K, int E, int A, const int32_t* counts,
@@ -587,8 +659,8 @@ cudaError_t feplb_launch_permute(const int32_t* ids, int64_t S, int K, int E, in
   cudaError_t err;
   const int nb = (int)((S + FEPLB_SLOTS_PER_BLOCK - 1) / FEPLB_SLOTS_PER_BLOCK);
   if (nb) {
-    err = launch(k_block_hist, nb, kThreads, sizeof(int) * kWarps * E, st, false, ids, S, E, E, block_hist,
-                 (int32_t*)nullptr, (int32_t*)nullptr, status, slot_to_row);
+    err = launch(k_block_hist, nb, kThreads, sizeof(int) * kWarps * E, st, true, ids, S, E, E, block_hist,
+                 (int32_t*)nullptr, (int32_t*)nullptr, (int32_t*)nullptr, status, slot_to_row);
     ++*n_launch;
     if (err != cudaSuccess) return err;
   }
@@ -643,7 +715,7 @@ cudaError_t feplb_launch_route_fused(const int32_t* ids, int64_t S, int E, int R
   const int nb = (int)((S + FEPLB_SLOTS_PER_BLOCK - 1) / FEPLB_SLOTS_PER_BLOCK);
   if (nb) {
     err = launch(k_block_hist, nb, kThreads, sizeof(int) * kWarps * E, st, true, ids, S, E, E, block_hist,
-                 (int32_t*)nullptr, (int32_t*)nullptr, status, slot_to_row);
+                 (int32_t*)nullptr, (int32_t*)nullptr, (int32_t*)nullptr, status, slot_to_row);
     ++*n_launch;
     if (err != cudaSuccess) return err;
   }
@@ -659,8 +731,8 @@ bool feplb_front_is_small(int64_t S, int E) { return S > 0 && S <= kSmallMaxSlot
 
 template <int CH>
 static cudaError_t launch_small(const void* x, const int32_t* ids, int T, int K, int E, int R, int d, int A, int dyn,
-                                const uint8_t* mask_in, int32_t* counts, int32_t* rank_load, int32_t* pad_off, feplb_group* groups,
-                                int32_t* slot_to_row, int32_t* row_to_token, void* x_perm, int64_t s_cap, uint32_t* status,
+                                const uint8_t* mask_in, const int32_t* counts_in, int32_t* counts, int32_t* rank_load, int32_t* pad_off,
+                                feplb_group* groups, int32_t* slot_to_row, int32_t* row_to_token, void* x_perm, int64_t s_cap, uint32_t* status,
                                 unsigned long long* counts_host_tagged, int32_t seq, unsigned long long* t_counts, int num_sms,
                                 cudaStream_t st) {
   static bool ready[64] = {};                // per instantiation and device: the shared-memory attribute
@@ -678,18 +750,18 @@ static cudaError_t launch_small(const void* x, const int32_t* ids, int T, int K,
   const int grid = (int)(want < num_sms ? want : num_sms);
   const size_t smem = sizeof(int) * ((size_t)(kSmallWarps + 2) * E + (size_t)kSmallThreads * CH);
   return launch(k_route_small<CH>, grid, kSmallThreads, smem, st, true, (const uint4*)x, ids, T, K, E, E / R, A, dyn, mask_in,
-                counts, rank_load, pad_off, groups, slot_to_row, row_to_token, (uint4*)x_perm, chunks, s_cap, status,
+                counts_in, counts, rank_load, pad_off, groups, slot_to_row, row_to_token, (uint4*)x_perm, chunks, s_cap, status,
                 counts_host_tagged, seq, t_counts);
 }
 
 cudaError_t feplb_launch_front_small(const void* x, const int32_t* ids, int T, int K, int E, int R, int d, int A, int dyn,
-                                     const uint8_t* mask_in, int32_t* counts, int32_t* rank_load, int32_t* pad_off,
-                                     feplb_group* groups, int32_t* slot_to_row, int32_t* row_to_token, void* x_perm,
+                                     const uint8_t* mask_in, const int32_t* counts_in, int32_t* counts, int32_t* rank_load,
+                                     int32_t* pad_off, feplb_group* groups, int32_t* slot_to_row, int32_t* row_to_token, void* x_perm,
                                      int64_t s_cap, uint32_t* status, unsigned long long* counts_host_tagged, int32_t seq,
                                      unsigned long long* t_counts, int num_sms, cudaStream_t st, int64_t* n_launch) {
   const int S = T * K;
   auto go = [&](auto fn) {
-    return fn(x, ids, T, K, E, R, d, A, dyn, mask_in, counts, rank_load, pad_off, groups, slot_to_row, row_to_token, x_perm,
+    return fn(x, ids, T, K, E, R, d, A, dyn, mask_in, counts_in, counts, rank_load, pad_off, groups, slot_to_row, row_to_token, x_perm,
               s_cap, status, counts_host_tagged, seq, t_counts, num_sms, st);
   };
   ++*n_launch;
@@ -706,12 +778,8 @@ cudaError_t feplb_launch_route_topk(const float* logits, int T, int E, int K, in
   int blocks = (T + kWarps - 1) / kWarps;
   if (blocks > num_sms * 8) blocks = num_sms * 8;
   const int nper = (E + 31) / 32;
+  auto kernel = nper <= 1 ? k_route_topk<1> : nper <= 2 ? k_route_topk<2> : nper <= 4 ? k_route_topk<4>
+                : nper <= 8 ? k_route_topk<8> : nper <= 16 ? k_route_topk<16> : k_route_topk<32>;
   ++*n_launch;
-  if (nper <= 1) k_route_topk<1><<<blocks, kThreads, 0, st>>>(logits, T, E, K, ids, gates);
-  else if (nper <= 2) k_route_topk<2><<<blocks, kThreads, 0, st>>>(logits, T, E, K, ids, gates);
-  else if (nper <= 4) k_route_topk<4><<<blocks, kThreads, 0, st>>>(logits, T, E, K, ids, gates);
-  else if (nper <= 8) k_route_topk<8><<<blocks, kThreads, 0, st>>>(logits, T, E, K, ids, gates);
-  else if (nper <= 16) k_route_topk<16><<<blocks, kThreads, 0, st>>>(logits, T, E, K, ids, gates);
-  else k_route_topk<32><<<blocks, kThreads, 0, st>>>(logits, T, E, K, ids, gates);
-  return cudaGetLastError();
+  return launch(kernel, blocks, kThreads, 0, st, true, logits, T, E, K, ids, gates);
 }

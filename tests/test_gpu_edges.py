@@ -136,3 +136,39 @@ def test_backward_overhanging_n_tile(d, f, pair):
         _close(got.cpu().numpy().astype(np.float64)[: len(want)], want, what)
     _close(W.bf16_bits_to_f64(F.bf16_bits(bwd.d_x)), ref[0], "dx")
     case.close()
+
+
+@pytest.mark.parametrize("T,K,E,R", [(1, 1, 2, 1), (700, 3, 48, 3), (4097, 4, 60, 5), (1500, 8, 1024, 16), (20000, 2, 8, 2)])
+def test_route_hist_and_dispatch_repeat(T, K, E, R):
+    """The histogram's accumulators are left zero (the second call counts other ids from scratch); dispatch from one CTA
+    to many, few and many experts per scanning thread."""
+    import torch
+    w = W.get_workload("cfg1").with_(T=T, K=K, E=E, R=R, d=128, f=64)
+    cfg = F.config_from_workload(w)
+    ctx, buf = F.Context(cfg), F.Buffers(cfg)
+    x = W.gen_activations(w, 0)
+    for seed in (1, 2):
+        ids = np.random.default_rng(seed).integers(0, E, size=(T, K)).astype(np.int32)
+        d_ids = torch.from_numpy(ids).cuda()
+        ctx.route_hist(d_ids, buf.counts, buf.rank_load)
+        ctx.dispatch(F.bf16_tensor(x), d_ids, buf.counts, buf.x_perm, buf.slot_to_row, buf.row_to_token)
+        ctx.check_status()
+        counts, load = O.route_hist(ids, E, R)
+        assert np.array_equal(buf.counts.cpu().numpy(), counts) and np.array_equal(buf.rank_load.cpu().numpy(), load)
+        s2r, r2t, _, n = O.permute(ids, E, 1)
+        assert np.array_equal(buf.slot_to_row.cpu().numpy(), s2r) and np.array_equal(buf.row_to_token.cpu().numpy()[:n], r2t)
+        assert np.array_equal(F.bf16_bits(buf.x_perm)[:n], O.gather_rows(x, r2t))
+    ctx.close()
+
+
+def test_route_topk_signed_zeros_and_extremes():
+    """-0 and +0 tie (lower id first); largest, smallest and subnormal magnitudes keep their order."""
+    import torch
+    row = np.array([0.0, -0.0, 3.4e38, -3.4e38, 1e-42, -1e-42, -0.0, 0.0], np.float32)
+    logits = np.stack([row, row[::-1], np.roll(row, 3)])
+    ctx = F.Context(F.make_config(3, 8, 8, 1, 128, 64))
+    ids = torch.zeros(3, 8, dtype=torch.int32, device="cuda")
+    gates = torch.zeros(3, 8, device="cuda")
+    ctx.route_topk(torch.from_numpy(logits.copy()).cuda(), ids, gates)
+    assert np.array_equal(ids.cpu().numpy(), O.route_topk(logits, 8)[0])
+    ctx.close()
