@@ -363,7 +363,9 @@ int feplb_moe_forward(feplb_ctx* ctx, const void* x, const int32_t* topk_ids, co
 
 /* Same pass with HOST inputs and output: copies x, topk_ids, gates (host, ideally pinned) to
  * the device buffers x_dev, ids_dev, gates_dev, runs feplb_moe_forward, copies out_dev to
- * out_host, all on `stream`; returns after the stream has drained.  Weights stay resident. */
+ * out_host; returns after all of it has drained.  Weights stay resident.  Where the copies of a large batch take long
+ * enough beside its kernels it is processed in up to four token ranges, so that the copies of one (on the context's
+ * copy streams, ordered behind `stream`) run under the kernels of another; results are the same bit for bit. */
 int feplb_moe_forward_host(feplb_ctx* ctx, const void* x_host, const int32_t* topk_ids_host,
                            const float* gates_host, void* x_dev, int32_t* ids_dev, float* gates_dev,
                            const void* w1, const void* w3, const void* w2, const uint8_t* dyn_mask_host,

@@ -11,6 +11,7 @@
 #define FEPLB_MAX_GROUPS 1024
 #define FEPLB_SLOTS_PER_BLOCK 1024   // slots ranked by one CTA of the permutation kernels
 #define FEPLB_FRONT_SMALL_SLOTS 8192 // most slots of a batch whose routing and gather run as one launch
+#define FEPLB_MAX_RANGES 4           // token ranges a host-buffer forward is cut into at most
 #define FEPLB_TILE_M 128             // rows of one GEMM tile
 #ifndef FEPLB_NOALLOC_MAX_HIST_INTS
 #error "feplb.h must define FEPLB_NOALLOC_MAX_HIST_INTS"
@@ -48,7 +49,7 @@ cudaError_t feplb_launch_permute(const int32_t* ids, int64_t S, int K, int E, in
 cudaError_t feplb_launch_gather(const void* x, const int32_t* ids, const int32_t* block_base, int32_t* slot_to_row,
                                 const int32_t* counts, const int32_t* pad_off, void* x_perm, int T, int K, int E, int d,
                                 int A, int64_t s_cap, int num_sms, cudaStream_t st, int64_t* n_launch,
-                                int32_t* row_to_token, bool programmatic);
+                                int32_t* row_to_token, bool programmatic, int t0 = 0);   // tokens [t0, t0 + T)
 // Whole-layer path: histogram (+ ranks inside each CTA's slots) + one scan kernel that emits counts, rank
 // loads, offsets, the home group table and the -1 tail of row_to_token.
 cudaError_t feplb_launch_route_fused(const int32_t* ids, int64_t S, int E, int R, int A, int dyn,
@@ -57,6 +58,10 @@ cudaError_t feplb_launch_route_fused(const int32_t* ids, int64_t S, int E, int R
                                      int32_t* slot_to_row, int32_t* row_to_token, int64_t s_cap, uint32_t* status,
                                      unsigned long long* counts_host_tagged, int32_t seq, unsigned long long* t_counts,
                                      cudaStream_t st, int64_t* n_launch);
+// A batch processed in n_ranges token ranges (first_token[r] * K a multiple of FEPLB_SLOTS_PER_BLOCK): the group table of
+// range r goes to out + r * E.  block_base and home as feplb_launch_route_fused leaves them.
+cudaError_t feplb_launch_range_groups(const int32_t* block_base, int64_t S, int K, int E, const feplb_group* home,
+                                      const int* first_token, int n_ranges, feplb_group* out, cudaStream_t st, int64_t* n_launch);
 // Small batches: feplb_launch_route_fused and feplb_launch_gather in one launch; with groups == nullptr (and no mask,
 // counts, rank_load, pad_off) feplb_launch_permute and feplb_launch_gather, counts_in being the caller's counts.
 bool feplb_front_is_small(int64_t S, int E);

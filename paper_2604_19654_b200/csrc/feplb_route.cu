@@ -18,6 +18,8 @@
 
 namespace {
 
+struct RangeBlocks { int first[FEPLB_MAX_RANGES + 1]; };   // first CTA-of-1024-slots of every token range, and the end
+
 // Programmatic dependent launch: a kernel launched with the attribute below may be scheduled
 // while the kernel before it in the stream drains; pdl_sync() holds it until that kernel's
 // results are complete (a no-op for ordinary launches) and lets its own successor do the same.
@@ -331,7 +333,7 @@ __device__ __forceinline__ uint4 ld_nc_v4(const uint4* p) {
 // writes it to the K rows of its slots.  A slot's row = segment offset of its expert + first row of
 // its CTA-of-1024-slots within the segment (both from the scan) + its rank inside that CTA (left in
 // slot_to_row by k_block_hist); the warp that copies the first slice of a token writes the final
-// slot_to_row and row_to_token entries.  Another warp working on a later slice of the same token may
+// slot_to_row and row_to_token entries (tokens [t0, t0 + T) of the batch).  Another warp working on a later slice of the same token may
 // read either form of the entry, and gets the same row from both.
 constexpr int kGatherUnroll = 4;
 // Work unit = (token, slice of 4 x 32 chunks = 2 KiB of its row).  Unit u goes to warp u mod #warps of a grid
@@ -343,7 +345,8 @@ constexpr int kGatherUnroll = 4;
 __global__ void __launch_bounds__(kThreads)
 k_gather(const uint4* __restrict__ x, const int32_t* __restrict__ ids, const int32_t* __restrict__ pad_off,
          const int32_t* __restrict__ block_base, int32_t* slot_to_row, int32_t* __restrict__ row_to_token,
-         uint4* __restrict__ x_perm, int T, int K, int E, int chunks, int64_t s_cap, const int32_t* __restrict__ counts, int A) {
+         uint4* __restrict__ x_perm, int t0, int T, int K, int E, int chunks, int64_t s_cap, const int32_t* __restrict__ counts,
+         int A) {
   pdl_sync();
   const int lane = threadIdx.x & 31;
   const int64_t warp = ((int64_t)blockIdx.x * kThreads + threadIdx.x) >> 5;
@@ -351,8 +354,8 @@ k_gather(const uint4* __restrict__ x, const int32_t* __restrict__ ids, const int
   const int slices = (chunks + 32 * kGatherUnroll - 1) / (32 * kGatherUnroll);
   const int64_t units = (int64_t)T * slices;
   for (int64_t u = warp; u < units; u += nwarps) {
-    const int t = (int)(u / slices);
-    const int c0 = (int)(u - (int64_t)t * slices) * 32 * kGatherUnroll;
+    const int tu = (int)(u / slices), t = t0 + tu;
+    const int c0 = (int)(u - (int64_t)tu * slices) * 32 * kGatherUnroll;
     const uint4* src = x + (int64_t)t * chunks;
     uint4 v[kGatherUnroll];
 #pragma unroll
@@ -577,6 +580,21 @@ k_home_groups(const int32_t* __restrict__ counts, const uint8_t* __restrict__ ma
   if (mask_out) mask_out[e] = (uint8_t)is_dyn;
 }
 
+// Group tables of a batch processed in token ranges whose first slots are multiples of 1024: range r (one CTA) holds, per
+// expert, the rows of its slots, which lie side by side in the expert's segment because rows follow the slots.
+__global__ void __launch_bounds__(1024)
+k_range_groups(const int32_t* __restrict__ block_base, int nb, int E, const feplb_group* __restrict__ home, RangeBlocks rb,
+               feplb_group* __restrict__ out) {
+  pdl_sync();
+  const int e = threadIdx.x, b0 = rb.first[blockIdx.x], b1 = rb.first[blockIdx.x + 1];
+  if (e >= E) return;
+  feplb_group g = home[e];
+  const int lo = b0 < nb ? block_base[(int64_t)b0 * E + e] : g.rows, hi = b1 < nb ? block_base[(int64_t)b1 * E + e] : g.rows;
+  g.row_start += lo;
+  g.rows = hi - lo;
+  out[(int64_t)blockIdx.x * E + e] = g;
+}
+
 // Order-preserving map of finite floats to unsigned integers > 0; -0 and +0 map to the same value.
 __device__ __forceinline__ unsigned sortable(float f) {
   const unsigned u = __float_as_uint(f + 0.f);
@@ -672,7 +690,7 @@ cudaError_t feplb_launch_permute(const int32_t* ids, int64_t S, int K, int E, in
 cudaError_t feplb_launch_gather(const void* x, const int32_t* ids, const int32_t* block_base, int32_t* slot_to_row,
                                 const int32_t* counts, const int32_t* pad_off, void* x_perm, int T, int K, int E, int d,
                                 int A, int64_t s_cap, int num_sms, cudaStream_t st, int64_t* n_launch,
-                                int32_t* row_to_token, bool programmatic) {
+                                int32_t* row_to_token, bool programmatic, int t0) {
   const int chunks = d / 8;
   if (T == 0 && A == 1) return cudaSuccess;
   const int64_t units = (int64_t)T * ((chunks + 32 * kGatherUnroll - 1) / (32 * kGatherUnroll));
@@ -681,7 +699,7 @@ cudaError_t feplb_launch_gather(const void* x, const int32_t* ids, const int32_t
   if (need < blocks) blocks = (int)need;
   ++*n_launch;
   return launch(k_gather, blocks, kThreads, 0, st, programmatic, (const uint4*)x, ids, pad_off, block_base, slot_to_row,
-                row_to_token, (uint4*)x_perm, T, K, E, chunks, s_cap, counts, A);
+                row_to_token, (uint4*)x_perm, t0, T, K, E, chunks, s_cap, counts, A);
 }
 
 // Copies the planner's table of dynamic groups from mapped pinned host memory to the device.  A
@@ -722,6 +740,16 @@ cudaError_t feplb_launch_route_fused(const int32_t* ids, int64_t S, int E, int R
   ++*n_launch;
   return launch(k_scan_fused, 1, 1024, 0, st, true, block_hist, nb, E, E / R, A, dyn, mask_in, counts, rank_load, pad_off,
                 groups, mask_out, row_to_token, s_cap, counts_host_tagged, seq, t_counts);
+}
+
+cudaError_t feplb_launch_range_groups(const int32_t* block_base, int64_t S, int K, int E, const feplb_group* home,
+                                      const int* first_token, int n_ranges, feplb_group* out, cudaStream_t st, int64_t* n_launch) {
+  RangeBlocks rb = {};
+  const int nb = (int)((S + FEPLB_SLOTS_PER_BLOCK - 1) / FEPLB_SLOTS_PER_BLOCK);
+  for (int i = 0; i <= n_ranges; ++i)
+    rb.first[i] = i == n_ranges ? nb : (int)((int64_t)first_token[i] * K / FEPLB_SLOTS_PER_BLOCK);
+  ++*n_launch;
+  return launch(k_range_groups, n_ranges, 1024, 0, st, true, block_base, nb, E, home, rb, out);
 }
 
 // The one-launch front pays while the routing that every CTA repeats is short: its eight match rounds at 8192

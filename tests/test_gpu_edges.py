@@ -172,3 +172,41 @@ def test_route_topk_signed_zeros_and_extremes():
     ctx.route_topk(torch.from_numpy(logits.copy()).cuda(), ids, gates)
     assert np.array_equal(ids.cpu().numpy(), O.route_topk(logits, 8)[0])
     ctx.close()
+
+
+@pytest.mark.parametrize("T,K,E,d,f,A", [
+    (4096, 2, 8, 1024, 64, 1),        # four ranges of 1024 tokens
+    (5000, 3, 16, 1024, 64, 128),     # boundaries at multiples of 1024 tokens, padding rows, a ragged last range
+    (3000, 6, 24, 1920, 192, 1),      # boundaries at multiples of 512 tokens
+    (2049, 1, 8, 3072, 64, 1),        # ranges of 1024 and 1025 tokens
+])
+def test_host_forward_in_token_ranges(T, K, E, d, f, A):
+    """Batches whose host copies dominate are processed in token ranges; every buffer and the plan equal those of the
+    whole-batch path (device-resident forward) bit for bit."""
+    import torch
+    w = W.get_workload("cfg1").with_(T=T, K=K, E=E, d=d, f=f, tau=1)
+    case = DeviceCase(w, row_align=A)
+    p0 = case.ctx.moe_forward(case.d_x, case.d_ids, case.d_gates, case.d_w1, case.d_w3, case.d_w2, case.buf)
+    case.ctx.check_status()
+    n = int(p0.groups[-1][1] + p0.groups[-1][2])
+    names = ("counts", "rank_load", "slot_to_row", "row_to_token", "x_perm", "y_perm", "out")
+    want = {k: getattr(case.buf, k).clone() for k in names}
+    live = case.buf.row_to_token[:n] >= 0
+    for k in names:
+        getattr(case.buf, k).fill_(3)
+    host = [t.cpu().pin_memory() for t in (case.d_x, case.d_ids, case.d_gates)]
+    dev = [torch.zeros_like(t) for t in (case.d_x, case.d_ids, case.d_gates)]
+    out = torch.zeros(T, d, dtype=torch.bfloat16).pin_memory()
+    before = case.ctx.launch_count()
+    p1 = case.ctx.moe_forward_host(*host, *dev, case.d_w1, case.d_w3, case.d_w2, case.buf, out, want_plan=True)
+    case.ctx.check_status()
+    assert case.ctx.launch_count() - before >= 11                            # 3 + 4 per range: at least two ranges
+    assert (p1.moves, p1.groups) == (p0.moves, p0.groups)
+    assert torch.equal(out, want["out"].cpu())
+    for k in names:
+        got = getattr(case.buf, k)
+        if k in ("x_perm", "y_perm"):
+            assert torch.equal(got[:n][live], want[k][:n][live]), k
+        else:
+            assert torch.equal(got, want[k]), k
+    case.close()
