@@ -356,9 +356,11 @@ k_grouped_gemm(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__
       return true;
     };
     // The loads of one K block of one tile.  Pair form: both CTAs credit the LEADER's barrier; the leader
-    // announces the bytes of both.  A tile whose second 128 rows hold no valid row (a group of at most
-    // 128 rows, or a ragged tail) needs no A rows in the peer: it skips that load (the MMA then multiplies
-    // whatever its stage holds into accumulator rows nobody stores).
+    // announces the bytes of both.  For a tile whose second 128 rows hold no valid row (a group of at most
+    // 128 rows, or a ragged tail) the peer's A box lies past the end of the tensor: zeros arrive without
+    // any traffic from L2, and multiplying zeros takes less power than multiplying what a skipped load would
+    // leave in the stage, which is clock at the power cap (64 experts, d = 2048, T = 4096: 343.2 -> 337.1 us per
+    // layer).  Zeros for the partly valid 128 rows as well, by boxes of 32 rows, cost 4 % instead.
     auto few_rows = [&](const TileCoord& c) { return !PAIR && c.slot < 0 && c.rows_valid <= kFewRows; };
     auto load_b = [&](const TileCoord& c, int kb, int st) {      // announces the stage's bytes, loads the weights
       // weights of a migrated expert come from its slot of the receive buffer
@@ -370,7 +372,7 @@ k_grouped_gemm(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__
       const uint32_t half = (uint32_t)c.bn * BK * 2, box = (uint32_t)p.b_box * BK * 2;
       if (PAIR) {
         const uint32_t full0 = map_to_cta(full, 0);
-        if (cta_rank == 0) mbar_expect_tx(full, (c.rows_valid > BM ? 2 * kABytes : kABytes) + 2 * half);
+        if (cta_rank == 0) mbar_expect_tx(full, 2 * kABytes + 2 * half);
         const CUtensorMap* mb = cta_rank == 0 ? mb0 : mb1;
         const int r0 = row + (!SWIGLU && cta_rank ? c.bn : 0);
         for (uint32_t o = 0, r = 0; o < half; o += box, r += p.b_box) tma_load_2d_pair(sb + o, mb, full0, kb * BK, r0 + (int)r);
@@ -387,7 +389,8 @@ k_grouped_gemm(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__
       const uint32_t full = smem_u32(&tail->full[st]);
       const uint32_t sa = smem_u32(smem + (size_t)st * kStageBytes);
       if (PAIR) {
-        if (cta_rank == 0 || c.rows_valid > BM) tma_load_2d_pair(sa, ma, map_to_cta(full, 0), kb * BK, c.row0 + (int)cta_rank * BM);
+        tma_load_2d_pair(sa, ma, map_to_cta(full, 0), kb * BK,
+                         cta_rank == 0 ? c.row0 : c.rows_valid > BM ? c.row0 + BM : (int)p.s_cap);
       } else {
         tma_load_2d(sa, few_rows(c) ? &tm_as : ma, full, kb * BK, c.row0);
       }

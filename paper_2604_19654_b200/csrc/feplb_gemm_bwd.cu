@@ -333,7 +333,8 @@ k_ffn_bwd_gemm(const __grid_constant__ Maps<KIND> maps, const __grid_constant__ 
               const CUtensorMap* mb = (KIND == KIND_DX && kb >= p.k_switch) ? &maps.b[1] : &maps.b[0];
               const int kb_b = (KIND == KIND_DX && kb >= p.k_switch) ? kb - p.k_switch : kb;
               const int brow = c.expert * p.b_rows_per_expert + c.nt * 2 * bn + (int)cta_rank * bn;
-              tma_load_2d_pair(sa, ma, full0, kb * BK, c.row0 + (int)cta_rank * BM);
+              // (no valid row among the second 128: past the end of the tensor, zeros; see feplb_gemm.cu)
+              tma_load_2d_pair(sa, ma, full0, kb * BK, cta_rank == 0 ? c.row0 : c.rows_valid > BM ? c.row0 + BM : (int)p.s_cap);
               tma_load_2d_pair(sb, mb, full0, kb_b * BK, brow);
             }
             if (++stage == NS) { stage = 0; phase ^= 1u; }
