@@ -119,7 +119,8 @@ typedef struct {
   /* Merged launches only (one launch per pass walks the static, then the dynamic groups); the
    * marks are taken inside the kernels from the GPU's global timer.  There dev_static_ffn_us is the
    * whole expert FFN, dev_dynamic_ffn_us is 0, dev_counts_to_static_start_us ends at the first CTA's
-   * start and dev_counts_to_static_end_us at the first moment a CTA ran out of static work. */
+   * start and dev_counts_to_static_end_us at the first moment a CTA ran out of static work -- or
+   * at the end of pass 1, when the planner's table was on the device before the launch. */
   double dev_ffn_pass1_us, dev_ffn_pass2_us; /* device: first CTA's start -> last CTA's end of each pass */
   double dev_plan_wait_us;              /* device: longest time a CTA spent waiting for the dynamic table */
   double ffn_launches;                  /* GEMM launches of the forward: 4 (static, dynamic x 2 passes) or 2 */
@@ -428,11 +429,14 @@ int feplb_set_gemm_form(feplb_ctx* ctx, int32_t forward_form, int32_t backward_p
 /* How feplb_moe_forward launches the expert GEMMs.  merged = 1: one launch per pass runs the static
  * groups (Section 2.3: while the CPU balancer works) and then the dynamic groups, whose table it
  * picks up on the device with a bounded wait on a word the planner thread writes into mapped host
- * memory -- two launches per forward, everything enqueued before the planner is joined, the
- * static-first order kept inside each launch.  merged = 0: static and dynamic groups in launches of
+ * memory -- two launches per forward, everything enqueued before the planner is joined.  Usually the
+ * planner is done while the rows are gathered; the gather then brings its table to the device and
+ * each launch runs static and dynamic groups side by side, otherwise static first.  merged = 0: static and dynamic groups in launches of
  * their own (four per forward), the dynamic ones enqueued after the planner has been joined and
  * each table in the form that suits it.  -1 (default): merged while a forward's groups are small
- * (below ~768 rows per expert).  With cfg.phase2_copy the four-launch order is always used.
+ * (below ~768 rows per expert), and for the smallest batches (below 128 rows per expert, or ~150 us
+ * of expert FFN) two launches over the home groups that do not depend on the plan at all, which the
+ * calling thread makes after it has enqueued them.  With cfg.phase2_copy the four-launch order is always used.
  * merged = 1 needs 2*E + R*max_num_dyn <= 1024.  Not allowed while a plan is pending. */
 int feplb_set_launch_merging(feplb_ctx* ctx, int32_t merged);
 /* Test and tuning aid for the merged launches of feplb_moe_forward.  planner_delay_us: the

@@ -57,7 +57,7 @@ struct feplb_ctx {
   int32_t* h_dyn_tab32 = nullptr;                    // pinned + mapped: the dynamic table as 32-byte entries tagged with the sequence number
   int32_t* h_dyn_tab32_dev = nullptr;                // its device address
   int32_t* d_dyn_tab32 = nullptr;                    // device copy, made by the GEMM's claiming CTA
-  unsigned long long* d_dyn_ready = nullptr;         // device words: [0] ready, [1] claim
+  unsigned long long* d_dyn_ready = nullptr;         // device words: [0] ready, [1] claim, [2] early
   unsigned long long* h_dyn_ready = nullptr;         // pinned + mapped word, set by the planner thread
   unsigned long long* h_dyn_ready_dev = nullptr;     // its device address
   unsigned long long* d_stamps = nullptr;            // [kEvRing][kStampWords] globaltimer marks of the kernels
@@ -398,8 +398,8 @@ extern "C" int feplb_create(const feplb_config* cfg, feplb_ctx** out) {
   const double ffn_us = 6.0 * cfg->d * cfg->f * ((double)cfg->E / 6.5e6 + (double)S / 1e9);
   c->direct_auto = c->direct = S < (int64_t)FEPLB_DIRECT_ROWS_PER_EXPERT * cfg->E || ffn_us < FEPLB_DIRECT_FFN_US;
   bool ok = true;
-  ok = ok && cudaMalloc(&c->d_dyn_ready, 2 * sizeof(unsigned long long)) == cudaSuccess &&     // [0] ready word, [1] claim word
-       cudaMemset(c->d_dyn_ready, 0, 2 * sizeof(unsigned long long)) == cudaSuccess;
+  ok = ok && cudaMalloc(&c->d_dyn_ready, 3 * sizeof(unsigned long long)) == cudaSuccess &&     // [0] ready word, [1] claim word, [2] early word
+       cudaMemset(c->d_dyn_ready, 0, 3 * sizeof(unsigned long long)) == cudaSuccess;
   ok = ok && cudaHostAlloc(&c->h_dyn_ready, sizeof(unsigned long long), cudaHostAllocMapped) == cudaSuccess &&
        cudaHostGetDevicePointer(&c->h_dyn_ready_dev, c->h_dyn_ready, 0) == cudaSuccess;
   if (ok) *c->h_dyn_ready = 0;
@@ -854,13 +854,20 @@ extern "C" int feplb_moe_forward(feplb_ctx* c, const void* x, const int32_t* top
   if (!direct && (rc = plan_kick_flag(c, dyn_mask_host, seq, wm)) != FEPLB_OK) return rc;
   TL_EVENT(EV_COUNTS);
   TL_EVENT(EV_HIST);
+  // how the merged launches, and the gather in front of them, get the planner's table
+  feplb_wm_dyn dyn;
+  dyn.table_dev = c->d_dyn_tab32; dyn.table_host = c->h_dyn_tab32_dev;
+  dyn.ready_dev = c->d_dyn_ready; dyn.ready_host = c->h_dyn_ready_dev;
+  dyn.claim = reinterpret_cast<uint32_t*>(c->d_dyn_ready + 1); dyn.early = c->d_dyn_ready + 2;
+  dyn.seq = direct || !wm ? 0u : (uint32_t)seq; dyn.max_groups = direct ? 0 : c->plan.cap_groups; dyn.stamps = stamps;
+  dyn.wait_limit_ns = 1000ull * (unsigned long long)c->device_wait_limit_us;
   // step 3: permutation (does not depend on the plan: a migration relabels rows, it does not move
   // them here).  From here on a failure must still join the planner, so errors are carried in rc.
   {
     cudaError_t e = cudaSuccess;
     if (!small_front)
       e = feplb_launch_gather(x, topk_ids, c->d_block_hist, slot_to_row, counts, c->d_pad_off, x_perm, g.T, g.K, g.E, g.d,
-                              g.row_align, (int64_t)c->s_cap, c->num_sms, st, &c->launches, row_to_token, true);
+                              g.row_align, (int64_t)c->s_cap, c->num_sms, st, &c->launches, row_to_token, true, 0, &dyn, c->d_status);
     if (e == cudaSuccess && g.phase2_copy) {
       // the planner's row copies of Phase 2 wait for the permuted rows
       e = cudaEventRecord(c->ev_gather, st);
@@ -873,12 +880,6 @@ extern "C" int feplb_moe_forward(feplb_ctx* c, const void* x, const int32_t* top
   if (wm) {
     // steps 4 + 5 in two launches: static groups from the table built on the device, then the dynamic
     // groups as soon as the planner has published them (bounded wait inside the kernel)
-    feplb_wm_dyn dyn;
-    dyn.table_dev = c->d_dyn_tab32; dyn.table_host = c->h_dyn_tab32_dev;
-    dyn.ready_dev = c->d_dyn_ready; dyn.ready_host = c->h_dyn_ready_dev;
-    dyn.claim = reinterpret_cast<uint32_t*>(c->d_dyn_ready + 1);
-    dyn.seq = direct ? 0u : (uint32_t)seq; dyn.max_groups = direct ? 0 : c->plan.cap_groups; dyn.stamps = stamps;
-    dyn.wait_limit_ns = 1000ull * (unsigned long long)c->device_wait_limit_us;
     if (rc == FEPLB_OK)
       rc = ffn_impl(c, x_perm, w1, w3, w2, c->d_home_groups, g.E, direct ? FEPLB_FFN_ALL : FEPLB_FFN_STATIC, h_scratch, y_perm, st,
                     c->gemm_pair_forced >= 0 ? c->gemm_pair_forced : (int)c->merged_pair, &dyn);

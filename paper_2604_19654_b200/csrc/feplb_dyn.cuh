@@ -2,6 +2,10 @@
 // the CPU balancer computes the plan while the GPU runs the static experts, so the launch that
 // goes on from the static to the dynamic groups is enqueued before the table exists).
 //
+// Usually the table is there before the GEMM starts: a CTA of the row gather, which runs while the planner works, picks it
+// up (dyn_deliver_early), and the launches walk static and dynamic groups together, in expert order.  What follows is
+// for a table that comes later than that.
+//
 // The planner thread writes the table -- 32-byte entries {expert, row_start, rows, exec_rank,
 // is_dynamic, seq, 0, 0} -- and then the word (seq << 32) | number of groups into mapped host
 // memory.  Of the CTAs that have run out of static work, the first one claims the transfer: it alone
@@ -32,6 +36,7 @@ struct DynTable {
   const int4* dyn_host;                 // ... the planner's own table in mapped host memory
   unsigned long long* ready_dev;        // (seq << 32) | number of dynamic groups
   const unsigned long long* ready_host;
+  unsigned long long* early;            // seq of the forward whose table was on the device before its GEMM launches started
   uint32_t* claim;                      // device word: seq of the forward whose table transfer has been claimed
   int dyn_cap;                          // capacity of dyn_dev in groups
   uint32_t seq;                         // 0: no dynamic table in this launch
@@ -59,6 +64,35 @@ __device__ __forceinline__ bool dyn_entry(const DynTable& d, int i, int& expert,
 // The number of groups a peek at the device-side word shows, or -1 if the word is not this forward's.
 __device__ __forceinline__ int dyn_peek_count(const DynTable& d, unsigned long long word) {
   return (uint32_t)(word >> 32) == d.seq && (int)(uint32_t)word != kDynGaveUp ? (int)(uint32_t)word : -1;
+}
+
+// Warp-collective: copies the planner's table to its device copy and sets the device-side word.  Ordinary (weak) 16-byte
+// loads coalesce into a few PCIe reads; entries that do not carry the sequence number yet are read again.
+__device__ __forceinline__ int dyn_bring_table(const DynTable& d, int lane, uint32_t* status, int n_dyn) {
+  if (n_dyn < 0 || n_dyn > d.dyn_cap) {
+    if (lane == 0) atomicOr(status, FEPLB_ST_GROUP);
+    n_dyn = 0;
+  }
+  bool good = false;
+  for (int attempt = 0; attempt < 64 && !good; ++attempt) {
+    good = true;
+    for (int i = lane; i < n_dyn; i += 32) {
+      const int4 lo = __ldcv(d.dyn_host + 2 * i), hi = __ldcv(d.dyn_host + 2 * i + 1);
+      if ((uint32_t)hi.y != d.seq) { good = false; continue; }
+      d.dyn_dev[2 * i] = lo;
+      d.dyn_dev[2 * i + 1] = hi;
+    }
+    good = __all_sync(0xffffffffu, good);
+  }
+  if (!good) {
+    if (lane == 0) atomicOr(status, FEPLB_ST_GROUP);
+    n_dyn = 0;
+  }
+  __syncwarp();                      // the lanes' stores happen before lane 0's release below
+  if (lane == 0)
+    asm volatile("st.release.gpu.global.u64 [%0], %1;" ::"l"(d.ready_dev),
+                 "l"(((unsigned long long)d.seq << 32) | (uint32_t)n_dyn) : "memory");
+  return n_dyn;
 }
 
 // Warp-collective, called by a CTA that has nothing left to do without the table.  Waits (bounded by
@@ -106,32 +140,26 @@ __device__ __forceinline__ int dyn_wait_table(const DynTable& d, int lane, volat
     if (n_dyn == kDynGaveUp && lane == 0) atomicOr(status, FEPLB_ST_PLAN);
     return n_dyn;
   }
-  // got == 2: bring the table over.  Ordinary (weak) 16-byte loads coalesce into a few PCIe reads;
-  // entries that do not carry the sequence number yet are read again.
-  if (n_dyn < 0 || n_dyn > d.dyn_cap) {
-    if (lane == 0) atomicOr(status, FEPLB_ST_GROUP);
-    n_dyn = 0;
+  return dyn_bring_table(d, lane, status, n_dyn);          // got == 2
+}
+
+// Warp-collective, by one CTA of the kernel in front of the GEMM (the row gather, which usually takes longer than the
+// planner): waits at most limit_ns for the planner's table and brings it over, so that the GEMM launches know it from
+// the start and need not run the static groups first.  When it is late nothing is left behind.
+__device__ __forceinline__ void dyn_deliver_early(const DynTable& d, int lane, uint32_t* status, unsigned long long limit_ns) {
+  unsigned long long v = 0;
+  int there = 0;
+  if (lane == 0) {
+    const unsigned long long t0 = global_timer_ns();
+    do {
+      v = ld_relaxed_sys_u64(d.ready_host);
+      there = (uint32_t)(v >> 32) == d.seq;
+      if (!there) __nanosleep(100);
+    } while (!there && global_timer_ns() - t0 <= limit_ns);
   }
-  bool good = false;
-  for (int attempt = 0; attempt < 64 && !good; ++attempt) {
-    good = true;
-    for (int i = lane; i < n_dyn; i += 32) {
-      const int4 lo = __ldcv(d.dyn_host + 2 * i), hi = __ldcv(d.dyn_host + 2 * i + 1);
-      if ((uint32_t)hi.y != d.seq) { good = false; continue; }
-      d.dyn_dev[2 * i] = lo;
-      d.dyn_dev[2 * i + 1] = hi;
-    }
-    good = __all_sync(0xffffffffu, good);
-  }
-  if (!good) {
-    if (lane == 0) atomicOr(status, FEPLB_ST_GROUP);
-    n_dyn = 0;
-  }
-  __syncwarp();                      // the lanes' stores happen before lane 0's release below
-  if (lane == 0)
-    asm volatile("st.release.gpu.global.u64 [%0], %1;" ::"l"(d.ready_dev),
-                 "l"(((unsigned long long)d.seq << 32) | (uint32_t)n_dyn) : "memory");
-  return n_dyn;
+  if (!__shfl_sync(0xffffffffu, there, 0)) return;
+  dyn_bring_table(d, lane, status, __shfl_sync(0xffffffffu, (int)(uint32_t)v, 0));
+  if (lane == 0) *reinterpret_cast<volatile unsigned long long*>(d.early) = d.seq;
 }
 
 // Kernel parameter from the host-side description.
@@ -142,6 +170,7 @@ inline DynTable feplb_dyn_table(const feplb_wm_dyn& dyn) {
   d.ready_dev = dyn.ready_dev;
   d.ready_host = dyn.ready_host;
   d.claim = dyn.claim;
+  d.early = dyn.early;
   d.dyn_cap = dyn.max_groups;
   d.seq = dyn.seq;
   d.wait_limit_ns = dyn.wait_limit_ns ? dyn.wait_limit_ns : kWaitLimitNs;

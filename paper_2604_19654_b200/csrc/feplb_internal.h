@@ -43,13 +43,30 @@ cudaError_t feplb_launch_permute(const int32_t* ids, int64_t S, int K, int E, in
                                  int32_t* block_hist, int32_t* pad_off, int32_t* slot_to_row,
                                  int32_t* row_to_token, int64_t s_cap, uint32_t* status,
                                  cudaStream_t st, int64_t* n_launch);
+// A launch per pass walks a.groups (filtered by a.which) and then, if dyn.seq != 0, the planner's dynamic
+// table, which it picks up on the device once the host-side ready word carries (seq << 32) | number of
+// groups; the CTA that wins `claim` copies it to table_dev (feplb_dyn.cuh).
+struct feplb_wm_dyn {
+  // the table travels as 32-byte entries {expert, row_start, rows, exec_rank, is_dynamic, seq, 0, 0}
+  void* table_dev = nullptr;                         // device copy of the table, written by the claiming CTA
+  const void* table_host = nullptr;                  // device address of the planner's table in mapped host memory
+  unsigned long long* ready_dev = nullptr;           // set by the claiming CTA after table_dev
+  const unsigned long long* ready_host = nullptr;    // device address of the word the planner thread sets after table_host
+  uint32_t* claim = nullptr;                         // device word the CTAs race for
+  unsigned long long* early = nullptr;               // device word: seq of the forward whose table the gather brought over
+  uint32_t seq = 0;                                  // 0: no dynamic table
+  int max_groups = 0;                                // capacity of the tables
+  unsigned long long* stamps = nullptr;              // optional, 8 words: globaltimer marks of the two launches
+  unsigned long long wait_limit_ns = 0;              // bound of the wait for the table (0: the library's default)
+};
 // Must follow feplb_launch_permute or feplb_launch_route_fused on the same stream: turns the ranks those
 // left in slot_to_row into rows (block_base = the scanned per-CTA histograms), fills row_to_token and
 // copies the rows of x.
 cudaError_t feplb_launch_gather(const void* x, const int32_t* ids, const int32_t* block_base, int32_t* slot_to_row,
                                 const int32_t* counts, const int32_t* pad_off, void* x_perm, int T, int K, int E, int d,
                                 int A, int64_t s_cap, int num_sms, cudaStream_t st, int64_t* n_launch,
-                                int32_t* row_to_token, bool programmatic, int t0 = 0);   // tokens [t0, t0 + T)
+                                int32_t* row_to_token, bool programmatic, int t0 = 0,          // tokens [t0, t0 + T)
+                                const feplb_wm_dyn* dyn = nullptr, uint32_t* status = nullptr);   // pick the planner's table up along the way
 // Whole-layer path: histogram (+ ranks inside each CTA's slots) + one scan kernel that emits counts, rank
 // loads, offsets, the home group table and the -1 tail of row_to_token.
 cudaError_t feplb_launch_route_fused(const int32_t* ids, int64_t S, int E, int R, int A, int dyn,
@@ -95,21 +112,6 @@ struct feplb_gemm_args {
 // Returns FEPLB_OK or a feplb_status; text of a failure goes to err (size errn).
 // One thread waits (bounded by limit_ns) on an mbarrier nobody completes; *gave_up = 1 and FEPLB_ST_WAIT expected.
 cudaError_t feplb_launch_wait_selftest(uint32_t* status, unsigned long long limit_ns, int* gave_up, cudaStream_t st);
-// A launch per pass walks a.groups (filtered by a.which) and then, if dyn.seq != 0, the planner's dynamic
-// table, which it picks up on the device once the host-side ready word carries (seq << 32) | number of
-// groups; the CTA that wins `claim` copies it to table_dev (feplb_dyn.cuh).
-struct feplb_wm_dyn {
-  // the table travels as 32-byte entries {expert, row_start, rows, exec_rank, is_dynamic, seq, 0, 0}
-  void* table_dev = nullptr;                         // device copy of the table, written by the claiming CTA
-  const void* table_host = nullptr;                  // device address of the planner's table in mapped host memory
-  unsigned long long* ready_dev = nullptr;           // set by the claiming CTA after table_dev
-  const unsigned long long* ready_host = nullptr;    // device address of the word the planner thread sets after table_host
-  uint32_t* claim = nullptr;                         // device word the CTAs race for
-  uint32_t seq = 0;                                  // 0: no dynamic table
-  int max_groups = 0;                                // capacity of the tables
-  unsigned long long* stamps = nullptr;              // optional, 8 words: globaltimer marks of the two launches
-  unsigned long long wait_limit_ns = 0;              // bound of the wait for the table (0: the library's default)
-};
 // Tokens-on-M forms (feplb_gemm.cu): single CTA per 128-row tile or, with a.pair, clusters of two on 256-row tiles.
 int feplb_launch_expert_ffn(const feplb_gemm_args& a, cudaStream_t st, int64_t* n_launch, char* err, size_t errn,
                             const feplb_wm_dyn* dyn = nullptr);

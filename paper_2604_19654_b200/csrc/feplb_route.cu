@@ -14,6 +14,7 @@
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 
+#include "feplb_dyn.cuh"
 #include "feplb_internal.h"
 
 namespace {
@@ -336,6 +337,7 @@ __device__ __forceinline__ uint4 ld_nc_v4(const uint4* p) {
 // slot_to_row and row_to_token entries (tokens [t0, t0 + T) of the batch).  Another warp working on a later slice of the same token may
 // read either form of the entry, and gets the same row from both.
 constexpr int kGatherUnroll = 4;
+constexpr unsigned long long kEarlyTableNs = 15000;   // the planner publishes its table about 5 us after the scan
 // Work unit = (token, slice of 4 x 32 chunks = 2 KiB of its row).  Unit u goes to warp u mod #warps of a grid
 // sized to the machine: all warps work on neighbouring tokens at any time, and the rows of an expert, which
 // follow the token order, are written in one moving window per expert, so that DRAM pages are written while
@@ -346,11 +348,16 @@ __global__ void __launch_bounds__(kThreads)
 k_gather(const uint4* __restrict__ x, const int32_t* __restrict__ ids, const int32_t* __restrict__ pad_off,
          const int32_t* __restrict__ block_base, int32_t* slot_to_row, int32_t* __restrict__ row_to_token,
          uint4* __restrict__ x_perm, int t0, int T, int K, int E, int chunks, int64_t s_cap, const int32_t* __restrict__ counts,
-         int A) {
+         int A, const DynTable dyn, uint32_t* status) {
   pdl_sync();
   const int lane = threadIdx.x & 31;
-  const int64_t warp = ((int64_t)blockIdx.x * kThreads + threadIdx.x) >> 5;
-  const int64_t nwarps = ((int64_t)gridDim.x * kThreads) >> 5;
+  const int first = dyn.seq != 0;        // the first CTA picks the planner's table up
+  if (first && blockIdx.x == 0) {
+    if (threadIdx.x < 32) dyn_deliver_early(dyn, lane, status, kEarlyTableNs);
+    return;
+  }
+  const int64_t warp = ((int64_t)(blockIdx.x - first) * kThreads + threadIdx.x) >> 5;
+  const int64_t nwarps = ((int64_t)(gridDim.x - first) * kThreads) >> 5;
   const int slices = (chunks + 32 * kGatherUnroll - 1) / (32 * kGatherUnroll);
   const int64_t units = (int64_t)T * slices;
   for (int64_t u = warp; u < units; u += nwarps) {
@@ -690,16 +697,19 @@ cudaError_t feplb_launch_permute(const int32_t* ids, int64_t S, int K, int E, in
 cudaError_t feplb_launch_gather(const void* x, const int32_t* ids, const int32_t* block_base, int32_t* slot_to_row,
                                 const int32_t* counts, const int32_t* pad_off, void* x_perm, int T, int K, int E, int d,
                                 int A, int64_t s_cap, int num_sms, cudaStream_t st, int64_t* n_launch,
-                                int32_t* row_to_token, bool programmatic, int t0) {
+                                int32_t* row_to_token, bool programmatic, int t0, const feplb_wm_dyn* dyn, uint32_t* status) {
   const int chunks = d / 8;
   if (T == 0 && A == 1) return cudaSuccess;
   const int64_t units = (int64_t)T * ((chunks + 32 * kGatherUnroll - 1) / (32 * kGatherUnroll));
   int blocks = num_sms * 8;   // 8 CTAs of 256 threads per SM are resident
   const int64_t need = ((A > 1 && units < (int64_t)E * A ? (int64_t)E * A : units) + kWarps - 1) / kWarps;
   if (need < blocks) blocks = (int)need;
+  const feplb_wm_dyn none;
+  if (dyn && dyn->seq && blocks < num_sms * 8) ++blocks;
   ++*n_launch;
   return launch(k_gather, blocks, kThreads, 0, st, programmatic, (const uint4*)x, ids, pad_off, block_base, slot_to_row,
-                row_to_token, (uint4*)x_perm, t0, T, K, E, chunks, s_cap, counts, A);
+                row_to_token, (uint4*)x_perm, t0, T, K, E, chunks, s_cap, counts, A,
+                feplb_dyn_table(dyn ? *dyn : none), status);
 }
 
 // Copies the planner's table of dynamic groups from mapped pinned host memory to the device.  A

@@ -210,3 +210,21 @@ def test_host_forward_in_token_ranges(T, K, E, d, f, A):
         else:
             assert torch.equal(got, want[k]), k
     case.close()
+
+
+@pytest.mark.parametrize("form", [F.FORM_SINGLE, F.FORM_PAIR, F.FORM_WEIGHT_M])
+@pytest.mark.parametrize("E,R,split", [(16, 4, 0), (16, 4, 1), (6, 3, 1), (64, 2, 0)])
+def test_table_brought_over_by_the_gather(E, R, split, form):
+    """The planner's table on the device before the GEMM (merged into the home table, whole experts and several pieces of
+    one) and after its start (planner held back): the same integers and the same rows bit for bit."""
+    w = W.get_workload("cfg4").with_(T=3000, K=4, E=E, R=R, d=256, f=128, dyn=3, max_num_dyn=4, tau=8, routing="dirichlet", alpha=0.3)
+    case = DeviceCase(w, split=split, split_granule=64)
+    case.ctx.set_gemm_form(form)
+    case.ctx.set_launch_merging(1)
+    p0, _ = _check_forward(case, sample=200)
+    out = F.bf16_bits(case.buf.out).copy()
+    case.ctx.set_planner_timing(planner_delay_us=2000)
+    p1, _ = _check_forward(case, sample=20)
+    assert p0.groups == p1.groups and len(p0.moves) > 0
+    assert np.array_equal(F.bf16_bits(case.buf.out), out)
+    case.close()
