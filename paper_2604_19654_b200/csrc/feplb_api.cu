@@ -374,18 +374,22 @@ extern "C" int feplb_create(const feplb_config* cfg, feplb_ctx** out) {
   c->nb = (int)((S + FEPLB_SLOTS_PER_BLOCK - 1) / FEPLB_SLOTS_PER_BLOCK);
   const int cap_moves = cfg->R * cfg->max_num_dyn;
   const int cap_groups = cfg->E + cap_moves;
-  // Weights-on-M form: pays while groups are a few hundred rows (less padding, an expert's weights cross
-  // the L2 port once per 256 rows); from ~1000 rows per expert the two-CTA form keeps its lead because
-  // it can overlap every tile's epilogue with the next tile's MMAs.
+  // Weights-on-M form: no padding rows to speak of, and an expert's weights cross the L2 ports once per 256 rows; its units
+  // are only worth their transposed epilogue where they are long.  Steady state, tokens-on-M -> weights-on-M, us per
+  // layer: d = 6144, f = 2048, 128 experts: 64 rows per expert 1384 -> 1368, 128 2007 -> 1913, 256 3204 -> 2971, 512 5149 ->
+  // 5001, 1024 9070 -> 9061; d = 6144, f = 512, 384 rows 705 -> 681; d = 4096, f = 1024, 256 rows 1138 -> 1084;
+  // d = f = 2048, 384 rows 745 -> 730; but d = 2048, f = 768: 187 rows 210 -> 212, 384 327 -> 328, 562 437 -> 440, and
+  // below 64 rows weights stream as fast in 128-row tiles (32 rows 1189 -> 1200).
   c->wm_ok = feplb_wm_supported(cfg->E, cfg->d, cfg->f, cfg->E + cap_groups);
-  c->wm_auto = c->wm = false;      // measured a few percent behind the tokens-on-M forms at every benchmarked size: on request only
+  c->wm_auto = c->wm = c->wm_ok && S >= (int64_t)FEPLB_WM_MIN_ROWS_PER_EXPERT * cfg->E &&
+                       S < (int64_t)FEPLB_MERGED_MAX_ROWS_PER_EXPERT * cfg->E && (int64_t)cfg->d * cfg->f >= FEPLB_WM_MIN_WEIGHT;
   // One launch per pass over the static and then the dynamic groups (the table of the latter is
   // picked up on the device): saves two launch ramps and two partly filled last waves per forward,
   // which matters while a forward's GEMMs take a few hundred microseconds; one form serves both
   // tables then, so it stays off where the dynamic groups want the two-CTA form and the static ones
   // do not (from ~1000 rows per expert).
   c->merged_ok = cfg->E + cap_groups <= FEPLB_MAX_GROUPS;
-  c->merged_auto = c->merged = c->merged_ok && S < (int64_t)FEPLB_WM_AUTO_ROWS_PER_EXPERT * cfg->E;
+  c->merged_auto = c->merged = c->merged_ok && S < (int64_t)FEPLB_MERGED_MAX_ROWS_PER_EXPERT * cfg->E;
   // Small batches: a migration only relabels the rank that executes rows whose weights are the same everywhere, so
   // the launches need not wait for the plan at all.  They do where the static groups keep the GPU busy for longer
   // than the planner takes (its table is then there in time); below that the wait and the table's way to the

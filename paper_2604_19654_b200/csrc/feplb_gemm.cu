@@ -238,32 +238,6 @@ __device__ __forceinline__ void warp_scan_prefix(SmemTail* t, int first, int n, 
   __syncwarp();
 }
 
-// The planner's table is there already: its groups join the home table, one group of each dynamic expert (the first piece
-// of its segment) in the expert's own entry, which the static selection left empty, further pieces behind the
-// others.  In expert order the large dynamic groups, bound by the tensor pipe and the power cap, run side by side with
-// the small static ones, bound by weight traffic: 64 experts, d = 2048, T = 4096 348.9 -> 338.2 us per layer against all
-// static groups first.  Returns the number of entries.  One warp.
-template <int kRows>
-__device__ __forceinline__ int merge_table(SmemTail* t, const GemmParams& p, int lane) {
-  const int n_dyn = min((int)(uint32_t)ld_relaxed_gpu_u64(p.dyn.ready_dev), FEPLB_MAX_GROUPS - p.n_groups);
-  int n = p.n_groups;
-  for (int i0 = 0; i0 < n_dyn; i0 += 32) {
-    int e = 0, rs = 0, rw = 0, dy = 0;
-    const bool have = i0 + lane < n_dyn;
-    if (have && !dyn_entry(p.dyn, i0 + lane, e, rs, rw, dy)) {
-      atomicOr(p.status, FEPLB_ST_GROUP);
-      rw = 0;
-    }
-    const bool own = have && e >= 0 && e < p.n_groups && t->g_row_start[e] == rs && t->prefix[e + 1] == 0;
-    const unsigned others = __ballot_sync(0xffffffffu, have && !own);
-    const int idx = own ? e : n + __popc(others & ((1u << lane) - 1u));
-    if (have) t->prefix[idx + 1] = put_group<kRows>(t, idx, e, rs, rw, dy, true, p);
-    n += __popc(others);
-    __syncwarp();
-  }
-  return n;
-}
-
 template <bool SWIGLU, bool PAIR>
 __global__ void __launch_bounds__(kThreads, 1)
 k_grouped_gemm(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__ CUtensorMap tm_as,
@@ -330,12 +304,14 @@ k_grouped_gemm(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__
     tail->prefix[g + 1] = put_group<kTileRows>(tail, g, gr.expert, gr.row_start, gr.rows, gr.is_dynamic, selected, p);   // scanned below
   }
   if (threadIdx.x == 0) tail->prefix[0] = 0;
-  // the same answer in every CTA and in both passes: the word is written by a kernel that has finished, or not at all
-  const bool early = p.dyn.seq != 0 && ld_relaxed_gpu_u64(p.dyn.early) == p.dyn.seq;
+  const bool early = dyn_is_early(p.dyn);
   tc_fence_before();
   __syncthreads();
   if (warp == 0) {
-    const int n = early ? merge_table<kTileRows>(tail, p, lane) : p.n_groups;
+    const int n = !early ? p.n_groups : dyn_merge_table(
+        p.dyn, p.n_groups, FEPLB_MAX_GROUPS, p.status, lane,
+        [&](int e, int rs) { return tail->g_row_start[e] == rs && tail->prefix[e + 1] == 0; },
+        [&](int i, int e, int rs, int rw, int dy) { tail->prefix[i + 1] = put_group<kTileRows>(tail, i, e, rs, rw, dy, true, p); });
     warp_scan_prefix(tail, 0, n, lane);
     if (lane == 0) {
       tail->n_entries = n;

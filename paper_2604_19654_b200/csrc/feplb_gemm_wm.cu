@@ -58,7 +58,8 @@ constexpr int kTmemCols = 512;
 constexpr int kEpiWarps = 8;            // two warps per TMEM lane quarter
 constexpr int kThreads = 64 + 32 * kEpiWarps;
 constexpr int kEpiStageBytes = 32 * 64; // per epilogue warp: 32 tokens x 32 units of bf16
-constexpr int kXchgBytes = 32 * 32 * 4; // per pair of epilogue warps (pass 1): 32 tokens x 32 units of fp32
+constexpr int kXchgPitch = 144;         // bytes of a lane's 32 fp32 values in the exchange buffer, 16 apart from a bank's multiple
+constexpr int kXchgBytes = 32 * kXchgPitch;   // per pair of epilogue warps (pass 1)
 constexpr int kXchg = 4;
 constexpr int kMaxEntries = FEPLB_WM_MAX_ENTRIES;   // group entries of both tables together
 constexpr int kBoxes = 4;               // token-row boxes of 128, 64, 32 and 16 rows
@@ -175,15 +176,47 @@ __device__ __forceinline__ void warp_scan_prefix(Tail* t, int first, int n, int 
   __syncwarp();
 }
 
-// 32 values of one weight row (this lane) for 32 consecutive token rows -> global rows, transposed
-// through the warp's staging area: token j at byte j*64, this lane's unit at +lane*2; read back in
-// 16-byte pieces, 8 tokens per instruction, so that a token's 32 units leave as one 64-byte run.
+// 16 TMEM lanes x 32 fp32 columns in the layout of matrix fragments: registers 4g .. 4g + 3 of a thread are columns
+// 8g + 2 (lane % 4) and the next of row lane / 4, then the same columns of row lane / 4 + 8.
+__device__ __forceinline__ void tmem_ld_frag(uint32_t taddr, uint32_t* r) {
+  asm volatile(
+      "tcgen05.ld.sync.aligned.16x256b.x4.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, [%16];"
+      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]), "=r"(r[9]),
+        "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
+      : "r"(taddr) : "memory");
+}
+
+// The warp's staging area may still be read by the TMA store of its previous chunk.
+__device__ __forceinline__ void staging_ready(int lane) {
+  if (lane == 0) asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
+  __syncwarp();
+}
+
+// 32 weight rows x 32 consecutive token rows (two fragment halves of 16 weight rows) -> token rows of global memory.  The
+// transposition happens in stmatrix: the fragments of four octets of weight rows and one octet of tokens go to 8
+// token rows of 64 bytes, whose four 16-byte pieces are exchanged by bits 1 and 2 of the row number -- the
+// 64-byte swizzle of the tensor map, free of bank conflicts.  A full chunk leaves through one TMA store (m); a ragged
+// one, or one without a map, is read back in 16-byte pieces, 8 tokens per instruction.
 __device__ __forceinline__ void store_transposed(uint32_t stg, const float (&v)[32], __nv_bfloat16* out, int64_t ld, int n_valid,
-                                                 int lane) {
+                                                 int lane, const CUtensorMap* m, int col, int row) {
+  staging_ready(lane);
+  const uint32_t octet = lane >> 3, tok = lane & 7;
 #pragma unroll
-  for (int j = 0; j < 32; ++j) {
-    const unsigned short h = __bfloat16_as_ushort(__float2bfloat16_rn(v[j]));
-    asm volatile("st.shared.u16 [%0], %1;" ::"r"(stg + (uint32_t)(j * 64 + lane * 2)), "h"(h) : "memory");
+  for (int g = 0; g < 4; ++g) {
+    const uint32_t addr = stg + (8 * g + tok) * 64 + ((octet ^ ((tok >> 1) & 3)) << 4);
+    asm volatile("stmatrix.sync.aligned.m8n8.x4.trans.shared.b16 [%0], {%1, %2, %3, %4};" ::"r"(addr),
+                 "r"(pack_bf16x2(v[4 * g], v[4 * g + 1])), "r"(pack_bf16x2(v[4 * g + 2], v[4 * g + 3])),
+                 "r"(pack_bf16x2(v[16 + 4 * g], v[16 + 4 * g + 1])), "r"(pack_bf16x2(v[16 + 4 * g + 2], v[16 + 4 * g + 3])) : "memory");
+  }
+  if (m != nullptr && n_valid >= 32) {
+    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+    __syncwarp();
+    if (lane == 0) {
+      asm volatile("cp.async.bulk.tensor.2d.global.shared::cta.bulk_group [%0, {%2, %3}], [%1];"
+                   ::"l"(reinterpret_cast<uint64_t>(m)), "r"(stg), "r"(col), "r"(row) : "memory");
+      asm volatile("cp.async.bulk.commit_group;" ::: "memory");
+    }
+    return;
   }
   __syncwarp();
   const int tj = lane >> 2, piece = lane & 3;
@@ -192,7 +225,7 @@ __device__ __forceinline__ void store_transposed(uint32_t stg, const float (&v)[
     const int j = it * 8 + tj;
     uint4 w;
     asm volatile("ld.shared.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(w.x), "=r"(w.y), "=r"(w.z), "=r"(w.w)
-                 : "r"(stg + (uint32_t)(j * 64 + piece * 16)));
+                 : "r"(stg + (uint32_t)(j * 64 + ((piece ^ ((j >> 1) & 3)) << 4))));
     if (j < n_valid) *reinterpret_cast<uint4*>(out + (int64_t)j * ld + piece * 8) = w;
   }
   __syncwarp();
@@ -202,7 +235,8 @@ template <bool SWIGLU>
 __global__ void __launch_bounds__(kThreads, 1)
 k_ffn_wm(const __grid_constant__ CUtensorMap tm_a0, const __grid_constant__ CUtensorMap tm_a1,
          const __grid_constant__ CUtensorMap tm_r0, const __grid_constant__ CUtensorMap tm_r1,
-         const __grid_constant__ BMaps tm_b, const __grid_constant__ BMaps tm_rb, const WmParams p) {
+         const __grid_constant__ BMaps tm_b, const __grid_constant__ BMaps tm_rb, const __grid_constant__ CUtensorMap tm_out,
+         const WmParams p) {
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
   uint8_t* epi_smem = smem + (size_t)kRingBytes;
@@ -212,7 +246,6 @@ k_ffn_wm(const __grid_constant__ CUtensorMap tm_a0, const __grid_constant__ CUte
   const uint32_t cta_rank = cluster_ctarank();          // 0 = leader: issues the MMAs of the pair
   const int worker = (int)(blockIdx.x >> 1), n_workers = (int)(gridDim.x >> 1);
   volatile int* abort_flag = &tail->abort_flag;
-  const bool has_dyn = p.dyn.seq != 0;
 
   asm volatile("griddepcontrol.launch_dependents;");
 
@@ -250,21 +283,27 @@ k_ffn_wm(const __grid_constant__ CUtensorMap tm_a0, const __grid_constant__ CUte
     tail->prefix[g + 1] = put_entry(tail, g, gr.expert, gr.row_start, gr.rows, gr.is_dynamic, selected, p);
   }
   if (threadIdx.x == 0) tail->prefix[0] = 0;
+  const bool early = dyn_is_early(p.dyn);
   tc_fence_before();
   __syncthreads();
   if (warp == 0) {
-    warp_scan_prefix(tail, 0, p.n_groups, lane);
+    const int n = !early ? p.n_groups : dyn_merge_table(
+        p.dyn, p.n_groups, kMaxEntries, p.status, lane,
+        [&](int e, int rs) { return tail->row_start[e] == rs && tail->prefix[e + 1] == 0; },
+        [&](int i, int e, int rs, int rw, int dy) { tail->prefix[i + 1] = put_entry(tail, i, e, rs, rw, dy, true, p); });
+    warp_scan_prefix(tail, 0, n, lane);
     if (lane == 0) {
-      tail->n_entries = p.n_groups;
-      tail->total_units = tail->prefix[p.n_groups];
+      tail->n_entries = n;
+      tail->total_units = tail->prefix[n];
     }
   }
   __syncthreads();
   cluster_sync_all();                    // the peer's barriers are initialised before anything signals them
   tc_fence_after();
   const uint32_t tmem_base = tail->tmem_base;
-  const int n_static_entries = p.n_groups;
-  const int n_static_units = tail->prefix[p.n_groups];
+  const bool has_dyn = p.dyn.seq != 0 && !early;
+  const int n_static_entries = early ? tail->n_entries : p.n_groups;
+  const int n_static_units = tail->prefix[n_static_entries];
 
   if (warp == 0) {
     // ---- TMA producer (lane 0 issues; the whole warp fetches the dynamic table) --------------------
@@ -404,7 +443,7 @@ k_ffn_wm(const __grid_constant__ CUtensorMap tm_a0, const __grid_constant__ CUte
     }
   } else {
     // ---- epilogue: TMEM -> registers -> (SwiGLU) -> bf16 -> transposed rows in global memory ---------
-    // A thread owns one weight row of its CTA and gets 32 token rows per tcgen05.ld; two warps share
+    // A warp owns 32 weight rows of its CTA and takes 32 token rows at a time as matrix fragments; two warps share
     // each TMEM lane quarter and take alternate chunks of 32 tokens.  Pass 1: lanes 0-63 hold a, lanes
     // 64-127 b of the same 64 hidden units, so the warps of quarters 2 and 3 hand their b values to the
     // warps of quarters 0 and 1 through an exchange buffer (fp32), and those compute and store H.
@@ -443,14 +482,18 @@ k_ffn_wm(const __grid_constant__ CUtensorMap tm_a0, const __grid_constant__ CUte
       const int n_chunks = c.n_pad >> 5;
       uint32_t r[32];
       int ch = half;
-      if (ch < n_chunks) tmem_ld32(taddr + (uint32_t)(ch * 32), r);
+      auto load_chunk = [&](int chunk) {
+        tmem_ld_frag(taddr + (uint32_t)(chunk * 32), r);
+        tmem_ld_frag(taddr + (16u << 16) + (uint32_t)(chunk * 32), r + 16);
+      };
+      if (ch < n_chunks) load_chunk(ch);
       for (; ch < n_chunks && ok; ch += 2) {
         tmem_ld_wait();
         float v[32];
 #pragma unroll
         for (int j = 0; j < 32; ++j) v[j] = __uint_as_float(r[j]);
         if (ch + 2 < n_chunks) {                 // the next chunk's TMEM load flies while this one is converted and stored
-          tmem_ld32(taddr + (uint32_t)((ch + 2) * 32), r);
+          load_chunk(ch + 2);
         } else {
           // every TMEM read of this unit by this warp has completed: the accumulator may be overwritten
           tc_fence_before();
@@ -460,35 +503,38 @@ k_ffn_wm(const __grid_constant__ CUtensorMap tm_a0, const __grid_constant__ CUte
         const int r0 = c.row0 + ch * 32;
         const int n_valid = c.n_rows - ch * 32;  // valid token rows among this chunk's 32
         if (!SWIGLU) {
-          store_transposed(stg, v, p.out + (int64_t)r0 * p.ld_out + col0, p.ld_out, n_valid, lane);
+          store_transposed(stg, v, p.out + (int64_t)r0 * p.ld_out + col0, p.ld_out, n_valid, lane, &tm_out, col0, r0);
         } else if (gives_b) {
           ok = mbar_wait(xempty, xphase ^ 1u, abort_flag, p.status);
           ok = __all_sync(0xffffffffu, ok);
           if (!ok) break;
 #pragma unroll
-          for (int j = 0; j < 32; ++j)
-            asm volatile("st.shared.f32 [%0], %1;" ::"r"(xb + (uint32_t)(j * 128 + lane * 4)), "f"(v[j]) : "memory");
+          for (int j = 0; j < 32; j += 4)            // the partner's same lane holds a of the same units and tokens
+            asm volatile("st.shared.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(xb + (uint32_t)(lane * kXchgPitch + j * 4)), "f"(v[j]),
+                         "f"(v[j + 1]), "f"(v[j + 2]), "f"(v[j + 3]) : "memory");
           __syncwarp();
           if (lane == 0) mbar_arrive(xfull);
           xphase ^= 1u;
           if (p.ab_out != nullptr)
-            store_transposed(stg, v, p.ab_out + (int64_t)r0 * (2 * p.ld_out) + p.ld_out + col0, 2 * p.ld_out, n_valid, lane);
+            store_transposed(stg, v, p.ab_out + (int64_t)r0 * (2 * p.ld_out) + p.ld_out + col0, 2 * p.ld_out, n_valid, lane, nullptr, 0, 0);
         } else {
           if (p.ab_out != nullptr)
-            store_transposed(stg, v, p.ab_out + (int64_t)r0 * (2 * p.ld_out) + col0, 2 * p.ld_out, n_valid, lane);
+            store_transposed(stg, v, p.ab_out + (int64_t)r0 * (2 * p.ld_out) + col0, 2 * p.ld_out, n_valid, lane, nullptr, 0, 0);
           ok = mbar_wait(xfull, xphase, abort_flag, p.status);
           ok = __all_sync(0xffffffffu, ok);
           if (!ok) break;
 #pragma unroll
-          for (int j = 0; j < 32; ++j) {
-            float b;
-            asm volatile("ld.shared.f32 %0, [%1];" : "=f"(b) : "r"(xb + (uint32_t)(j * 128 + lane * 4)));
-            v[j] = silu_f(v[j]) * b;
+          for (int j = 0; j < 32; j += 4) {
+            float b[4];
+            asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(b[0]), "=f"(b[1]), "=f"(b[2]), "=f"(b[3])
+                         : "r"(xb + (uint32_t)(lane * kXchgPitch + j * 4)));
+#pragma unroll
+            for (int i = 0; i < 4; ++i) v[j + i] = silu_f(v[j + i]) * b[i];
           }
           __syncwarp();
           if (lane == 0) mbar_arrive(xempty);
           xphase ^= 1u;
-          store_transposed(stg, v, p.out + (int64_t)r0 * p.ld_out + col0, p.ld_out, n_valid, lane);
+          store_transposed(stg, v, p.out + (int64_t)r0 * p.ld_out + col0, p.ld_out, n_valid, lane, &tm_out, col0, r0);
         }
       }
       if (!ok) break;
@@ -499,6 +545,7 @@ k_ffn_wm(const __grid_constant__ CUtensorMap tm_a0, const __grid_constant__ CUte
       }
       if (++as == 2) { as = 0; aphase ^= 1u; }
     }
+    staging_ready(lane);      // the staging area must outlive the last TMA store that reads it
   }
 
   // ---- teardown --------------------------------------------------------------------------------------
@@ -531,16 +578,17 @@ encode_tiled_fn get_encode_fn() {
   return fn;
 }
 
-// Row-major bf16 matrix [rows, inner] -> tensor map with a [box_rows, 64] box, 128-byte swizzle.
-bool make_tmap(CUtensorMap* m, const void* base, uint64_t rows, uint64_t inner, uint32_t box_rows) {
+// Row-major bf16 matrix [rows, inner] -> tensor map with a [box_rows, box_cols] box (64 or 32 columns), swizzled by its width.
+bool make_tmap(CUtensorMap* m, const void* base, uint64_t rows, uint64_t inner, uint32_t box_rows, uint32_t box_cols = BK) {
   encode_tiled_fn fn = get_encode_fn();
   if (!fn) return false;
   cuuint64_t dims[2] = {inner, rows};
   cuuint64_t strides[1] = {inner * 2};
-  cuuint32_t box[2] = {(cuuint32_t)BK, box_rows};
+  cuuint32_t box[2] = {box_cols, box_rows};
   cuuint32_t estr[2] = {1, 1};
   return fn(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void*>(base), dims, strides, box, estr,
-            CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+            CU_TENSOR_MAP_INTERLEAVE_NONE, box_cols == 32 ? CU_TENSOR_MAP_SWIZZLE_64B : CU_TENSOR_MAP_SWIZZLE_128B,
+            CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
             CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
@@ -552,7 +600,7 @@ bool make_bmaps(BMaps* b, const void* base, uint64_t rows, uint64_t inner) {
 
 template <bool SWIGLU>
 cudaError_t launch_wm(const CUtensorMap& a0, const CUtensorMap& a1, const CUtensorMap& r0, const CUtensorMap& r1,
-                      const BMaps& b, const BMaps& rb, const WmParams& p, int num_sms, cudaStream_t st) {
+                      const BMaps& b, const BMaps& rb, const CUtensorMap& out, const WmParams& p, int num_sms, cudaStream_t st) {
   // per instantiation and device: the shared-memory attribute and the resident grid are set on first use
   static int grid_of[64] = {};
   int dev = 0;
@@ -583,7 +631,7 @@ cudaError_t launch_wm(const CUtensorMap& a0, const CUtensorMap& a1, const CUtens
     grid = 2 * (n_clusters < num_sms / 2 ? n_clusters : num_sms / 2);
   }
   cfg.gridDim = dim3(grid);
-  return cudaLaunchKernelEx(&cfg, k_ffn_wm<SWIGLU>, a0, a1, r0, r1, b, rb, p);
+  return cudaLaunchKernelEx(&cfg, k_ffn_wm<SWIGLU>, a0, a1, r0, r1, b, rb, out, p);
 }
 
 }  // namespace
@@ -599,11 +647,13 @@ int feplb_launch_expert_ffn_wm(const feplb_gemm_args& a, const feplb_wm_dyn& dyn
     snprintf(err, errn, "expert_ffn: shape not supported by the weights-on-M form");
     return FEPLB_E_INVALID;
   }
-  CUtensorMap tm_w1, tm_w3, tm_w2;      // weights in boxes of 64 rows
+  CUtensorMap tm_w1, tm_w3, tm_w2, tm_h, tm_y;      // weights in boxes of 64 rows, outputs in boxes of 32 x 32
   BMaps bx, bh;
   if (!make_tmap(&tm_w1, a.w1, (uint64_t)a.E * a.f, (uint64_t)a.d, WM / 2) ||
       !make_tmap(&tm_w3, a.w3, (uint64_t)a.E * a.f, (uint64_t)a.d, WM / 2) ||
       !make_tmap(&tm_w2, a.w2, (uint64_t)a.E * a.d, (uint64_t)a.f, WM) ||
+      !make_tmap(&tm_h, a.h, (uint64_t)a.s_cap, (uint64_t)a.f, 32, 32) ||
+      !make_tmap(&tm_y, a.y, (uint64_t)a.s_cap, (uint64_t)a.d, 32, 32) ||
       !make_bmaps(&bx, a.x_perm, (uint64_t)a.s_cap, (uint64_t)a.d) ||
       !make_bmaps(&bh, a.h, (uint64_t)a.s_cap, (uint64_t)a.f)) {
     snprintf(err, errn, "cuTensorMapEncodeTiled failed (driver entry point missing or bad pointer/shape)");
@@ -637,10 +687,10 @@ int feplb_launch_expert_ffn_wm(const feplb_gemm_args& a, const feplb_wm_dyn& dyn
   p2.out = (__nv_bfloat16*)a.y; p2.ld_out = a.d; p2.ab_out = nullptr;
   p2.stamps = dyn.stamps ? dyn.stamps + 4 : nullptr;
 
-  cudaError_t e = launch_wm<true>(tm_w1, tm_w3, tm_r1, tm_r3, bx, brx, p1, a.num_sms, st);
+  cudaError_t e = launch_wm<true>(tm_w1, tm_w3, tm_r1, tm_r3, bx, brx, tm_h, p1, a.num_sms, st);
   ++*n_launch;
   if (e == cudaSuccess) {
-    e = launch_wm<false>(tm_w2, tm_w2, tm_r2, tm_r2, bh, bh, p2, a.num_sms, st);
+    e = launch_wm<false>(tm_w2, tm_w2, tm_r2, tm_r2, bh, bh, tm_y, p2, a.num_sms, st);
     ++*n_launch;
   }
   if (e != cudaSuccess) {

@@ -23,7 +23,9 @@
 #define FEPLB_ST_WAIT 4u       // a bounded mbarrier wait gave up inside the GEMM
 #define FEPLB_ST_GROUP 8u      // a group entry was malformed (expert or rows out of range)
 #define FEPLB_ST_PLAN 16u      // the GEMM's bounded wait for the planner's dynamic group table gave up
-#define FEPLB_WM_AUTO_ROWS_PER_EXPERT 768   // the weights-on-M form is the default below this many rows per expert
+#define FEPLB_MERGED_MAX_ROWS_PER_EXPERT 768   // static and dynamic groups share launches below this many rows per expert
+#define FEPLB_WM_MIN_ROWS_PER_EXPERT 64        // the weights-on-M form is the default from here (up to the line above) ...
+#define FEPLB_WM_MIN_WEIGHT (3 << 20)          // ... for weight matrices of at least so many elements
 // No launch of a forward waits for the plan below this many rows per expert, or where the expert FFN takes less than this long
 #define FEPLB_DIRECT_ROWS_PER_EXPERT 128
 #define FEPLB_DIRECT_FFN_US 150
