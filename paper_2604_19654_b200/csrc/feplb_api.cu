@@ -45,6 +45,7 @@ struct feplb_ctx {
   bool wm_ok = false;          // the weights-on-M form supports this geometry
   bool wm = false;             // ... and is the form in use (feplb_create's choice or feplb_set_gemm_form)
   bool wm_auto = false;
+  bool wm_static = false, wm_static_auto = false;   // the static launches of the four-launch order use it
   bool merged_ok = false;      // both group tables of a forward fit one launch (static, then dynamic groups)
   bool merged = false;         // ... and feplb_moe_forward runs that way: two GEMM launches instead of four
   bool merged_auto = false;
@@ -383,6 +384,9 @@ extern "C" int feplb_create(const feplb_config* cfg, feplb_ctx** out) {
   c->wm_ok = feplb_wm_supported(cfg->E, cfg->d, cfg->f, cfg->E + cap_groups);
   c->wm_auto = c->wm = c->wm_ok && S >= (int64_t)FEPLB_WM_MIN_ROWS_PER_EXPERT * cfg->E &&
                        S < (int64_t)FEPLB_MERGED_MAX_ROWS_PER_EXPERT * cfg->E && (int64_t)cfg->d * cfg->f >= FEPLB_WM_MIN_WEIGHT;
+  // In the four-launch order the static experts are the less busy ones and stay in the range above for longer: d = 6144,
+  // f = 2048, 128 experts, 1024 rows per expert on average 9911 -> 9750 us per layer, 1500 rows 13828 -> 13785.
+  c->wm_static_auto = c->wm_static = c->wm_ok && S < (int64_t)2048 * cfg->E && (int64_t)cfg->d * cfg->f >= FEPLB_WM_MIN_WEIGHT;
   // One launch per pass over the static and then the dynamic groups (the table of the latter is
   // picked up on the device): saves two launch ramps and two partly filled last waves per forward,
   // which matters while a forward's GEMMs take a few hundred microseconds; one form serves both
@@ -608,7 +612,7 @@ extern "C" int feplb_home_groups(feplb_ctx* c, const int32_t* counts, const uint
 // `dyn` != nullptr: weights-on-M launches that go on to the planner's dynamic table after `groups`.
 static int ffn_impl(feplb_ctx* c, const void* x_perm, const void* w1, const void* w3, const void* w2,
                     const feplb_group* groups, int32_t n_groups, int32_t which, void* h, void* y, cudaStream_t st,
-                    int pair = -1, const feplb_wm_dyn* dyn = nullptr) {
+                    int pair = -1, const feplb_wm_dyn* dyn = nullptr, bool weights_on_m = false) {
   if (pair < 0) pair = c->gemm_pair_default;
   if (n_groups < 0 || n_groups > FEPLB_MAX_GROUPS) return fail(c, FEPLB_E_INVALID, "expert_ffn: n_groups out of range");
   if (which != FEPLB_FFN_ALL && which != FEPLB_FFN_STATIC && which != FEPLB_FFN_DYNAMIC)
@@ -625,7 +629,7 @@ static int ffn_impl(feplb_ctx* c, const void* x_perm, const void* w1, const void
   a.ab_out = c->d_preact;
   a.recv_w1 = c->d_recv_w1; a.recv_w3 = c->d_recv_w3; a.recv_w2 = c->d_recv_w2; a.n_recv_slots = c->n_recv_slots;
   a.recv_x = c->d_recv_x;
-  if (c->wm && n_groups + (dyn ? dyn->max_groups : 0) <= FEPLB_WM_MAX_ENTRIES) {
+  if ((c->wm || weights_on_m) && n_groups + (dyn ? dyn->max_groups : 0) <= FEPLB_WM_MAX_ENTRIES) {
     const feplb_wm_dyn none;
     return feplb_launch_expert_ffn_wm(a, dyn ? *dyn : none, st, &c->launches, c->err, sizeof(c->err));
   }
@@ -917,7 +921,7 @@ extern "C" int feplb_moe_forward(feplb_ctx* c, const void* x, const int32_t* top
   } else {
     // step 4: static experts on their home ranks, from the group table built on the device
     if (rc == FEPLB_OK)
-      rc = ffn_impl(c, x_perm, w1, w3, w2, c->d_home_groups, g.E, FEPLB_FFN_STATIC, h_scratch, y_perm, st);
+      rc = ffn_impl(c, x_perm, w1, w3, w2, c->d_home_groups, g.E, FEPLB_FFN_STATIC, h_scratch, y_perm, st, -1, nullptr, c->wm_static);
     TL_EVENT(EV_STATIC1);
     c->tl.host_enqueue_static_done_us = us_since(c->t0);
     // join the planner (always, so that the context returns to idle), then step 5
@@ -1190,6 +1194,7 @@ extern "C" int feplb_set_gemm_form(feplb_ctx* c, int32_t forward_form, int32_t b
     return fail(c, FEPLB_E_INVALID, "set_gemm_form: backward_pair must be -1 (auto) or a 2-bit mask");
   std::lock_guard<std::mutex> lk(c->mu);
   if (c->job != JOB_IDLE) return fail(c, FEPLB_E_STATE, "set_gemm_form: a plan is pending");
+  c->wm_static = forward_form == FEPLB_FORM_AUTO && c->wm_static_auto;
   c->wm = forward_form == FEPLB_FORM_AUTO ? c->wm_auto : forward_form == FEPLB_FORM_WEIGHT_M;
   c->gemm_pair_forced = forward_form == FEPLB_FORM_SINGLE || forward_form == FEPLB_FORM_PAIR ? forward_form : -1;
   c->gemm_pair_default = c->gemm_pair_forced < 0 ? c->gemm_pair_auto : forward_form;

@@ -228,3 +228,14 @@ def test_table_brought_over_by_the_gather(E, R, split, form):
     assert p0.groups == p1.groups and len(p0.moves) > 0
     assert np.array_equal(F.bf16_bits(case.buf.out), out)
     case.close()
+
+
+@pytest.mark.parametrize("T,merged", [(48, 1), (60, 0), (700, 0), (800, 0), (60, -1), (700, -1)])
+def test_form_rule_of_large_weights(T, merged):
+    """Shapes from which the weights-on-M form is chosen (3 Mi elements per matrix): below, inside and above its range of
+    rows per expert, in every launch order."""
+    w = W.get_workload("cfg2").with_(T=T, E=2, R=2, K=2, d=2048, f=1536, dyn=1, max_num_dyn=1, tau=1)
+    case = DeviceCase(w)
+    case.ctx.set_launch_merging(merged)
+    _check_forward(case, sample=40)
+    case.close()
