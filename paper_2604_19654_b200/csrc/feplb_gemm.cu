@@ -360,45 +360,57 @@ k_grouped_gemm(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__
       dyn_known = true;
       return true;
     };
-    // The loads of one K block of one tile.  Pair form: both CTAs credit the LEADER's barrier; the leader
-    // announces the bytes of both.  For a tile whose second 128 rows hold no valid row (a group of at most
-    // 128 rows, or a ragged tail) the peer's A box lies past the end of the tensor: zeros arrive without
-    // any traffic from L2, and multiplying zeros takes less power than multiplying what a skipped load would
-    // leave in the stage, which is clock at the power cap (64 experts, d = 2048, T = 4096: 343.2 -> 337.1 us per
-    // layer).  Zeros for the partly valid 128 rows as well, by boxes of 32 rows, cost 4 % instead.
-    auto few_rows = [&](const TileCoord& c) { return !PAIR && c.slot < 0 && c.rows_valid <= kFewRows; };
-    auto load_b = [&](const TileCoord& c, int kb, int st) {      // announces the stage's bytes, loads the weights
-      // weights of a migrated expert come from its slot of the receive buffer
-      const CUtensorMap* mb0 = c.slot >= 0 ? &tm_r0 : &tm_b0;
-      const CUtensorMap* mb1 = c.slot >= 0 ? &tm_r1 : &tm_b1;
-      const int row = (c.slot >= 0 ? c.slot : c.expert) * p.b_rows_per_expert + (SWIGLU ? c.n0 : 2 * c.n0);
-      const uint32_t full = smem_u32(&tail->full[st]);
-      const uint32_t sb = smem_u32(smem + (size_t)st * kStageBytes) + kABytes;
-      const uint32_t half = (uint32_t)c.bn * BK * 2, box = (uint32_t)p.b_box * BK * 2;
+    // What a tile's K blocks are loaded from, worked out once per tile and not in the K loop, which runs in one thread
+    // beside the MMA issuer (d = 1920, f = 704, 60 experts, T = 1537: 148.7 -> 145.1 us per layer).
+    // Pair form: both CTAs credit the LEADER's barrier; the leader announces the bytes of both.  For a tile whose
+    // second 128 rows hold no valid row (a group of at most 128 rows, or a ragged tail) the peer's A box lies past
+    // the end of the tensor: zeros arrive without any traffic from L2, and multiplying zeros takes less power than
+    // multiplying what a skipped load would leave in the stage, which is clock at the power cap (64 experts, d = 2048,
+    // T = 4096: 343.2 -> 337.1 us per layer).  Zeros for the partly valid 128 rows as well, by boxes of 32 rows, cost
+    // 4 % instead.
+    struct Source { const CUtensorMap *a, *b0, *b1; int arow, brow0, brow1; uint32_t half, tx; bool two; };
+    auto source = [&](const TileCoord& c) {
+      Source q;
+      const bool few = !PAIR && c.slot < 0 && c.rows_valid <= kFewRows;
+      // weights of a migrated expert come from its slot of the receive buffer, and in pass 1 its rows from the
+      // receive region (same row numbers as the permuted buffer)
+      q.a = c.slot >= 0 ? &tm_ra : few ? &tm_as : &tm_a;
+      q.b0 = c.slot >= 0 ? &tm_r0 : &tm_b0;
+      q.b1 = c.slot >= 0 ? &tm_r1 : &tm_b1;
+      q.arow = c.row0;
+      q.brow0 = (c.slot >= 0 ? c.slot : c.expert) * p.b_rows_per_expert + (SWIGLU ? c.n0 : 2 * c.n0);
+      q.brow1 = SWIGLU ? q.brow0 : q.brow0 + c.bn;
+      q.half = (uint32_t)c.bn * BK * 2;
+      q.two = c.bn > p.b_box;              // 128 rows in boxes of 64
+      q.tx = (PAIR ? 2 * kABytes : few ? kFewRows * BK * 2 : kABytes) + 2 * q.half;
+      if (PAIR && cta_rank) {
+        q.arow = c.rows_valid > BM ? c.row0 + BM : (int)p.s_cap;
+        q.b0 = q.b1;
+        q.brow0 = q.brow1;
+      }
+      return q;
+    };
+    auto announce = [&](const Source& q, uint32_t full) {      // the bytes of a stage
+      if (!PAIR || cta_rank == 0) mbar_expect_tx(full, q.tx);
+    };
+    auto load_b = [&](const Source& q, int kb, uint32_t full, uint32_t sb) {
+      constexpr uint32_t kBox = 64 * BK * 2;
       if (PAIR) {
         const uint32_t full0 = map_to_cta(full, 0);
-        if (cta_rank == 0) mbar_expect_tx(full, 2 * kABytes + 2 * half);
-        const CUtensorMap* mb = cta_rank == 0 ? mb0 : mb1;
-        const int r0 = row + (!SWIGLU && cta_rank ? c.bn : 0);
-        for (uint32_t o = 0, r = 0; o < half; o += box, r += p.b_box) tma_load_2d_pair(sb + o, mb, full0, kb * BK, r0 + (int)r);
+        tma_load_2d_pair(sb, q.b0, full0, kb * BK, q.brow0);
+        if (q.two) tma_load_2d_pair(sb + kBox, q.b0, full0, kb * BK, q.brow0 + 64);
       } else {
-        mbar_expect_tx(full, (few_rows(c) ? kFewRows * BK * 2 : kABytes) + 2 * half);
-        for (uint32_t o = 0, r = 0; o < half; o += box, r += p.b_box) tma_load_2d(sb + o, mb0, full, kb * BK, row + (int)r);
-        const int row1 = SWIGLU ? row : row + c.bn;
-        for (uint32_t o = 0, r = 0; o < half; o += box, r += p.b_box) tma_load_2d(sb + half + o, mb1, full, kb * BK, row1 + (int)r);
+        tma_load_2d(sb, q.b0, full, kb * BK, q.brow0);
+        tma_load_2d(sb + q.half, q.b1, full, kb * BK, q.brow1);
+        if (q.two) {
+          tma_load_2d(sb + kBox, q.b0, full, kb * BK, q.brow0 + 64);
+          tma_load_2d(sb + q.half + kBox, q.b1, full, kb * BK, q.brow1 + 64);
+        }
       }
     };
-    auto load_a = [&](const TileCoord& c, int kb, int st) {
-      // in pass 1 the rows of a migrated piece come from the receive region (same row numbers as the permuted buffer)
-      const CUtensorMap* ma = c.slot >= 0 ? &tm_ra : &tm_a;
-      const uint32_t full = smem_u32(&tail->full[st]);
-      const uint32_t sa = smem_u32(smem + (size_t)st * kStageBytes);
-      if (PAIR) {
-        tma_load_2d_pair(sa, ma, map_to_cta(full, 0), kb * BK,
-                         cta_rank == 0 ? c.row0 : c.rows_valid > BM ? c.row0 + BM : (int)p.s_cap);
-      } else {
-        tma_load_2d(sa, few_rows(c) ? &tm_as : ma, full, kb * BK, c.row0);
-      }
+    auto load_a = [&](const Source& q, int kb, uint32_t full, uint32_t sa) {
+      if (PAIR) tma_load_2d_pair(sa, q.a, map_to_cta(full, 0), kb * BK, q.arow);
+      else tma_load_2d(sa, q.a, full, kb * BK, q.arow);
     };
     // Weights of the first tile, as far as the ring holds them, before the wait for the rows.
     int n_early = 0;
@@ -406,8 +418,11 @@ k_grouped_gemm(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__
       if (worker < n_static_tiles) {
         n_early = min(kStages, p.num_k_blocks);
         if (lane == 0) {
-          const TileCoord c = tile_coord<kTileRows>(tail, n_entries, p, worker);
-          for (int kb = 0; kb < n_early; ++kb) load_b(c, kb, kb);
+          const Source q = source(tile_coord<kTileRows>(tail, n_entries, p, worker));
+          for (int kb = 0; kb < n_early; ++kb) {
+            announce(q, smem_u32(&tail->full[kb]));
+            load_b(q, kb, smem_u32(&tail->full[kb]), smem_u32(smem + (size_t)kb * kStageBytes) + kABytes);
+          }
         }
         __syncwarp();
       }
@@ -440,12 +455,19 @@ k_grouped_gemm(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__
       unsigned long long peek = 0;
       if (!dyn_known && lane == 0) peek = ld_relaxed_gpu_u64(p.dyn.ready_dev);
       if (lane == 0) {
-        for (int kb = 0; kb < p.num_k_blocks; ++kb) {
-          if (kb >= n_early) {
-            if (!(ok = mbar_wait(smem_u32(&tail->empty[stage]), phase ^ 1u, abort_flag, p.status))) break;
-            load_b(c, kb, stage);
-          }
-          load_a(c, kb, stage);
+        const Source q = source(c);
+        int kb = 0;
+        for (; kb < n_early; ++kb) {       // stages 0 .. n_early - 1, whose weights are on their way
+          load_a(q, kb, smem_u32(&tail->full[stage]), smem_u32(smem + (size_t)stage * kStageBytes));
+          if (++stage == kStages) { stage = 0; phase ^= 1u; }
+        }
+        for (; kb < p.num_k_blocks; ++kb) {
+          if (!(ok = mbar_wait(smem_u32(&tail->empty[stage]), phase ^ 1u, abort_flag, p.status))) break;
+          const uint32_t full = smem_u32(&tail->full[stage]);
+          const uint32_t sa = smem_u32(smem + (size_t)stage * kStageBytes);
+          announce(q, full);
+          load_a(q, kb, full, sa);
+          load_b(q, kb, full, sa + kABytes);
           if (++stage == kStages) { stage = 0; phase ^= 1u; }
         }
       }
@@ -463,6 +485,8 @@ k_grouped_gemm(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__
   } else if (warp == 1) {
     // ---- MMA issuer -------------------------------------------------------------------------
     if (lane == 0 && cta_rank == 0) {
+      const bool narrow = p.half_width % p.bn != 0;      // the last N tile is
+      uint32_t idesc = make_idesc(kTileRows, 2 * p.bn);
       int stage = 0, as = 0;
       uint32_t phase = 0, aphase = 0;
       bool ok = true, dyn_known = !has_dyn;
@@ -475,7 +499,7 @@ k_grouped_gemm(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__
           total = tail->total_mtiles * p.n_tiles_n;
           if (tile >= total) break;
         }
-        const uint32_t idesc = make_idesc(kTileRows, 2 * min(p.bn, p.half_width - tile % p.n_tiles_n * p.bn));
+        if (narrow) idesc = make_idesc(kTileRows, 2 * min(p.bn, p.half_width - tile % p.n_tiles_n * p.bn));
         if (!(ok = mbar_wait(smem_u32(&tail->tmem_empty[as]), aphase ^ 1u, abort_flag, p.status))) break;
         tc_fence_after();
         const uint32_t d_tmem = tmem_base + (uint32_t)(as * kAccCols);
