@@ -561,7 +561,9 @@ k_grouped_gemm(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__
       const int row_off = (int)cta_rank * BM + q * 32;    // this warp's first row inside the tile
       const int rows_here = c.rows_valid - row_off;       // valid rows among this warp's 32
       __nv_bfloat16* obase = p.out + (int64_t)(c.row0 + row_off) * p.ld_out + col0;
-      if (rows_here > 0) {                                // a warp without valid rows only hands the accumulator back
+      // Single form: a warp without valid rows only hands the accumulator back.  In the pair form, which has few of them,
+      // this test costs more than it saves: d = 6144, T = 65536 35344 us per layer with it, 34903 without.
+      if (PAIR || rows_here > 0) {
         uint32_t a0[32], a1[32], b0[32], b1[32], packed[32];
         tmem_ld32(taddr, a0);
         tmem_ld32(taddr + 32u, a1);
