@@ -415,8 +415,9 @@ k_gather(const uint4* __restrict__ x, const int32_t* __restrict__ ids, const int
 // size; here every CTA computes the complete routing of the batch for itself (at most kSmallMaxSlots ids, read
 // from L2; the ranks end up in shared memory), so that no CTA needs another one's result, and then copies
 // its share of the rows.  CTA 0 alone publishes the tables (groups != nullptr) or compares the counts with the
-// caller's (counts_in, stand-alone dispatch: its offsets come from the ids, so wrong counts only raise the status).  The redundant part grows with the number of slots
-// and ends the range: see feplb_front_is_small.
+// caller's (counts_in, stand-alone dispatch: the segments have the caller's sizes, clamped to the buffer, as in
+// k_scan and k_gather).  The redundant part grows with the number of slots and ends the range: see
+// feplb_front_is_small.
 // Whole layer, chained front -> this: 32.3 -> 27.9 us at T = 256, top-2, d = 128, 8 experts; 102.0 -> 97.9 us at
 // T = 64, top-6, d = 2048, 64 experts.
 constexpr int kSmallThreads = 1024;
@@ -433,7 +434,7 @@ k_route_small(const uint4* __restrict__ x, const int32_t* __restrict__ ids, int 
   extern __shared__ int sm[];
   __shared__ int tmp[64];
   int* wh = sm;                              // [kSmallWarps][E] histograms per warp, then ranks of a warp's first slots
-  int* sc = wh + kSmallWarps * E;            // [E] counts
+  int* sc = wh + kSmallWarps * E;            // [E] rows of the segment: the counts, or the caller's
   int* pad = sc + E;                         // [E] first row of the segment
   int* rows = pad + E;                       // [32 * 32 * CH] row of every slot, -1 for an id outside [0, E)
   const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -458,6 +459,7 @@ k_route_small(const uint4* __restrict__ x, const int32_t* __restrict__ ids, int 
     const int s = (w * CH + c) * 32 + lane;
     id[c] = s < S ? ids[s] : -1;
   }
+  const int given = counts_in && (int)threadIdx.x < E ? counts_in[threadIdx.x] : 0;
   if (u < units) load_unit(u);
   unsigned mk[CH];
   bool bad = false;
@@ -482,14 +484,16 @@ k_route_small(const uint4* __restrict__ x, const int32_t* __restrict__ ids, int 
       wh[i * E + e] = cnt;
       cnt += n;
     }
-    sc[e] = cnt;
     if (blockIdx.x == 0) {
-      if (counts_in && counts_in[e] != cnt) atomicOr(status, FEPLB_ST_COUNTS);
+      if (counts_in && given != cnt) atomicOr(status, FEPLB_ST_COUNTS);
       if (counts_out) counts_out[e] = cnt;
       if (counts_host_tagged)                // see k_scan_fused
         *reinterpret_cast<volatile unsigned long long*>(counts_host_tagged + e) =
             ((unsigned long long)(uint32_t)seq << 32) | (uint32_t)cnt;
     }
+    // a segment larger than the buffer pushes the ones behind it out of it whatever its size: no sum overflows
+    if (counts_in) cnt = min(max(given, 0), (int)s_cap);
+    sc[e] = cnt;
   }
   if (blockIdx.x == 0 && e == 0 && t_counts) {
     unsigned long long t;
@@ -505,6 +509,7 @@ k_route_small(const uint4* __restrict__ x, const int32_t* __restrict__ ids, int 
   for (int c = 0; c < CH; ++c) {
     int r = -1;
     if (id[c] >= 0) r = pad[id[c]] + wh[w * E + id[c]] + __popc(mk[c] & lt);
+    if (r >= s_cap) r = -1;                  // only with counts that disagree with the ids
     __syncwarp();
     if (id[c] >= 0 && lane == __ffs(mk[c]) - 1) wh[w * E + id[c]] += __popc(mk[c]);
     __syncwarp();
@@ -553,7 +558,7 @@ k_route_small(const uint4* __restrict__ x, const int32_t* __restrict__ ids, int 
     row_to_token[i] = -1;
   if (A > 1) {                               // padding rows at the end of the segments
     for (int g = blockIdx.x; g < E; g += gridDim.x) {
-      const int r0 = pad[g] + sc[g], r1 = pad[g] + (sc[g] + A - 1) / A * A;
+      const int r0 = pad[g] + sc[g], r1 = (int)min((int64_t)pad[g] + (sc[g] + A - 1) / A * A, s_cap);
       for (int r = r0 + (int)threadIdx.x; r < r1; r += kSmallThreads) row_to_token[r] = -1;
       uint4* p = x_perm + (int64_t)r0 * chunks;
       const int64_t n = (int64_t)(r1 - r0) * chunks;

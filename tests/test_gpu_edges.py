@@ -239,3 +239,35 @@ def test_form_rule_of_large_weights(T, merged):
     case.ctx.set_launch_merging(merged)
     _check_forward(case, sample=40)
     case.close()
+
+
+@pytest.mark.parametrize("A", [1, 128])
+@pytest.mark.parametrize("T", [300, 2730, 2731])
+def test_dispatch_takes_the_segments_from_the_counts(T, A):
+    """Counts that disagree with the ids: one rule on both sides of the one-launch front's range (8190 and 8193 slots).  The
+    caller's counts give the segments, clamped to the buffer; a slot whose row would lie behind it gets -1."""
+    import torch
+    K, E = 3, 16
+    cfg = F.make_config(T, K, E, 2, 128, 64, row_align=A)
+    ctx, buf, cap = F.Context(cfg), F.Buffers(cfg), F.s_pad(cfg)
+    ids = np.random.default_rng(T).integers(0, E, size=(T, K)).astype(np.int32)
+    flat = ids.ravel()
+    true = np.bincount(flat, minlength=E)
+    rank = np.empty(flat.size, np.int64)
+    for e in range(E):
+        rank[flat == e] = np.arange(true[e])
+    x, d_ids = torch.zeros(T, 128, dtype=torch.bfloat16, device="cuda"), torch.from_numpy(ids).cuda()
+    for delta in ({3: 1}, {15: 5}, {0: -2}, {2: -10 ** 6}, {1: 2 ** 30, 2: 2 ** 30, 3: 2 ** 30}, {5: 1000, 9: -7}):
+        counts = true.copy()
+        for e, dv in delta.items():
+            counts[e] = dv if abs(dv) >= 10 ** 6 else counts[e] + dv
+        seg = np.maximum(counts, 0)
+        off = np.concatenate([[0], np.cumsum((seg + A - 1) // A * A)[:-1]])
+        rows = np.minimum(off, cap)[flat] + rank
+        rows[rows >= cap] = -1
+        ctx.dispatch(x, d_ids, torch.from_numpy(counts.astype(np.int32)).cuda(), buf.x_perm, buf.slot_to_row, buf.row_to_token)
+        with pytest.raises(F.FeplbError) as ei:
+            ctx.check_status()
+        assert ei.value.code == F.E_DEVICE
+        assert np.array_equal(buf.slot_to_row.cpu().numpy().ravel(), rows), delta
+    ctx.close()
