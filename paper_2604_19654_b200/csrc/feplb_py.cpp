@@ -1,5 +1,5 @@
 // CPython module with the per-micro-batch calls of the binding: takes tensors (anything with is_contiguous() and
-// data_ptr()), addresses or None, and calls the C ABI with their pointers, without the GIL.  The ctypes route
+// data_ptr()), numpy arrays, addresses or None, and calls the C ABI with their pointers, without the GIL.  The ctypes route
 // does the same in Python and costs 10 us for the 19 arguments of feplb_moe_forward, as much as the whole
 // GPU work of a small batch; through this module the call overhead is about 2 us.
 #define PY_SSIZE_T_CLEAN
@@ -12,7 +12,7 @@
 
 namespace {
 
-PyObject *s_is_contiguous, *s_data_ptr;
+PyObject *s_is_contiguous, *s_data_ptr, *s_ctypes, *s_data;
 PyObject *s_buf[8], *s_bwd[6];      // attribute names of Buffers / BackwardBuffers, in the order of the C arguments
 
 decltype(&feplb_moe_forward) p_forward;
@@ -22,7 +22,27 @@ decltype(&feplb_route_hist) p_hist;
 decltype(&feplb_dispatch) p_dispatch;
 decltype(&feplb_combine) p_combine;
 
-// Address of a tensor or int, NULL for None; false with a Python error set.
+// Address of a numpy array (page-locked host memory is addressable from the GPU), which has no is_contiguous();
+// the AttributeError that said so stays set for any other object.
+bool array_ptr(PyObject* o, void** out) {
+  PyObject *type, *value, *trace;
+  PyErr_Fetch(&type, &value, &trace);
+  PyObject* c = PyObject_GetAttr(o, s_ctypes);
+  PyObject* d = c ? PyObject_GetAttr(c, s_data) : nullptr;
+  Py_XDECREF(c);
+  if (!d) {
+    PyErr_Restore(type, value, trace);
+    return false;
+  }
+  Py_XDECREF(type);
+  Py_XDECREF(value);
+  Py_XDECREF(trace);
+  *out = PyLong_AsVoidPtr(d);
+  Py_DECREF(d);
+  return !PyErr_Occurred();
+}
+
+// Address of a tensor, array or int, NULL for None; false with a Python error set.
 bool ptr_of(PyObject* o, void** out) {
   if (o == Py_None) { *out = nullptr; return true; }
   if (PyLong_Check(o)) {
@@ -30,7 +50,7 @@ bool ptr_of(PyObject* o, void** out) {
     return !(PyErr_Occurred());
   }
   PyObject* r = PyObject_CallMethodNoArgs(o, s_is_contiguous);
-  if (!r) return false;
+  if (!r) return PyErr_ExceptionMatches(PyExc_AttributeError) && array_ptr(o, out);
   const int yes = PyObject_IsTrue(r);
   Py_DECREF(r);
   if (yes <= 0) {
@@ -83,15 +103,16 @@ PyObject* moe_forward(PyObject*, PyObject* const* args, Py_ssize_t n) {
                      (feplb_plan_out*)t[0], t[1]));
 }
 
-// (ctx, d_out, gates, w1t, w3t, w2t, buf, bwd, dw1, dw3, dw2, accumulate, stream)
+// (ctx, d_out, gates, w1t, w3t, w2t, buf, bwd, dw1, dw3, dw2, accumulate, stream); of buf only x_perm, h_scratch, y_perm
+// and slot_to_row
 PyObject* moe_backward(PyObject*, PyObject* const* args, Py_ssize_t n) {
-  void *a[6], *b[8], *g[6], *t[3], *st;
-  if (!want(n, 13, "moe_backward") || !ptrs_of(args, 6, a) || !attrs_of(args[6], s_buf, 8, b) || !attrs_of(args[7], s_bwd, 6, g) ||
+  void *a[6], *b[4], *g[6], *t[3], *st;
+  if (!want(n, 13, "moe_backward") || !ptrs_of(args, 6, a) || !attrs_of(args[6], s_buf + 2, 4, b) || !attrs_of(args[7], s_bwd, 6, g) ||
       !ptrs_of(args + 8, 3, t) || !ptr_of(args[12], &st))
     return nullptr;
   const long acc = PyLong_AsLong(args[11]);
   if (acc == -1 && PyErr_Occurred()) return nullptr;
-  CALL(rc, p_backward((feplb_ctx*)a[0], a[1], (const float*)a[2], a[3], a[4], a[5], b[2], g[0], b[3], b[4], (const int32_t*)b[5],
+  CALL(rc, p_backward((feplb_ctx*)a[0], a[1], (const float*)a[2], a[3], a[4], a[5], b[0], g[0], b[1], b[2], (const int32_t*)b[3],
                       g[1], g[2], g[3], g[4], (float*)g[5], (float*)t[0], (float*)t[1], (float*)t[2], (int32_t)acc, st));
 }
 
@@ -156,6 +177,8 @@ PyMODINIT_FUNC PyInit__feplb_py(void) {
   const char* bwd[6] = {"ab", "d_y_perm", "d_ab", "d_x_perm", "d_x", "d_gates"};
   s_is_contiguous = PyUnicode_InternFromString("is_contiguous");
   s_data_ptr = PyUnicode_InternFromString("data_ptr");
+  s_ctypes = PyUnicode_InternFromString("ctypes");
+  s_data = PyUnicode_InternFromString("data");
   for (int i = 0; i < 8; ++i) s_buf[i] = PyUnicode_InternFromString(buf[i]);
   for (int i = 0; i < 6; ++i) s_bwd[i] = PyUnicode_InternFromString(bwd[i]);
   return PyModule_Create(&module);

@@ -335,7 +335,8 @@ class Context:
     def _stream(stream) -> Optional[int]:
         if stream is None:
             return _current_stream()
-        return getattr(stream, "cuda_stream", stream) or None
+        h = getattr(stream, "cuda_stream", stream)
+        return (h.value if isinstance(h, C.c_void_p) else h) or None
 
     def check_status(self, stream=None):
         self._chk(lib().feplb_check_status(self._h, self._stream(stream)), "feplb_check_status")
