@@ -1,5 +1,5 @@
-"""Builds libfeplb.so (C ABI + sm_100a kernels) in-tree with nvcc, and with g++ the CPython module the binding
-makes its per-micro-batch calls through.
+"""Builds libfeplb.so (C ABI + sm_100a kernels) in-tree with nvcc, and with g++, where there are Python headers, the
+CPython module the binding makes its per-micro-batch calls through (without it they go through ctypes).
 
 ``python -m paper_2604_19654_b200.build [--force] [-v] [--nvcc-flag=FLAG ...]`` or ``build()``;
 nvcc cross-compiles without a GPU.  ``-v`` prints ptxas resource usage; ``--nvcc-flag`` appends one
@@ -8,6 +8,7 @@ reads no environment variable besides NVCC, the compiler's path).
 """
 from __future__ import annotations
 
+import importlib.machinery
 import os
 import shutil
 import subprocess
@@ -18,7 +19,7 @@ HERE = os.path.dirname(os.path.abspath(__file__))
 ROOT = os.path.dirname(HERE)
 CSRC = os.path.join(HERE, "csrc")
 LIB = os.path.join(HERE, "libfeplb.so")
-PY_LIB = os.path.join(HERE, "_feplb_py.so")
+PY_LIB = os.path.join(HERE, "_feplb_py" + importlib.machinery.EXTENSION_SUFFIXES[0])   # this interpreter's ABI alone loads it
 SOURCES = ["feplb_plan.cpp", "feplb_api.cu", "feplb_route.cu", "feplb_combine.cu", "feplb_gemm.cu",
            "feplb_noalloc.cu", "feplb_gemm_bwd.cu", "feplb_gemm_wm.cu"]
 
@@ -30,10 +31,17 @@ def _nvcc() -> str:
     raise RuntimeError("nvcc not found: libfeplb cannot be built (there is no CPU fallback)")
 
 
+def _python_include():
+    """Directory of this interpreter's headers, or None where the module cannot be built."""
+    inc = sysconfig.get_paths()["include"]
+    return inc if shutil.which("g++") and os.path.exists(os.path.join(inc, "Python.h")) else None
+
+
 def needs_build() -> bool:
-    if not os.path.exists(LIB) or not os.path.exists(PY_LIB):
+    targets = [LIB, PY_LIB] if _python_include() else [LIB]
+    if not all(os.path.exists(p) for p in targets):
         return True
-    t = min(os.path.getmtime(LIB), os.path.getmtime(PY_LIB))
+    t = min(os.path.getmtime(p) for p in targets)
     deps = [os.path.join(CSRC, f) for f in os.listdir(CSRC)] + [os.path.join(ROOT, "include", "feplb.h")]
     return any(os.path.getmtime(p) > t for p in deps)
 
@@ -62,9 +70,6 @@ def build(force: bool = False, verbose: bool = False, extra_flags=()) -> str:
         try:
             if not force and not needs_build():
                 return LIB
-            _run([shutil.which("g++") or "g++", "-shared", "-fPIC", "-O2", "-std=c++17", "-I", sysconfig.get_paths()["include"],
-                  "-I", os.path.join(ROOT, "include"), "-o", f"{PY_LIB}.{os.getpid()}.tmp", os.path.join(CSRC, "feplb_py.cpp"),
-                  "-ldl"], PY_LIB, verbose)
             tmp = f"{LIB}.{os.getpid()}.tmp"
             cmd = [_nvcc(), "-shared", "-O3", "-std=c++17", "-lineinfo",
                    "-gencode", "arch=compute_100a,code=sm_100a",
@@ -75,6 +80,12 @@ def build(force: bool = False, verbose: bool = False, extra_flags=()) -> str:
             if verbose:
                 cmd.insert(1, "-Xptxas=-v")
             _run(cmd, LIB, verbose)
+            inc = _python_include()
+            if inc:
+                _run(["g++", "-shared", "-fPIC", "-O2", "-std=c++17", "-I", inc, "-I", os.path.join(ROOT, "include"),
+                      "-o", f"{PY_LIB}.{os.getpid()}.tmp", os.path.join(CSRC, "feplb_py.cpp"), "-ldl"], PY_LIB, verbose)
+            elif os.path.exists(PY_LIB):
+                os.remove(PY_LIB)          # of an older library
             return LIB
         finally:
             fcntl.flock(lock, fcntl.LOCK_UN)

@@ -1,5 +1,5 @@
 """Thin binding over the C ABI of ``libfeplb.so`` (see ``include/feplb.h``): ctypes, and for the calls a program
-makes per micro-batch a small CPython module (``csrc/feplb_py.cpp``).
+makes per micro-batch a small CPython module (``csrc/feplb_py.cpp``) where one was built for this interpreter.
 
 Argument marshalling only: every step of the path runs in the library's CUDA kernels (or, for
 the plan, in its C++ host code).  PyTorch supplies device memory and streams.  If the library is
@@ -8,6 +8,7 @@ missing the import of a symbol fails loudly -- there is no fallback.
 from __future__ import annotations
 
 import ctypes as C
+import importlib.machinery
 import importlib.util
 import os
 from typing import Optional, Sequence
@@ -16,7 +17,7 @@ import numpy as np
 
 _HERE = os.path.dirname(os.path.abspath(__file__))
 LIB_PATH = os.path.join(_HERE, "libfeplb.so")
-PY_LIB_PATH = os.path.join(_HERE, "_feplb_py.so")
+PY_LIB_PATH = os.path.join(_HERE, "_feplb_py" + importlib.machinery.EXTENSION_SUFFIXES[0])
 
 OK, E_INVALID, E_RANGE, E_CUDA, E_NOMEM, E_TIMEOUT, E_STATE, E_DEVICE = 0, -1, -2, -3, -4, -5, -6, -7
 POLICY_LITERAL, POLICY_FIRST_FIT = 0, 1
@@ -134,9 +135,31 @@ def lib() -> C.CDLL:
 _fast_mod = None
 
 
+class _CtypesCalls:
+    """The calls of the CPython module, argument for argument, through ctypes."""
+
+    _BUF = ("counts", "rank_load", "x_perm", "h_scratch", "y_perm", "slot_to_row", "row_to_token", "out")
+
+    def __getattr__(self, name):
+        fn = getattr(lib(), "feplb_" + name)
+        return lambda h, *a: fn(h, *map(_ptr, a[:-1]), a[-1])
+
+    def moe_forward(self, h, *a):
+        *first, buf, plan, stream = a
+        return lib().feplb_moe_forward(h, *map(_ptr, first), *(_ptr(getattr(buf, n)) for n in self._BUF),
+                                       C.cast(plan, C.POINTER(PlanOut)), stream)
+
+    def moe_backward(self, h, d_out, gates, w1t, w3t, w2t, buf, bwd, dw1, dw3, dw2, accumulate, stream):
+        t = (d_out, gates, w1t, w3t, w2t, buf.x_perm, bwd.ab, buf.h_scratch, buf.y_perm, buf.slot_to_row, bwd.d_y_perm,
+             bwd.d_ab, bwd.d_x_perm, bwd.d_x, bwd.d_gates, dw1, dw3, dw2)
+        return lib().feplb_moe_backward(h, *map(_ptr, t), accumulate, stream)
+
+
 def _fast():
     """The CPython module of the per-micro-batch calls, bound to the same library as lib() (once)."""
     global _fast_mod
+    if _fast_mod is None and not os.path.exists(PY_LIB_PATH):
+        return _CtypesCalls()
     if _fast_mod is None:
         lib()
         spec = importlib.util.spec_from_file_location("_feplb_py", PY_LIB_PATH)

@@ -1,7 +1,9 @@
-"""The per-micro-batch calls of the binding take the same objects and hand on the same addresses as the ctypes route they
-stand for.  A recording stub takes the library's place; no call touches a GPU."""
+"""The per-micro-batch calls of the binding, through the CPython module and through ctypes, take the same objects and hand
+on the same addresses.  A recording stub takes the library's place; no call touches a GPU."""
 import ctypes as C
+import os
 import subprocess
+import sysconfig
 from types import SimpleNamespace
 
 import numpy as np
@@ -18,8 +20,8 @@ BUF = ["counts", "rank_load", "x_perm", "h_scratch", "y_perm", "slot_to_row", "r
 BWD = ["ab", "d_y_perm", "d_ab", "d_x_perm", "d_x", "d_gates"]
 
 
-@pytest.fixture(scope="module")
-def calls(tmp_path_factory):
+@pytest.fixture(scope="module", params=["module", "ctypes"])
+def calls(tmp_path_factory, request):
     """(module, function that returns what the stub was given last)"""
     B.build()
     src = tmp_path_factory.mktemp("stub") / "stub.cpp"
@@ -31,11 +33,21 @@ def calls(tmp_path_factory):
     src.write_text(text + "}\n")
     lib = str(src.with_suffix(".so"))
     subprocess.run(["g++", "-shared", "-fPIC", "-o", lib, str(src)], check=True)
-    mod = F._fast()
-    mod.load(lib)
-    seen = (C.c_ulonglong * 32).in_dll(C.CDLL(lib), "seen")
-    yield mod, lambda name: [v or None for v in seen[:ARITY[name]]]
-    mod.load(F.LIB_PATH)
+    stub = C.CDLL(lib)
+    for name in ARITY:
+        getattr(stub, name).argtypes = getattr(F.lib(), name).argtypes
+    seen = (C.c_ulonglong * 32).in_dll(stub, "seen")
+    read = lambda name: [v or None for v in seen[:ARITY[name]]]       # noqa: E731
+    if request.param == "module":
+        mod = F._fast()
+        assert not isinstance(mod, F._CtypesCalls)
+        mod.load(lib)
+        yield mod, read
+        mod.load(F.LIB_PATH)
+    else:
+        with pytest.MonkeyPatch.context() as m:
+            m.setattr(F, "lib", lambda: stub)
+            yield F._CtypesCalls(), read
 
 
 def _objects(n, kind):
@@ -85,3 +97,17 @@ def test_refused_objects(calls):
                                            (SimpleNamespace(cuda_stream=12), 12), (SimpleNamespace(cuda_stream=0), None)])
 def test_stream_handles(stream, handle):
     assert F.Context._stream(stream) == handle
+
+
+def test_interpreter_without_the_module(monkeypatch, tmp_path):
+    """The module's file name carries the interpreter's ABI; without that file the calls go through ctypes, and without
+    Python headers the library alone makes the build complete."""
+    B.build()
+    assert F.PY_LIB_PATH == B.PY_LIB and F.PY_LIB_PATH.endswith(sysconfig.get_config_var("EXT_SUFFIX"))
+    monkeypatch.setattr(F, "_fast_mod", None)
+    monkeypatch.setattr(F, "PY_LIB_PATH", str(tmp_path / "none.so"))
+    assert isinstance(F._fast(), F._CtypesCalls) and F._fast().combine(None, None, None, None, None, None) == F.E_INVALID
+    monkeypatch.setattr(B, "PY_LIB", str(tmp_path / "none.so"))
+    assert B.needs_build()
+    monkeypatch.setattr(B, "_python_include", lambda: None)
+    assert not B.needs_build() and os.path.exists(B.LIB)
