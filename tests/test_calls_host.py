@@ -20,9 +20,8 @@ BUF = ["counts", "rank_load", "x_perm", "h_scratch", "y_perm", "slot_to_row", "r
 BWD = ["ab", "d_y_perm", "d_ab", "d_x_perm", "d_x", "d_gates"]
 
 
-@pytest.fixture(scope="module", params=["module", "ctypes"])
-def calls(tmp_path_factory, request):
-    """(module, function that returns what the stub was given last)"""
+@pytest.fixture(scope="module")
+def stub_path(tmp_path_factory):
     B.build()
     src = tmp_path_factory.mktemp("stub") / "stub.cpp"
     text = "extern \"C\" { unsigned long long seen[32];\n"
@@ -33,7 +32,13 @@ def calls(tmp_path_factory, request):
     src.write_text(text + "}\n")
     lib = str(src.with_suffix(".so"))
     subprocess.run(["g++", "-shared", "-fPIC", "-o", lib, str(src)], check=True)
-    stub = C.CDLL(lib)
+    return lib
+
+
+@pytest.fixture(params=["module", "ctypes"])
+def calls(stub_path, request):
+    """(module, function that returns what the stub was given last)"""
+    stub = C.CDLL(stub_path)
     for name in ARITY:
         getattr(stub, name).argtypes = getattr(F.lib(), name).argtypes
     seen = (C.c_ulonglong * 32).in_dll(stub, "seen")
@@ -41,7 +46,7 @@ def calls(tmp_path_factory, request):
     if request.param == "module":
         mod = F._fast()
         assert not isinstance(mod, F._CtypesCalls)
-        mod.load(lib)
+        mod.load(stub_path)
         yield mod, read
         mod.load(F.LIB_PATH)
     else:
