@@ -123,7 +123,8 @@ typedef struct {
    * at the end of pass 1, when the planner's table was on the device before the launch. */
   double dev_ffn_pass1_us, dev_ffn_pass2_us; /* device: first CTA's start -> last CTA's end of each pass */
   double dev_plan_wait_us;              /* device: longest time a CTA spent waiting for the dynamic table */
-  double ffn_launches;                  /* GEMM launches of the forward: 4 (static, dynamic x 2 passes) or 2 */
+  double ffn_launches;                  /* GEMM launches of the forward: 4 (static, dynamic x 2 passes) or 2 (a host-buffer
+                                         * forward in token ranges: 2 per range) */
 } feplb_timeline;
 
 typedef struct feplb_ctx feplb_ctx;

@@ -991,6 +991,8 @@ static int host_forward_ranges(feplb_ctx* c, int n, const int* first, const void
   }
   c->t0 = clk::now();
   c->timeline_valid = true;
+  memset(&c->tl, 0, sizeof(c->tl));
+  c->tl.ffn_launches = 2 * n;
   // inputs: after whatever `st` still does with the staging buffers
   CUDA_TRY(c, cudaEventRecord(c->ev_range_ids, st));
   CUDA_TRY(c, cudaStreamWaitEvent(c->in_stream, c->ev_range_ids, 0));
@@ -1040,7 +1042,9 @@ static int host_forward_ranges(feplb_ctx* c, int n, const int* first, const void
   rc = await_counts(c, c->flag_seq);
   if (rc == FEPLB_OK) rc = make_plan(c, dyn_mask_host);
   if (rc != FEPLB_OK) return fail(c, rc, "planner failed: %s", feplb_strerror(rc));
-  return copy_plan(c, plan_copy);
+  rc = copy_plan(c, plan_copy);
+  c->tl.host_upload_enqueued_us = c->tl.host_join_us = c->tl.host_return_us = us_since(c->t0);
+  return rc;
 }
 
 extern "C" int feplb_moe_forward_host(feplb_ctx* c, const void* x_host, const int32_t* topk_ids_host,

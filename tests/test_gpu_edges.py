@@ -271,3 +271,22 @@ def test_dispatch_takes_the_segments_from_the_counts(T, A):
         assert ei.value.code == F.E_DEVICE
         assert np.array_equal(buf.slot_to_row.cpu().numpy().ravel(), rows), delta
     ctx.close()
+
+
+def test_host_times_of_a_forward_in_token_ranges():
+    """feplb_get_timeline after a host-buffer forward in token ranges: this call's host times, none left by another."""
+    import torch
+    w = W.get_workload("cfg1").with_(T=4096, K=2, E=8, d=1024, f=64, tau=1)
+    case = DeviceCase(w)
+    case.ctx.moe_forward(case.d_x, case.d_ids, case.d_gates, case.d_w1, case.d_w3, case.d_w2, case.buf)
+    host = [t.cpu().pin_memory() for t in (case.d_x, case.d_ids, case.d_gates)]
+    out = torch.zeros(w.T, w.d, dtype=torch.bfloat16).pin_memory()
+    torch.cuda.synchronize()
+    before = case.ctx.launch_count()
+    case.ctx.moe_forward_host(*host, case.d_x, case.d_ids, case.d_gates, case.d_w1, case.d_w3, case.d_w2, case.buf, out)
+    ranges = (case.ctx.launch_count() - before - 3) // 4                     # 3 launches for the batch, 4 per range
+    t = case.ctx.get_timeline()
+    assert ranges > 1 and t["ffn_launches"] == 2 * ranges
+    assert 0 < t["host_enqueue_static_done_us"] <= t["host_counts_ready_us"] <= t["host_plan_done_us"]
+    assert t["host_plan_done_us"] <= t["host_upload_enqueued_us"] <= t["host_join_us"] <= t["host_return_us"]
+    case.close()
