@@ -297,7 +297,7 @@ k_grouped_gemm(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__
   // the group table: the kernel before this one had itself waited for the table's writer when it let this
   // one start.  For the same reason this kernel lets its successor start only after its own wait.
   if (!p.early_weights) asm volatile("griddepcontrol.wait;" ::: "memory");
-  if (p.stamps && threadIdx.x == 0) atomicMin(&p.stamps[0], global_timer_ns());
+  if (p.stamps && !p.early_weights && threadIdx.x == 0) atomicMin(&p.stamps[0], global_timer_ns());
   for (int g = threadIdx.x; g < p.n_groups; g += kThreads) {
     const feplb_group gr = p.groups[g];
     const bool selected = p.which == FEPLB_FFN_ALL || (p.which == FEPLB_FFN_STATIC) == (gr.is_dynamic == 0);
@@ -326,7 +326,10 @@ k_grouped_gemm(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__
   const int n_static_entries = early ? tail->n_entries : p.n_groups;
   const int n_static_tiles = tail->prefix[n_static_entries] * p.n_tiles_n;
   // (the producer waits on its own, after its first weight loads)
-  if (p.early_weights && warp != 0) asm volatile("griddepcontrol.wait;" ::: "memory");
+  if (p.early_weights && warp != 0) {
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    if (p.stamps && threadIdx.x == 32) atomicMin(&p.stamps[0], global_timer_ns());
+  }
   if (warp != 0) asm volatile("griddepcontrol.launch_dependents;");
 
   if (warp == 0) {

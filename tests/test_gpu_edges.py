@@ -290,3 +290,22 @@ def test_host_times_of_a_forward_in_token_ranges():
     assert 0 < t["host_enqueue_static_done_us"] <= t["host_counts_ready_us"] <= t["host_plan_done_us"]
     assert t["host_plan_done_us"] <= t["host_upload_enqueued_us"] <= t["host_join_us"] <= t["host_return_us"]
     case.close()
+
+
+@pytest.mark.parametrize("form", [F.FORM_PAIR, F.FORM_WEIGHT_M])
+def test_pass_times_do_not_overlap(form):
+    """The two passes' own times fit into the interval between the events around their launches: a CTA of pass 2 that is
+    resident but still waits for pass 1 does not count."""
+    w = W.get_workload("cfg2")
+    case = DeviceCase(w)
+    case.ctx.set_gemm_form(form)
+    case.ctx.set_launch_merging(1)
+    case.ctx.set_timeline(True)
+    slack = []
+    for _ in range(15):
+        case.ctx.moe_forward(case.d_x, case.d_ids, case.d_gates, case.d_w1, case.d_w3, case.d_w2, case.buf, want_plan=False)
+        t = case.ctx.get_timeline()
+        slack.append(t["dev_static_ffn_us"] - t["dev_ffn_pass1_us"] - t["dev_ffn_pass2_us"])
+    case.ctx.check_status()
+    assert np.median(slack) > 0, slack
+    case.close()
