@@ -390,13 +390,15 @@ def merged_timeline(st):
             ["host: dynamic table published / upload enqueued", counts_at + st["host_upload_enqueued_us"] - h0,
              counts_at + st["host_upload_enqueued_us"] - h0]]
     if st.get("ffn_launches", 4) < 3:
-        # weights-on-M form: one launch per pass; the marks inside the launches come from the GPU's timer
+        # one launch per pass; the marks inside the launches come from the GPU's timer.  A forward whose table came with the
+        # gather has no static part of its own (static end = static start)
         p1e = s0 + st["dev_ffn_pass1_us"]
+        both = "static and dynamic groups side by side, the table from the gather" if s1 - s0 < 1.0 else "remaining static and dynamic groups"
         tl = [["hist+scan (counts to host)", 0.0, counts_at],
               ["rank+gather (dispatch)", counts_at, counts_at + st["dev_dispatch_us"]],
-              ["FFN pass 1: static groups (until the first CTA runs out of them)", s0, s1]] + host + [
-              ["FFN pass 1: remaining static and dynamic groups", s1, p1e],
-              ["FFN pass 2: static, then dynamic groups", d1 - st["dev_ffn_pass2_us"], d1],
+              ["FFN pass 1: static groups alone (until the first CTA runs out of them)", s0, s1]] + host + [
+              [f"FFN pass 1: {both}", s1, p1e],
+              ["FFN pass 2: static and dynamic groups", d1 - st["dev_ffn_pass2_us"], d1],
               ["longest device-side wait for the dynamic table", s1, s1 + st["dev_plan_wait_us"]],
               ["combine", d1, st["dev_total_us"]]]
         return [[n, round(a, 2), round(b, 2)] for n, a, b in tl]

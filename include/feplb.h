@@ -119,8 +119,9 @@ typedef struct {
   /* Merged launches only (one launch per pass walks the static, then the dynamic groups); the
    * marks are taken inside the kernels from the GPU's global timer.  There dev_static_ffn_us is the
    * whole expert FFN, dev_dynamic_ffn_us is 0, dev_counts_to_static_start_us ends at the first CTA's
-   * start and dev_counts_to_static_end_us at the first moment a CTA ran out of static work -- or
-   * at the end of pass 1, when the planner's table was on the device before the launch. */
+   * start and dev_counts_to_static_end_us at the first moment a CTA ran out of static work.  When the
+   * planner's table was on the device before the launch, static and dynamic groups run side by side and
+   * the two are equal; when no launch needs the plan, the latter ends with pass 1. */
   double dev_ffn_pass1_us, dev_ffn_pass2_us; /* device: first CTA's start -> last CTA's end of each pass */
   double dev_plan_wait_us;              /* device: longest time a CTA spent waiting for the dynamic table */
   double ffn_launches;                  /* GEMM launches of the forward: 4 (static, dynamic x 2 passes) or 2 (a host-buffer

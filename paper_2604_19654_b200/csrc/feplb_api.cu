@@ -28,7 +28,8 @@ inline double us_since(clk::time_point t0) {
 enum JobState { JOB_IDLE = 0, JOB_PENDING = 1, JOB_RUNNING = 2, JOB_DONE = 3 };
 enum { EV_T0 = 0, EV_HIST, EV_DISPATCH, EV_STATIC0, EV_STATIC1, EV_DYN0, EV_DYN1, EV_COMBINE, EV_COUNTS, EV_COPIES, EV_STAMPS, EV_N };
 constexpr int kEvRing = 16;   // forwards whose stage events may be outstanding
-constexpr int kStampWords = 16;   // [0..3] pass 1, [4..7] pass 2 (see WmParams::stamps), [8] counts left the device
+constexpr int kStampWords = 16;   // [0..3] pass 1, [4..7] pass 2 (see WmParams::stamps), [8] counts left the device, [9] table
+                                  // brought over by the gather
 }  // namespace
 
 struct feplb_ctx {
@@ -765,7 +766,9 @@ static int harvest_slot(feplb_ctx* c, int r) {
     t.dev_ffn_pass1_us = span(p1_start, p1_end);
     t.dev_ffn_pass2_us = span(p2_start, p2_end);
     t.dev_counts_to_static_start_us = span(t_counts, p1_start);
-    t.dev_counts_to_static_end_us = span(t_counts, p1_first_dyn != none ? p1_first_dyn : p1_end);
+    // table there before the launch: static and dynamic groups side by side, no static part of its own;
+    // no CTA ran out of static work otherwise: every group counts as static (the order that does not need the plan)
+    t.dev_counts_to_static_end_us = span(t_counts, sp[9] != none ? p1_start : p1_first_dyn != none ? p1_first_dyn : p1_end);
     const unsigned long long w1 = sp[3] == none ? 0 : ~sp[3], w2 = sp[7] == none ? 0 : ~sp[7];
     t.dev_plan_wait_us = (w1 > w2 ? w1 : w2) * 1e-3;
   }

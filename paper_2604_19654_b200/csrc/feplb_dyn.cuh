@@ -37,6 +37,7 @@ struct DynTable {
   unsigned long long* ready_dev;        // (seq << 32) | number of dynamic groups
   const unsigned long long* ready_host;
   unsigned long long* early;            // seq of the forward whose table was on the device before its GEMM launches started
+  unsigned long long* delivered;        // optional: when it got there (globaltimer, ns)
   uint32_t* claim;                      // device word: seq of the forward whose table transfer has been claimed
   int dyn_cap;                          // capacity of dyn_dev in groups
   uint32_t seq;                         // 0: no dynamic table in this launch
@@ -159,7 +160,10 @@ __device__ __forceinline__ void dyn_deliver_early(const DynTable& d, int lane, u
   }
   if (!__shfl_sync(0xffffffffu, there, 0)) return;
   dyn_bring_table(d, lane, status, __shfl_sync(0xffffffffu, (int)(uint32_t)v, 0));
-  if (lane == 0) *reinterpret_cast<volatile unsigned long long*>(d.early) = d.seq;
+  if (lane == 0) {
+    *reinterpret_cast<volatile unsigned long long*>(d.early) = d.seq;
+    if (d.delivered) *d.delivered = global_timer_ns();
+  }
 }
 
 // The planner's table is there already: its groups join the home table, one group of each dynamic expert (the first piece
@@ -201,6 +205,7 @@ inline DynTable feplb_dyn_table(const feplb_wm_dyn& dyn) {
   d.ready_host = dyn.ready_host;
   d.claim = dyn.claim;
   d.early = dyn.early;
+  d.delivered = dyn.stamps ? dyn.stamps + 9 : nullptr;
   d.dyn_cap = dyn.max_groups;
   d.seq = dyn.seq;
   d.wait_limit_ns = dyn.wait_limit_ns ? dyn.wait_limit_ns : kWaitLimitNs;

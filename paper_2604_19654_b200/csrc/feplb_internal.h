@@ -58,7 +58,7 @@ struct feplb_wm_dyn {
   unsigned long long* early = nullptr;               // device word: seq of the forward whose table the gather brought over
   uint32_t seq = 0;                                  // 0: no dynamic table
   int max_groups = 0;                                // capacity of the tables
-  unsigned long long* stamps = nullptr;              // optional, 8 words: globaltimer marks of the two launches
+  unsigned long long* stamps = nullptr;              // optional: globaltimer marks, [0..7] of the two launches, [9] early delivery
   unsigned long long wait_limit_ns = 0;              // bound of the wait for the table (0: the library's default)
 };
 // Must follow feplb_launch_permute or feplb_launch_route_fused on the same stream: turns the ranks those

@@ -144,24 +144,28 @@ def test_sweep_points(cfg3_weights, T, R):
 
 @pytest.mark.parametrize("name", ["cfg2", "cfg3"])
 def test_plan_upload_lands_inside_the_static_window(name, cfg3_weights):
-    """Section 2.3's overlap condition, asserted: the planner thread has enqueued the upload of the
-    dynamic group table before the static-expert GEMM ends.  Both intervals start when the counts
-    leave the device: the host one is (upload enqueued - counts seen by the planner thread), the
-    device one (counts written -> static tiles done).  Median over 20 forwards after warm-up."""
+    """Section 2.3's overlap condition, asserted: the planner thread has published the dynamic group
+    table before the GPU can use it.  Both intervals start when the counts leave the device: the
+    host one is (published - counts seen by the planner thread), the device one (counts written ->
+    static tiles done), or, in forwards whose launches have the table from their start, (counts
+    written -> first CTA of pass 1), i.e. the end of the gather.  Median over 20 forwards after
+    warm-up.  At cfg2 the table comes with the gather, in most forwards at least."""
     w = W.get_workload(name)
     case = DeviceCase(w, mb=0, weights=cfg3_weights if name == "cfg3" else None)
     for _ in range(3):
         case.ctx.moe_forward(case.d_x, case.d_ids, case.d_gates, case.d_w1, case.d_w3, case.d_w2, case.buf, want_plan=False)
     case.ctx.check_status()
     case.ctx.set_timeline(True)
-    host, dev, plan_us = [], [], []
+    host, dev, plan_us, early = [], [], [], []
     for _ in range(20):
         case.ctx.moe_forward(case.d_x, case.d_ids, case.d_gates, case.d_w1, case.d_w3, case.d_w2, case.buf, want_plan=False)
         tl = case.ctx.get_timeline()
         host.append(tl["host_upload_enqueued_us"] - tl["host_counts_ready_us"])
         dev.append(tl["dev_counts_to_static_end_us"])
         plan_us.append(tl["plan_us"])
+        early.append(tl["dev_counts_to_static_end_us"] == tl["dev_counts_to_static_start_us"])
     case.ctx.check_status()
+    assert np.median(early) == (name == "cfg2"), early           # cfg3: four launches
     assert min(host) >= 0 and min(dev) > 0
     assert np.median(host) < np.median(dev), (np.median(host), np.median(dev))
     # the greedy itself is tens of microseconds at most (the paper quotes ~50 us on one core)
