@@ -453,6 +453,16 @@ int feplb_set_planner_timing(feplb_ctx* ctx, int32_t planner_delay_us, int32_t d
  * Returns FEPLB_OK if the wait gave up, raised the status bit and the kernel returned normally;
  * FEPLB_E_STATE otherwise.  The status word is clear afterwards.  Synchronises `stream`. */
 int feplb_selftest_bounded_wait(feplb_ctx* ctx, int32_t limit_us, void* stream);
+/* How the last forward on `ctx` was launched, FEPLB_PATH_* bits: the order of its launches and every form that its
+ * expert GEMMs took (0 before the first one). */
+#define FEPLB_PATH_SMALL_FRONT 1   /* routing and gather in one launch */
+#define FEPLB_PATH_HOME_TABLE 2    /* no launch needs the plan: both passes walk the home groups */
+#define FEPLB_PATH_MERGED 4        /* one launch per pass over static and dynamic groups */
+#define FEPLB_PATH_RANGES 8        /* host-buffer forward in token ranges */
+#define FEPLB_PATH_SINGLE 16       /* single-CTA tiles of 128 rows */
+#define FEPLB_PATH_PAIR 32         /* two-CTA tiles of 256 rows */
+#define FEPLB_PATH_WEIGHT_M 64     /* weights-on-M units */
+int32_t feplb_forward_path(const feplb_ctx* ctx);
 /* Number of kernels this library has launched on `ctx` since creation. */
 int64_t feplb_launch_count(const feplb_ctx* ctx);
 

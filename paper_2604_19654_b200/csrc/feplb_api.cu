@@ -39,6 +39,7 @@ struct feplb_ctx {
   int nb = 0;   // CTAs of the permutation kernels
   char err[512] = {0};
   int64_t launches = 0;
+  int32_t path = 0;            // FEPLB_PATH_* of the last forward
   int gemm_pair_default = 0;   // GEMM form for launches whose group sizes the host does not know
   int gemm_pair_forced = -1;   // feplb_set_gemm_form: 0/1 forces one form everywhere, -1 = chosen per table
   int bwd_pair = 0;            // backward GEMMs in the pair form: bit 0 activation gradients, bit 1 weight gradients
@@ -543,6 +544,8 @@ extern "C" int feplb_destroy(feplb_ctx* c) {
 
 extern "C" const char* feplb_last_error(const feplb_ctx* c) { return c ? c->err : ""; }
 
+extern "C" int32_t feplb_forward_path(const feplb_ctx* c) { return c ? c->path : 0; }
+
 extern "C" int64_t feplb_launch_count(const feplb_ctx* c) { return c ? c->launches : 0; }
 
 extern "C" int feplb_check_status(feplb_ctx* c, void* stream) {
@@ -631,9 +634,11 @@ static int ffn_impl(feplb_ctx* c, const void* x_perm, const void* w1, const void
   a.recv_w1 = c->d_recv_w1; a.recv_w3 = c->d_recv_w3; a.recv_w2 = c->d_recv_w2; a.n_recv_slots = c->n_recv_slots;
   a.recv_x = c->d_recv_x;
   if ((c->wm || weights_on_m) && n_groups + (dyn ? dyn->max_groups : 0) <= FEPLB_WM_MAX_ENTRIES) {
+    c->path |= FEPLB_PATH_WEIGHT_M;
     const feplb_wm_dyn none;
     return feplb_launch_expert_ffn_wm(a, dyn ? *dyn : none, st, &c->launches, c->err, sizeof(c->err));
   }
+  c->path |= pair ? FEPLB_PATH_PAIR : FEPLB_PATH_SINGLE;
   return feplb_launch_expert_ffn(a, st, &c->launches, c->err, sizeof(c->err), dyn);
 }
 
@@ -850,6 +855,7 @@ extern "C" int feplb_moe_forward(feplb_ctx* c, const void* x, const int32_t* top
   c->flag_seq = c->flag_seq == INT32_MAX ? 1 : c->flag_seq + 1;
   const int32_t seq = c->flag_seq;
   const bool small_front = feplb_front_is_small(S, g.E);
+  c->path = (small_front ? FEPLB_PATH_SMALL_FRONT : 0) | (direct ? FEPLB_PATH_HOME_TABLE : wm ? FEPLB_PATH_MERGED : 0);
   if (small_front)
     CUDA_TRY(c, feplb_launch_front_small(x, topk_ids, g.T, g.K, g.E, g.R, g.d, g.row_align, g.dyn, mask_dev, nullptr, counts, rank_load,
                                          c->d_pad_off, c->d_home_groups, slot_to_row, row_to_token, x_perm, (int64_t)c->s_cap,
@@ -996,6 +1002,7 @@ static int host_forward_ranges(feplb_ctx* c, int n, const int* first, const void
   c->timeline_valid = true;
   memset(&c->tl, 0, sizeof(c->tl));
   c->tl.ffn_launches = 2 * n;
+  c->path = FEPLB_PATH_RANGES;
   // inputs: after whatever `st` still does with the staging buffers
   CUDA_TRY(c, cudaEventRecord(c->ev_range_ids, st));
   CUDA_TRY(c, cudaStreamWaitEvent(c->in_stream, c->ev_range_ids, 0));

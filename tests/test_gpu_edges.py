@@ -201,6 +201,7 @@ def test_host_forward_in_token_ranges(T, K, E, d, f, A):
     p1 = case.ctx.moe_forward_host(*host, *dev, case.d_w1, case.d_w3, case.d_w2, case.buf, out, want_plan=True)
     case.ctx.check_status()
     assert case.ctx.launch_count() - before >= 11                            # 3 + 4 per range: at least two ranges
+    assert case.ctx.forward_path() & F.PATH_RANGES
     assert (p1.moves, p1.groups) == (p0.moves, p0.groups)
     assert torch.equal(out, want["out"].cpu())
     for k in names:
@@ -258,15 +259,44 @@ def test_merged_orders_of_random_shapes_beyond_the_one_launch_front(seed):
     case.close()
 
 
-@pytest.mark.parametrize("T,merged", [(48, 1), (60, 0), (700, 0), (800, 0), (60, -1), (700, -1)])
-def test_form_rule_of_large_weights(T, merged):
+@pytest.mark.parametrize("T,merged,path", [
+    (48, 1, F.PATH_MERGED | F.PATH_SINGLE),                     # T rows per expert on average: below 64
+    (60, 0, F.PATH_WEIGHT_M | F.PATH_SINGLE),                   # four launches, static | dynamic
+    (700, 0, F.PATH_WEIGHT_M),
+    (800, 0, F.PATH_WEIGHT_M | F.PATH_PAIR),                    # above 768; the one dynamic expert of a rank has more than 512 rows
+    (60, -1, F.PATH_HOME_TABLE | F.PATH_SINGLE),
+    (700, -1, F.PATH_HOME_TABLE | F.PATH_WEIGHT_M),
+])
+def test_form_rule_of_large_weights(T, merged, path):
     """Shapes from which the weights-on-M form is chosen (3 Mi elements per matrix): below, inside and above its range of
     rows per expert, in every launch order."""
     w = W.get_workload("cfg2").with_(T=T, E=2, R=2, K=2, d=2048, f=1536, dyn=1, max_num_dyn=1, tau=1)
     case = DeviceCase(w)
+    assert case.ctx.forward_path() == 0
     case.ctx.set_launch_merging(merged)
     _check_forward(case, sample=40)
+    assert case.ctx.forward_path() == path | F.PATH_SMALL_FRONT
     case.close()
+
+
+@pytest.mark.parametrize("T,K,E,d,f,path", [
+    (1024, 2, 16, 256, 128, F.PATH_HOME_TABLE | F.PATH_SMALL_FRONT | F.PATH_SINGLE),      # 128 rows per expert, a short FFN
+    (2048, 2, 16, 256, 128, F.PATH_HOME_TABLE | F.PATH_SMALL_FRONT | F.PATH_PAIR),        # 256 rows per expert: two-CTA tiles
+    (2047, 1, 16, 4096, 2048, F.PATH_HOME_TABLE | F.PATH_SMALL_FRONT | F.PATH_WEIGHT_M),  # below 128 rows per expert
+    (2048, 1, 16, 4096, 2048, F.PATH_MERGED | F.PATH_SMALL_FRONT | F.PATH_WEIGHT_M),      # 128, and an FFN of 230 us
+    (6144, 1, 8, 4096, 2048, F.PATH_SMALL_FRONT | F.PATH_WEIGHT_M | F.PATH_PAIR),         # 768: four launches
+])
+def test_order_rule(T, K, E, d, f, path):
+    """The launch order on both sides of its lines."""
+    import torch
+    ctx, buf = (c(F.make_config(T, K, E, 2, d, f, dyn=1, tau=1)) for c in (F.Context, F.Buffers))
+    rng = torch.Generator(device="cuda").manual_seed(1)
+    z = lambda *s: torch.zeros(*s, dtype=torch.bfloat16, device="cuda")       # noqa: E731
+    ids = torch.rand(T, E, generator=rng, device="cuda").topk(K, dim=1)[1].int()
+    ctx.moe_forward(z(T, d), ids, torch.ones(T, K, device="cuda"), z(E, f, d), z(E, f, d), z(E, d, f), buf)
+    ctx.check_status()
+    assert ctx.forward_path() == path
+    ctx.close()
 
 
 @pytest.mark.parametrize("A", [1, 128])
