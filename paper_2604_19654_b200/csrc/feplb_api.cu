@@ -60,7 +60,7 @@ struct feplb_ctx {
   int32_t* h_dyn_tab32 = nullptr;                    // pinned + mapped: the dynamic table as 32-byte entries tagged with the sequence number
   int32_t* h_dyn_tab32_dev = nullptr;                // its device address
   int32_t* d_dyn_tab32 = nullptr;                    // device copy, made by the GEMM's claiming CTA
-  unsigned long long* d_dyn_ready = nullptr;         // device words: [0] ready, [1] claim, [2] early
+  unsigned long long* d_dyn_ready = nullptr;         // device words: [0] ready, [1] claim, [2] early, [3] gather done
   unsigned long long* h_dyn_ready = nullptr;         // pinned + mapped word, set by the planner thread
   unsigned long long* h_dyn_ready_dev = nullptr;     // its device address
   unsigned long long* d_stamps = nullptr;            // [kEvRing][kStampWords] globaltimer marks of the kernels
@@ -408,8 +408,8 @@ extern "C" int feplb_create(const feplb_config* cfg, feplb_ctx** out) {
   const double ffn_us = 6.0 * cfg->d * cfg->f * ((double)cfg->E / 6.5e6 + (double)S / 1e9);
   c->direct_auto = c->direct = S < (int64_t)FEPLB_DIRECT_ROWS_PER_EXPERT * cfg->E || ffn_us < FEPLB_DIRECT_FFN_US;
   bool ok = true;
-  ok = ok && cudaMalloc(&c->d_dyn_ready, 3 * sizeof(unsigned long long)) == cudaSuccess &&     // [0] ready word, [1] claim word, [2] early word
-       cudaMemset(c->d_dyn_ready, 0, 3 * sizeof(unsigned long long)) == cudaSuccess;
+  ok = ok && cudaMalloc(&c->d_dyn_ready, 4 * sizeof(unsigned long long)) == cudaSuccess &&
+       cudaMemset(c->d_dyn_ready, 0, 4 * sizeof(unsigned long long)) == cudaSuccess;
   ok = ok && cudaHostAlloc(&c->h_dyn_ready, sizeof(unsigned long long), cudaHostAllocMapped) == cudaSuccess &&
        cudaHostGetDevicePointer(&c->h_dyn_ready_dev, c->h_dyn_ready, 0) == cudaSuccess;
   if (ok) *c->h_dyn_ready = 0;
@@ -876,6 +876,7 @@ extern "C" int feplb_moe_forward(feplb_ctx* c, const void* x, const int32_t* top
   dyn.table_dev = c->d_dyn_tab32; dyn.table_host = c->h_dyn_tab32_dev;
   dyn.ready_dev = c->d_dyn_ready; dyn.ready_host = c->h_dyn_ready_dev;
   dyn.claim = reinterpret_cast<uint32_t*>(c->d_dyn_ready + 1); dyn.early = c->d_dyn_ready + 2;
+  dyn.gather_done = reinterpret_cast<uint32_t*>(c->d_dyn_ready + 3);
   dyn.seq = direct || !wm ? 0u : (uint32_t)seq; dyn.max_groups = direct ? 0 : c->plan.cap_groups; dyn.stamps = stamps;
   dyn.wait_limit_ns = 1000ull * (unsigned long long)c->device_wait_limit_us;
   // step 3: permutation (does not depend on the plan: a migration relabels rows, it does not move

@@ -4,7 +4,8 @@
 //
 // Usually the table is there before the GEMM starts: a CTA of the row gather, which runs while the planner works, picks it
 // up (dyn_deliver_early), and the launches walk static and dynamic groups together, in expert order.  What follows is
-// for a table that comes later than that.
+// for a table that comes later than that, and for batches whose routing and gather are one launch (k_route_small), which
+// has no such CTA.
 //
 // The planner thread writes the table -- 32-byte entries {expert, row_start, rows, exec_rank,
 // is_dynamic, seq, 0, 0} -- and then the word (seq << 32) | number of groups into mapped host
@@ -39,6 +40,7 @@ struct DynTable {
   unsigned long long* early;            // seq of the forward whose table was on the device before its GEMM launches started
   unsigned long long* delivered;        // optional: when it got there (globaltimer, ns)
   uint32_t* claim;                      // device word: seq of the forward whose table transfer has been claimed
+  uint32_t* gather_done;                // seq of the forward whose gather has a CTA without work left
   int dyn_cap;                          // capacity of dyn_dev in groups
   uint32_t seq;                         // 0: no dynamic table in this launch
   unsigned long long wait_limit_ns;     // bound of the wait for the table
@@ -145,18 +147,22 @@ __device__ __forceinline__ int dyn_wait_table(const DynTable& d, int lane, volat
 }
 
 // Warp-collective, by one CTA of the kernel in front of the GEMM (the row gather, which usually takes longer than the
-// planner): waits at most limit_ns for the planner's table and brings it over, so that the GEMM launches know it from
-// the start and need not run the static groups first.  When it is late nothing is left behind.
-__device__ __forceinline__ void dyn_deliver_early(const DynTable& d, int lane, uint32_t* status, unsigned long long limit_ns) {
+// planner): waits for the planner's table until the first of the other CTAs is done, but for least_ns at any rate, and
+// brings it over, so that the GEMM launches know it from the start and need not run the static groups first.  When it
+// is late nothing is left behind, and next to nothing has waited for it.
+__device__ __forceinline__ void dyn_deliver_early(const DynTable& d, int lane, uint32_t* status, unsigned long long least_ns) {
+  constexpr unsigned long long kLimitNs = 1000000;      // the other CTAs do not depend on this one; a bound all the same
   unsigned long long v = 0;
   int there = 0;
   if (lane == 0) {
     const unsigned long long t0 = global_timer_ns();
-    do {
+    for (;;) {
       v = ld_relaxed_sys_u64(d.ready_host);
       there = (uint32_t)(v >> 32) == d.seq;
-      if (!there) __nanosleep(100);
-    } while (!there && global_timer_ns() - t0 <= limit_ns);
+      const unsigned long long waited = global_timer_ns() - t0;
+      if (there || waited > kLimitNs || (waited > least_ns && *reinterpret_cast<volatile uint32_t*>(d.gather_done) == d.seq)) break;
+      __nanosleep(100);
+    }
   }
   if (!__shfl_sync(0xffffffffu, there, 0)) return;
   dyn_bring_table(d, lane, status, __shfl_sync(0xffffffffu, (int)(uint32_t)v, 0));
@@ -205,6 +211,7 @@ inline DynTable feplb_dyn_table(const feplb_wm_dyn& dyn) {
   d.ready_host = dyn.ready_host;
   d.claim = dyn.claim;
   d.early = dyn.early;
+  d.gather_done = dyn.gather_done;
   d.delivered = dyn.stamps ? dyn.stamps + 9 : nullptr;
   d.dyn_cap = dyn.max_groups;
   d.seq = dyn.seq;

@@ -56,6 +56,7 @@ struct feplb_wm_dyn {
   const unsigned long long* ready_host = nullptr;    // device address of the word the planner thread sets after table_host
   uint32_t* claim = nullptr;                         // device word the CTAs race for
   unsigned long long* early = nullptr;               // device word: seq of the forward whose table the gather brought over
+  uint32_t* gather_done = nullptr;                   // device word: seq of the forward whose gather has a CTA without work left
   uint32_t seq = 0;                                  // 0: no dynamic table
   int max_groups = 0;                                // capacity of the tables
   unsigned long long* stamps = nullptr;              // optional: globaltimer marks, [0..7] of the two launches, [9] early delivery

@@ -337,7 +337,11 @@ __device__ __forceinline__ uint4 ld_nc_v4(const uint4* p) {
 // slot_to_row and row_to_token entries (tokens [t0, t0 + T) of the batch).  Another warp working on a later slice of the same token may
 // read either form of the entry, and gets the same row from both.
 constexpr int kGatherUnroll = 4;
-constexpr unsigned long long kEarlyTableNs = 15000;   // the planner publishes its table about 5 us after the scan
+// How long the gather's first CTA looks for the planner's table even if the rows are copied in less: a planner whose
+// thread has a core to itself publishes it 2-3 us after the scan.  When the planner is late (held back 60 us), 64 experts,
+// d = 2048, us per layer without an early table -> a fixed wait of 15 us -> this: T = 1400 193 -> 196 -> 192, T = 2000
+// 230 -> 236 -> 233, T = 4096 350 in all three; when it is not: 193 -> 186 -> 185, 231 -> 223 -> 223, 350 -> 340 -> 340.
+constexpr unsigned long long kEarlyTableNs = 4000;
 // Work unit = (token, slice of 4 x 32 chunks = 2 KiB of its row).  Unit u goes to warp u mod #warps of a grid
 // sized to the machine: all warps work on neighbouring tokens at any time, and the rows of an expert, which
 // follow the token order, are written in one moving window per expert, so that DRAM pages are written while
@@ -398,6 +402,7 @@ k_gather(const uint4* __restrict__ x, const int32_t* __restrict__ ids, const int
       }
     }
   }
+  if (first && threadIdx.x == 0) *reinterpret_cast<volatile uint32_t*>(dyn.gather_done) = dyn.seq;
   if (A > 1) {                   // zeros for the padding rows at the end of every expert's segment, one row per warp at a time
     for (int64_t q = warp; q < (int64_t)E * A; q += nwarps) {
       const int e = (int)(q / A), c = counts[e] > 0 ? counts[e] : 0;

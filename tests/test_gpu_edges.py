@@ -228,14 +228,15 @@ def test_table_brought_over_by_the_gather(E, R, split, form):
         t = case.ctx.get_timeline()
         return t["dev_counts_to_static_end_us"] == t["dev_counts_to_static_start_us"]
 
-    for attempt in range(20):                                    # a busy host can be late by itself
-        p0, _ = _check_forward(case, sample=200)
-        out = F.bf16_bits(case.buf.out).copy()
+    for attempt in range(100):                                   # a busy host can be late by itself
+        for _ in range(4):                                       # the planner thread is up before the last one's counts are
+            p0 = case.ctx.moe_forward(case.d_x, case.d_ids, case.d_gates, case.d_w1, case.d_w3, case.d_w2, case.buf)
         if early():
             break
     assert early()
+    out = F.bf16_bits(case.buf.out).copy()
     case.ctx.set_planner_timing(planner_delay_us=2000)
-    p1, _ = _check_forward(case, sample=20)
+    p1, _ = _check_forward(case, sample=200)
     assert not early()
     assert p0.groups == p1.groups and len(p0.moves) > 0
     assert np.array_equal(F.bf16_bits(case.buf.out), out)
@@ -366,4 +367,21 @@ def test_pass_times_do_not_overlap(form):
         slack.append(t["dev_static_ffn_us"] - t["dev_ffn_pass1_us"] - t["dev_ffn_pass2_us"])
     case.ctx.check_status()
     assert np.median(slack) > 0, slack
+    case.close()
+
+
+def test_late_planner_does_not_hold_the_gather_up():
+    """The CTA that waits for the planner's table gives up soon after the rows are copied (here in about 3 us, under an
+    event interval of about 10): with the planner held back, the gather stays far below 15 us."""
+    w = W.get_workload("cfg1").with_(T=3000, K=4, E=16, R=4, d=256, f=128, tau=1)
+    case = DeviceCase(w)
+    case.ctx.set_launch_merging(1)
+    case.ctx.set_planner_timing(planner_delay_us=200)
+    case.ctx.set_timeline(True)
+    gather = []
+    for _ in range(15):
+        case.ctx.moe_forward(case.d_x, case.d_ids, case.d_gates, case.d_w1, case.d_w3, case.d_w2, case.buf, want_plan=False)
+        gather.append(case.ctx.get_timeline()["dev_dispatch_us"])
+    case.ctx.check_status()
+    assert np.median(gather) < 15, gather
     case.close()
