@@ -348,7 +348,7 @@ constexpr unsigned long long kEarlyTableNs = 4000;
 // they are open.  With a contiguous range of units per warp (every warp in a place of its own) the gather and
 // the combine together, T = 8192, top-8, d = 6144, ran at 5.5 TB/s; this way at 6.0 (route + gather +
 // combine 353 -> 330 us).  Slices of 1 KiB: 347 us, of 4 KiB: the same.
-__global__ void __launch_bounds__(kThreads)
+__global__ void __launch_bounds__(kThreads, 6)     // 40 registers; with 48 (five CTAs per SM) route + gather + combine 310 -> 315 us
 k_gather(const uint4* __restrict__ x, const int32_t* __restrict__ ids, const int32_t* __restrict__ pad_off,
          const int32_t* __restrict__ block_base, int32_t* slot_to_row, int32_t* __restrict__ row_to_token,
          uint4* __restrict__ x_perm, int t0, int T, int K, int E, int chunks, int64_t s_cap, const int32_t* __restrict__ counts,
