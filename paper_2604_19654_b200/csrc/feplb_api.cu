@@ -402,8 +402,11 @@ extern "C" int feplb_create(const feplb_config* cfg, feplb_ctx** out) {
   // device cost up to 10 us per forward, and the plan (returned as ever) is made by the calling thread
   // instead.  Whole layer, table order -> this: 27.9 -> 19.6 us (T = 256, top-2, d = 128, 8 experts), 30.8 ->
   // 20.3 (the same at T = 1200), 97.9 -> 88.7 (T = 64, top-6, d = 2048, 64 experts), 156.7 -> 148.9 (102 rows
-  // per expert, d = 1920).  At 384 rows per expert of d = 2048 (325 us by the estimate) the gain would be 3 %,
-  // at 1024 of d = 6144 the order that gives the static groups launches of their own is 4 % ahead.
+  // per expert, d = 1920), 181 -> 170 (128 of d = 2048).  Above the line, where the table comes with the gather, the two
+  // are level: 173.6 and 172.0 at 131 rows per expert of d = 2048, 211 and 211 at 188, 286 and 284 at 281, 2001 and 1989
+  // at 128 of d = 6144; at 1024 of d = 6144 the order that gives the static groups launches of their own is 4 % ahead.
+  // (Up to 8192 slots no CTA of the front picks the table up: 16 experts of d = 4096, f = 1024, 384 rows each, would
+  // gain from this order, 227 -> 199.)
   // The time is an estimate: all weights streamed at 6.5 TB/s plus the products at 1 PFLOP/s.
   const double ffn_us = 6.0 * cfg->d * cfg->f * ((double)cfg->E / 6.5e6 + (double)S / 1e9);
   c->direct_auto = c->direct = S < (int64_t)FEPLB_DIRECT_ROWS_PER_EXPERT * cfg->E || ffn_us < FEPLB_DIRECT_FFN_US;

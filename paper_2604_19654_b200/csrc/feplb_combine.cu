@@ -1,7 +1,7 @@
 // Gated combine of the FEPLB hot path on sm_100a (paper Section 2.3: the Combine phase returns
 // the expert results to their tokens): out[t,:] = sum_k gates[t,k] * y_perm[slot_to_row[t,k],:],
 // k ascending, fp32 accumulation, one bf16 rounding.  HBM-bound: every y_perm row is read once
-// with 16-byte loads (K independent loads in flight per lane), every out row written once.
+// with 16-byte loads (up to 8 independent ones in flight per lane), every out row written once.
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 

@@ -24,10 +24,11 @@
 // box of 16, 32, 64 or 128 rows).  Per CTA: warp 0 = TMA producer, warp 1 = tcgen05.mma issuer
 // (even CTA only) and TMEM owner, warps 2..9 = epilogue.
 //
-// One launch walks TWO group tables in order: the table known at launch (static experts on their
-// home ranks, built on the device from the counts) and then the planner's table of dynamic
+// One launch walks TWO group tables: the table known at launch (static experts on their
+// home ranks, built on the device from the counts) and the planner's table of dynamic
 // groups, which does not exist yet when the launch is enqueued (Section 2.3: the CPU balancer runs
-// while the GPU computes the static experts).  A CTA that runs out of static units looks the
+// while the GPU computes the static experts).  Usually the row gather has brought it to the device when the
+// launch starts, and both are walked together.  Otherwise a CTA that runs out of static units looks the
 // dynamic table up with a bounded wait on a word in mapped host memory that the planner thread
 // itself writes after the table (no kernel waits for another kernel); the first CTA to see it copies
 // the table into device memory for all the others.  Every wait is bounded and ends in a status bit,
@@ -100,7 +101,6 @@ struct WmParams {
   int a_rows_per_expert;                // rows of one expert in the weight maps
   int unit_rows;                        // weight-map rows a unit advances by: 128 (pass 1, in W1 and in W3) or 256 (pass 2)
   int cta_rows;                         // ... and the second CTA's offset inside it: 64 or 128
-  int a1_row_off;                       // row offset of a CTA's second 64-row box inside the same map (pass 2: 64), 0 in pass 1
   int n_recv_slots;
   __nv_bfloat16* out;
   int ld_out;
@@ -366,10 +366,8 @@ k_ffn_wm(const __grid_constant__ CUtensorMap tm_a0, const __grid_constant__ CUte
       if (lane == 0) {
         const CUtensorMap* ma0 = c.slot >= 0 ? &tm_r0 : &tm_a0;
         const CUtensorMap* ma1 = c.slot >= 0 ? &tm_r1 : &tm_a1;
-        // this CTA's 128 weight rows as two boxes of 64: pass 1 W1 rows, then the same rows of W3;
-        // pass 2 two consecutive boxes of W2
-        const int arow0 = (c.slot >= 0 ? c.slot : c.expert) * p.a_rows_per_expert + c.wt * p.unit_rows + (int)cta_rank * p.cta_rows;
-        const int arow1 = arow0 + p.a1_row_off;
+        // this CTA's 128 weight rows: 64 of W1 and the same 64 of W3 (pass 1), one box of W2 (pass 2)
+        const int arow = (c.slot >= 0 ? c.slot : c.expert) * p.a_rows_per_expert + c.wt * p.unit_rows + (int)cta_rank * p.cta_rows;
         const int n_half = c.n_pad >> 1;                  // token rows this CTA stages
         const int brow0 = c.row0 + (int)cta_rank * n_half;
         // one box per operand and stage (every TMA instruction costs about a hundred cycles on top of its
@@ -386,10 +384,10 @@ k_ffn_wm(const __grid_constant__ CUtensorMap tm_a0, const __grid_constant__ CUte
           const uint32_t sa = smem_u32(smem + (size_t)stage * kStageBytes);
           if (cta_rank == 0) mbar_expect_tx(smem_u32(&tail->full[stage]), tx);
           if (SWIGLU) {
-            tma_load_2d_pair(sa, ma0, full, kb * BK, arow0);                  // 64 rows of W1
-            tma_load_2d_pair(sa + kATile / 2, ma1, full, kb * BK, arow1);     // the same 64 rows of W3
+            tma_load_2d_pair(sa, ma0, full, kb * BK, arow);                   // 64 rows of W1
+            tma_load_2d_pair(sa + kATile / 2, ma1, full, kb * BK, arow);      // the same 64 rows of W3
           } else {
-            tma_load_2d_pair(sa, ma0, full, kb * BK, arow0);                  // 128 rows of W2
+            tma_load_2d_pair(sa, ma0, full, kb * BK, arow);                   // 128 rows of W2
           }
           tma_load_2d_pair(sa + kATile, c.slot >= 0 ? &tm_rb.m[bi] : &tm_b.m[bi], full, kb * BK, brow0);
           if (++stage == kStages) { stage = 0; phase ^= 1u; }
@@ -647,7 +645,7 @@ int feplb_launch_expert_ffn_wm(const feplb_gemm_args& a, const feplb_wm_dyn& dyn
     snprintf(err, errn, "expert_ffn: shape not supported by the weights-on-M form");
     return FEPLB_E_INVALID;
   }
-  CUtensorMap tm_w1, tm_w3, tm_w2, tm_h, tm_y;      // weights in boxes of 64 rows, outputs in boxes of 32 x 32
+  CUtensorMap tm_w1, tm_w3, tm_w2, tm_h, tm_y;      // W1, W3 in boxes of 64 rows, W2 of 128, outputs of 32 x 32
   BMaps bx, bh;
   if (!make_tmap(&tm_w1, a.w1, (uint64_t)a.E * a.f, (uint64_t)a.d, WM / 2) ||
       !make_tmap(&tm_w3, a.w3, (uint64_t)a.E * a.f, (uint64_t)a.d, WM / 2) ||
@@ -677,13 +675,13 @@ int feplb_launch_expert_ffn_wm(const feplb_gemm_args& a, const feplb_wm_dyn& dyn
   p1.dyn = feplb_dyn_table(dyn);
   p1.E = a.E; p1.s_cap = a.s_cap;
   // pass 1: a unit covers 128 hidden units, 64 per CTA, each CTA taking its rows of W1 and of W3
-  p1.n_pairs = a.f / 128; p1.num_k_blocks = a.d / BK; p1.a_rows_per_expert = a.f; p1.unit_rows = 128; p1.cta_rows = 64; p1.a1_row_off = 0;
+  p1.n_pairs = a.f / 128; p1.num_k_blocks = a.d / BK; p1.a_rows_per_expert = a.f; p1.unit_rows = 128; p1.cta_rows = 64;
   p1.n_recv_slots = has_recv ? a.n_recv_slots : 0;
   p1.out = (__nv_bfloat16*)a.h; p1.ld_out = a.f; p1.ab_out = (__nv_bfloat16*)a.ab_out;
   p1.status = a.status; p1.stamps = dyn.stamps;
-  // pass 2: a unit covers 256 output columns, 128 per CTA as two consecutive boxes of W2
+  // pass 2: a unit covers 256 output columns, 128 per CTA
   WmParams p2 = p1;
-  p2.n_pairs = a.d / 256; p2.num_k_blocks = a.f / BK; p2.a_rows_per_expert = a.d; p2.unit_rows = 256; p2.cta_rows = 128; p2.a1_row_off = 64;
+  p2.n_pairs = a.d / 256; p2.num_k_blocks = a.f / BK; p2.a_rows_per_expert = a.d; p2.unit_rows = 256; p2.cta_rows = 128;
   p2.out = (__nv_bfloat16*)a.y; p2.ld_out = a.d; p2.ab_out = nullptr;
   p2.stamps = dyn.stamps ? dyn.stamps + 4 : nullptr;
 
