@@ -367,9 +367,9 @@ k_grouped_gemm(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__
     // beside the MMA issuer (d = 1920, f = 704, 60 experts, T = 1537: 148.7 -> 145.1 us per layer).
     // Pair form: both CTAs credit the LEADER's barrier; the leader announces the bytes of both.  For a tile whose
     // second 128 rows hold no valid row (a group of at most 128 rows, or a ragged tail) the peer's A box lies past
-    // the end of the tensor: zeros arrive without any traffic from L2, and multiplying zeros takes less power than
-    // multiplying what a skipped load would leave in the stage, which is clock at the power cap (64 experts, d = 2048,
-    // T = 4096: 343.2 -> 337.1 us per layer).  Zeros for the partly valid 128 rows as well, by boxes of 32 rows, cost
+    // the end of the tensor and brings zeros (the counter of bytes from L2 to the SMs counts them like rows: 1.53 ->
+    // 1.65 GB in pass 1).  Multiplying zeros takes less power than multiplying what a skipped load would leave in the
+    // stage, which is clock at the power cap (64 experts, d = 2048, T = 4096: 343.2 -> 337.1 us per layer).  Zeros for the partly valid 128 rows as well, by boxes of 32 rows, cost
     // 4 % instead.
     struct Source { const CUtensorMap *a, *b0, *b1; int arow, brow0, brow1; uint32_t half, tx; bool two; };
     auto source = [&](const TileCoord& c) {
