@@ -405,7 +405,8 @@ int feplb_host_stage_inputs(feplb_ctx* ctx, int32_t slot, const void* x_host, co
 /* Blocks until the result of the last feplb_moe_forward_host_async on `slot` is in its out_host. */
 int feplb_host_wait(feplb_ctx* ctx, int32_t slot);
 
-/* Turns CUDA-event timing of the stages of feplb_moe_forward on (1) or off (0, default). */
+/* Turns CUDA-event timing of the stages of feplb_moe_forward on (1) or off (0, default).  While it is on,
+ * feplb_moe_forward_host processes its batch in one piece. */
 int feplb_set_timeline(feplb_ctx* ctx, int32_t enable);
 /* Waits for the last forward's stage events and fills *out (device fields are 0 when timing was
  * off during that forward). */
