@@ -112,7 +112,7 @@ struct TileCoord { int row0, rows_valid, expert, slot, n0, bn; };   // slot >= 0
 
 // tile -> (group, M tile, N tile); N tiles of one M tile are consecutive so that CTAs running at
 // the same time share the A rows and sweep one expert's weights together (both stay in L2).
-template <int kRows>
+template <int kRows, bool NARROW>
 __device__ __forceinline__ TileCoord tile_coord(const SmemTail* t, int n_groups, const GemmParams& p, int tile) {
   const int mt = tile / p.n_tiles_n;
   int lo = 0, hi = n_groups;   // largest g with prefix[g] <= mt
@@ -127,7 +127,7 @@ __device__ __forceinline__ TileCoord tile_coord(const SmemTail* t, int n_groups,
   c.expert = t->g_expert[lo] & 0xffff;
   c.slot = (t->g_expert[lo] >> 16) - 1;
   c.n0 = (tile - mt * p.n_tiles_n) * p.bn;
-  c.bn = min(p.bn, p.half_width - c.n0);
+  c.bn = NARROW ? min(p.bn, p.half_width - c.n0) : p.bn;
   return c;
 }
 
@@ -238,7 +238,11 @@ __device__ __forceinline__ void warp_scan_prefix(SmemTail* t, int first, int n, 
   __syncwarp();
 }
 
-template <bool SWIGLU, bool PAIR>
+// NARROW: the last N tile of a row of tiles has fewer columns than the others.  An instantiation of its own, because a
+// width that differs per tile costs the roles more than it saves where it does not: both passes of a large batch in the
+// single form, 64 experts, d = 2048, f = 768, 1536 / 3750 rows per expert on average: 950 / 2204 us with one kernel
+// for all widths, 922 / 2142 this way; the pair form 868 / 1972 and 857 / 1960.
+template <bool SWIGLU, bool PAIR, bool NARROW>
 __global__ void __launch_bounds__(kThreads, 1)
 k_grouped_gemm(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__ CUtensorMap tm_as,
                const __grid_constant__ CUtensorMap tm_ra,
@@ -384,7 +388,7 @@ k_grouped_gemm(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__
       q.brow0 = (c.slot >= 0 ? c.slot : c.expert) * p.b_rows_per_expert + (SWIGLU ? c.n0 : 2 * c.n0);
       q.brow1 = SWIGLU ? q.brow0 : q.brow0 + c.bn;
       q.half = (uint32_t)c.bn * BK * 2;
-      q.two = c.bn > p.b_box;              // 128 rows in boxes of 64
+      q.two = NARROW && c.bn > p.b_box;    // 128 rows in boxes of 64
       q.tx = (PAIR ? 2 * kABytes : few ? kFewRows * BK * 2 : kABytes) + 2 * q.half;
       if (PAIR && cta_rank) {
         q.arow = c.rows_valid > BM ? c.row0 + BM : (int)p.s_cap;
@@ -421,7 +425,7 @@ k_grouped_gemm(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__
       if (worker < n_static_tiles) {
         n_early = min(kStages, p.num_k_blocks);
         if (lane == 0) {
-          const Source q = source(tile_coord<kTileRows>(tail, n_entries, p, worker));
+          const Source q = source(tile_coord<kTileRows, NARROW>(tail, n_entries, p, worker));
           for (int kb = 0; kb < n_early; ++kb) {
             announce(q, smem_u32(&tail->full[kb]));
             load_b(q, kb, smem_u32(&tail->full[kb]), smem_u32(smem + (size_t)kb * kStageBytes) + kABytes);
@@ -452,7 +456,7 @@ k_grouped_gemm(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__
         if (p.stamps && lane == 0) atomicMin(&p.stamps[3], ~(global_timer_ns() - t0));
       }
       if (tile >= total) break;
-      const TileCoord c = tile_coord<kTileRows>(tail, n_entries, p, tile);
+      const TileCoord c = tile_coord<kTileRows, NARROW>(tail, n_entries, p, tile);
       // While static tiles remain, peek at the device-side word once per tile: the load is in flight
       // during the K loop below and is looked at after it, so it costs the pipeline nothing.
       unsigned long long peek = 0;
@@ -488,7 +492,6 @@ k_grouped_gemm(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__
   } else if (warp == 1) {
     // ---- MMA issuer -------------------------------------------------------------------------
     if (lane == 0 && cta_rank == 0) {
-      const bool narrow = p.half_width % p.bn != 0;      // the last N tile is
       uint32_t idesc = make_idesc(kTileRows, 2 * p.bn);
       int stage = 0, as = 0;
       uint32_t phase = 0, aphase = 0;
@@ -502,7 +505,7 @@ k_grouped_gemm(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__
           total = tail->total_mtiles * p.n_tiles_n;
           if (tile >= total) break;
         }
-        if (narrow) idesc = make_idesc(kTileRows, 2 * min(p.bn, p.half_width - tile % p.n_tiles_n * p.bn));
+        if (NARROW) idesc = make_idesc(kTileRows, 2 * min(p.bn, p.half_width - tile % p.n_tiles_n * p.bn));
         if (!(ok = mbar_wait(smem_u32(&tail->tmem_empty[as]), aphase ^ 1u, abort_flag, p.status))) break;
         tc_fence_after();
         const uint32_t d_tmem = tmem_base + (uint32_t)(as * kAccCols);
@@ -553,7 +556,7 @@ k_grouped_gemm(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__
         total = tail->total_mtiles * p.n_tiles_n;
         if (tile >= total) break;
       }
-      const TileCoord c = tile_coord<kTileRows>(tail, n_entries, p, tile);
+      const TileCoord c = tile_coord<kTileRows, NARROW>(tail, n_entries, p, tile);
       const int out_cols = SWIGLU ? c.bn : 2 * c.bn;
       const int col0 = SWIGLU ? c.n0 : 2 * c.n0;          // first output column of the tile
       ok = mbar_wait(smem_u32(&tail->tmem_full[as]), aphase, abort_flag, p.status);
@@ -677,8 +680,8 @@ bool make_tmap(CUtensorMap* m, const void* base, uint64_t rows, uint64_t inner, 
             CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
-template <bool SWIGLU, bool PAIR>
-cudaError_t launch_one(const CUtensorMap& ta, const CUtensorMap& tas, const CUtensorMap& tra, const CUtensorMap& tb0, const CUtensorMap& tb1, const CUtensorMap& tr0,
+template <bool SWIGLU, bool PAIR, bool NARROW>
+cudaError_t launch_form(const CUtensorMap& ta, const CUtensorMap& tas, const CUtensorMap& tra, const CUtensorMap& tb0, const CUtensorMap& tb1, const CUtensorMap& tr0,
                        const CUtensorMap& tr1, const CUtensorMap& tout, const GemmParams& p, int num_sms, cudaStream_t st) {
   // per instantiation and device: the shared-memory attribute and the resident grid are set on first use
   static int grid_of[64] = {};
@@ -702,7 +705,7 @@ cudaError_t launch_one(const CUtensorMap& ta, const CUtensorMap& tas, const CUte
     cfg.numAttrs = 2;
   }
   if (!grid) {
-    cudaError_t e = cudaFuncSetAttribute(k_grouped_gemm<SWIGLU, PAIR>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+    cudaError_t e = cudaFuncSetAttribute(k_grouped_gemm<SWIGLU, PAIR, NARROW>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          (int)kSmemBytes);
     if (e != cudaSuccess) return e;
     int g = num_sms;
@@ -710,7 +713,7 @@ cudaError_t launch_one(const CUtensorMap& ta, const CUtensorMap& tas, const CUte
       // as many clusters of two as can be resident at once (one CTA per SM, both SMs in one GPC)
       int n_clusters = 0;
       cfg.gridDim = dim3(num_sms / 2 * 2);
-      e = cudaOccupancyMaxActiveClusters(&n_clusters, k_grouped_gemm<SWIGLU, PAIR>, &cfg);
+      e = cudaOccupancyMaxActiveClusters(&n_clusters, k_grouped_gemm<SWIGLU, PAIR, NARROW>, &cfg);
       if (e != cudaSuccess) return e;
       if (n_clusters < 1) return cudaErrorLaunchOutOfResources;
       g = 2 * (n_clusters < num_sms / 2 ? n_clusters : num_sms / 2);
@@ -718,7 +721,14 @@ cudaError_t launch_one(const CUtensorMap& ta, const CUtensorMap& tas, const CUte
     grid = g;
   }
   cfg.gridDim = dim3(grid);
-  return cudaLaunchKernelEx(&cfg, k_grouped_gemm<SWIGLU, PAIR>, ta, tas, tra, tb0, tb1, tr0, tr1, tout, p);
+  return cudaLaunchKernelEx(&cfg, k_grouped_gemm<SWIGLU, PAIR, NARROW>, ta, tas, tra, tb0, tb1, tr0, tr1, tout, p);
+}
+
+template <bool SWIGLU, bool PAIR>
+cudaError_t launch_one(const CUtensorMap& ta, const CUtensorMap& tas, const CUtensorMap& tra, const CUtensorMap& tb0, const CUtensorMap& tb1, const CUtensorMap& tr0,
+                       const CUtensorMap& tr1, const CUtensorMap& tout, const GemmParams& p, int num_sms, cudaStream_t st) {
+  auto form = p.half_width % p.bn ? launch_form<SWIGLU, PAIR, true> : launch_form<SWIGLU, PAIR, false>;
+  return form(ta, tas, tra, tb0, tb1, tr0, tr1, tout, p, num_sms, st);
 }
 
 }  // namespace
