@@ -32,7 +32,7 @@ UNIT = "tokens/s"
 # DRAM bytes (read + write) of one k_grouped_gemm launch at the benchmarked workload, from the ncu
 # capture summarised under profiles/; none (null in the line) where no capture exists.
 NCU_TRAFFIC_BYTES_PER_LAUNCH = {     # keyed by (workload, GEMM launches per forward)
-    ("cfg2", 2): {"bytes": 380.9e6, "source": "profiles/k_grouped_gemm_cfg2.md: 761.7 MB over the 2 launches of one forward "
+    ("cfg2", 2): {"bytes": 380.7e6, "source": "profiles/k_grouped_gemm_cfg2.md: 761.4 MB over the 2 launches of one forward "
                                               "(capture of the merged two-CTA launches)"},
     ("cfg2", 4): {"bytes": 190.0e6, "source": "capture of the four-launch form: 760 MB over the 4 launches of one forward"},
 }

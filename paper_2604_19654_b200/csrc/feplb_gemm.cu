@@ -240,8 +240,8 @@ __device__ __forceinline__ void warp_scan_prefix(SmemTail* t, int first, int n, 
 
 // NARROW: the last N tile of a row of tiles has fewer columns than the others.  An instantiation of its own, because a
 // width that differs per tile costs the roles more than it saves where it does not: both passes of a large batch in the
-// single form, 64 experts, d = 2048, f = 768, 1536 / 3750 rows per expert on average: 950 / 2204 us with one kernel
-// for all widths, 922 / 2142 this way; the pair form 868 / 1972 and 857 / 1960.
+// single form, 64 experts, d = 2048, f = 768, 1536 / 3750 rows per expert on average: 950 / 2187 us with one kernel
+// for all widths, 920 / 2118 this way; the pair form 864 / 1967 and 851 / 1938.
 template <bool SWIGLU, bool PAIR, bool NARROW>
 __global__ void __launch_bounds__(kThreads, 1)
 k_grouped_gemm(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__ CUtensorMap tm_as,

@@ -339,8 +339,8 @@ __device__ __forceinline__ uint4 ld_nc_v4(const uint4* p) {
 constexpr int kGatherUnroll = 4;
 // How long the gather's first CTA looks for the planner's table even if the rows are copied in less: a planner whose
 // thread has a core to itself publishes it 2-3 us after the scan.  When the planner is late (held back 60 us), 64 experts,
-// d = 2048, us per layer without an early table -> a fixed wait of 15 us -> this: T = 1400 193 -> 196 -> 192, T = 2000
-// 230 -> 236 -> 233, T = 4096 350 in all three; when it is not: 193 -> 186 -> 185, 231 -> 223 -> 223, 350 -> 340 -> 340.
+// d = 2048, us per layer without an early table -> a fixed wait of 15 us -> this: T = 1400 190 -> 194 -> 188, T = 2000
+// 227 -> 231 -> 227, T = 4096 343 -> 343 -> 341; when it is not: 191 -> 185 -> 181, 228 -> 220 -> 216, 343 -> 334 -> 333.
 constexpr unsigned long long kEarlyTableNs = 4000;
 // Work unit = (token, slice of 4 x 32 chunks = 2 KiB of its row).  Unit u goes to warp u mod #warps of a grid
 // sized to the machine: all warps work on neighbouring tokens at any time, and the rows of an expert, which
