@@ -125,6 +125,7 @@ struct feplb_ctx {
   std::condition_variable cv;
   bool quit = false;
   int job = JOB_IDLE;
+  std::atomic<bool> job_abort{false};   // the counts of the pending job will not come: its launches failed
   const uint8_t* job_mask = nullptr;
   const void* job_w1 = nullptr;   // weights of the current forward (sources of the Phase-2 copies)
   const void* job_w3 = nullptr;
@@ -176,6 +177,7 @@ int await_counts(feplb_ctx* c, int32_t seq) {
         c->h_counts[e] = (int32_t)(uint32_t)v;
       }
       if (e == c->cfg.E) break;
+      if (c->job_abort.load(std::memory_order_relaxed)) { rc = FEPLB_E_CUDA; break; }
     } else {
       cudaError_t q = cudaEventQuery(c->ev_counts);
       if (q == cudaSuccess) break;
@@ -696,6 +698,7 @@ static int plan_kick_flag(feplb_ctx* c, const uint8_t* dyn_mask_host, int32_t se
     c->job_mask = dyn_mask_host;
     c->job_wm = wm;
     c->job_flag_seq = seq;
+    c->job_abort.store(false, std::memory_order_relaxed);
     c->job = JOB_PENDING;
   }
   c->cv.notify_all();
@@ -859,19 +862,30 @@ extern "C" int feplb_moe_forward(feplb_ctx* c, const void* x, const int32_t* top
   const int32_t seq = c->flag_seq;
   const bool small_front = feplb_front_is_small(S, g.E);
   c->path = (small_front ? FEPLB_PATH_SMALL_FRONT : 0) | (direct ? FEPLB_PATH_HOME_TABLE : wm ? FEPLB_PATH_MERGED : 0);
-  if (small_front)
-    CUDA_TRY(c, feplb_launch_front_small(x, topk_ids, g.T, g.K, g.E, g.R, g.d, g.row_align, g.dyn, mask_dev, nullptr, counts, rank_load,
-                                         c->d_pad_off, c->d_home_groups, slot_to_row, row_to_token, x_perm, (int64_t)c->s_cap,
-                                         c->d_status, c->h_counts_tagged, seq, stamps ? stamps + 8 : nullptr, c->num_sms, st,
-                                         &c->launches));
-  else
-    CUDA_TRY(c, feplb_launch_route_fused(topk_ids, S, g.E, g.R, g.row_align, g.dyn, mask_dev, c->d_block_hist, counts,
-                                         rank_load, c->d_pad_off, c->d_home_groups, nullptr, slot_to_row, row_to_token,
-                                         (int64_t)c->s_cap, c->d_status, c->h_counts_tagged, seq,
-                                         stamps ? stamps + 8 : nullptr, st, &c->launches));
   c->job_w1 = w1; c->job_w3 = w3; c->job_w2 = w2;   // read by the planner thread after it is woken
   c->job_x_perm = x_perm;
-  if (!direct && (rc = plan_kick_flag(c, dyn_mask_host, seq, wm)) != FEPLB_OK) return rc;
+  // Where the gather looks for the planner's table the thread is woken before the launches whose counts it waits for: a
+  // forward on an idle GPU has its counts about 10 us after them, as long as a sleeping thread takes to wake.  Elsewhere
+  // the launches go first.
+  const bool kick_first = wm && !direct && !small_front;
+  if (kick_first && (rc = plan_kick_flag(c, dyn_mask_host, seq, wm)) != FEPLB_OK) return rc;
+  const cudaError_t front =
+      small_front ? feplb_launch_front_small(x, topk_ids, g.T, g.K, g.E, g.R, g.d, g.row_align, g.dyn, mask_dev, nullptr, counts,
+                                             rank_load, c->d_pad_off, c->d_home_groups, slot_to_row, row_to_token, x_perm,
+                                             (int64_t)c->s_cap, c->d_status, c->h_counts_tagged, seq, stamps ? stamps + 8 : nullptr,
+                                             c->num_sms, st, &c->launches)
+                  : feplb_launch_route_fused(topk_ids, S, g.E, g.R, g.row_align, g.dyn, mask_dev, c->d_block_hist, counts,
+                                             rank_load, c->d_pad_off, c->d_home_groups, nullptr, slot_to_row, row_to_token,
+                                             (int64_t)c->s_cap, c->d_status, c->h_counts_tagged, seq,
+                                             stamps ? stamps + 8 : nullptr, st, &c->launches);
+  if (front != cudaSuccess) {
+    if (kick_first) {
+      c->job_abort.store(true, std::memory_order_relaxed);
+      join_planner(c, c->planner_timeout_ms + 500, nullptr);
+    }
+    return fail(c, FEPLB_E_CUDA, "routing launch: %s", cudaGetErrorString(front));
+  }
+  if (!direct && !kick_first && (rc = plan_kick_flag(c, dyn_mask_host, seq, wm)) != FEPLB_OK) return rc;
   TL_EVENT(EV_COUNTS);
   TL_EVENT(EV_HIST);
   // how the merged launches, and the gather in front of them, get the planner's table

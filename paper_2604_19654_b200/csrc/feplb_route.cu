@@ -338,10 +338,12 @@ __device__ __forceinline__ uint4 ld_nc_v4(const uint4* p) {
 // read either form of the entry, and gets the same row from both.
 constexpr int kGatherUnroll = 4;
 // How long the gather's first CTA looks for the planner's table even if the rows are copied in less: a planner whose
-// thread has a core to itself publishes it 2-3 us after the scan.  When the planner is late (held back 60 us), 64 experts,
+// thread is awake publishes it 2-3 us after the scan, one that has to be woken (a forward on an idle GPU) some 5 us later.
+// One such forward and the wait for it, T = 2000 / 4096: 208 / 298 us with a fixed wait of 15 us, 216 / 299 with 4 us at
+// least, 205 / 296 with 8 and the thread woken before the routing launches.  When the planner is late (held back 60 us), 64 experts,
 // d = 2048, us per layer without an early table -> a fixed wait of 15 us -> this: T = 1400 190 -> 194 -> 188, T = 2000
 // 227 -> 231 -> 227, T = 4096 343 -> 343 -> 341; when it is not: 191 -> 185 -> 181, 228 -> 220 -> 216, 343 -> 334 -> 333.
-constexpr unsigned long long kEarlyTableNs = 4000;
+constexpr unsigned long long kEarlyTableNs = 8000;
 // Work unit = (token, slice of 4 x 32 chunks = 2 KiB of its row).  Unit u goes to warp u mod #warps of a grid
 // sized to the machine: all warps work on neighbouring tokens at any time, and the rows of an expert, which
 // follow the token order, are written in one moving window per expert, so that DRAM pages are written while

@@ -371,8 +371,9 @@ def test_pass_times_do_not_overlap(form):
 
 
 def test_late_planner_does_not_hold_the_gather_up():
-    """The CTA that waits for the planner's table gives up soon after the rows are copied (here in about 3 us, under an
-    event interval of about 10): with the planner held back, the gather stays far below 15 us."""
+    """The CTA that waits for the planner's table gives up when the rows are copied, after 8 us at least (here the copies take
+    about 3): with the planner held back, the interval between the events around the gather is about 17 us -- the 8,
+    one more look across PCIe and the launch -- against 11 with the table on time and 23 with a fixed wait of 15 us."""
     w = W.get_workload("cfg1").with_(T=3000, K=4, E=16, R=4, d=256, f=128, tau=1)
     case = DeviceCase(w)
     case.ctx.set_launch_merging(1)
@@ -383,5 +384,5 @@ def test_late_planner_does_not_hold_the_gather_up():
         case.ctx.moe_forward(case.d_x, case.d_ids, case.d_gates, case.d_w1, case.d_w3, case.d_w2, case.buf, want_plan=False)
         gather.append(case.ctx.get_timeline()["dev_dispatch_us"])
     case.ctx.check_status()
-    assert np.median(gather) < 15, gather
+    assert np.median(gather) < 20, gather
     case.close()
