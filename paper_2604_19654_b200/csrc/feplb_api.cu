@@ -651,7 +651,10 @@ extern "C" int feplb_expert_ffn(feplb_ctx* c, const void* x_perm, const void* w1
                                 const feplb_group* groups, int32_t n_groups, int32_t which,
                                 void* h_scratch, void* y_perm, void* stream) {
   if (!c) return FEPLB_E_INVALID;
-  return ffn_impl(c, x_perm, w1, w3, w2, groups, n_groups, which, h_scratch, y_perm, (cudaStream_t)stream);
+  const int32_t path = c->path;         // of the last forward, which this call is not
+  const int rc = ffn_impl(c, x_perm, w1, w3, w2, groups, n_groups, which, h_scratch, y_perm, (cudaStream_t)stream);
+  c->path = path;
+  return rc;
 }
 
 extern "C" int feplb_combine(feplb_ctx* c, const void* y_perm, const int32_t* slot_to_row, const float* gates,
@@ -882,6 +885,7 @@ extern "C" int feplb_moe_forward(feplb_ctx* c, const void* x, const int32_t* top
     if (kick_first) {
       c->job_abort.store(true, std::memory_order_relaxed);
       join_planner(c, c->planner_timeout_ms + 500, nullptr);
+      c->job_abort.store(false, std::memory_order_relaxed);      // the next forward may wait for its counts by itself
     }
     return fail(c, FEPLB_E_CUDA, "routing launch: %s", cudaGetErrorString(front));
   }

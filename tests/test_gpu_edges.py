@@ -294,7 +294,15 @@ def test_order_rule(T, K, E, d, f, path):
     rng = torch.Generator(device="cuda").manual_seed(1)
     z = lambda *s: torch.zeros(*s, dtype=torch.bfloat16, device="cuda")       # noqa: E731
     ids = torch.rand(T, E, generator=rng, device="cuda").topk(K, dim=1)[1].int()
-    ctx.moe_forward(z(T, d), ids, torch.ones(T, K, device="cuda"), z(E, f, d), z(E, f, d), z(E, d, f), buf)
+    w = z(E, f, d), z(E, f, d), z(E, d, f)
+    ctx.moe_forward(z(T, d), ids, torch.ones(T, K, device="cuda"), *w, buf)
+    ctx.check_status()
+    assert ctx.forward_path() == path
+    groups = torch.zeros(E, 5, dtype=torch.int32, device="cuda")
+    ctx.home_groups(buf.counts, None, groups)
+    for form in (F.FORM_SINGLE, F.FORM_PAIR):
+        ctx.set_gemm_form(form)
+        ctx.expert_ffn(buf.x_perm, *w, groups, E, buf.h_scratch, buf.y_perm)       # not a forward
     ctx.check_status()
     assert ctx.forward_path() == path
     ctx.close()
