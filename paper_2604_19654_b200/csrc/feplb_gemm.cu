@@ -27,7 +27,7 @@
 namespace {
 
 constexpr int BM = FEPLB_TILE_M;       // rows per MMA (UMMA M) = rows of one sub-tile
-constexpr int BK = 64;                 // K elements per stage = one 128-byte swizzle row
+constexpr int kChunk = 64;             // K elements of a 128-byte swizzle row
 constexpr int UMMA_K = 16;             // K per tcgen05.mma for 16-bit inputs
 constexpr int kAccCols = 256;          // TMEM columns of one accumulator
 constexpr int kTmemCols = 512;         // all of TMEM: one CTA per SM
@@ -35,8 +35,8 @@ constexpr int kTmemCols = 512;         // all of TMEM: one CTA per SM
 // padding rows of full boxes would be a third of the bytes through an SM's L2 port.  Whole layer at T = 128, top-8,
 // d = 6144, 128 experts: 966 -> 947 us; T = 300, top-6, d = 2048, 64 experts: 110.3 -> 108.6.
 constexpr int kFewRows = 32;
-constexpr int kABytes = BM * BK * 2;               // 16 KiB per sub-tile
-constexpr int kBBytesMax = 256 * BK * 2;           // 32 KiB
+constexpr int kABytes = BM * kChunk * 2;           // 16 KiB per sub-tile and chunk
+constexpr int kBBytesMax = 256 * kChunk * 2;       // 32 KiB
 
 // Two forms of one kernel.
 //   single (PAIR = false): one CTA computes a 128 x 256 tile (UMMA M x N, cta_group::1); K step 64;
@@ -44,16 +44,21 @@ constexpr int kBBytesMax = 256 * BK * 2;           // 32 KiB
 //   pair (PAIR = true): a cluster of two CTAs computes a 256 x 256 tile with cta_group::2 MMAs
 //     issued by the even CTA: each CTA stages its own 128 rows of A and HALF of the B tile (the
 //     W1 tile in the even CTA and the W3 tile in the odd one in pass 1), so a CTA needs only
-//     64 bytes per MMA cycle from L2 and the ring holds 6 stages of 32 KiB.  No load is shared
-//     between the CTAs: each brings its own halves.  Used for launches whose groups are large
-//     (a 256-row tile wastes more on a ragged tail).
+//     64 bytes per MMA cycle from L2.  K step 128, two 64-element chunks in one TMA instruction per operand (3-d
+//     maps), 3 stages of 64 KiB: a stage costs the producer and the issuer a fixed few hundred cycles, whatever
+//     it holds.  Against 6 stages of 32 KiB, us per layer: 64 experts, d = 2048, T = 4096 333.5 -> 330.0; 32 experts, d =
+//     4096, f = 1024, T = 4096 505 -> 494; 128 experts, d = 6144, T = 8192 5512 -> 5382.
+//     No load is shared between the CTAs: each brings its own halves.  Used for launches whose groups are large;
+//     the last tile of a group shrinks to 128 rows, 64 per CTA, where no more are valid.
 // Both keep two accumulators in TMEM so that the epilogue of tile i overlaps the MMAs of tile i+1.
 template <bool PAIR> struct Ring {
-  static constexpr int kStages = PAIR ? 6 : 4;
-  static constexpr int kStageBytes = kABytes + (PAIR ? kBBytesMax / 2 : kBBytesMax);   // multiple of 1024
+  static constexpr int kChunks = PAIR ? 2 : 1;
+  static constexpr int BK = kChunks * kChunk;                                          // K elements per stage
+  static constexpr int kStages = PAIR ? 3 : 4;
+  static constexpr int kStageBytes = kChunks * (kABytes + (PAIR ? kBBytesMax / 2 : kBBytesMax));   // multiple of 1024
   static constexpr int kTileRows = PAIR ? 2 * BM : BM;
 };
-constexpr int kMaxStages = 6;
+constexpr int kMaxStages = 4;
 constexpr int kAccStages = 2;
 constexpr int kRingBytes = 4 * (kABytes + kBBytesMax);   // 192 KiB in both forms
 static_assert(Ring<false>::kStages * Ring<false>::kStageBytes == kRingBytes &&
@@ -68,6 +73,7 @@ struct SmemTail {
   unsigned long long tmem_full[kAccStages];
   unsigned long long tmem_empty[kAccStages];
   unsigned long long dyn_bar;         // completed by warp 0 once the dynamic entries are in place
+  uint32_t idesc[kMaxStages];         // instruction descriptor of the tile whose first K block is in the stage (leader)
   uint32_t tmem_base;
   int abort_flag;
   int n_entries;                      // entries in use (the table known at launch, then the planner's dynamic groups)
@@ -90,10 +96,14 @@ struct GemmParams {
   int64_t s_cap;        // rows of the A and output buffers
   int n_tiles_n;        // N tiles per M tile
   int half_width;       // rows of B over all half tiles of one M tile: f (pass 1), d / 2 (pass 2); a multiple of 64
-  int b_box;            // rows of one box of the B tensor maps (64 or 128); divides every half tile
+  int b_box;            // single form: rows of one box of the B tensor maps (64 or 128), which divides every half tile; in the
+                        // pair form a box has bn rows, and a narrow last tile leaves some of them unused
   int early_weights;    // the group table was complete before this kernel's predecessor let it start: B loads of the
                         // first tile may be issued before griddepcontrol.wait
-  int num_k_blocks;     // K / 64
+  int num_k_blocks;     // K / 64, pair form K / 128 rounded up (the chunk past the end reads as zeros and is not multiplied)
+  int num_chunks;       // K / 64
+  int halves;           // pair form: tiles of at most 128 valid rows take the 128-row MMA (in pass 1 it needs tm_h ...
+  int b_first;          // ... which begins at W3 where that lies in front of W1)
   int b_rows_per_expert;  // rows of one expert in the B tensor maps
   int n_recv_slots;     // slots of the receive buffer of migrated experts' weights (0 = none)
   int bn;               // rows of one B half tile (64 or 128; the last N tile may be narrower); the MMA has N = 2 * rows
@@ -129,6 +139,15 @@ __device__ __forceinline__ TileCoord tile_coord(const SmemTail* t, int n_groups,
   c.n0 = (tile - mt * p.n_tiles_n) * p.bn;
   c.bn = NARROW ? min(p.bn, p.half_width - c.n0) : p.bn;
   return c;
+}
+
+// Pair form: a tile of at most 128 valid rows is a 128 x 256 MMA over the two CTAs, 64 rows of A each.  In pass 1 both
+// halves of B then hold W1 and W3 rows of the same 64 hidden units (see the producer), which takes a full-width tile.
+// Half the MMA time and half the A rows against a 256-row tile whose second half is empty: 64 experts, d = 2048, T =
+// 4096 (a third of the tiles) 345.9 -> 340.2 us per layer, three hot experts 355.9 -> 345.0.
+template <bool SWIGLU, bool PAIR>
+__device__ __forceinline__ bool is_half(const TileCoord& c, const GemmParams& p) {
+  return PAIR && c.rows_valid <= BM && c.slot < 0 && p.halves && (!SWIGLU || c.bn == 128);
 }
 
 // fp32 accumulator registers of 32 columns -> 16 packed bf16 pairs (SwiGLU: silu(a) * b first).
@@ -248,9 +267,10 @@ k_grouped_gemm(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__
                const __grid_constant__ CUtensorMap tm_ra,
                const __grid_constant__ CUtensorMap tm_b0,
                const __grid_constant__ CUtensorMap tm_b1, const __grid_constant__ CUtensorMap tm_r0,
-               const __grid_constant__ CUtensorMap tm_r1, const __grid_constant__ CUtensorMap tm_out, const GemmParams p) {
+               const __grid_constant__ CUtensorMap tm_r1, const __grid_constant__ CUtensorMap tm_h,
+               const __grid_constant__ CUtensorMap tm_out, const GemmParams p) {
   constexpr int kStages = Ring<PAIR>::kStages, kStageBytes = Ring<PAIR>::kStageBytes;
-  constexpr int kTileRows = Ring<PAIR>::kTileRows;
+  constexpr int kTileRows = Ring<PAIR>::kTileRows, kChunks = Ring<PAIR>::kChunks, BK = Ring<PAIR>::BK;
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
   uint8_t* epi_smem = smem + (size_t)kRingBytes;
@@ -272,6 +292,7 @@ k_grouped_gemm(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__
     prefetch_tmap(&tm_b1);
     prefetch_tmap(&tm_r0);
     prefetch_tmap(&tm_r1);
+    prefetch_tmap(&tm_h);
     prefetch_tmap(&tm_out);
     for (int s = 0; s < kStages; ++s) {
       mbar_init(smem_u32(&tail->full[s]), 1);
@@ -375,7 +396,7 @@ k_grouped_gemm(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__
     // 1.65 GB in pass 1).  Multiplying zeros takes less power than multiplying what a skipped load would leave in the
     // stage, which is clock at the power cap (64 experts, d = 2048, T = 4096: 343.2 -> 337.1 us per layer).  Zeros for the partly valid 128 rows as well, by boxes of 32 rows, cost
     // 4 % instead.
-    struct Source { const CUtensorMap *a, *b0, *b1; int arow, brow0, brow1; uint32_t half, tx; bool two; };
+    struct Source { const CUtensorMap *a, *b0, *b1; int arow, brow0, brow1; uint32_t half, tx, idesc; bool two, split; };
     auto source = [&](const TileCoord& c) {
       Source q;
       const bool few = !PAIR && c.slot < 0 && c.rows_valid <= kFewRows;
@@ -387,25 +408,42 @@ k_grouped_gemm(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__
       q.arow = c.row0;
       q.brow0 = (c.slot >= 0 ? c.slot : c.expert) * p.b_rows_per_expert + (SWIGLU ? c.n0 : 2 * c.n0);
       q.brow1 = SWIGLU ? q.brow0 : q.brow0 + c.bn;
-      q.half = (uint32_t)c.bn * BK * 2;
-      q.two = NARROW && c.bn > p.b_box;    // 128 rows in boxes of 64
-      q.tx = (PAIR ? 2 * kABytes : few ? kFewRows * BK * 2 : kABytes) + 2 * q.half;
+      q.half = (uint32_t)(PAIR ? p.bn : c.bn) * BK * 2;
+      q.two = !PAIR && NARROW && c.bn > p.b_box;    // 128 rows in boxes of 64
+      q.tx = (PAIR ? 2 * kChunks * kABytes : few ? kFewRows * kChunk * 2 : kABytes) + 2 * q.half;
       if (PAIR && cta_rank) {
         q.arow = c.rows_valid > BM ? c.row0 + BM : (int)p.s_cap;
         q.b0 = q.b1;
         q.brow0 = q.brow1;
       }
+      q.idesc = make_idesc(kTileRows, 2 * c.bn);
+      q.split = false;
+      if (is_half<SWIGLU, PAIR>(c, p)) {
+        // 64 rows of A per CTA (zeros where none of them is valid); pass 1: 64 rows of W1 and the same 64 of W3
+        q.a = &tm_as;
+        q.arow = !cta_rank ? c.row0 : c.rows_valid > BM / 2 ? c.row0 + BM / 2 : (int)p.s_cap;
+        q.tx = kChunks * kABytes + 2 * q.half;
+        q.idesc = make_idesc(BM, 2 * c.bn);
+        q.split = SWIGLU;
+        if (SWIGLU) q.brow0 = c.expert * p.b_rows_per_expert + c.n0 + (int)cta_rank * 64;
+      }
       return q;
     };
-    auto announce = [&](const Source& q, uint32_t full) {      // the bytes of a stage
-      if (!PAIR || cta_rank == 0) mbar_expect_tx(full, q.tx);
+    auto announce = [&](const Source& q, int st) {      // the bytes of a stage, and what the issuer does with them
+      if (PAIR && cta_rank) return;
+      if (PAIR || NARROW) tail->idesc[st] = q.idesc;
+      mbar_expect_tx(smem_u32(&tail->full[st]), q.tx);
     };
     auto load_b = [&](const Source& q, int kb, uint32_t full, uint32_t sb) {
       constexpr uint32_t kBox = 64 * BK * 2;
       if (PAIR) {
         const uint32_t full0 = map_to_cta(full, 0);
-        tma_load_2d_pair(sb, q.b0, full0, kb * BK, q.brow0);
-        if (q.two) tma_load_2d_pair(sb + kBox, q.b0, full0, kb * BK, q.brow0 + 64);
+        if (SWIGLU && q.split)      // 64 rows of W1 and of W3, chunk after chunk
+          asm volatile(
+              "cp.async.bulk.tensor.4d.cta_group::2.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4, %3, %5}], [%2];"
+              ::"r"(sb), "l"(reinterpret_cast<uint64_t>(&tm_h)), "r"(full0), "r"(0), "r"(q.brow0), "r"(kb * kChunks) : "memory");
+        else
+          tma_load_3d_pair(sb, q.b0, full0, 0, q.brow0, kb * kChunks);
       } else {
         tma_load_2d(sb, q.b0, full, kb * BK, q.brow0);
         tma_load_2d(sb + q.half, q.b1, full, kb * BK, q.brow1);
@@ -416,7 +454,7 @@ k_grouped_gemm(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__
       }
     };
     auto load_a = [&](const Source& q, int kb, uint32_t full, uint32_t sa) {
-      if (PAIR) tma_load_2d_pair(sa, q.a, map_to_cta(full, 0), kb * BK, q.arow);
+      if (PAIR) tma_load_3d_pair(sa, q.a, map_to_cta(full, 0), 0, q.arow, kb * kChunks);
       else tma_load_2d(sa, q.a, full, kb * BK, q.arow);
     };
     // Weights of the first tile, as far as the ring holds them, before the wait for the rows.
@@ -427,8 +465,8 @@ k_grouped_gemm(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__
         if (lane == 0) {
           const Source q = source(tile_coord<kTileRows, NARROW>(tail, n_entries, p, worker));
           for (int kb = 0; kb < n_early; ++kb) {
-            announce(q, smem_u32(&tail->full[kb]));
-            load_b(q, kb, smem_u32(&tail->full[kb]), smem_u32(smem + (size_t)kb * kStageBytes) + kABytes);
+            announce(q, kb);
+            load_b(q, kb, smem_u32(&tail->full[kb]), smem_u32(smem + (size_t)kb * kStageBytes) + kChunks * kABytes);
           }
         }
         __syncwarp();
@@ -472,9 +510,9 @@ k_grouped_gemm(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__
           if (!(ok = mbar_wait(smem_u32(&tail->empty[stage]), phase ^ 1u, abort_flag, p.status))) break;
           const uint32_t full = smem_u32(&tail->full[stage]);
           const uint32_t sa = smem_u32(smem + (size_t)stage * kStageBytes);
-          announce(q, full);
+          announce(q, stage);
           load_a(q, kb, full, sa);
-          load_b(q, kb, full, sa + kABytes);
+          load_b(q, kb, full, sa + kChunks * kABytes);
           if (++stage == kStages) { stage = 0; phase ^= 1u; }
         }
       }
@@ -493,6 +531,9 @@ k_grouped_gemm(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__
     // ---- MMA issuer -------------------------------------------------------------------------
     if (lane == 0 && cta_rank == 0) {
       uint32_t idesc = make_idesc(kTileRows, 2 * p.bn);
+      // between the chunks of a stage's A (64 rows in a tile of 128) and B, >> 4
+      uint32_t a_chunk = kABytes >> 4;
+      const uint32_t b_chunk = (uint32_t)(p.bn * kChunk * 2) >> 4;
       int stage = 0, as = 0;
       uint32_t phase = 0, aphase = 0;
       bool ok = true, dyn_known = !has_dyn;
@@ -505,20 +546,25 @@ k_grouped_gemm(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__
           total = tail->total_mtiles * p.n_tiles_n;
           if (tile >= total) break;
         }
-        if (NARROW) idesc = make_idesc(kTileRows, 2 * min(p.bn, p.half_width - tile % p.n_tiles_n * p.bn));
         if (!(ok = mbar_wait(smem_u32(&tail->tmem_empty[as]), aphase ^ 1u, abort_flag, p.status))) break;
         tc_fence_after();
         const uint32_t d_tmem = tmem_base + (uint32_t)(as * kAccCols);
         for (int kb = 0; kb < p.num_k_blocks; ++kb) {
           if (!(ok = mbar_wait(smem_u32(&tail->full[stage]), phase, abort_flag, p.status))) break;
           tc_fence_after();
+          if ((PAIR || NARROW) && kb == 0) {
+            idesc = *reinterpret_cast<volatile uint32_t*>(&tail->idesc[stage]);
+            if (PAIR) a_chunk = idesc >> 24 == BM >> 4 ? kABytes / 2 >> 4 : kABytes >> 4;
+          }
           const uint32_t sa = smem_u32(smem + (size_t)stage * kStageBytes);
           const uint64_t da = make_smem_desc(sa);
-          const uint64_t db = make_smem_desc(sa + kABytes);
+          const uint64_t db = make_smem_desc(sa + kChunks * kABytes);
 #pragma unroll
           for (int k = 0; k < BK / UMMA_K; ++k) {
             // +32 bytes (>> 4 = 2) per K step inside the 128-byte swizzle row
-            if (PAIR) umma_bf16_pair(d_tmem, da + (uint64_t)(k * 2), db + (uint64_t)(k * 2), idesc, (uint32_t)((kb | k) != 0));
+            const int ch = k / (kChunk / UMMA_K), ks = 2 * (k % (kChunk / UMMA_K));
+            if (ch > 0 && kb * kChunks + ch >= p.num_chunks) break;
+            if (PAIR) umma_bf16_pair(d_tmem, da + (uint64_t)(ch * a_chunk + ks), db + (uint64_t)(ch * b_chunk + ks), idesc, (uint32_t)((kb | k) != 0));
             else umma_bf16(d_tmem, da + (uint64_t)(k * 2), db + (uint64_t)(k * 2), idesc, (uint32_t)((kb | k) != 0));
           }
           // stage reusable (in both CTAs of a pair) once these MMAs have read it
@@ -557,25 +603,30 @@ k_grouped_gemm(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__
         if (tile >= total) break;
       }
       const TileCoord c = tile_coord<kTileRows, NARROW>(tail, n_entries, p, tile);
-      const int out_cols = SWIGLU ? c.bn : 2 * c.bn;
-      const int col0 = SWIGLU ? c.n0 : 2 * c.n0;          // first output column of the tile
+      // In a tile of 128 rows over two CTAs TMEM lanes 0-63 hold the CTA's 64 rows for the columns of the even CTA's half
+      // of B, lanes 64-127 the same rows for those of the odd CTA's.
+      const bool half = is_half<SWIGLU, PAIR>(c, p);
+      // pass 1: TMEM columns of a and of b
+      const uint32_t a_off = SWIGLU && half && p.b_first ? 64 : 0, b_off = half ? 64 - a_off : (uint32_t)c.bn;
+      const int out_cols = half ? (SWIGLU ? 64 : c.bn) : SWIGLU ? c.bn : 2 * c.bn;
+      const int col0 = (SWIGLU ? c.n0 : 2 * c.n0) + (half ? (q >> 1) * out_cols : 0);   // this warp's first output column
       ok = mbar_wait(smem_u32(&tail->tmem_full[as]), aphase, abort_flag, p.status);
       ok = __all_sync(0xffffffffu, ok);
       if (!ok) break;
       tc_fence_after();
       const uint32_t taddr = tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)(as * kAccCols);
-      const int row_off = (int)cta_rank * BM + q * 32;    // this warp's first row inside the tile
+      const int row_off = half ? (int)cta_rank * (BM / 2) + (q & 1) * 32 : (int)cta_rank * BM + q * 32;    // this warp's first row inside the tile
       const int rows_here = c.rows_valid - row_off;       // valid rows among this warp's 32
       __nv_bfloat16* obase = p.out + (int64_t)(c.row0 + row_off) * p.ld_out + col0;
       // Single form: a warp without valid rows only hands the accumulator back.  In the pair form, which has few of them,
       // this test costs more than it saves: d = 6144, T = 65536 35344 us per layer with it, 34903 without.
       if (PAIR || rows_here > 0) {
         uint32_t a0[32], a1[32], b0[32], b1[32], packed[32];
-        tmem_ld32(taddr, a0);
-        tmem_ld32(taddr + 32u, a1);
+        tmem_ld32(taddr + a_off, a0);
+        tmem_ld32(taddr + a_off + 32u, a1);
         if (SWIGLU) {
-          tmem_ld32(taddr + (uint32_t)c.bn, b0);
-          tmem_ld32(taddr + (uint32_t)c.bn + 32u, b1);
+          tmem_ld32(taddr + b_off, b0);
+          tmem_ld32(taddr + b_off + 32u, b1);
         }
         for (int col = 0; col < out_cols; col += 64) {
           tmem_ld_wait();
@@ -600,11 +651,11 @@ k_grouped_gemm(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__
           convert_slice<SWIGLU>(a0, b0, packed);
           convert_slice<SWIGLU>(a1, b1, packed + 16);
           if (col + 64 < out_cols) {           // next slice's TMEM loads fly while this one is stored
-            tmem_ld32(taddr + (uint32_t)(col + 64), a0);
-            tmem_ld32(taddr + (uint32_t)(col + 96), a1);
+            tmem_ld32(taddr + a_off + (uint32_t)(col + 64), a0);
+            tmem_ld32(taddr + a_off + (uint32_t)(col + 96), a1);
             if (SWIGLU) {
-              tmem_ld32(taddr + (uint32_t)(c.bn + col + 64), b0);
-              tmem_ld32(taddr + (uint32_t)(c.bn + col + 96), b1);
+              tmem_ld32(taddr + b_off + (uint32_t)(col + 64), b0);
+              tmem_ld32(taddr + b_off + (uint32_t)(col + 96), b1);
             }
           }
           if (rows_here >= 32) stage_and_tma_store(stg, packed, &tm_out, col0 + col, c.row0 + row_off, lane);
@@ -667,22 +718,39 @@ encode_tiled_fn get_encode_fn() {
   return fn;
 }
 
+bool encode(CUtensorMap* m, int rank, const void* base, const cuuint64_t* dims, const cuuint64_t* strides, const cuuint32_t* box) {
+  encode_tiled_fn fn = get_encode_fn();
+  const cuuint32_t estr[5] = {1, 1, 1, 1, 1};
+  return fn && fn(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, (cuuint32_t)rank, const_cast<void*>(base), dims, strides, box, estr,
+                  CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+                  CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
 // Row-major bf16 matrix [rows, inner] -> tensor map with a [box_rows, 64] box, 128-byte swizzle.
 bool make_tmap(CUtensorMap* m, const void* base, uint64_t rows, uint64_t inner, uint32_t box_rows) {
-  encode_tiled_fn fn = get_encode_fn();
-  if (!fn) return false;
-  cuuint64_t dims[2] = {inner, rows};
-  cuuint64_t strides[1] = {inner * 2};
-  cuuint32_t box[2] = {(cuuint32_t)BK, box_rows};
-  cuuint32_t estr[2] = {1, 1};
-  return fn(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void*>(base), dims, strides, box, estr,
-            CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-            CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+  const cuuint64_t dims[2] = {inner, rows}, strides[1] = {inner * 2};
+  const cuuint32_t box[2] = {(cuuint32_t)kChunk, box_rows};
+  return encode(m, 2, base, dims, strides, box);
+}
+// The same with boxes of two 64-element chunks, chunk after chunk (pair form).
+bool make_tmap_chunks(CUtensorMap* m, const void* base, uint64_t rows, uint64_t inner, uint32_t box_rows) {
+  const cuuint64_t dims[3] = {(cuuint64_t)kChunk, rows, inner / kChunk}, strides[2] = {inner * 2, kChunk * 2};
+  const cuuint32_t box[3] = {(cuuint32_t)kChunk, box_rows, 2};
+  return encode(m, 3, base, dims, strides, box);
+}
+// 64 rows of W1 and the same 64 of W3, two chunks: {64 columns, rows, W1 and W3, chunks}, beginning at the one in
+// front.  Fails where they are further apart than a map's stride reaches, or the same.
+bool make_tmap_w13(CUtensorMap* m, const void* w1, const void* w3, uint64_t rows, uint64_t inner) {
+  const char *lo = (const char*)(w1 < w3 ? w1 : w3), *hi = (const char*)(w1 < w3 ? w3 : w1);
+  const uint64_t apart = (uint64_t)(hi - lo);
+  if (apart == 0 || apart >= (1ull << 40)) return false;
+  const cuuint64_t dims[4] = {(cuuint64_t)kChunk, rows, 2, inner / kChunk}, strides[3] = {inner * 2, apart, kChunk * 2};
+  const cuuint32_t box[4] = {(cuuint32_t)kChunk, 64, 2, 2};
+  return encode(m, 4, lo, dims, strides, box);
 }
 
 template <bool SWIGLU, bool PAIR, bool NARROW>
 cudaError_t launch_form(const CUtensorMap& ta, const CUtensorMap& tas, const CUtensorMap& tra, const CUtensorMap& tb0, const CUtensorMap& tb1, const CUtensorMap& tr0,
-                       const CUtensorMap& tr1, const CUtensorMap& tout, const GemmParams& p, int num_sms, cudaStream_t st) {
+                       const CUtensorMap& tr1, const CUtensorMap& th, const CUtensorMap& tout, const GemmParams& p, int num_sms, cudaStream_t st) {
   // per instantiation and device: the shared-memory attribute and the resident grid are set on first use
   static int grid_of[64] = {};
   int dev = 0;
@@ -721,14 +789,14 @@ cudaError_t launch_form(const CUtensorMap& ta, const CUtensorMap& tas, const CUt
     grid = g;
   }
   cfg.gridDim = dim3(grid);
-  return cudaLaunchKernelEx(&cfg, k_grouped_gemm<SWIGLU, PAIR, NARROW>, ta, tas, tra, tb0, tb1, tr0, tr1, tout, p);
+  return cudaLaunchKernelEx(&cfg, k_grouped_gemm<SWIGLU, PAIR, NARROW>, ta, tas, tra, tb0, tb1, tr0, tr1, th, tout, p);
 }
 
 template <bool SWIGLU, bool PAIR>
 cudaError_t launch_one(const CUtensorMap& ta, const CUtensorMap& tas, const CUtensorMap& tra, const CUtensorMap& tb0, const CUtensorMap& tb1, const CUtensorMap& tr0,
-                       const CUtensorMap& tr1, const CUtensorMap& tout, const GemmParams& p, int num_sms, cudaStream_t st) {
+                       const CUtensorMap& tr1, const CUtensorMap& th, const CUtensorMap& tout, const GemmParams& p, int num_sms, cudaStream_t st) {
   auto form = p.half_width % p.bn ? launch_form<SWIGLU, PAIR, true> : launch_form<SWIGLU, PAIR, false>;
-  return form(ta, tas, tra, tb0, tb1, tr0, tr1, tout, p, num_sms, st);
+  return form(ta, tas, tra, tb0, tb1, tr0, tr1, th, tout, p, num_sms, st);
 }
 
 }  // namespace
@@ -747,32 +815,37 @@ int feplb_launch_expert_ffn(const feplb_gemm_args& a, cudaStream_t st, int64_t* 
   // top-4: 171.2 -> 150.9 us together with the early weight loads of pass 2.
   const int hw1 = a.f, hw2 = a.d / 2;
   const int bn1 = hw1 < 128 ? 64 : 128, bn2 = hw2 < 128 ? 64 : 128;
-  const int bb1 = hw1 % 128 ? 64 : 128, bb2 = hw2 % 128 ? 64 : 128;
+  const int bb1 = a.pair ? bn1 : hw1 % 128 ? 64 : 128, bb2 = a.pair ? bn2 : hw2 % 128 ? 64 : 128;
   CUtensorMap tm_x, tm_xs, tm_hs, tm_w1, tm_w3, tm_h, tm_w2, tm_ho, tm_yo;     // tm_ho, tm_yo: outputs in boxes of 32 rows x 64 columns
-  if (!make_tmap(&tm_x, a.x_perm, (uint64_t)a.s_cap, (uint64_t)a.d, BM) ||
-      !make_tmap(&tm_xs, a.x_perm, (uint64_t)a.s_cap, (uint64_t)a.d, kFewRows) ||
-      !make_tmap(&tm_hs, a.h, (uint64_t)a.s_cap, (uint64_t)a.f, kFewRows) ||
-      !make_tmap(&tm_w1, a.w1, (uint64_t)a.E * a.f, (uint64_t)a.d, bb1) ||
-      !make_tmap(&tm_w3, a.w3, (uint64_t)a.E * a.f, (uint64_t)a.d, bb1) ||
-      !make_tmap(&tm_h, a.h, (uint64_t)a.s_cap, (uint64_t)a.f, BM) ||
-      !make_tmap(&tm_w2, a.w2, (uint64_t)a.E * a.d, (uint64_t)a.f, bb2) ||
+  const auto map = a.pair ? make_tmap_chunks : make_tmap;
+  const int few = a.pair ? BM / 2 : kFewRows;            // rows of the smaller boxes of A
+  if (!map(&tm_x, a.x_perm, (uint64_t)a.s_cap, (uint64_t)a.d, BM) ||
+      !map(&tm_xs, a.x_perm, (uint64_t)a.s_cap, (uint64_t)a.d, few) ||
+      !map(&tm_hs, a.h, (uint64_t)a.s_cap, (uint64_t)a.f, few) ||
+      !map(&tm_w1, a.w1, (uint64_t)a.E * a.f, (uint64_t)a.d, bb1) ||
+      !map(&tm_w3, a.w3, (uint64_t)a.E * a.f, (uint64_t)a.d, bb1) ||
+      !map(&tm_h, a.h, (uint64_t)a.s_cap, (uint64_t)a.f, BM) ||
+      !map(&tm_w2, a.w2, (uint64_t)a.E * a.d, (uint64_t)a.f, bb2) ||
       !make_tmap(&tm_ho, a.h, (uint64_t)a.s_cap, (uint64_t)a.f, 32) ||
       !make_tmap(&tm_yo, a.y, (uint64_t)a.s_cap, (uint64_t)a.d, 32)) {
     snprintf(err, errn, "cuTensorMapEncodeTiled failed (driver entry point missing or bad pointer/shape)");
     return FEPLB_E_CUDA;
   }
+  // pass 1 of the pair form, tiles of at most 128 rows
+  CUtensorMap tm_w13 = tm_w1;
+  const bool halves = a.pair && make_tmap_w13(&tm_w13, a.w1, a.w3, (uint64_t)a.E * a.f, (uint64_t)a.d);
   // receive buffer of migrated experts' weights, addressed by slot like the home weights by expert
   CUtensorMap tm_r1 = tm_w1, tm_r3 = tm_w3, tm_r2 = tm_w2;
   const bool has_recv = a.recv_w1 && a.recv_w3 && a.recv_w2 && a.n_recv_slots > 0;
-  if (has_recv && (!make_tmap(&tm_r1, a.recv_w1, (uint64_t)a.n_recv_slots * a.f, (uint64_t)a.d, bb1) ||
-                   !make_tmap(&tm_r3, a.recv_w3, (uint64_t)a.n_recv_slots * a.f, (uint64_t)a.d, bb1) ||
-                   !make_tmap(&tm_r2, a.recv_w2, (uint64_t)a.n_recv_slots * a.d, (uint64_t)a.f, bb2))) {
+  if (has_recv && (!map(&tm_r1, a.recv_w1, (uint64_t)a.n_recv_slots * a.f, (uint64_t)a.d, bb1) ||
+                   !map(&tm_r3, a.recv_w3, (uint64_t)a.n_recv_slots * a.f, (uint64_t)a.d, bb1) ||
+                   !map(&tm_r2, a.recv_w2, (uint64_t)a.n_recv_slots * a.d, (uint64_t)a.f, bb2))) {
     snprintf(err, errn, "cuTensorMapEncodeTiled failed for the receive buffer");
     return FEPLB_E_CUDA;
   }
   // rows of migrated pieces: pass 1 reads them from the receive region when there is one
   CUtensorMap tm_rx = tm_x;
-  if (has_recv && a.recv_x && !make_tmap(&tm_rx, a.recv_x, (uint64_t)a.s_cap, (uint64_t)a.d, BM)) {
+  if (has_recv && a.recv_x && !map(&tm_rx, a.recv_x, (uint64_t)a.s_cap, (uint64_t)a.d, BM)) {
     snprintf(err, errn, "cuTensorMapEncodeTiled failed for the receive region of the rows");
     return FEPLB_E_CUDA;
   }
@@ -780,23 +853,26 @@ int feplb_launch_expert_ffn(const feplb_gemm_args& a, cudaStream_t st, int64_t* 
   p1.n_recv_slots = has_recv ? a.n_recv_slots : 0;
   p1.groups = a.groups; p1.n_groups = a.n_groups; p1.which = a.which; p1.E = a.E; p1.s_cap = a.s_cap;
   p1.n_tiles_n = (hw1 + bn1 - 1) / bn1; p1.half_width = hw1; p1.b_box = bb1; p1.early_weights = 0;
-  p1.num_k_blocks = a.d / BK; p1.b_rows_per_expert = a.f; p1.bn = bn1;
+  const int bk = a.pair ? Ring<true>::BK : Ring<false>::BK;
+  p1.halves = halves; p1.b_first = a.w3 < a.w1;
+  p1.num_k_blocks = (a.d + bk - 1) / bk; p1.num_chunks = a.d / kChunk; p1.b_rows_per_expert = a.f; p1.bn = bn1;
   p1.out = (__nv_bfloat16*)a.h; p1.ld_out = a.f; p1.status = a.status; p1.ab_out = (__nv_bfloat16*)a.ab_out;
   const feplb_wm_dyn none;
   p1.dyn = feplb_dyn_table(dyn ? *dyn : none);
   p1.stamps = dyn ? dyn->stamps : nullptr;
   GemmParams p2 = p1;
   p2.n_tiles_n = (hw2 + bn2 - 1) / bn2; p2.half_width = hw2; p2.b_box = bb2; p2.early_weights = 1;
-  p2.num_k_blocks = a.f / BK; p2.b_rows_per_expert = a.d; p2.bn = bn2;
+  p2.halves = 1;
+  p2.num_k_blocks = (a.f + bk - 1) / bk; p2.num_chunks = a.f / kChunk; p2.b_rows_per_expert = a.d; p2.bn = bn2;
   p2.out = (__nv_bfloat16*)a.y; p2.ld_out = a.d; p2.ab_out = nullptr;
   p2.stamps = p1.stamps ? p1.stamps + 4 : nullptr;
 
-  cudaError_t e = a.pair ? launch_one<true, true>(tm_x, tm_xs, tm_rx, tm_w1, tm_w3, tm_r1, tm_r3, tm_ho, p1, a.num_sms, st)
-                         : launch_one<true, false>(tm_x, tm_xs, tm_rx, tm_w1, tm_w3, tm_r1, tm_r3, tm_ho, p1, a.num_sms, st);
+  cudaError_t e = a.pair ? launch_one<true, true>(tm_x, tm_xs, tm_rx, tm_w1, tm_w3, tm_r1, tm_r3, tm_w13, tm_ho, p1, a.num_sms, st)
+                         : launch_one<true, false>(tm_x, tm_xs, tm_rx, tm_w1, tm_w3, tm_r1, tm_r3, tm_w13, tm_ho, p1, a.num_sms, st);
   ++*n_launch;
   if (e == cudaSuccess) {
-    e = a.pair ? launch_one<false, true>(tm_h, tm_hs, tm_h, tm_w2, tm_w2, tm_r2, tm_r2, tm_yo, p2, a.num_sms, st)
-               : launch_one<false, false>(tm_h, tm_hs, tm_h, tm_w2, tm_w2, tm_r2, tm_r2, tm_yo, p2, a.num_sms, st);
+    e = a.pair ? launch_one<false, true>(tm_h, tm_hs, tm_h, tm_w2, tm_w2, tm_r2, tm_r2, tm_w2, tm_yo, p2, a.num_sms, st)
+               : launch_one<false, false>(tm_h, tm_hs, tm_h, tm_w2, tm_w2, tm_r2, tm_r2, tm_w2, tm_yo, p2, a.num_sms, st);
     ++*n_launch;
   }
   if (e != cudaSuccess) {

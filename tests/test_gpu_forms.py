@@ -1,0 +1,72 @@
+"""The forms of the expert FFN at the edges of their tiles, against the oracle: segments around the row counts at which a
+tile changes its shape, weights in either order in memory, widths that leave the last weight block or K block
+half empty."""
+import numpy as np
+import pytest
+
+from oracle import feplb_oracle as O
+from paper_2604_19654_b200 import build as B
+from paper_2604_19654_b200 import feplb as F
+from paper_2604_19654_b200 import workloads as W
+
+from gpu_utils import assert_close
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _built():
+    B.build()
+
+
+def _run(rows, d, f, form, w3_first=False, same=False, preact=False):
+    """One forward whose expert e has rows[e] rows (top-1); returns the context's launch path."""
+    import torch
+    E, T = len(rows), sum(rows)
+    w = W.get_workload("cfg1").with_(T=T, E=E, K=1, R=1, d=d, f=f, dyn=0)
+    ids = np.repeat(np.arange(E, dtype=np.int32), rows)[np.random.default_rng(T).permutation(T)].reshape(T, 1)
+    gates = np.ones((T, 1), np.float32)
+    x = W.gen_activations(w, 0)
+    w1, w3, w2 = W.gen_weights(w)
+    pair = torch.empty(2, E, f, d, dtype=torch.bfloat16, device="cuda")          # one allocation: the order is known
+    d_w1, d_w3 = (pair[1], pair[0]) if w3_first else (pair[0], pair[0] if same else pair[1])
+    d_w1.copy_(F.bf16_tensor(w1))
+    if same:
+        w3 = w1
+    else:
+        d_w3.copy_(F.bf16_tensor(w3))
+    cfg = F.config_from_workload(w)
+    ctx, buf = F.Context(cfg), F.Buffers(cfg)
+    if form is not None:
+        ctx.set_gemm_form(form)
+    ab = torch.full((T, 2 * f), 7.0, dtype=torch.bfloat16, device="cuda")
+    if preact:
+        ctx.set_preact_buffer(ab)
+    buf.h_scratch.fill_(float("nan"))
+    buf.y_perm.fill_(float("nan"))
+    ctx.moe_forward(F.bf16_tensor(x), torch.from_numpy(ids).cuda(), torch.from_numpy(gates).cuda(), d_w1, d_w3, F.bf16_tensor(w2), buf)
+    ctx.check_status()
+    assert_close(W.bf16_bits_to_f64(F.bf16_bits(buf.out)), O.moe_layer(x, ids, gates, w1, w3, w2, E), f"{rows} {d} {f} {form}")
+    if preact:
+        x64, order = W.bf16_bits_to_f64(x), np.argsort(ids[:, 0], kind="stable")
+        for e in range(E):
+            xe, got = x64[order][ids[order, 0] == e], W.bf16_bits_to_f64(F.bf16_bits(ab))[:T][ids[order, 0] == e]
+            assert_close(got[:, :f], xe @ W.bf16_bits_to_f64(w1[e]).T, "a")
+            assert_close(got[:, f:], xe @ W.bf16_bits_to_f64(w3[e]).T, "b")
+    path = ctx.forward_path()
+    ctx.close()
+    return path
+
+
+@pytest.mark.parametrize("w3_first", [False, True])
+@pytest.mark.parametrize("d,f", [(256, 128), (384, 320), (128, 64)])
+def test_pair_form_tiles_of_128_and_256_rows(d, f, w3_first):
+    """Tiles of at most 128 rows go through the 128-row MMA, 64 rows per CTA; f = 320: K blocks and N tiles half empty."""
+    path = _run([1, 32, 63, 64, 65, 96, 127, 128, 129, 255, 256, 257, 384, 385], d, f, F.FORM_PAIR, w3_first)
+    assert path & F.PATH_PAIR
+
+
+@pytest.mark.parametrize("form", [F.FORM_PAIR, None])
+def test_weights_in_one_buffer(form):
+    """W1 and W3 the same tensor: no map covers both side by side, the launches go without."""
+    _run([1, 40, 64, 65, 130], 256, 128, form, same=True)
