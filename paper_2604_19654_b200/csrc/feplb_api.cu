@@ -44,7 +44,7 @@ struct feplb_ctx {
   int gemm_pair_forced = -1;   // feplb_set_gemm_form: 0/1 forces one form everywhere, -1 = chosen per table
   int bwd_pair = 0;            // backward GEMMs in the pair form: bit 0 activation gradients, bit 1 weight gradients
   int gemm_pair_auto = 0, bwd_pair_auto = 0;   // the choices feplb_create derived from the geometry
-  bool wm_ok = false;          // the weights-on-M form supports this geometry
+  bool wm_ok = false;          // the weights-on-M form may be asked for: widths of whole units
   bool wm = false;             // ... and is the form in use (feplb_create's choice or feplb_set_gemm_form)
   bool wm_auto = false;
   bool wm_static = false, wm_static_auto = false;   // the static launches of the four-launch order use it
@@ -379,18 +379,21 @@ extern "C" int feplb_create(const feplb_config* cfg, feplb_ctx** out) {
   c->nb = (int)((S + FEPLB_SLOTS_PER_BLOCK - 1) / FEPLB_SLOTS_PER_BLOCK);
   const int cap_moves = cfg->R * cfg->max_num_dyn;
   const int cap_groups = cfg->E + cap_moves;
-  // Weights-on-M form: no padding rows to speak of, and an expert's weights cross the L2 ports once per 256 rows; its units
-  // are only worth their transposed epilogue where they are long.  Steady state, tokens-on-M -> weights-on-M, us per
-  // layer: d = 6144, f = 2048, 128 experts: 64 rows per expert 1384 -> 1368, 128 2007 -> 1913, 256 3204 -> 2971, 512 5149 ->
-  // 5001, 1024 9070 -> 9061; d = 6144, f = 512, 384 rows 705 -> 681; d = 4096, f = 1024, 256 rows 1138 -> 1084;
-  // d = f = 2048, 384 rows 745 -> 730; but d = 2048, f = 768: 187 rows 210 -> 212, 384 327 -> 328, 562 437 -> 440, and
-  // below 64 rows weights stream as fast in 128-row tiles (32 rows 1189 -> 1200).
-  c->wm_ok = feplb_wm_supported(cfg->E, cfg->d, cfg->f, cfg->E + cap_groups);
-  c->wm_auto = c->wm = c->wm_ok && S >= (int64_t)FEPLB_WM_MIN_ROWS_PER_EXPERT * cfg->E &&
+  // Weights-on-M form: no padding rows to speak of, and an expert's weights cross the L2 ports once per 256 rows.
+  // us per layer, single-CTA 128-row tiles / two-CTA 256-row tiles / weights on M:
+  //   128 experts, d = 6144, f = 2048: 64 rows per expert 1498 / 1485 / 1363, 128 2212 / 2160 / 1940, 512 5645 / 5383 / 5163,
+  //     1024 10110 / 9500 / 9622;  32 experts, d = 4096, f = 1024: 88 194 / 193 / 178, 512 525 / 494 / 478
+  //   64 experts, d = 2048, f = 768: 66 136.6 / 142.0 / 132.9, 131 188.7 / 184.2 / 173.5, 384 342 / 330 / 322, 768 607 / 577 / 572,
+  //     2812 1917 / 1815 / 1832
+  //   half-empty last weight blocks (60 experts, d = 1920, f = 704): 102 145.8 / 152.4 / 140.0, 400 312 / 304 / 298
+  //   32 experts, d = 1024, f = 512: 112 44.8 / 44.6 / 43.2, 250 63.2 / 61.4 / 59.6;  16, d = 512, f = 256: 375 28.4 / 30.9 / 31.3
+  const bool wm_can = feplb_wm_supported(cfg->E, cfg->E + cap_groups);
+  c->wm_ok = wm_can && cfg->f % 128 == 0 && cfg->d % 256 == 0;
+  c->wm_auto = c->wm = wm_can && S >= (int64_t)FEPLB_WM_MIN_ROWS_PER_EXPERT * cfg->E &&
                        S < (int64_t)FEPLB_MERGED_MAX_ROWS_PER_EXPERT * cfg->E && (int64_t)cfg->d * cfg->f >= FEPLB_WM_MIN_WEIGHT;
   // In the four-launch order the static experts are the less busy ones and stay in the range above for longer: d = 6144,
   // f = 2048, 128 experts, 1024 rows per expert on average 9911 -> 9750 us per layer, 1500 rows 13828 -> 13785.
-  c->wm_static_auto = c->wm_static = c->wm_ok && S < (int64_t)2048 * cfg->E && (int64_t)cfg->d * cfg->f >= FEPLB_WM_MIN_WEIGHT;
+  c->wm_static_auto = c->wm_static = wm_can && S < (int64_t)2048 * cfg->E && (int64_t)cfg->d * cfg->f >= FEPLB_WM_MIN_WEIGHT;
   // One launch per pass over the static and then the dynamic groups (the table of the latter is
   // picked up on the device): saves two launch ramps and two partly filled last waves per forward,
   // which matters while a forward's GEMMs take a few hundred microseconds; one form serves both
@@ -639,9 +642,12 @@ static int ffn_impl(feplb_ctx* c, const void* x_perm, const void* w1, const void
   a.recv_w1 = c->d_recv_w1; a.recv_w3 = c->d_recv_w3; a.recv_w2 = c->d_recv_w2; a.n_recv_slots = c->n_recv_slots;
   a.recv_x = c->d_recv_x;
   if ((c->wm || weights_on_m) && n_groups + (dyn ? dyn->max_groups : 0) <= FEPLB_WM_MAX_ENTRIES) {
-    c->path |= FEPLB_PATH_WEIGHT_M;
     const feplb_wm_dyn none;
-    return feplb_launch_expert_ffn_wm(a, dyn ? *dyn : none, st, &c->launches, c->err, sizeof(c->err));
+    rc = feplb_launch_expert_ffn_wm(a, dyn ? *dyn : none, st, &c->launches, c->err, sizeof(c->err));
+    if (rc != FEPLB_E_STATE) {
+      c->path |= FEPLB_PATH_WEIGHT_M;
+      return rc;
+    }
   }
   c->path |= pair ? FEPLB_PATH_PAIR : FEPLB_PATH_SINGLE;
   return feplb_launch_expert_ffn(a, st, &c->launches, c->err, sizeof(c->err), dyn);

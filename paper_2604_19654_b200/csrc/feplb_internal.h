@@ -25,7 +25,7 @@
 #define FEPLB_ST_PLAN 16u      // the GEMM's bounded wait for the planner's dynamic group table gave up
 #define FEPLB_MERGED_MAX_ROWS_PER_EXPERT 768   // static and dynamic groups share launches below this many rows per expert
 #define FEPLB_WM_MIN_ROWS_PER_EXPERT 64        // the weights-on-M form is the default from here (up to the line above) ...
-#define FEPLB_WM_MIN_WEIGHT (3 << 20)          // ... for weight matrices of at least so many elements
+#define FEPLB_WM_MIN_WEIGHT (1 << 19)          // ... for weight matrices of at least so many elements
 // No launch of a forward waits for the plan below this many rows per expert, or where the expert FFN takes less than this long
 #define FEPLB_DIRECT_ROWS_PER_EXPERT 128
 #define FEPLB_DIRECT_FFN_US 150
@@ -118,8 +118,8 @@ cudaError_t feplb_launch_wait_selftest(uint32_t* status, unsigned long long limi
 // Tokens-on-M forms (feplb_gemm.cu): single CTA per 128-row tile or, with a.pair, clusters of two on 256-row tiles.
 int feplb_launch_expert_ffn(const feplb_gemm_args& a, cudaStream_t st, int64_t* n_launch, char* err, size_t errn,
                             const feplb_wm_dyn* dyn = nullptr);
-// Weights-on-M form (feplb_gemm_wm.cu).
-bool feplb_wm_supported(int E, int d, int f, int n_entries_max);
+// Weights-on-M form (feplb_gemm_wm.cu).  FEPLB_E_STATE, with nothing launched, where no tensor map covers W1 and W3 together.
+bool feplb_wm_supported(int E, int n_entries_max);
 int feplb_launch_expert_ffn_wm(const feplb_gemm_args& a, const feplb_wm_dyn& dyn, cudaStream_t st, int64_t* n_launch,
                                char* err, size_t errn);
 // ---- backward pass ---------------------------------------------------------------------------

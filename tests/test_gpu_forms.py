@@ -70,3 +70,11 @@ def test_pair_form_tiles_of_128_and_256_rows(d, f, w3_first):
 def test_weights_in_one_buffer(form):
     """W1 and W3 the same tensor: no map covers both side by side, the launches go without."""
     _run([1, 40, 64, 65, 130], 256, 128, form, same=True)
+
+
+@pytest.mark.parametrize("w3_first", [False, True])
+def test_weights_on_m_units_of_any_width(w3_first):
+    """d = 4.5 x 256, f = 4.5 x 128: the second CTA's half of the last weight block lies past the width, the last K block of
+    pass 2 is half empty; segments around the multiples of 32 and 256 rows; saved pre-activations."""
+    rows = [1, 31, 32, 33, 64, 65, 128, 129, 200, 255, 256, 257, 300]
+    assert _run(rows, 1152, 576, None, w3_first, preact=True) & F.PATH_WEIGHT_M
