@@ -460,7 +460,7 @@ int feplb_selftest_bounded_wait(feplb_ctx* ctx, int32_t limit_us, void* stream);
 #define FEPLB_PATH_HOME_TABLE 2    /* no launch needs the plan: both passes walk the home groups */
 #define FEPLB_PATH_MERGED 4        /* one launch per pass over static and dynamic groups */
 #define FEPLB_PATH_RANGES 8        /* host-buffer forward in token ranges */
-#define FEPLB_PATH_SINGLE 16       /* single-CTA tiles of 128 rows */
+#define FEPLB_PATH_SINGLE 16       /* single-CTA tiles of 128 rows (of tokens or, with few rows per expert, of weights) */
 #define FEPLB_PATH_PAIR 32         /* two-CTA tiles of 256 rows */
 #define FEPLB_PATH_WEIGHT_M 64     /* weights-on-M units */
 int32_t feplb_forward_path(const feplb_ctx* ctx);

@@ -21,7 +21,7 @@ CSRC = os.path.join(HERE, "csrc")
 LIB = os.path.join(HERE, "libfeplb.so")
 PY_LIB = os.path.join(HERE, "_feplb_py" + importlib.machinery.EXTENSION_SUFFIXES[0])   # this interpreter's ABI alone loads it
 SOURCES = ["feplb_plan.cpp", "feplb_api.cu", "feplb_route.cu", "feplb_combine.cu", "feplb_gemm.cu",
-           "feplb_noalloc.cu", "feplb_gemm_bwd.cu", "feplb_gemm_wm.cu"]
+           "feplb_noalloc.cu", "feplb_gemm_bwd.cu", "feplb_gemm_wm.cu", "feplb_gemm_few.cu"]
 
 
 def _nvcc() -> str:

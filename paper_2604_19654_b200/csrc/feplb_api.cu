@@ -45,6 +45,7 @@ struct feplb_ctx {
   int bwd_pair = 0;            // backward GEMMs in the pair form: bit 0 activation gradients, bit 1 weight gradients
   int gemm_pair_auto = 0, bwd_pair_auto = 0;   // the choices feplb_create derived from the geometry
   bool wm_ok = false;          // the weights-on-M form may be asked for: widths of whole units
+  int few = 0, few_auto = 0;   // > 0: single group tables go through the form for few rows per expert, in units of that many
   bool wm = false;             // ... and is the form in use (feplb_create's choice or feplb_set_gemm_form)
   bool wm_auto = false;
   bool wm_static = false, wm_static_auto = false;   // the static launches of the four-launch order use it
@@ -336,6 +337,28 @@ int check_dev_ptrs(feplb_ctx* c, std::initializer_list<const void*> ptrs) {
 
 }  // namespace
 
+// Most token rows per unit of the form for few rows per expert (feplb_gemm_few.cu), or 0 where the others are better.
+// us per layer, single-CTA 128-row tiles -> units of 32 / 64 / 128 rows:
+//   one wave of units: 8 experts, d = 128, f = 64: T = 256 18.7 -> 15.6 / 16.8 / 18.5, T = 1000 18.6 -> 16.6 / 17.6 / 20.0;
+//     16 experts, d = 512, f = 256, 125 rows per expert 23.9 -> 24.5 / 23.0 / 21.4: the smallest units that fit
+//   T <= 64 (an expert has two units of 32 at most): 64 experts, d = 2048, f = 768, top-6, T = 64 82.5 -> 77.0 / 81.0 / 82.7;
+//     T = 96 83.5 -> 78.0 / 78.4 / 82.6; 64 experts, d = 4096, T = 90 134.7 -> 134.9 / 122.5 / 126.8
+//   128 experts, d = 6144, f = 2048: 8 rows per expert 925 -> 855 / 815 / 822, 16 1052 -> 1140 / 984 / 961, 32 1225 -> 1641 /
+//     1293 / 1144, 64 1402 -> 2427 / 1719 / 1386 (weights-on-M form 1334): small units leave room for more weights in flight,
+//     but a busy expert's weights are read again for each
+//   128 experts, d = 2560: f = 128 8 rows 55.1 -> 57.5 (64), 22 rows 65.1 -> 68.3; f = 192 8 rows 75.4 -> 66.1; f = 256 38
+//     rows 106 -> 105 (128); f = 320 130 -> 123: units of a short second pass have mostly fixed costs
+static int few_rows(const feplb_config& g, int num_sms) {
+  const int64_t S = (int64_t)g.T * g.K, E = g.E, touched = S < E ? S : E, weight = (int64_t)g.d * g.f;
+  const int64_t blocks = g.f / 64 > g.d / 128 ? g.f / 64 : g.d / 128;        // weight blocks of the wider pass
+  for (int n = 32; n <= 128 && S < FEPLB_PAIR_MIN_ROWS_PER_EXPERT * E; n *= 2)
+    if ((touched + S / n) * blocks <= num_sms) return n;
+  if (S < 7 * E) return g.T <= 64 ? 32 : 64;
+  if (g.f <= 128) return 0;
+  if (weight < FEPLB_FEW_LARGE_WEIGHT) return S < 24 * E ? 64 : 0;
+  return S < 14 * E ? 64 : S < FEPLB_WM_MIN_ROWS_PER_EXPERT * E ? 128 : 0;
+}
+
 extern "C" int feplb_version(void) { return 100; }
 
 extern "C" const char* feplb_strerror(int s) {
@@ -371,7 +394,7 @@ extern "C" int feplb_create(const feplb_config* cfg, feplb_ctx** out) {
   // 256-row pair tiles pay off when an expert's segment is several tiles long on average
   c->gemm_pair_auto = c->gemm_pair_default = (int64_t)cfg->T * cfg->K >= (int64_t)2048 * cfg->E;
   // a merged launch runs static and dynamic groups in one form: the two-CTA form from 256 rows per expert
-  c->merged_pair = (int64_t)cfg->T * cfg->K >= (int64_t)256 * cfg->E;
+  c->merged_pair = (int64_t)cfg->T * cfg->K >= (int64_t)FEPLB_PAIR_MIN_ROWS_PER_EXPERT * cfg->E;
   // backward GEMMs: the pair form pays once an expert's segment spans several 256-row tiles
   // (measured: -7.5 % backward time at 1024 rows per expert, slower at 384)
   c->bwd_pair_auto = c->bwd_pair = (int64_t)cfg->T * cfg->K >= (int64_t)512 * cfg->E ? 3 : 0;
@@ -388,6 +411,7 @@ extern "C" int feplb_create(const feplb_config* cfg, feplb_ctx** out) {
   //   half-empty last weight blocks (60 experts, d = 1920, f = 704): 102 145.8 / 152.4 / 140.0, 400 312 / 304 / 298
   //   32 experts, d = 1024, f = 512: 112 44.8 / 44.6 / 43.2, 250 63.2 / 61.4 / 59.6;  16, d = 512, f = 256: 375 28.4 / 30.9 / 31.3
   const bool wm_can = feplb_wm_supported(cfg->E, cfg->E + cap_groups);
+  c->few_auto = c->few = few_rows(*cfg, c->num_sms);
   c->wm_ok = wm_can && cfg->f % 128 == 0 && cfg->d % 256 == 0;
   c->wm_auto = c->wm = wm_can && S >= (int64_t)FEPLB_WM_MIN_ROWS_PER_EXPERT * cfg->E &&
                        S < (int64_t)FEPLB_MERGED_MAX_ROWS_PER_EXPERT * cfg->E && (int64_t)cfg->d * cfg->f >= FEPLB_WM_MIN_WEIGHT;
@@ -641,6 +665,13 @@ static int ffn_impl(feplb_ctx* c, const void* x_perm, const void* w1, const void
   a.ab_out = c->d_preact;
   a.recv_w1 = c->d_recv_w1; a.recv_w3 = c->d_recv_w3; a.recv_w2 = c->d_recv_w2; a.n_recv_slots = c->n_recv_slots;
   a.recv_x = c->d_recv_x;
+  if (c->few && !weights_on_m && !a.n_recv_slots && !(dyn && dyn->seq)) {
+    rc = feplb_launch_expert_ffn_few(a, st, &c->launches, c->err, sizeof(c->err), c->few, dyn ? dyn->stamps : nullptr);
+    if (rc != FEPLB_E_STATE) {
+      c->path |= FEPLB_PATH_SINGLE;
+      return rc;
+    }
+  }
   if ((c->wm || weights_on_m) && n_groups + (dyn ? dyn->max_groups : 0) <= FEPLB_WM_MAX_ENTRIES) {
     const feplb_wm_dyn none;
     rc = feplb_launch_expert_ffn_wm(a, dyn ? *dyn : none, st, &c->launches, c->err, sizeof(c->err));
@@ -1237,6 +1268,7 @@ extern "C" int feplb_set_gemm_form(feplb_ctx* c, int32_t forward_form, int32_t b
   std::lock_guard<std::mutex> lk(c->mu);
   if (c->job != JOB_IDLE) return fail(c, FEPLB_E_STATE, "set_gemm_form: a plan is pending");
   c->wm_static = forward_form == FEPLB_FORM_AUTO && c->wm_static_auto;
+  c->few = forward_form == FEPLB_FORM_AUTO ? c->few_auto : 0;
   c->wm = forward_form == FEPLB_FORM_AUTO ? c->wm_auto : forward_form == FEPLB_FORM_WEIGHT_M;
   c->gemm_pair_forced = forward_form == FEPLB_FORM_SINGLE || forward_form == FEPLB_FORM_PAIR ? forward_form : -1;
   c->gemm_pair_default = c->gemm_pair_forced < 0 ? c->gemm_pair_auto : forward_form;

@@ -24,7 +24,9 @@
 #define FEPLB_ST_GROUP 8u      // a group entry was malformed (expert or rows out of range)
 #define FEPLB_ST_PLAN 16u      // the GEMM's bounded wait for the planner's dynamic group table gave up
 #define FEPLB_MERGED_MAX_ROWS_PER_EXPERT 768   // static and dynamic groups share launches below this many rows per expert
-#define FEPLB_WM_MIN_ROWS_PER_EXPERT 64        // the weights-on-M form is the default from here (up to the line above) ...
+#define FEPLB_PAIR_MIN_ROWS_PER_EXPERT 256     // launches over static and dynamic groups, or all: two-CTA tiles from here
+#define FEPLB_FEW_LARGE_WEIGHT (1 << 20)       // weight matrices of at least so many elements: the form for few rows per expert up to ...
+#define FEPLB_WM_MIN_ROWS_PER_EXPERT 64        // ... this many; from here (up to the line above) the weights-on-M form ...
 #define FEPLB_WM_MIN_WEIGHT (1 << 19)          // ... for weight matrices of at least so many elements
 // No launch of a forward waits for the plan below this many rows per expert, or where the expert FFN takes less than this long
 #define FEPLB_DIRECT_ROWS_PER_EXPERT 128
@@ -122,6 +124,10 @@ int feplb_launch_expert_ffn(const feplb_gemm_args& a, cudaStream_t st, int64_t* 
 bool feplb_wm_supported(int E, int n_entries_max);
 int feplb_launch_expert_ffn_wm(const feplb_gemm_args& a, const feplb_wm_dyn& dyn, cudaStream_t st, int64_t* n_launch,
                                char* err, size_t errn);
+// The same for few rows per expert (feplb_gemm_few.cu): one table, no receive slots.  stamps: as feplb_wm_dyn::stamps.
+// nmax: most token rows per unit, 32, 64 or 128.  FEPLB_E_STATE, with nothing launched, where no tensor map covers W1 and W3 together.
+int feplb_launch_expert_ffn_few(const feplb_gemm_args& a, cudaStream_t st, int64_t* n_launch, char* err, size_t errn,
+                                int nmax, unsigned long long* stamps);
 // ---- backward pass ---------------------------------------------------------------------------
 struct feplb_bwd_args {
   const void* x_perm; const void* ab_saved; void* h; void* d_y_perm;   // padding rows of h, d_y_perm, d_ab get zeros

@@ -49,7 +49,7 @@ def _run(rows, d, f, form, w3_first=False, same=False, preact=False):
     assert_close(W.bf16_bits_to_f64(F.bf16_bits(buf.out)), O.moe_layer(x, ids, gates, w1, w3, w2, E), f"{rows} {d} {f} {form}")
     if preact:
         x64, order = W.bf16_bits_to_f64(x), np.argsort(ids[:, 0], kind="stable")
-        for e in range(E):
+        for e in np.flatnonzero(rows):
             xe, got = x64[order][ids[order, 0] == e], W.bf16_bits_to_f64(F.bf16_bits(ab))[:T][ids[order, 0] == e]
             assert_close(got[:, :f], xe @ W.bf16_bits_to_f64(w1[e]).T, "a")
             assert_close(got[:, f:], xe @ W.bf16_bits_to_f64(w3[e]).T, "b")
@@ -78,3 +78,15 @@ def test_weights_on_m_units_of_any_width(w3_first):
     pass 2 is half empty; segments around the multiples of 32 and 256 rows; saved pre-activations."""
     rows = [1, 31, 32, 33, 64, 65, 128, 129, 200, 255, 256, 257, 300]
     assert _run(rows, 1152, 576, None, w3_first, preact=True) & F.PATH_WEIGHT_M
+
+
+@pytest.mark.parametrize("w3_first", [False, True])
+@pytest.mark.parametrize("d,f,rows", [
+    (256, 320, [1, 15, 16, 17, 31, 32, 33, 40]),                             # one wave of units of 32 rows
+    (1024, 1024, [1, 15, 16, 17, 33, 63, 64, 65] + [0] * 14),                # units of 64 rows
+    (1024, 1088, [1, 16, 31, 32, 33, 64, 65, 127, 128, 129]),                # units of 128 rows, K blocks half empty
+])
+def test_units_for_few_rows_per_expert(d, f, rows, w3_first):
+    """Segments around the multiples of 16 rows and of a unit, in each size of the units that the rule picks; saved
+    pre-activations."""
+    assert _run(rows, d, f, None, w3_first, preact=True) & F.PATH_SINGLE
