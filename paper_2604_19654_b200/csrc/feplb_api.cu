@@ -48,6 +48,7 @@ struct feplb_ctx {
   int few = 0, few_auto = 0;   // > 0: single group tables go through the form for few rows per expert, in units of that many
   bool wm = false;             // ... and is the form in use (feplb_create's choice or feplb_set_gemm_form)
   bool wm_auto = false;
+  bool wm_merged = false, wm_merged_auto = false;   // the same for launches over static and dynamic groups together
   bool wm_static = false, wm_static_auto = false;   // the static launches of the four-launch order use it
   bool merged_ok = false;      // both group tables of a forward fit one launch (static, then dynamic groups)
   bool merged = false;         // ... and feplb_moe_forward runs that way: two GEMM launches instead of four
@@ -393,8 +394,12 @@ extern "C" int feplb_create(const feplb_config* cfg, feplb_ctx** out) {
   c->s_cap = feplb_s_pad(cfg);
   // 256-row pair tiles pay off when an expert's segment is several tiles long on average
   c->gemm_pair_auto = c->gemm_pair_default = (int64_t)cfg->T * cfg->K >= (int64_t)2048 * cfg->E;
-  // a merged launch runs static and dynamic groups in one form: the two-CTA form from 256 rows per expert
-  c->merged_pair = (int64_t)cfg->T * cfg->K >= (int64_t)FEPLB_PAIR_MIN_ROWS_PER_EXPERT * cfg->E;
+  // a launch over static and dynamic groups runs them in one form: the two-CTA form from 256 rows per expert, but small
+  // weights and many rows, where a tile is short, in single-CTA tiles (16 experts, d = 512, f = 256, T = 8000 / 30000, top-2
+  // 45.9 -> 42.2 / 107.9 -> 99.4 us per layer; 8 experts, d = 128, f = 64, T = 40000 64.1 -> 54.9)
+  const int64_t weight = (int64_t)cfg->d * cfg->f;
+  const bool short_tiles = weight < FEPLB_SHORT_TILE_WEIGHT && (int64_t)cfg->T * cfg->K >= (int64_t)512 * cfg->E;
+  c->merged_pair = (int64_t)cfg->T * cfg->K >= (int64_t)FEPLB_PAIR_MIN_ROWS_PER_EXPERT * cfg->E && !short_tiles;
   // backward GEMMs: the pair form pays once an expert's segment spans several 256-row tiles
   // (measured: -7.5 % backward time at 1024 rows per expert, slower at 384)
   c->bwd_pair_auto = c->bwd_pair = (int64_t)cfg->T * cfg->K >= (int64_t)512 * cfg->E ? 3 : 0;
@@ -413,18 +418,22 @@ extern "C" int feplb_create(const feplb_config* cfg, feplb_ctx** out) {
   const bool wm_can = feplb_wm_supported(cfg->E, cfg->E + cap_groups);
   c->few_auto = c->few = few_rows(*cfg, c->num_sms);
   c->wm_ok = wm_can && cfg->f % 128 == 0 && cfg->d % 256 == 0;
-  c->wm_auto = c->wm = wm_can && S >= (int64_t)FEPLB_WM_MIN_ROWS_PER_EXPERT * cfg->E &&
-                       S < (int64_t)FEPLB_MERGED_MAX_ROWS_PER_EXPERT * cfg->E && (int64_t)cfg->d * cfg->f >= FEPLB_WM_MIN_WEIGHT;
+  const bool large = weight >= FEPLB_MERGED_ANY_ROWS_WEIGHT;
+  c->wm_merged_auto = c->wm_merged = wm_can && S >= (int64_t)FEPLB_WM_MIN_ROWS_PER_EXPERT * cfg->E &&
+                                     S < (int64_t)FEPLB_WM_MAX_ROWS_PER_EXPERT * cfg->E && weight >= FEPLB_WM_MIN_WEIGHT;
+  c->wm_auto = c->wm = c->wm_merged && S < (int64_t)FEPLB_MERGED_MAX_ROWS_PER_EXPERT * cfg->E;
   // In the four-launch order the static experts are the less busy ones and stay in the range above for longer: d = 6144,
   // f = 2048, 128 experts, 1024 rows per expert on average 9911 -> 9750 us per layer, 1500 rows 13828 -> 13785.
-  c->wm_static_auto = c->wm_static = wm_can && S < (int64_t)2048 * cfg->E && (int64_t)cfg->d * cfg->f >= FEPLB_WM_MIN_WEIGHT;
+  c->wm_static_auto = c->wm_static = wm_can && S < (int64_t)2048 * cfg->E && weight >= FEPLB_WM_MIN_WEIGHT;
   // One launch per pass over the static and then the dynamic groups (the table of the latter is
   // picked up on the device): saves two launch ramps and two partly filled last waves per forward,
-  // which matters while a forward's GEMMs take a few hundred microseconds; one form serves both
-  // tables then, so it stays off where the dynamic groups want the two-CTA form and the static ones
-  // do not (from ~1000 rows per expert).
+  // which matters while a forward's GEMMs take up to a few milliseconds.  Launches of their own -> one, us per layer
+  // (weights on M / two-CTA tiles): 64 experts, d = 2048, f = 768, 768 rows per expert 549 -> 533 / 535, 1536 994 ->
+  // 979 / 978, 2812 1735 -> 1717 / 1687, 6144 3654 -> 3656 / 3611; 32, d = 4096, f = 1024, 1024 rows 866 -> 834 / 841, 2048
+  // 1555 -> 1562 / 1543; 64, d = 3072, f = 1536, 1250 2087 -> 2065 / 2103.  At large weights (d = 6144, f = 2048) the two
+  // are within 1 %, and static and dynamic groups keep a form each from 768 rows per expert.
   c->merged_ok = cfg->E + cap_groups <= FEPLB_MAX_GROUPS;
-  c->merged_auto = c->merged = c->merged_ok && S < (int64_t)FEPLB_MERGED_MAX_ROWS_PER_EXPERT * cfg->E;
+  c->merged_auto = c->merged = c->merged_ok && (!large || S < (int64_t)FEPLB_MERGED_MAX_ROWS_PER_EXPERT * cfg->E);
   // Small batches: a migration only relabels the rank that executes rows whose weights are the same everywhere, so
   // the launches need not wait for the plan at all.  They do where the static groups keep the GPU busy for longer
   // than the planner takes (its table is then there in time); below that the wait and the table's way to the
@@ -672,7 +681,7 @@ static int ffn_impl(feplb_ctx* c, const void* x_perm, const void* w1, const void
       return rc;
     }
   }
-  if ((c->wm || weights_on_m) && n_groups + (dyn ? dyn->max_groups : 0) <= FEPLB_WM_MAX_ENTRIES) {
+  if ((weights_on_m || (dyn ? c->wm_merged : c->wm)) && n_groups + (dyn ? dyn->max_groups : 0) <= FEPLB_WM_MAX_ENTRIES) {
     const feplb_wm_dyn none;
     rc = feplb_launch_expert_ffn_wm(a, dyn ? *dyn : none, st, &c->launches, c->err, sizeof(c->err));
     if (rc != FEPLB_E_STATE) {
@@ -1270,6 +1279,7 @@ extern "C" int feplb_set_gemm_form(feplb_ctx* c, int32_t forward_form, int32_t b
   c->wm_static = forward_form == FEPLB_FORM_AUTO && c->wm_static_auto;
   c->few = forward_form == FEPLB_FORM_AUTO ? c->few_auto : 0;
   c->wm = forward_form == FEPLB_FORM_AUTO ? c->wm_auto : forward_form == FEPLB_FORM_WEIGHT_M;
+  c->wm_merged = forward_form == FEPLB_FORM_AUTO ? c->wm_merged_auto : c->wm;
   c->gemm_pair_forced = forward_form == FEPLB_FORM_SINGLE || forward_form == FEPLB_FORM_PAIR ? forward_form : -1;
   c->gemm_pair_default = c->gemm_pair_forced < 0 ? c->gemm_pair_auto : forward_form;
   c->bwd_pair = backward_pair < 0 ? c->bwd_pair_auto : backward_pair;

@@ -431,7 +431,7 @@ k_grouped_gemm(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__
     };
     auto announce = [&](const Source& q, int st) {      // the bytes of a stage, and what the issuer does with them
       if (PAIR && cta_rank) return;
-      if (PAIR || NARROW) tail->idesc[st] = q.idesc;
+      if (PAIR) tail->idesc[st] = q.idesc;
       mbar_expect_tx(smem_u32(&tail->full[st]), q.tx);
     };
     auto load_b = [&](const Source& q, int kb, uint32_t full, uint32_t sb) {
@@ -546,15 +546,16 @@ k_grouped_gemm(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__
           total = tail->total_mtiles * p.n_tiles_n;
           if (tile >= total) break;
         }
+        if (!PAIR && NARROW) idesc = make_idesc(kTileRows, 2 * min(p.bn, p.half_width - tile % p.n_tiles_n * p.bn));
         if (!(ok = mbar_wait(smem_u32(&tail->tmem_empty[as]), aphase ^ 1u, abort_flag, p.status))) break;
         tc_fence_after();
         const uint32_t d_tmem = tmem_base + (uint32_t)(as * kAccCols);
         for (int kb = 0; kb < p.num_k_blocks; ++kb) {
           if (!(ok = mbar_wait(smem_u32(&tail->full[stage]), phase, abort_flag, p.status))) break;
           tc_fence_after();
-          if ((PAIR || NARROW) && kb == 0) {
+          if (PAIR && kb == 0) {
             idesc = *reinterpret_cast<volatile uint32_t*>(&tail->idesc[stage]);
-            if (PAIR) a_chunk = idesc >> 24 == BM >> 4 ? kABytes / 2 >> 4 : kABytes >> 4;
+            a_chunk = idesc >> 24 == BM >> 4 ? kABytes / 2 >> 4 : kABytes >> 4;
           }
           const uint32_t sa = smem_u32(smem + (size_t)stage * kStageBytes);
           const uint64_t da = make_smem_desc(sa);

@@ -23,7 +23,10 @@
 #define FEPLB_ST_WAIT 4u       // a bounded mbarrier wait gave up inside the GEMM
 #define FEPLB_ST_GROUP 8u      // a group entry was malformed (expert or rows out of range)
 #define FEPLB_ST_PLAN 16u      // the GEMM's bounded wait for the planner's dynamic group table gave up
-#define FEPLB_MERGED_MAX_ROWS_PER_EXPERT 768   // static and dynamic groups share launches below this many rows per expert
+#define FEPLB_MERGED_MAX_ROWS_PER_EXPERT 768   // static and dynamic groups share launches below this many rows per expert ...
+#define FEPLB_MERGED_ANY_ROWS_WEIGHT (6 << 20)  // ... and at any number where a weight matrix has fewer elements than this
+#define FEPLB_WM_MAX_ROWS_PER_EXPERT 1280       // the weights-on-M form ends here in such launches
+#define FEPLB_SHORT_TILE_WEIGHT (1 << 18)       // below this many elements tiles are short: see feplb_create
 #define FEPLB_PAIR_MIN_ROWS_PER_EXPERT 256     // launches over static and dynamic groups, or all: two-CTA tiles from here
 #define FEPLB_FEW_LARGE_WEIGHT (1 << 20)       // weight matrices of at least so many elements: the form for few rows per expert up to ...
 #define FEPLB_WM_MIN_ROWS_PER_EXPERT 64        // ... this many; from here (up to the line above) the weights-on-M form ...
