@@ -90,3 +90,14 @@ def test_units_for_few_rows_per_expert(d, f, rows, w3_first):
     """Segments around the multiples of 16 rows and of a unit, in each size of the units that the rule picks; saved
     pre-activations."""
     assert _run(rows, d, f, None, w3_first, preact=True) & F.PATH_SINGLE
+
+
+@pytest.mark.parametrize("d,f,rows,form", [
+    (128, 64, [300, 200, 280], F.PATH_PAIR),              # 256 rows per expert and more: two-CTA tiles ...
+    (128, 64, [600, 500, 450], F.PATH_SINGLE),            # ... and from 512 single-CTA tiles again for small weights
+    (1024, 512, [900, 641, 768], F.PATH_WEIGHT_M),        # weights on M up to 1280 rows per expert
+    (1024, 512, [1281, 1279, 1280], F.PATH_PAIR),
+])
+def test_forms_of_larger_batches(d, f, rows, form):
+    path = _run(rows, d, f, None)
+    assert path & (F.PATH_SINGLE | F.PATH_PAIR | F.PATH_WEIGHT_M) == form
