@@ -29,12 +29,12 @@ from paper_2604_19654_b200 import workloads as W  # noqa: E402
 
 METRIC = "moe_layer_tokens_per_s"
 UNIT = "tokens/s"
-# DRAM bytes (read + write) of one k_grouped_gemm launch at the benchmarked workload, from the ncu
+# DRAM bytes (read + write) of one expert GEMM launch at the benchmarked workload, from the ncu
 # capture summarised under profiles/; none (null in the line) where no capture exists.
-NCU_TRAFFIC_BYTES_PER_LAUNCH = {     # keyed by (workload, GEMM launches per forward)
-    ("cfg2", 2): {"bytes": 380.7e6, "source": "profiles/k_grouped_gemm_cfg2.md: 761.4 MB over the 2 launches of one forward "
-                                              "(capture of the merged two-CTA launches)"},
-    ("cfg2", 4): {"bytes": 190.0e6, "source": "capture of the four-launch form: 760 MB over the 4 launches of one forward"},
+NCU_TRAFFIC_BYTES_PER_LAUNCH = {     # keyed by (workload, GEMM launches per forward, kernels)
+    ("cfg2", 2, "k_ffn_wm"): {"bytes": 380.6e6, "source": "profiles/k_ffn_wm_cfg2.md: 761.2 MB over the 2 launches of one forward"},
+    ("cfg2", 2, "k_grouped_gemm (pair)"): {"bytes": 380.7e6, "source": "profiles/k_grouped_gemm_cfg2.md: 761.4 MB over the 2 launches of one forward "
+                                                                      "(merged two-CTA launches, 256-row tiles)"},
 }
 
 
@@ -291,6 +291,7 @@ def run_cuda(args, w):
     ctx.timeline_totals(reset=True)
     blocks2 = timed_blocks(args.min_timed_ms)
     totals, n_fw = ctx.timeline_totals(reset=True)
+    args.ffn_kernels = _ffn_kernels(ctx.forward_path())
     ctx.set_timeline(False)
     m2 = sampler.mark() if rank == 0 else 0
     ctx.check_status()
@@ -617,6 +618,13 @@ def time_oracle_single_thread(w, sample_tokens, weights):
     return {"value": val, "sample_tokens": n_tok}
 
 
+def _ffn_kernels(path):
+    """The kernels behind the expert GEMM launches of a forward, from its path bits."""
+    from paper_2604_19654_b200 import feplb as F
+    names = ((F.PATH_SINGLE, "k_grouped_gemm (single) or k_ffn_few"), (F.PATH_PAIR, "k_grouped_gemm (pair)"), (F.PATH_WEIGHT_M, "k_ffn_wm"))
+    return ", ".join(n for bit, n in names if path & bit)
+
+
 def _report(args, w, ctx, rank, world, value, ms_total, launches, clocks, totals, n_fw, e2e_value, h2d, d2h, strag, weights, n_mb):
     if rank == 0:
         peaks = _peaks()
@@ -631,8 +639,8 @@ def _report(args, w, ctx, rank, world, value, ms_total, launches, clocks, totals
         sus = peaks["bf16_tflops_sustained"] or peaks["bf16_tflops"]
         io_bytes = 2.0 * (w.T * w.d + w.S * w.d) + 12.0 * w.S
         cold = getattr(args, "cold", None) or {}
-        traffic = NCU_TRAFFIC_BYTES_PER_LAUNCH.get((w.name, per_fw)) if args.form in ("auto", "pair") else None
-        roof = {"bound": "tensor", "kernel": ("k_grouped_gemm, static + dynamic groups per launch" if per_fw == 2 else "k_grouped_gemm") if args.form != "weight_m" else "k_ffn_wm",
+        traffic = NCU_TRAFFIC_BYTES_PER_LAUNCH.get((w.name, per_fw, args.ffn_kernels))
+        roof = {"bound": "tensor", "kernel": args.ffn_kernels + (", static + dynamic groups per launch" if per_fw == 2 else ""),
                 "achieved": achieved, "peak": peak, "unit": "TFLOP/s",
                 "frac": achieved / peak if achieved else None,
                 "peak_source": f"{peaks['source']} ({regime}: chosen from the SM clock and power-cap state sampled during this pass)",
