@@ -438,7 +438,7 @@ int feplb_set_gemm_form(feplb_ctx* ctx, int32_t forward_form, int32_t backward_p
  * their own (four per forward), the dynamic ones enqueued after the planner has been joined and
  * each table in the form that suits it.  -1 (default): merged, except for large weights (6 Mi elements
  * per matrix) from 768 rows per expert, and for the smallest batches (below 128 rows per expert, or ~150 us
- * of expert FFN) two launches over the home groups that do not depend on the plan at all, which the
+ * of expert FFN, or up to 8192 slots from 192 on) two launches over the home groups that do not depend on the plan at all, which the
  * calling thread makes after it has enqueued them.  With cfg.phase2_copy the four-launch order is always used.
  * merged = 1 needs 2*E + R*max_num_dyn <= 1024.  Not allowed while a plan is pending. */
 int feplb_set_launch_merging(feplb_ctx* ctx, int32_t merged);

@@ -443,11 +443,15 @@ extern "C" int feplb_create(const feplb_config* cfg, feplb_ctx** out) {
   // per expert, d = 1920), 181 -> 170 (128 of d = 2048).  Above the line, where the table comes with the gather, the two
   // are level: 173.6 and 172.0 at 131 rows per expert of d = 2048, 211 and 211 at 188, 286 and 284 at 281, 2001 and 1989
   // at 128 of d = 6144; at 1024 of d = 6144 the order that gives the static groups launches of their own is 4 % ahead.
-  // (Up to 8192 slots no CTA of the front picks the table up: 16 experts of d = 4096, f = 1024, 384 rows each, would
-  // gain from this order, 227 -> 199.)
+  // Up to 8192 slots no CTA of the front picks the table up, the launches always take the late way, and the line lies
+  // elsewhere: 192 rows per expert.  Table order -> this: 32 experts of d = 6144, f = 2048, 256 rows each 789 -> 764 us, 32 of
+  // d = f = 2048, 256 rows 285 -> 266, 24 of d = 3072, f = 1536, 333 rows 321 -> 296, 16 of d = 6144, f = 2048, 512 rows
+  // 707 -> 678; at 171 rows (48 experts, d = 6144) 952 -> 932, within the runs of one side.  From 768 rows per expert of large weights static and dynamic groups keep the launches of
+  // their own that feplb_forward_path reports there.
   // The time is an estimate: all weights streamed at 6.5 TB/s plus the products at 1 PFLOP/s.
   const double ffn_us = 6.0 * cfg->d * cfg->f * ((double)cfg->E / 6.5e6 + (double)S / 1e9);
-  c->direct_auto = c->direct = S < (int64_t)FEPLB_DIRECT_ROWS_PER_EXPERT * cfg->E || ffn_us < FEPLB_DIRECT_FFN_US;
+  c->direct_auto = c->direct = S < (int64_t)FEPLB_DIRECT_ROWS_PER_EXPERT * cfg->E || ffn_us < FEPLB_DIRECT_FFN_US ||
+                                (c->merged && feplb_front_is_small(S, cfg->E) && S >= (int64_t)FEPLB_DIRECT_SMALL_FRONT_ROWS * cfg->E);
   bool ok = true;
   ok = ok && cudaMalloc(&c->d_dyn_ready, 4 * sizeof(unsigned long long)) == cudaSuccess &&
        cudaMemset(c->d_dyn_ready, 0, 4 * sizeof(unsigned long long)) == cudaSuccess;

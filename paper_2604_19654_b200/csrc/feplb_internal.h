@@ -33,6 +33,7 @@
 #define FEPLB_WM_MIN_WEIGHT (1 << 19)          // ... for weight matrices of at least so many elements
 // No launch of a forward waits for the plan below this many rows per expert, or where the expert FFN takes less than this long
 #define FEPLB_DIRECT_ROWS_PER_EXPERT 128
+#define FEPLB_DIRECT_SMALL_FRONT_ROWS 192      // ... or, in the merged order behind the one-launch front, from this many
 #define FEPLB_DIRECT_FFN_US 150
 #define FEPLB_WM_MAX_ENTRIES 1024    // group entries (static + dynamic table) one weights-on-M launch can hold
 

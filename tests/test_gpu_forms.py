@@ -101,3 +101,13 @@ def test_units_for_few_rows_per_expert(d, f, rows, w3_first):
 def test_forms_of_larger_batches(d, f, rows, form):
     path = _run(rows, d, f, None)
     assert path & (F.PATH_SINGLE | F.PATH_PAIR | F.PATH_WEIGHT_M) == form
+
+
+@pytest.mark.parametrize("rows,order", [
+    ([191] * 8, F.PATH_MERGED),                # an FFN of more than 150 us behind the one-launch front: 192 rows per expert
+    ([192] * 8, F.PATH_HOME_TABLE),
+    ([640, 0, 1, 128, 300, 255, 200, 12], F.PATH_HOME_TABLE),
+])
+def test_order_behind_the_one_launch_front(rows, order):
+    path = _run(rows, 4096, 4096, None)
+    assert path & (F.PATH_MERGED | F.PATH_HOME_TABLE | F.PATH_SMALL_FRONT) == order | F.PATH_SMALL_FRONT
