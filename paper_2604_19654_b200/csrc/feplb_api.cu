@@ -354,10 +354,21 @@ static int few_rows(const feplb_config& g, int num_sms) {
   const int64_t blocks = g.f / 64 > g.d / 128 ? g.f / 64 : g.d / 128;        // weight blocks of the wider pass
   for (int n = 32; n <= 128 && S < FEPLB_PAIR_MIN_ROWS_PER_EXPERT * E; n *= 2)
     if ((touched + S / n) * blocks <= num_sms) return n;
-  if (S < 7 * E) return g.T <= 64 ? 32 : 64;
-  if (g.f <= 128) return 0;
-  if (weight < FEPLB_FEW_LARGE_WEIGHT) return S < 24 * E ? 64 : 0;
-  return S < 14 * E ? 64 : S < FEPLB_WM_MIN_ROWS_PER_EXPERT * E ? 128 : 0;
+  int n = 0;
+  if (S < 7 * E) n = g.T <= 64 ? 32 : 64;
+  else if (g.f <= 128) n = 0;
+  else if (weight < FEPLB_FEW_LARGE_WEIGHT) n = S < 24 * E ? 64 : 0;
+  else n = S < 14 * E ? 64 : S < FEPLB_WM_MIN_ROWS_PER_EXPERT * E ? 128 : 0;
+  // A second wave of units that is mostly empty costs a whole one where units are long (their weights' 64 rows of f; the
+  // single form's tiles are twice as wide): 1.2 to 1.8 waves in pass 1 32 experts, d = 5376, f = 448, T = 65 80 -> 90, 60, d =
+  // 3712, f = 192, T = 114 68 -> 77, 16, d = 1408, f = 576, T = 174 30.1 -> 31.7, 1.1 waves 16, d = 3072, f = 640, T = 3 1.28 times
+  // faster, 2.4 waves 1.05 times.  Units of 128 rows need more of them: 4.4 waves 64 experts, d = 2944, f = 576, T = 178 104
+  // -> 112, 4.7 waves 128, d = 4992, f = 256, T = 745 224 -> 238, 5.0 waves 128, d = 5888, f = 320, T = 330 1.03 times faster.
+  if (n && weight >= FEPLB_WM_MIN_WEIGHT) {
+    const int64_t units = g.f / 64 * (touched + S / n);
+    if (5 * units > 6 * num_sms && units < (n == 128 ? 5 : 2) * num_sms) return 0;
+  }
+  return n;
 }
 
 extern "C" int feplb_version(void) { return 100; }
@@ -395,10 +406,12 @@ extern "C" int feplb_create(const feplb_config* cfg, feplb_ctx** out) {
   // 256-row pair tiles pay off when an expert's segment is several tiles long on average
   c->gemm_pair_auto = c->gemm_pair_default = (int64_t)cfg->T * cfg->K >= (int64_t)2048 * cfg->E;
   // a launch over static and dynamic groups runs them in one form: the two-CTA form from 256 rows per expert, but small
-  // weights and many rows, where a tile is short, in single-CTA tiles (16 experts, d = 512, f = 256, T = 8000 / 30000, top-2
-  // 45.9 -> 42.2 / 107.9 -> 99.4 us per layer; 8 experts, d = 128, f = 64, T = 40000 64.1 -> 54.9)
+  // weights, where a tile is short, from 288 rows in single-CTA tiles (us per layer: 16 experts, d = 512, f = 256, T = 30000,
+  // top-2 107.9 -> 99.4; 48, d = 128, f = 64, 293 rows 33.6 -> 26.9; 24, d = 640, f = 256, 297 rows 107.9 -> 95.1; 128, d = 1792,
+  // f = 128, 330 rows 187 -> 173; 8, d = 6144, f = 64, 1761 rows 260 -> 245; 128, d = 1792, f = 256, 604 rows 396 -> 386; d = 2688,
+  // f = 192, 2262 rows 379 -> 361; d = 1152, f = 384, 1903 rows 92.6 -> 91.9; but d = 1536, f = 576, 6713 rows 302 -> 359)
   const int64_t weight = (int64_t)cfg->d * cfg->f;
-  const bool short_tiles = weight < FEPLB_SHORT_TILE_WEIGHT && (int64_t)cfg->T * cfg->K >= (int64_t)512 * cfg->E;
+  const bool short_tiles = weight < FEPLB_SHORT_TILE_WEIGHT && (int64_t)cfg->T * cfg->K >= (int64_t)FEPLB_SHORT_TILE_MIN_ROWS * cfg->E;
   c->merged_pair = (int64_t)cfg->T * cfg->K >= (int64_t)FEPLB_PAIR_MIN_ROWS_PER_EXPERT * cfg->E && !short_tiles;
   // backward GEMMs: the pair form pays once an expert's segment spans several 256-row tiles
   // (measured: -7.5 % backward time at 1024 rows per expert, slower at 384)
@@ -415,16 +428,23 @@ extern "C" int feplb_create(const feplb_config* cfg, feplb_ctx** out) {
   //     2812 1917 / 1815 / 1832
   //   half-empty last weight blocks (60 experts, d = 1920, f = 704): 102 145.8 / 152.4 / 140.0, 400 312 / 304 / 298
   //   32 experts, d = 1024, f = 512: 112 44.8 / 44.6 / 43.2, 250 63.2 / 61.4 / 59.6;  16, d = 512, f = 256: 375 28.4 / 30.9 / 31.3
+  // Below 3 Mi elements the launch must have six waves of units and at most an eighth of them empty: 24 experts, d = 2304, f =
+  // 320, 113 rows, 1.4 waves 48 -> 59; 16, d = 2944, f = 448, 132 rows, 1.3 waves 55 -> 65; 48, d = 2688, f = 384, 169 rows, 3.2
+  // waves 112 -> 123; 64, d = 2816, f = 512, 135 rows, 5.3 waves 163 -> 172; 128, d = 2560, f = 320 (a sixth empty), 264 rows,
+  // 10.5 waves 355 -> 365; but 60, d = 1920, f = 704, 6.8 waves 146 -> 141, 32, d = 1920, f = 448, 9 waves 1.08 times faster.
+  const int64_t f_blocks = (cfg->f + 127) / 128;
+  const bool wm_units = f_blocks * (cfg->E + S / 256) >= 6 * (c->num_sms / 2) && f_blocks * 128 * 7 <= (int64_t)cfg->f * 8;
   const bool wm_can = feplb_wm_supported(cfg->E, cfg->E + cap_groups);
   c->few_auto = c->few = few_rows(*cfg, c->num_sms);
   c->wm_ok = wm_can && cfg->f % 128 == 0 && cfg->d % 256 == 0;
   const bool large = weight >= FEPLB_MERGED_ANY_ROWS_WEIGHT;
   c->wm_merged_auto = c->wm_merged = wm_can && S >= (int64_t)FEPLB_WM_MIN_ROWS_PER_EXPERT * cfg->E &&
-                                     S < (int64_t)FEPLB_WM_MAX_ROWS_PER_EXPERT * cfg->E && weight >= FEPLB_WM_MIN_WEIGHT;
+                                     S < (int64_t)FEPLB_WM_MAX_ROWS_PER_EXPERT * cfg->E &&
+                                     (weight >= FEPLB_WM_ANY_UNITS_WEIGHT || (weight >= FEPLB_WM_MIN_WEIGHT && wm_units));
   c->wm_auto = c->wm = c->wm_merged && S < (int64_t)FEPLB_MERGED_MAX_ROWS_PER_EXPERT * cfg->E;
   // In the four-launch order the static experts are the less busy ones and stay in the range above for longer: d = 6144,
   // f = 2048, 128 experts, 1024 rows per expert on average 9911 -> 9750 us per layer, 1500 rows 13828 -> 13785.
-  c->wm_static_auto = c->wm_static = wm_can && S < (int64_t)2048 * cfg->E && weight >= FEPLB_WM_MIN_WEIGHT;
+  c->wm_static_auto = c->wm_static = wm_can && S < (int64_t)2048 * cfg->E && weight >= FEPLB_WM_ANY_UNITS_WEIGHT;
   // One launch per pass over the static and then the dynamic groups (the table of the latter is
   // picked up on the device): saves two launch ramps and two partly filled last waves per forward,
   // which matters while a forward's GEMMs take up to a few milliseconds.  Launches of their own -> one, us per layer

@@ -26,11 +26,13 @@
 #define FEPLB_MERGED_MAX_ROWS_PER_EXPERT 768   // static and dynamic groups share launches below this many rows per expert ...
 #define FEPLB_MERGED_ANY_ROWS_WEIGHT (6 << 20)  // ... and at any number where a weight matrix has fewer elements than this
 #define FEPLB_WM_MAX_ROWS_PER_EXPERT 1280       // the weights-on-M form ends here in such launches
-#define FEPLB_SHORT_TILE_WEIGHT (1 << 18)       // below this many elements tiles are short: see feplb_create
+#define FEPLB_SHORT_TILE_WEIGHT (1 << 19)       // below this many elements tiles are short, single-CTA tiles better ...
+#define FEPLB_SHORT_TILE_MIN_ROWS 288           // ... from this many rows per expert
 #define FEPLB_PAIR_MIN_ROWS_PER_EXPERT 256     // launches over static and dynamic groups, or all: two-CTA tiles from here
 #define FEPLB_FEW_LARGE_WEIGHT (1 << 20)       // weight matrices of at least so many elements: the form for few rows per expert up to ...
 #define FEPLB_WM_MIN_ROWS_PER_EXPERT 64        // ... this many; from here (up to the line above) the weights-on-M form ...
 #define FEPLB_WM_MIN_WEIGHT (1 << 19)          // ... for weight matrices of at least so many elements
+#define FEPLB_WM_ANY_UNITS_WEIGHT (3 << 20)     // ... and enough units; from this many elements whatever their number
 // No launch of a forward waits for the plan below this many rows per expert, or where the expert FFN takes less than this long
 #define FEPLB_DIRECT_ROWS_PER_EXPERT 128
 #define FEPLB_DIRECT_SMALL_FRONT_ROWS 192      // ... or, in the merged order behind the one-launch front, from this many

@@ -74,17 +74,17 @@ def test_weights_in_one_buffer(form):
 
 @pytest.mark.parametrize("w3_first", [False, True])
 def test_weights_on_m_units_of_any_width(w3_first):
-    """d = 4.5 x 256, f = 4.5 x 128: the second CTA's half of the last weight block lies past the width, the last K block of
+    """d = 7.5 x 256, f = 13.5 x 128: the second CTA's half of the last weight block lies past the width, the last K block of
     pass 2 is half empty; segments around the multiples of 32 and 256 rows; saved pre-activations."""
     rows = [1, 31, 32, 33, 64, 65, 128, 129, 200, 255, 256, 257, 300]
-    assert _run(rows, 1152, 576, None, w3_first, preact=True) & F.PATH_WEIGHT_M
+    assert _run(rows, 1920, 1728, None, w3_first, preact=True) & F.PATH_WEIGHT_M
 
 
 @pytest.mark.parametrize("w3_first", [False, True])
 @pytest.mark.parametrize("d,f,rows", [
     (256, 320, [1, 15, 16, 17, 31, 32, 33, 40]),                             # one wave of units of 32 rows
     (1024, 1024, [1, 15, 16, 17, 33, 63, 64, 65] + [0] * 14),                # units of 64 rows
-    (1024, 1088, [1, 16, 31, 32, 33, 64, 65, 127, 128, 129]),                # units of 128 rows, K blocks half empty
+    (1920, 576, [1, 16, 31, 32, 33, 64, 65, 127, 128, 129]),                 # units of 128 rows, K blocks half empty
 ])
 def test_units_for_few_rows_per_expert(d, f, rows, w3_first):
     """Segments around the multiples of 16 rows and of a unit, in each size of the units that the rule picks; saved
@@ -94,9 +94,10 @@ def test_units_for_few_rows_per_expert(d, f, rows, w3_first):
 
 @pytest.mark.parametrize("d,f,rows,form", [
     (128, 64, [300, 200, 280], F.PATH_PAIR),              # 256 rows per expert and more: two-CTA tiles ...
-    (128, 64, [600, 500, 450], F.PATH_SINGLE),            # ... and from 512 single-CTA tiles again for small weights
-    (1024, 512, [900, 641, 768], F.PATH_WEIGHT_M),        # weights on M up to 1280 rows per expert
-    (1024, 512, [1281, 1279, 1280], F.PATH_PAIR),
+    (128, 64, [300, 200, 364], F.PATH_SINGLE),            # ... and from 288 single-CTA tiles again for small weights
+    (2048, 1536, [900, 641, 768], F.PATH_WEIGHT_M),       # weights on M up to 1280 rows per expert
+    (2048, 1536, [1281, 1279, 1280], F.PATH_PAIR),
+    (1024, 512, [300, 257, 280], F.PATH_PAIR),            # too few units of weights on M
 ])
 def test_forms_of_larger_batches(d, f, rows, form):
     path = _run(rows, d, f, None)
