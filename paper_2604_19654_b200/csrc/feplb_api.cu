@@ -409,9 +409,10 @@ extern "C" int feplb_create(const feplb_config* cfg, feplb_ctx** out) {
   // weights, where a tile is short, from 288 rows in single-CTA tiles (us per layer: 16 experts, d = 512, f = 256, T = 30000,
   // top-2 107.9 -> 99.4; 48, d = 128, f = 64, 293 rows 33.6 -> 26.9; 24, d = 640, f = 256, 297 rows 107.9 -> 95.1; 128, d = 1792,
   // f = 128, 330 rows 187 -> 173; 8, d = 6144, f = 64, 1761 rows 260 -> 245; 128, d = 1792, f = 256, 604 rows 396 -> 386; d = 2688,
-  // f = 192, 2262 rows 379 -> 361; d = 1152, f = 384, 1903 rows 92.6 -> 91.9; but d = 1536, f = 576, 6713 rows 302 -> 359)
+  // f = 192, 2262 rows 379 -> 361; d = 1152, f = 384, 1903 rows 92.6 -> 91.9; but d = 1536, f = 576, 6713 rows 302 -> 359,
+  // and d = 512, f = 832, 6118 rows 150 -> 160: from 256 Ki elements on only where f is short)
   const int64_t weight = (int64_t)cfg->d * cfg->f;
-  const bool short_tiles = weight < FEPLB_SHORT_TILE_WEIGHT && (int64_t)cfg->T * cfg->K >= (int64_t)FEPLB_SHORT_TILE_MIN_ROWS * cfg->E;
+  const bool short_tiles = (weight < FEPLB_SHORT_TILE_WEIGHT / 2 || (weight < FEPLB_SHORT_TILE_WEIGHT && cfg->f <= 384)) && (int64_t)cfg->T * cfg->K >= (int64_t)FEPLB_SHORT_TILE_MIN_ROWS * cfg->E;
   c->merged_pair = (int64_t)cfg->T * cfg->K >= (int64_t)FEPLB_PAIR_MIN_ROWS_PER_EXPERT * cfg->E && !short_tiles;
   // backward GEMMs: the pair form pays once an expert's segment spans several 256-row tiles
   // (measured: -7.5 % backward time at 1024 rows per expert, slower at 384)
