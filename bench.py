@@ -291,7 +291,7 @@ def run_cuda(args, w):
     ctx.timeline_totals(reset=True)
     blocks2 = timed_blocks(args.min_timed_ms)
     totals, n_fw = ctx.timeline_totals(reset=True)
-    args.ffn_kernels = _ffn_kernels(ctx.forward_path())
+    args.ffn_kernels = _ffn_kernels(ctx.forward_path(), ctx.forward_detail())
     ctx.set_timeline(False)
     m2 = sampler.mark() if rank == 0 else 0
     ctx.check_status()
@@ -618,10 +618,11 @@ def time_oracle_single_thread(w, sample_tokens, weights):
     return {"value": val, "sample_tokens": n_tok}
 
 
-def _ffn_kernels(path):
-    """The kernels behind the expert GEMM launches of a forward, from its path bits."""
+def _ffn_kernels(path, detail):
+    """The kernels behind the expert GEMM launches of a forward, from its path and detail bits."""
     from paper_2604_19654_b200 import feplb as F
-    names = ((F.PATH_SINGLE, "k_grouped_gemm (single) or k_ffn_few"), (F.PATH_PAIR, "k_grouped_gemm (pair)"), (F.PATH_WEIGHT_M, "k_ffn_wm"))
+    few = detail & (F.DETAIL_UNITS_32 | F.DETAIL_UNITS_64 | F.DETAIL_UNITS_128)
+    names = ((F.PATH_SINGLE, "k_ffn_few" if few else "k_grouped_gemm (single)"), (F.PATH_PAIR, "k_grouped_gemm (pair)"), (F.PATH_WEIGHT_M, "k_ffn_wm"))
     return ", ".join(n for bit, n in names if path & bit)
 
 

@@ -464,6 +464,12 @@ int feplb_selftest_bounded_wait(feplb_ctx* ctx, int32_t limit_us, void* stream);
 #define FEPLB_PATH_PAIR 32         /* two-CTA tiles of 256 rows */
 #define FEPLB_PATH_WEIGHT_M 64     /* weights-on-M units */
 int32_t feplb_forward_path(const feplb_ctx* ctx);
+/* Which variants of those forms ran, FEPLB_DETAIL_* bits (0 before the first forward).  Units: with few rows per expert
+ * FEPLB_PATH_SINGLE stands for tiles of 128 weight rows by at most so many token rows. */
+#define FEPLB_DETAIL_UNITS_32 32
+#define FEPLB_DETAIL_UNITS_64 64
+#define FEPLB_DETAIL_UNITS_128 128
+int32_t feplb_forward_detail(const feplb_ctx* ctx);
 /* Number of kernels this library has launched on `ctx` since creation. */
 int64_t feplb_launch_count(const feplb_ctx* ctx);
 

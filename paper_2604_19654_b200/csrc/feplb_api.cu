@@ -40,6 +40,7 @@ struct feplb_ctx {
   char err[512] = {0};
   int64_t launches = 0;
   int32_t path = 0;            // FEPLB_PATH_* of the last forward
+  int32_t detail = 0;          // FEPLB_DETAIL_* of the last forward
   int gemm_pair_default = 0;   // GEMM form for launches whose group sizes the host does not know
   int gemm_pair_forced = -1;   // feplb_set_gemm_form: 0/1 forces one form everywhere, -1 = chosen per table
   int bwd_pair = 0;            // backward GEMMs in the pair form: bit 0 activation gradients, bit 1 weight gradients
@@ -612,6 +613,8 @@ extern "C" const char* feplb_last_error(const feplb_ctx* c) { return c ? c->err 
 
 extern "C" int32_t feplb_forward_path(const feplb_ctx* c) { return c ? c->path : 0; }
 
+extern "C" int32_t feplb_forward_detail(const feplb_ctx* c) { return c ? c->detail : 0; }
+
 extern "C" int64_t feplb_launch_count(const feplb_ctx* c) { return c ? c->launches : 0; }
 
 extern "C" int feplb_check_status(feplb_ctx* c, void* stream) {
@@ -703,6 +706,7 @@ static int ffn_impl(feplb_ctx* c, const void* x_perm, const void* w1, const void
     rc = feplb_launch_expert_ffn_few(a, st, &c->launches, c->err, sizeof(c->err), c->few, dyn ? dyn->stamps : nullptr);
     if (rc != FEPLB_E_STATE) {
       c->path |= FEPLB_PATH_SINGLE;
+      c->detail |= c->few;             // FEPLB_DETAIL_UNITS_*
       return rc;
     }
   }
@@ -722,9 +726,10 @@ extern "C" int feplb_expert_ffn(feplb_ctx* c, const void* x_perm, const void* w1
                                 const feplb_group* groups, int32_t n_groups, int32_t which,
                                 void* h_scratch, void* y_perm, void* stream) {
   if (!c) return FEPLB_E_INVALID;
-  const int32_t path = c->path;         // of the last forward, which this call is not
+  const int32_t path = c->path, detail = c->detail;         // of the last forward, which this call is not
   const int rc = ffn_impl(c, x_perm, w1, w3, w2, groups, n_groups, which, h_scratch, y_perm, (cudaStream_t)stream);
   c->path = path;
+  c->detail = detail;
   return rc;
 }
 
@@ -936,6 +941,7 @@ extern "C" int feplb_moe_forward(feplb_ctx* c, const void* x, const int32_t* top
   const int32_t seq = c->flag_seq;
   const bool small_front = feplb_front_is_small(S, g.E);
   c->path = (small_front ? FEPLB_PATH_SMALL_FRONT : 0) | (direct ? FEPLB_PATH_HOME_TABLE : wm ? FEPLB_PATH_MERGED : 0);
+  c->detail = 0;
   c->job_w1 = w1; c->job_w3 = w3; c->job_w2 = w2;   // read by the planner thread after it is woken
   c->job_x_perm = x_perm;
   // Where the gather looks for the planner's table the thread is woken before the launches whose counts it waits for: a
@@ -1098,6 +1104,7 @@ static int host_forward_ranges(feplb_ctx* c, int n, const int* first, const void
   memset(&c->tl, 0, sizeof(c->tl));
   c->tl.ffn_launches = 2 * n;
   c->path = FEPLB_PATH_RANGES;
+  c->detail = 0;
   // inputs: after whatever `st` still does with the staging buffers
   CUDA_TRY(c, cudaEventRecord(c->ev_range_ids, st));
   CUDA_TRY(c, cudaStreamWaitEvent(c->in_stream, c->ev_range_ids, 0));

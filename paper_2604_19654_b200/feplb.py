@@ -25,6 +25,7 @@ MASK_GIVEN, MASK_REACTIVE = 0, 1
 FFN_ALL, FFN_STATIC, FFN_DYNAMIC = 0, 1, 2
 FORM_AUTO, FORM_SINGLE, FORM_PAIR, FORM_WEIGHT_M = -1, 0, 1, 2
 PATH_SMALL_FRONT, PATH_HOME_TABLE, PATH_MERGED, PATH_RANGES, PATH_SINGLE, PATH_PAIR, PATH_WEIGHT_M = (1 << i for i in range(7))
+DETAIL_UNITS_32, DETAIL_UNITS_64, DETAIL_UNITS_128 = 32, 64, 128
 HOST_SLOTS = 4            # staging sets of the pipelined host-buffer forward (FEPLB_HOST_SLOTS)
 
 
@@ -126,6 +127,7 @@ def lib() -> C.CDLL:
             "feplb_selftest_bounded_wait": (C.c_int, [vp, i32, vp]),
             "feplb_launch_count": (i64, [vp]),
             "feplb_forward_path": (i32, [vp]),
+            "feplb_forward_detail": (i32, [vp]),
         }
         for name, (res, args) in sig.items():
             fn = getattr(L, name)
@@ -514,6 +516,10 @@ class Context:
     def forward_path(self) -> int:
         """PATH_* bits of the last forward: the order of its launches and the forms of its expert GEMMs."""
         return int(lib().feplb_forward_path(self._h))
+
+    def forward_detail(self) -> int:
+        """DETAIL_* bits of the last forward: the variants of those forms."""
+        return int(lib().feplb_forward_detail(self._h))
 
     def launch_count(self) -> int:
         return int(lib().feplb_launch_count(self._h))

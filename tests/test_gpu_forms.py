@@ -3,6 +3,7 @@ tile changes its shape, weights in either order in memory, widths that leave the
 half empty."""
 import numpy as np
 import pytest
+import torch
 
 from oracle import feplb_oracle as O
 from paper_2604_19654_b200 import build as B
@@ -19,9 +20,9 @@ def _built():
     B.build()
 
 
-def _run(rows, d, f, form, w3_first=False, same=False, preact=False):
-    """One forward whose expert e has rows[e] rows (top-1); returns the context's launch path."""
-    import torch
+def _run(rows, d, f, form, w3_first=False, same=False, preact=False, detail=None):
+    """One forward whose expert e has rows[e] rows (top-1), through the variants `detail` (None: any); returns the context's
+    launch path."""
     E, T = len(rows), sum(rows)
     w = W.get_workload("cfg1").with_(T=T, E=E, K=1, R=1, d=d, f=f, dyn=0)
     ids = np.repeat(np.arange(E, dtype=np.int32), rows)[np.random.default_rng(T).permutation(T)].reshape(T, 1)
@@ -54,8 +55,17 @@ def _run(rows, d, f, form, w3_first=False, same=False, preact=False):
             assert_close(got[:, :f], xe @ W.bf16_bits_to_f64(w1[e]).T, "a")
             assert_close(got[:, f:], xe @ W.bf16_bits_to_f64(w3[e]).T, "b")
     path = ctx.forward_path()
+    assert detail is None or ctx.forward_detail() == detail
     ctx.close()
     return path
+
+
+def _zeros(T, K, E, d, f):
+    """Context, buffers and inputs of a layer of zeros, tokens spread evenly at random: for what a forward does, not what it computes."""
+    z = lambda *s: torch.zeros(*s, dtype=torch.bfloat16, device="cuda")       # noqa: E731
+    cfg = F.make_config(T, K, E, 1, d, f, dyn=1, tau=1)
+    ids = torch.rand(T, E, generator=torch.Generator(device="cuda").manual_seed(1), device="cuda").topk(K, dim=1)[1].int()
+    return F.Context(cfg), F.Buffers(cfg), (z(T, d), ids, torch.ones(T, K, device="cuda")), (z(E, f, d), z(E, f, d), z(E, d, f))
 
 
 @pytest.mark.parametrize("w3_first", [False, True])
@@ -81,15 +91,48 @@ def test_weights_on_m_units_of_any_width(w3_first):
 
 
 @pytest.mark.parametrize("w3_first", [False, True])
-@pytest.mark.parametrize("d,f,rows", [
-    (256, 320, [1, 15, 16, 17, 31, 32, 33, 40]),                             # one wave of units of 32 rows
-    (1024, 1024, [1, 15, 16, 17, 33, 63, 64, 65] + [0] * 14),                # units of 64 rows
-    (1920, 576, [1, 16, 31, 32, 33, 64, 65, 127, 128, 129]),                 # units of 128 rows, K blocks half empty
+@pytest.mark.parametrize("d,f,rows,units", [
+    (256, 320, [1, 15, 16, 17, 31, 32, 33, 40], F.DETAIL_UNITS_32),          # one wave of units of 32 rows
+    (1024, 1024, [1, 15, 16, 17, 33, 63, 64, 65] + [0] * 14, F.DETAIL_UNITS_64),
+    (1920, 576, [1, 16, 31, 32, 33, 64, 65, 127, 128, 129], F.DETAIL_UNITS_128),      # K blocks half empty
 ])
-def test_units_for_few_rows_per_expert(d, f, rows, w3_first):
+def test_units_for_few_rows_per_expert(d, f, rows, units, w3_first):
     """Segments around the multiples of 16 rows and of a unit, in each size of the units that the rule picks; saved
     pre-activations."""
-    assert _run(rows, d, f, None, w3_first, preact=True) & F.PATH_SINGLE
+    assert _run(rows, d, f, None, w3_first, preact=True, detail=units) & F.PATH_SINGLE
+
+
+@pytest.mark.parametrize("d,f,rows,units", [
+    (2048, 1024, [33, 2] + [1] * 28 + [0] * 2, F.DETAIL_UNITS_32),           # 496 units in both passes
+    (2048, 1024, [65, 64, 63] + [1] * 26 + [0] * 3, F.DETAIL_UNITS_64),      # 480
+    (1024, 2048, [129, 128, 127] + [3] * 28 + [0], F.DETAIL_UNITS_128),      # 1024 and 256
+])
+def test_several_units_per_cta_for_few_rows(d, f, rows, units):
+    """More than three units for each of 148 CTAs, and more K blocks than stages: the accumulators and the ring go round, and
+    the weights loaded ahead of the first unit are followed by ordinary loads; saved pre-activations."""
+    assert _run(rows, d, f, None, preact=True, detail=units) & F.PATH_SINGLE
+
+
+@pytest.mark.parametrize("T,K,E,d,f,detail", [
+    (32, 4, 32, 2048, 1024, F.DETAIL_UNITS_32),
+    (16, 4, 16, 128, 64, F.DETAIL_UNITS_32),
+    (2048, 1, 16, 2048, 1024, 0),                  # 128 rows per expert
+])
+def test_detail_of_the_last_forward(T, K, E, d, f, detail):
+    """What a forward reports; asking for a form, or a call on a table of one's own, does not change it afterwards."""
+    ctx, buf, args, w = _zeros(T, K, E, d, f)
+    assert ctx.forward_detail() == 0
+    ctx.moe_forward(*args, *w, buf)
+    assert ctx.forward_detail() == detail
+    ctx.set_gemm_form(F.FORM_SINGLE)
+    groups = torch.zeros(E, 5, dtype=torch.int32, device="cuda")
+    ctx.home_groups(buf.counts, None, groups)
+    ctx.expert_ffn(buf.x_perm, *w, groups, E, buf.h_scratch, buf.y_perm)
+    assert ctx.forward_detail() == detail
+    ctx.moe_forward(*args, *w, buf)
+    assert ctx.forward_detail() == 0
+    ctx.check_status()
+    ctx.close()
 
 
 @pytest.mark.parametrize("d,f,rows,form", [
