@@ -6,6 +6,7 @@
 #include <atomic>
 #include <chrono>
 #include <climits>
+#include <cmath>
 #include <condition_variable>
 #include <cstdarg>
 #include <cstdio>
@@ -360,15 +361,30 @@ static int few_rows(const feplb_config& g, int num_sms) {
   else if (g.f <= 128) n = 0;
   else if (weight < FEPLB_FEW_LARGE_WEIGHT) n = S < 24 * E ? 64 : 0;
   else n = S < 14 * E ? 64 : S < FEPLB_WM_MIN_ROWS_PER_EXPERT * E ? 128 : 0;
-  // A second wave of units that is mostly empty costs a whole one where units are long (their weights' 64 rows of f; the
-  // single form's tiles are twice as wide): 1.2 to 1.8 waves in pass 1 32 experts, d = 5376, f = 448, T = 65 80 -> 90, 60, d =
-  // 3712, f = 192, T = 114 68 -> 77, 16, d = 1408, f = 576, T = 174 30.1 -> 31.7, 1.1 waves 16, d = 3072, f = 640, T = 3 1.28 times
-  // faster, 2.4 waves 1.05 times.  Units of 128 rows need more of them: 4.4 waves 64 experts, d = 2944, f = 576, T = 178 104
-  // -> 112, 4.7 waves 128, d = 4992, f = 256, T = 745 224 -> 238, 5.0 waves 128, d = 5888, f = 320, T = 330 1.03 times faster.
-  if (n && weight >= FEPLB_WM_MIN_WEIGHT) {
+  if (!n) return 0;
+  // A second wave of units that is mostly empty costs a whole one where units are long (their weights' 64 rows of f; the single
+  // form's tiles are twice as wide).  How many experts a batch touches is known on the device alone: from 2048 columns on the guard
+  // takes what an even routing would touch and stays clear of 1.125 to 2.25 waves of that, which are 1.0 to 1.4 waves of a skewed
+  // one; a single token's experts are certain, and a wave is the line.  us per layer, waves of pass 1: 24 experts, d = 6144, f =
+  // 1216, T = 1 (1.03) 83.4 -> 90.9; 60, d = 4608, f = 960, T = 21 (1.01) 69.4 -> 74.1; 128, d = 4992, f = 320, T = 10 (1.28) 80.8
+  // -> 87.6; 64, d = 3840, f = 384, T = 9 (1.22) 65.0 -> 69.4; 64, d = 3584, f = 640, T = 5 (1.08) 60.6 -> 63.9; 128, d = 2048, f =
+  // 192, T = 30 (1.38) 47.3 -> 51.2; 96, d = 2176, f = 192, T = 50 (1.07) 45.0 -> 48.2; below one wave and above 1.5 it gains 5 to
+  // 24 % (32, d = 4224, f = 320, T = 34, 0.54 waves, 1.04 if even, 53.7 -> 42.2; 96, d = 4864, f = 1920, T = 2, 1.62 waves 6 %).
+  // Shorter units lose less: 16, d = 1408, f = 576, T = 174 (1.3 waves if every expert is touched) 30.1 -> 31.7.  Units of 128 rows
+  // need more waves: 4.4 waves 64, d = 2944, f = 576, T = 178 104 -> 112, 4.7 waves 128, d = 4992, f = 256, T = 745 224 -> 238, 5.0
+  // waves 128, d = 5888, f = 320, T = 330 1.03 times faster.
+  if (n < 128 && g.d >= 2048) {
+    const double even = E * (1.0 - pow(1.0 - (double)g.K / E, g.T));
+    const double units = g.f / 64 * (even > (double)S / n ? even : (double)S / n);
+    if (weight >= FEPLB_FEW_GUARD_WEIGHT && units > (g.T == 1 ? 1.0 : 1.125) * num_sms && units < 2.25 * num_sms) return 0;
+  } else if (weight >= FEPLB_WM_MIN_WEIGHT) {
     const int64_t units = g.f / 64 * (touched + S / n);
     if (5 * units > 6 * num_sms && units < (n == 128 ? 5 : 2) * num_sms) return 0;
   }
+  // Narrow layers: a unit of pass 1 is its fixed costs, and busy experts have many: 128 experts, d = 128, f = 1152, T = 1679, top-1
+  // 35.3 -> 39.4; 96, d = 256, f = 384, T = 344, top-5 29.2 -> 30.8; 128, d = 128, f = 768, 10.5 rows per expert 35.7 -> 36.7; but 64, d =
+  // 128, f = 768, 9.98 rows 27.0 -> 25.4.
+  if (g.d <= 256 && S >= 10 * E && g.f / 64 * touched >= 3 * num_sms) return 0;
   return n;
 }
 

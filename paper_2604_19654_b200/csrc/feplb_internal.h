@@ -30,6 +30,7 @@
 #define FEPLB_SHORT_TILE_MIN_ROWS 288           // ... from this many rows per expert
 #define FEPLB_PAIR_MIN_ROWS_PER_EXPERT 256     // launches over static and dynamic groups, or all: two-CTA tiles from here
 #define FEPLB_FEW_LARGE_WEIGHT (1 << 20)       // weight matrices of at least so many elements: the form for few rows per expert up to ...
+#define FEPLB_FEW_GUARD_WEIGHT (3 << 17)        // its guard against a nearly empty wave of long units, from so many elements
 #define FEPLB_WM_MIN_ROWS_PER_EXPERT 64        // ... this many; from here (up to the line above) the weights-on-M form ...
 #define FEPLB_WM_MIN_WEIGHT (1 << 19)          // ... for weight matrices of at least so many elements
 #define FEPLB_WM_ANY_UNITS_WEIGHT (3 << 20)     // ... and enough units; from this many elements whatever their number

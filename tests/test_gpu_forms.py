@@ -113,6 +113,28 @@ def test_several_units_per_cta_for_few_rows(d, f, rows, units):
     assert _run(rows, d, f, None, preact=True, detail=units) & F.PATH_SINGLE
 
 
+@pytest.mark.parametrize("T,K,E,d,f,units", [
+    (1, 8, 24, 6144, 1216, 0),                     # 152 units of long weights: a wave and four
+    (1, 7, 24, 6144, 1216, F.DETAIL_UNITS_32),     # 133
+    (5, 8, 64, 3584, 640, 0),                      # 31 experts of 10 blocks
+    (10, 8, 64, 3584, 640, F.DETAIL_UNITS_32),     # 47
+    (34, 3, 32, 4224, 320, F.DETAIL_UNITS_32),     # 31 of 5: 1.04 waves if the routing is even
+    (30, 8, 128, 2048, 192, 0),
+    (30, 8, 128, 1920, 192, F.DETAIL_UNITS_32),    # shorter units
+    (96, 2, 96, 2048, 192, 0),                     # units of 64 rows
+    (1280, 1, 128, 128, 768, 0),                   # 10 rows per expert of a narrow layer
+    (1279, 1, 128, 128, 768, F.DETAIL_UNITS_64),
+    (240, 1, 24, 128, 768, F.DETAIL_UNITS_64),     # two waves
+])
+def test_rule_of_few_rows_per_expert(T, K, E, d, f, units):
+    """Single-CTA tiles of token rows where a second wave of units would be nearly empty, or a unit is its fixed costs."""
+    ctx, buf, args, w = _zeros(T, K, E, d, f)
+    ctx.moe_forward(*args, *w, buf)
+    assert ctx.forward_detail() == units and ctx.forward_path() & F.PATH_SINGLE
+    ctx.check_status()
+    ctx.close()
+
+
 @pytest.mark.parametrize("T,K,E,d,f,detail", [
     (32, 4, 32, 2048, 1024, F.DETAIL_UNITS_32),
     (16, 4, 16, 128, 64, F.DETAIL_UNITS_32),
