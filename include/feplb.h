@@ -466,6 +466,7 @@ int feplb_selftest_bounded_wait(feplb_ctx* ctx, int32_t limit_us, void* stream);
 int32_t feplb_forward_path(const feplb_ctx* ctx);
 /* Which variants of those forms ran, FEPLB_DETAIL_* bits (0 before the first forward).  Units: with few rows per expert
  * FEPLB_PATH_SINGLE stands for tiles of 128 weight rows by at most so many token rows. */
+#define FEPLB_DETAIL_DEEP_STAGES 1   /* two-CTA tiles: 128 elements of K per stage, 128-row tiles for the ends of segments */
 #define FEPLB_DETAIL_UNITS_32 32
 #define FEPLB_DETAIL_UNITS_64 64
 #define FEPLB_DETAIL_UNITS_128 128

@@ -4,6 +4,7 @@
 #include <cuda_runtime.h>
 
 #include <atomic>
+#include <algorithm>
 #include <chrono>
 #include <climits>
 #include <cmath>
@@ -52,6 +53,7 @@ struct feplb_ctx {
   bool wm_auto = false;
   bool wm_merged = false, wm_merged_auto = false;   // the same for launches over static and dynamic groups together
   bool wm_static = false, wm_static_auto = false;   // the static launches of the four-launch order use it
+  bool pair_deep = false;      // the two-CTA form runs with stages of 128 elements and 128-row last tiles
   bool merged_ok = false;      // both group tables of a forward fit one launch (static, then dynamic groups)
   bool merged = false;         // ... and feplb_moe_forward runs that way: two GEMM launches instead of four
   bool merged_auto = false;
@@ -431,6 +433,23 @@ extern "C" int feplb_create(const feplb_config* cfg, feplb_ctx** out) {
   const int64_t weight = (int64_t)cfg->d * cfg->f;
   const bool short_tiles = (weight < FEPLB_SHORT_TILE_WEIGHT / 2 || (weight < FEPLB_SHORT_TILE_WEIGHT && cfg->f <= 384)) && (int64_t)cfg->T * cfg->K >= (int64_t)FEPLB_SHORT_TILE_MIN_ROWS * cfg->E;
   c->merged_pair = (int64_t)cfg->T * cfg->K >= (int64_t)FEPLB_PAIR_MIN_ROWS_PER_EXPERT * cfg->E && !short_tiles;
+  // Deep stages of that form (128 elements of K, and tiles of 128 rows): the epilogue that serves both tile heights costs
+  // every tile a little, a stage of 128 elements is half empty where the width is an odd number of 64, and a ring of three is
+  // less in flight while weights stream.  us per layer at the power cap, 64-element stages / deep ones:
+  //   large: 128 experts, d = 6144, f = 2048, 1024 rows per expert 9735 / 9395, 4096 rows 36897 / 35963; 32, d = 4096, f = 1024,
+  //     4096 rows 3091 / 3035; 16, d = 6144, f = 768, 3000 rows 1404 / 1375; d = 1536, f = 1408, 300 rows 107.8 / 103.3
+  //   many groups, i.e. many last tiles: 128, d = 2560, f = 320, 264 rows 406 / 389; 96, d = 384, f = 1024, 313 rows 158 / 151
+  //   short second pass: 48, d = 3584, f = 192, 8300 rows 3187 / 3435; 24, d = 3072, f = 192, 15000 rows 2502 / 2676; 16, d = 2560,
+  //     f = 256, 1294 rows 199.5 / 205.0; 16, d = 4736, f = 256, 269 rows 85.5 / 87.9; short first pass: 96, d = 128, f = 512, 286
+  //     rows 58.3 / 61.7
+  //   less than two waves of tiles: 16, d = 1536, f = 640, 290 rows 55.2 / 57.9; 16, d = 3328, f = 320, 306 rows 89.4 / 90.5; 16, d =
+  //     512, f = 640, 441 rows 41.9 / 42.9; 16, d = 1664, f = 448, 304 rows 59.2 / 61.5
+  {
+    const int64_t m_tiles = (int64_t)cfg->T * cfg->K / 256 + cfg->E / 2, clusters = c->num_sms / 2;
+    const int64_t blocks = std::min((cfg->f + 127) / 128, (cfg->d + 255) / 256);     // N tiles of the narrower pass
+    c->pair_deep = cfg->f > 256 && cfg->d >= 256 &&
+                   (weight >= FEPLB_PAIR_DEEP_WEIGHT || cfg->E >= FEPLB_PAIR_DEEP_EXPERTS || m_tiles * blocks >= 2 * clusters);
+  }
   // backward GEMMs: the pair form pays once an expert's segment spans several 256-row tiles
   // (measured: -7.5 % backward time at 1024 rows per expert, slower at 384)
   c->bwd_pair_auto = c->bwd_pair = (int64_t)cfg->T * cfg->K >= (int64_t)512 * cfg->E ? 3 : 0;
@@ -714,7 +733,7 @@ static int ffn_impl(feplb_ctx* c, const void* x_perm, const void* w1, const void
   a.x_perm = x_perm; a.w1 = w1; a.w3 = w3; a.w2 = w2; a.h = h; a.y = y;
   a.groups = groups; a.n_groups = n_groups; a.which = which;
   a.E = c->cfg.E; a.d = c->cfg.d; a.f = c->cfg.f; a.s_cap = (int64_t)c->s_cap;
-  a.status = c->d_status; a.num_sms = c->num_sms; a.pair = pair;
+  a.status = c->d_status; a.num_sms = c->num_sms; a.pair = pair; a.deep = c->pair_deep;
   a.ab_out = c->d_preact;
   a.recv_w1 = c->d_recv_w1; a.recv_w3 = c->d_recv_w3; a.recv_w2 = c->d_recv_w2; a.n_recv_slots = c->n_recv_slots;
   a.recv_x = c->d_recv_x;
@@ -735,6 +754,7 @@ static int ffn_impl(feplb_ctx* c, const void* x_perm, const void* w1, const void
     }
   }
   c->path |= pair ? FEPLB_PATH_PAIR : FEPLB_PATH_SINGLE;
+  if (pair && a.deep) c->detail |= FEPLB_DETAIL_DEEP_STAGES;
   return feplb_launch_expert_ffn(a, st, &c->launches, c->err, sizeof(c->err), dyn);
 }
 

@@ -44,25 +44,25 @@ constexpr int kBBytesMax = 256 * kChunk * 2;       // 32 KiB
 //   pair (PAIR = true): a cluster of two CTAs computes a 256 x 256 tile with cta_group::2 MMAs
 //     issued by the even CTA: each CTA stages its own 128 rows of A and HALF of the B tile (the
 //     W1 tile in the even CTA and the W3 tile in the odd one in pass 1), so a CTA needs only
-//     64 bytes per MMA cycle from L2.  K step 128, two 64-element chunks in one TMA instruction per operand (3-d
-//     maps), 3 stages of 64 KiB: a stage costs the producer and the issuer a fixed few hundred cycles, whatever
-//     it holds.  Against 6 stages of 32 KiB, us per layer: 64 experts, d = 2048, T = 4096 333.5 -> 330.0; 32 experts, d =
-//     4096, f = 1024, T = 4096 505 -> 494; 128 experts, d = 6144, T = 8192 5512 -> 5382.
-//     No load is shared between the CTAs: each brings its own halves.  Used for launches whose groups are large;
-//     the last tile of a group shrinks to 128 rows, 64 per CTA, where no more are valid.
+//     64 bytes per MMA cycle from L2.  No load is shared between the CTAs: each brings its own halves.  Used for
+//     launches whose groups are large.  K step 64, 6 stages of 32 KiB, or with deep stages (DEEP) K step 128, two 64-element
+//     chunks in one TMA instruction per operand (3-d maps), 3 stages of 64 KiB: a stage costs the producer and the
+//     issuer a fixed few hundred cycles, whatever it holds.  The last tile of a group then shrinks to 128 rows, 64 per
+//     CTA, where no more are valid.  Which of the two: pair_deep in feplb_create.
 // Both keep two accumulators in TMEM so that the epilogue of tile i overlaps the MMAs of tile i+1.
-template <bool PAIR> struct Ring {
-  static constexpr int kChunks = PAIR ? 2 : 1;
+template <bool PAIR, bool DEEP> struct Ring {
+  static constexpr int kChunks = DEEP ? 2 : 1;
   static constexpr int BK = kChunks * kChunk;                                          // K elements per stage
-  static constexpr int kStages = PAIR ? 3 : 4;
+  static constexpr int kStages = DEEP ? 3 : PAIR ? 6 : 4;
   static constexpr int kStageBytes = kChunks * (kABytes + (PAIR ? kBBytesMax / 2 : kBBytesMax));   // multiple of 1024
   static constexpr int kTileRows = PAIR ? 2 * BM : BM;
 };
-constexpr int kMaxStages = 4;
+constexpr int kMaxStages = 6;
 constexpr int kAccStages = 2;
 constexpr int kRingBytes = 4 * (kABytes + kBBytesMax);   // 192 KiB in both forms
-static_assert(Ring<false>::kStages * Ring<false>::kStageBytes == kRingBytes &&
-              Ring<true>::kStages * Ring<true>::kStageBytes == kRingBytes, "ring size");
+static_assert(Ring<false, false>::kStages * Ring<false, false>::kStageBytes == kRingBytes &&
+              Ring<true, false>::kStages * Ring<true, false>::kStageBytes == kRingBytes &&
+              Ring<true, true>::kStages * Ring<true, true>::kStageBytes == kRingBytes, "ring size");
 constexpr int kEpiWarps = 4;
 constexpr int kThreads = 64 + 32 * kEpiWarps;
 constexpr int kEpiStageBytes = 32 * 128;            // per epilogue warp: 32 rows x 64 bf16
@@ -73,7 +73,7 @@ struct SmemTail {
   unsigned long long tmem_full[kAccStages];
   unsigned long long tmem_empty[kAccStages];
   unsigned long long dyn_bar;         // completed by warp 0 once the dynamic entries are in place
-  uint32_t idesc[kMaxStages];         // instruction descriptor of the tile whose first K block is in the stage (leader)
+  uint32_t idesc[kMaxStages];         // deep stages: instruction descriptor of the tile whose first K block is in the stage (leader)
   uint32_t tmem_base;
   int abort_flag;
   int n_entries;                      // entries in use (the table known at launch, then the planner's dynamic groups)
@@ -96,13 +96,13 @@ struct GemmParams {
   int64_t s_cap;        // rows of the A and output buffers
   int n_tiles_n;        // N tiles per M tile
   int half_width;       // rows of B over all half tiles of one M tile: f (pass 1), d / 2 (pass 2); a multiple of 64
-  int b_box;            // single form: rows of one box of the B tensor maps (64 or 128), which divides every half tile; in the
-                        // pair form a box has bn rows, and a narrow last tile leaves some of them unused
+  int b_box;            // rows of one box of the B tensor maps (64 or 128), which divides every half tile; with deep stages a
+                        // box has bn rows, and a narrow last tile leaves some of them unused
   int early_weights;    // the group table was complete before this kernel's predecessor let it start: B loads of the
                         // first tile may be issued before griddepcontrol.wait
-  int num_k_blocks;     // K / 64, pair form K / 128 rounded up (the chunk past the end reads as zeros and is not multiplied)
+  int num_k_blocks;     // K / 64, with deep stages K / 128 rounded up (the chunk past the end reads as zeros and is not multiplied)
   int num_chunks;       // K / 64
-  int halves;           // pair form: tiles of at most 128 valid rows take the 128-row MMA (in pass 1 it needs tm_h ...
+  int halves;           // deep stages: tiles of at most 128 valid rows take the 128-row MMA (in pass 1 it needs w13 ...
   int b_first;          // ... which begins at W3 where that lies in front of W1)
   int b_rows_per_expert;  // rows of one expert in the B tensor maps
   int n_recv_slots;     // slots of the receive buffer of migrated experts' weights (0 = none)
@@ -116,6 +116,11 @@ struct GemmParams {
                                 // ran out of static tiles, [2] ~(last CTA's end), [3] ~(longest wait for the dynamic table)
 };
 
+
+// Tensor maps of one pass: rows (whole boxes, fewer rows, receive region), the two halves of B, the same of the receive
+// buffer, the output in boxes of 32 rows x 64 columns.
+template <bool DEEP> struct Maps { CUtensorMap a, as, ra, b0, b1, r0, r1, out; };
+template <> struct Maps<true> : Maps<false> { CUtensorMap w13; };     // pass 1: W1 and W3 together, for tiles of 128 rows
 
 struct TileCoord { int row0, rows_valid, expert, slot, n0, bn; };   // slot >= 0: weights in that receive slot;
                                                                    // n0 = first column of the half tile, bn its rows
@@ -141,13 +146,13 @@ __device__ __forceinline__ TileCoord tile_coord(const SmemTail* t, int n_groups,
   return c;
 }
 
-// Pair form: a tile of at most 128 valid rows is a 128 x 256 MMA over the two CTAs, 64 rows of A each.  In pass 1 both
+// Pair form, deep stages: a tile of at most 128 valid rows is a 128 x 256 MMA over the two CTAs, 64 rows of A each.  In pass 1 both
 // halves of B then hold W1 and W3 rows of the same 64 hidden units (see the producer), which takes a full-width tile.
 // Half the MMA time and half the A rows against a 256-row tile whose second half is empty: 64 experts, d = 2048, T =
 // 4096 (a third of the tiles) 345.9 -> 340.2 us per layer, three hot experts 355.9 -> 345.0.
-template <bool SWIGLU, bool PAIR>
+template <bool SWIGLU, bool DEEP>
 __device__ __forceinline__ bool is_half(const TileCoord& c, const GemmParams& p) {
-  return PAIR && c.rows_valid <= BM && c.slot < 0 && p.halves && (!SWIGLU || c.bn == 128);
+  return DEEP && c.rows_valid <= BM && c.slot < 0 && p.halves && (!SWIGLU || c.bn == 128);
 }
 
 // fp32 accumulator registers of 32 columns -> 16 packed bf16 pairs (SwiGLU: silu(a) * b first).
@@ -261,16 +266,12 @@ __device__ __forceinline__ void warp_scan_prefix(SmemTail* t, int first, int n, 
 // width that differs per tile costs the roles more than it saves where it does not: both passes of a large batch in the
 // single form, 64 experts, d = 2048, f = 768, 1536 / 3750 rows per expert on average: 950 / 2187 us with one kernel
 // for all widths, 920 / 2118 this way; the pair form 864 / 1967 and 851 / 1938.
-template <bool SWIGLU, bool PAIR, bool NARROW>
+template <bool SWIGLU, bool PAIR, bool NARROW, bool DEEP>
 __global__ void __launch_bounds__(kThreads, 1)
-k_grouped_gemm(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__ CUtensorMap tm_as,
-               const __grid_constant__ CUtensorMap tm_ra,
-               const __grid_constant__ CUtensorMap tm_b0,
-               const __grid_constant__ CUtensorMap tm_b1, const __grid_constant__ CUtensorMap tm_r0,
-               const __grid_constant__ CUtensorMap tm_r1, const __grid_constant__ CUtensorMap tm_h,
-               const __grid_constant__ CUtensorMap tm_out, const GemmParams p) {
-  constexpr int kStages = Ring<PAIR>::kStages, kStageBytes = Ring<PAIR>::kStageBytes;
-  constexpr int kTileRows = Ring<PAIR>::kTileRows, kChunks = Ring<PAIR>::kChunks, BK = Ring<PAIR>::BK;
+k_grouped_gemm(const __grid_constant__ Maps<DEEP> tm, const GemmParams p) {
+  static_assert(PAIR || !DEEP, "deep stages: pair form only");
+  using F = Ring<PAIR, DEEP>;
+  constexpr int kStages = F::kStages, kStageBytes = F::kStageBytes, kTileRows = F::kTileRows, kChunks = F::kChunks, BK = F::BK;
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
   uint8_t* epi_smem = smem + (size_t)kRingBytes;
@@ -285,15 +286,15 @@ k_grouped_gemm(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__
 
   // ---- set-up: barriers, TMEM, group table ------------------------------------------------
   if (threadIdx.x == 0) {
-    prefetch_tmap(&tm_a);
-    prefetch_tmap(&tm_as);
-    prefetch_tmap(&tm_ra);
-    prefetch_tmap(&tm_b0);
-    prefetch_tmap(&tm_b1);
-    prefetch_tmap(&tm_r0);
-    prefetch_tmap(&tm_r1);
-    prefetch_tmap(&tm_h);
-    prefetch_tmap(&tm_out);
+    prefetch_tmap(&tm.a);
+    prefetch_tmap(&tm.as);
+    prefetch_tmap(&tm.ra);
+    prefetch_tmap(&tm.b0);
+    prefetch_tmap(&tm.b1);
+    prefetch_tmap(&tm.r0);
+    prefetch_tmap(&tm.r1);
+    prefetch_tmap(&tm.out);
+    if constexpr (DEEP) prefetch_tmap(&tm.w13);
     for (int s = 0; s < kStages; ++s) {
       mbar_init(smem_u32(&tail->full[s]), 1);
       mbar_init(smem_u32(&tail->empty[s]), 1);
@@ -402,14 +403,14 @@ k_grouped_gemm(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__
       const bool few = !PAIR && c.slot < 0 && c.rows_valid <= kFewRows;
       // weights of a migrated expert come from its slot of the receive buffer, and in pass 1 its rows from the
       // receive region (same row numbers as the permuted buffer)
-      q.a = c.slot >= 0 ? &tm_ra : few ? &tm_as : &tm_a;
-      q.b0 = c.slot >= 0 ? &tm_r0 : &tm_b0;
-      q.b1 = c.slot >= 0 ? &tm_r1 : &tm_b1;
+      q.a = c.slot >= 0 ? &tm.ra : few ? &tm.as : &tm.a;
+      q.b0 = c.slot >= 0 ? &tm.r0 : &tm.b0;
+      q.b1 = c.slot >= 0 ? &tm.r1 : &tm.b1;
       q.arow = c.row0;
       q.brow0 = (c.slot >= 0 ? c.slot : c.expert) * p.b_rows_per_expert + (SWIGLU ? c.n0 : 2 * c.n0);
       q.brow1 = SWIGLU ? q.brow0 : q.brow0 + c.bn;
-      q.half = (uint32_t)(PAIR ? p.bn : c.bn) * BK * 2;
-      q.two = !PAIR && NARROW && c.bn > p.b_box;    // 128 rows in boxes of 64
+      q.half = (uint32_t)(DEEP ? p.bn : c.bn) * BK * 2;
+      q.two = !DEEP && NARROW && c.bn > p.b_box;    // 128 rows in boxes of 64
       q.tx = (PAIR ? 2 * kChunks * kABytes : few ? kFewRows * kChunk * 2 : kABytes) + 2 * q.half;
       if (PAIR && cta_rank) {
         q.arow = c.rows_valid > BM ? c.row0 + BM : (int)p.s_cap;
@@ -418,9 +419,9 @@ k_grouped_gemm(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__
       }
       q.idesc = make_idesc(kTileRows, 2 * c.bn);
       q.split = false;
-      if (is_half<SWIGLU, PAIR>(c, p)) {
+      if (is_half<SWIGLU, DEEP>(c, p)) {
         // 64 rows of A per CTA (zeros where none of them is valid); pass 1: 64 rows of W1 and the same 64 of W3
-        q.a = &tm_as;
+        q.a = &tm.as;
         q.arow = !cta_rank ? c.row0 : c.rows_valid > BM / 2 ? c.row0 + BM / 2 : (int)p.s_cap;
         q.tx = kChunks * kABytes + 2 * q.half;
         q.idesc = make_idesc(BM, 2 * c.bn);
@@ -431,19 +432,23 @@ k_grouped_gemm(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__
     };
     auto announce = [&](const Source& q, int st) {      // the bytes of a stage, and what the issuer does with them
       if (PAIR && cta_rank) return;
-      if (PAIR) tail->idesc[st] = q.idesc;
+      if (DEEP) tail->idesc[st] = q.idesc;
       mbar_expect_tx(smem_u32(&tail->full[st]), q.tx);
     };
     auto load_b = [&](const Source& q, int kb, uint32_t full, uint32_t sb) {
       constexpr uint32_t kBox = 64 * BK * 2;
-      if (PAIR) {
+      if constexpr (DEEP) {
         const uint32_t full0 = map_to_cta(full, 0);
         if (SWIGLU && q.split)      // 64 rows of W1 and of W3, chunk after chunk
           asm volatile(
               "cp.async.bulk.tensor.4d.cta_group::2.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4, %3, %5}], [%2];"
-              ::"r"(sb), "l"(reinterpret_cast<uint64_t>(&tm_h)), "r"(full0), "r"(0), "r"(q.brow0), "r"(kb * kChunks) : "memory");
+              ::"r"(sb), "l"(reinterpret_cast<uint64_t>(&tm.w13)), "r"(full0), "r"(0), "r"(q.brow0), "r"(kb * kChunks) : "memory");
         else
           tma_load_3d_pair(sb, q.b0, full0, 0, q.brow0, kb * kChunks);
+      } else if (PAIR) {
+        const uint32_t full0 = map_to_cta(full, 0);
+        tma_load_2d_pair(sb, q.b0, full0, kb * BK, q.brow0);
+        if (q.two) tma_load_2d_pair(sb + kBox, q.b0, full0, kb * BK, q.brow0 + 64);
       } else {
         tma_load_2d(sb, q.b0, full, kb * BK, q.brow0);
         tma_load_2d(sb + q.half, q.b1, full, kb * BK, q.brow1);
@@ -454,7 +459,8 @@ k_grouped_gemm(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__
       }
     };
     auto load_a = [&](const Source& q, int kb, uint32_t full, uint32_t sa) {
-      if (PAIR) tma_load_3d_pair(sa, q.a, map_to_cta(full, 0), 0, q.arow, kb * kChunks);
+      if (DEEP) tma_load_3d_pair(sa, q.a, map_to_cta(full, 0), 0, q.arow, kb * kChunks);
+      else if (PAIR) tma_load_2d_pair(sa, q.a, map_to_cta(full, 0), kb * BK, q.arow);
       else tma_load_2d(sa, q.a, full, kb * BK, q.arow);
     };
     // Weights of the first tile, as far as the ring holds them, before the wait for the rows.
@@ -546,14 +552,14 @@ k_grouped_gemm(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__
           total = tail->total_mtiles * p.n_tiles_n;
           if (tile >= total) break;
         }
-        if (!PAIR && NARROW) idesc = make_idesc(kTileRows, 2 * min(p.bn, p.half_width - tile % p.n_tiles_n * p.bn));
+        if (!DEEP && NARROW) idesc = make_idesc(kTileRows, 2 * min(p.bn, p.half_width - tile % p.n_tiles_n * p.bn));
         if (!(ok = mbar_wait(smem_u32(&tail->tmem_empty[as]), aphase ^ 1u, abort_flag, p.status))) break;
         tc_fence_after();
         const uint32_t d_tmem = tmem_base + (uint32_t)(as * kAccCols);
         for (int kb = 0; kb < p.num_k_blocks; ++kb) {
           if (!(ok = mbar_wait(smem_u32(&tail->full[stage]), phase, abort_flag, p.status))) break;
           tc_fence_after();
-          if (PAIR && kb == 0) {
+          if (DEEP && kb == 0) {
             idesc = *reinterpret_cast<volatile uint32_t*>(&tail->idesc[stage]);
             a_chunk = idesc >> 24 == BM >> 4 ? kABytes / 2 >> 4 : kABytes >> 4;
           }
@@ -606,7 +612,7 @@ k_grouped_gemm(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__
       const TileCoord c = tile_coord<kTileRows, NARROW>(tail, n_entries, p, tile);
       // In a tile of 128 rows over two CTAs TMEM lanes 0-63 hold the CTA's 64 rows for the columns of the even CTA's half
       // of B, lanes 64-127 the same rows for those of the odd CTA's.
-      const bool half = is_half<SWIGLU, PAIR>(c, p);
+      const bool half = is_half<SWIGLU, DEEP>(c, p);
       // pass 1: TMEM columns of a and of b
       const uint32_t a_off = SWIGLU && half && p.b_first ? 64 : 0, b_off = half ? 64 - a_off : (uint32_t)c.bn;
       const int out_cols = half ? (SWIGLU ? 64 : c.bn) : SWIGLU ? c.bn : 2 * c.bn;
@@ -659,7 +665,7 @@ k_grouped_gemm(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__
               tmem_ld32(taddr + b_off + (uint32_t)(col + 96), b1);
             }
           }
-          if (rows_here >= 32) stage_and_tma_store(stg, packed, &tm_out, col0 + col, c.row0 + row_off, lane);
+          if (rows_here >= 32) stage_and_tma_store(stg, packed, &tm.out, col0 + col, c.row0 + row_off, lane);
           else stage_and_store(stg, packed, obase, p.ld_out, col, rows_here, lane);
         }
       }
@@ -732,7 +738,7 @@ bool make_tmap(CUtensorMap* m, const void* base, uint64_t rows, uint64_t inner, 
   const cuuint32_t box[2] = {(cuuint32_t)kChunk, box_rows};
   return encode(m, 2, base, dims, strides, box);
 }
-// The same with boxes of two 64-element chunks, chunk after chunk (pair form).
+// The same with boxes of two 64-element chunks, chunk after chunk (deep stages).
 bool make_tmap_chunks(CUtensorMap* m, const void* base, uint64_t rows, uint64_t inner, uint32_t box_rows) {
   const cuuint64_t dims[3] = {(cuuint64_t)kChunk, rows, inner / kChunk}, strides[2] = {inner * 2, kChunk * 2};
   const cuuint32_t box[3] = {(cuuint32_t)kChunk, box_rows, 2};
@@ -749,14 +755,14 @@ bool make_tmap_w13(CUtensorMap* m, const void* w1, const void* w3, uint64_t rows
   return encode(m, 4, lo, dims, strides, box);
 }
 
-template <bool SWIGLU, bool PAIR, bool NARROW>
-cudaError_t launch_form(const CUtensorMap& ta, const CUtensorMap& tas, const CUtensorMap& tra, const CUtensorMap& tb0, const CUtensorMap& tb1, const CUtensorMap& tr0,
-                       const CUtensorMap& tr1, const CUtensorMap& th, const CUtensorMap& tout, const GemmParams& p, int num_sms, cudaStream_t st) {
+template <bool SWIGLU, bool PAIR, bool NARROW, bool DEEP>
+cudaError_t launch_form(const Maps<DEEP>& m, const GemmParams& p, int num_sms, cudaStream_t st) {
   // per instantiation and device: the shared-memory attribute and the resident grid are set on first use
   static int grid_of[64] = {};
   int dev = 0;
   if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
   int& grid = grid_of[dev];
+  const auto kernel = k_grouped_gemm<SWIGLU, PAIR, NARROW, DEEP>;
   cudaLaunchConfig_t cfg = {};
   cfg.blockDim = dim3(kThreads);
   cfg.dynamicSmemBytes = kSmemBytes;
@@ -774,15 +780,14 @@ cudaError_t launch_form(const CUtensorMap& ta, const CUtensorMap& tas, const CUt
     cfg.numAttrs = 2;
   }
   if (!grid) {
-    cudaError_t e = cudaFuncSetAttribute(k_grouped_gemm<SWIGLU, PAIR, NARROW>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)kSmemBytes);
+    cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemBytes);
     if (e != cudaSuccess) return e;
     int g = num_sms;
     if (PAIR) {
       // as many clusters of two as can be resident at once (one CTA per SM, both SMs in one GPC)
       int n_clusters = 0;
       cfg.gridDim = dim3(num_sms / 2 * 2);
-      e = cudaOccupancyMaxActiveClusters(&n_clusters, k_grouped_gemm<SWIGLU, PAIR, NARROW>, &cfg);
+      e = cudaOccupancyMaxActiveClusters(&n_clusters, kernel, &cfg);
       if (e != cudaSuccess) return e;
       if (n_clusters < 1) return cudaErrorLaunchOutOfResources;
       g = 2 * (n_clusters < num_sms / 2 ? n_clusters : num_sms / 2);
@@ -790,14 +795,15 @@ cudaError_t launch_form(const CUtensorMap& ta, const CUtensorMap& tas, const CUt
     grid = g;
   }
   cfg.gridDim = dim3(grid);
-  return cudaLaunchKernelEx(&cfg, k_grouped_gemm<SWIGLU, PAIR, NARROW>, ta, tas, tra, tb0, tb1, tr0, tr1, th, tout, p);
+  return cudaLaunchKernelEx(&cfg, kernel, m, p);
 }
 
-template <bool SWIGLU, bool PAIR>
-cudaError_t launch_one(const CUtensorMap& ta, const CUtensorMap& tas, const CUtensorMap& tra, const CUtensorMap& tb0, const CUtensorMap& tb1, const CUtensorMap& tr0,
-                       const CUtensorMap& tr1, const CUtensorMap& th, const CUtensorMap& tout, const GemmParams& p, int num_sms, cudaStream_t st) {
-  auto form = p.half_width % p.bn ? launch_form<SWIGLU, PAIR, true> : launch_form<SWIGLU, PAIR, false>;
-  return form(ta, tas, tra, tb0, tb1, tr0, tr1, th, tout, p, num_sms, st);
+template <bool SWIGLU>
+cudaError_t launch_one(const Maps<true>& m, const GemmParams& p, bool pair, bool deep, int num_sms, cudaStream_t st) {
+  const bool narrow = p.half_width % p.bn != 0;
+  if (!pair) return (narrow ? launch_form<SWIGLU, false, true, false> : launch_form<SWIGLU, false, false, false>)(m, p, num_sms, st);
+  if (!deep) return (narrow ? launch_form<SWIGLU, true, true, false> : launch_form<SWIGLU, true, false, false>)(m, p, num_sms, st);
+  return (narrow ? launch_form<SWIGLU, true, true, true> : launch_form<SWIGLU, true, false, true>)(m, p, num_sms, st);
 }
 
 }  // namespace
@@ -816,47 +822,39 @@ int feplb_launch_expert_ffn(const feplb_gemm_args& a, cudaStream_t st, int64_t* 
   // top-4: 171.2 -> 150.9 us together with the early weight loads of pass 2.
   const int hw1 = a.f, hw2 = a.d / 2;
   const int bn1 = hw1 < 128 ? 64 : 128, bn2 = hw2 < 128 ? 64 : 128;
-  const int bb1 = a.pair ? bn1 : hw1 % 128 ? 64 : 128, bb2 = a.pair ? bn2 : hw2 % 128 ? 64 : 128;
-  CUtensorMap tm_x, tm_xs, tm_hs, tm_w1, tm_w3, tm_h, tm_w2, tm_ho, tm_yo;     // tm_ho, tm_yo: outputs in boxes of 32 rows x 64 columns
-  const auto map = a.pair ? make_tmap_chunks : make_tmap;
+  const bool deep = a.pair && a.deep;
+  const int bb1 = deep ? bn1 : hw1 % 128 ? 64 : 128, bb2 = deep ? bn2 : hw2 % 128 ? 64 : 128;
+  const auto map = deep ? make_tmap_chunks : make_tmap;
   const int few = a.pair ? BM / 2 : kFewRows;            // rows of the smaller boxes of A
-  if (!map(&tm_x, a.x_perm, (uint64_t)a.s_cap, (uint64_t)a.d, BM) ||
-      !map(&tm_xs, a.x_perm, (uint64_t)a.s_cap, (uint64_t)a.d, few) ||
-      !map(&tm_hs, a.h, (uint64_t)a.s_cap, (uint64_t)a.f, few) ||
-      !map(&tm_w1, a.w1, (uint64_t)a.E * a.f, (uint64_t)a.d, bb1) ||
-      !map(&tm_w3, a.w3, (uint64_t)a.E * a.f, (uint64_t)a.d, bb1) ||
-      !map(&tm_h, a.h, (uint64_t)a.s_cap, (uint64_t)a.f, BM) ||
-      !map(&tm_w2, a.w2, (uint64_t)a.E * a.d, (uint64_t)a.f, bb2) ||
-      !make_tmap(&tm_ho, a.h, (uint64_t)a.s_cap, (uint64_t)a.f, 32) ||
-      !make_tmap(&tm_yo, a.y, (uint64_t)a.s_cap, (uint64_t)a.d, 32)) {
+  const uint64_t rows = (uint64_t)a.s_cap, w1_rows = (uint64_t)a.E * a.f, w2_rows = (uint64_t)a.E * a.d, d = (uint64_t)a.d, f = (uint64_t)a.f;
+  Maps<true> m1, m2;
+  if (!map(&m1.a, a.x_perm, rows, d, BM) || !map(&m1.as, a.x_perm, rows, d, few) || !map(&m1.b0, a.w1, w1_rows, d, bb1) ||
+      !map(&m1.b1, a.w3, w1_rows, d, bb1) || !map(&m2.a, a.h, rows, f, BM) || !map(&m2.as, a.h, rows, f, few) ||
+      !map(&m2.b0, a.w2, w2_rows, f, bb2) || !make_tmap(&m1.out, a.h, rows, f, 32) || !make_tmap(&m2.out, a.y, rows, d, 32)) {
     snprintf(err, errn, "cuTensorMapEncodeTiled failed (driver entry point missing or bad pointer/shape)");
     return FEPLB_E_CUDA;
   }
-  // pass 1 of the pair form, tiles of at most 128 rows
-  CUtensorMap tm_w13 = tm_w1;
-  const bool halves = a.pair && make_tmap_w13(&tm_w13, a.w1, a.w3, (uint64_t)a.E * a.f, (uint64_t)a.d);
-  // receive buffer of migrated experts' weights, addressed by slot like the home weights by expert
-  CUtensorMap tm_r1 = tm_w1, tm_r3 = tm_w3, tm_r2 = tm_w2;
+  m2.b1 = m2.w13 = m2.b0;
+  m1.w13 = m1.b0;
+  const bool halves = deep && make_tmap_w13(&m1.w13, a.w1, a.w3, w1_rows, d);
+  // receive buffer of migrated experts' weights, addressed by slot like the home weights by expert, and the rows of
+  // migrated pieces: pass 1 reads them from the receive region when there is one
+  m1.r0 = m1.b0; m1.r1 = m1.b1; m2.r0 = m2.b0; m1.ra = m1.a; m2.ra = m2.a;
   const bool has_recv = a.recv_w1 && a.recv_w3 && a.recv_w2 && a.n_recv_slots > 0;
-  if (has_recv && (!map(&tm_r1, a.recv_w1, (uint64_t)a.n_recv_slots * a.f, (uint64_t)a.d, bb1) ||
-                   !map(&tm_r3, a.recv_w3, (uint64_t)a.n_recv_slots * a.f, (uint64_t)a.d, bb1) ||
-                   !map(&tm_r2, a.recv_w2, (uint64_t)a.n_recv_slots * a.d, (uint64_t)a.f, bb2))) {
+  const uint64_t slots = (uint64_t)a.n_recv_slots;
+  if (has_recv && (!map(&m1.r0, a.recv_w1, slots * f, d, bb1) || !map(&m1.r1, a.recv_w3, slots * f, d, bb1) ||
+                   !map(&m2.r0, a.recv_w2, slots * d, f, bb2) || (a.recv_x && !map(&m1.ra, a.recv_x, rows, d, BM)))) {
     snprintf(err, errn, "cuTensorMapEncodeTiled failed for the receive buffer");
     return FEPLB_E_CUDA;
   }
-  // rows of migrated pieces: pass 1 reads them from the receive region when there is one
-  CUtensorMap tm_rx = tm_x;
-  if (has_recv && a.recv_x && !map(&tm_rx, a.recv_x, (uint64_t)a.s_cap, (uint64_t)a.d, BM)) {
-    snprintf(err, errn, "cuTensorMapEncodeTiled failed for the receive region of the rows");
-    return FEPLB_E_CUDA;
-  }
+  m2.r1 = m2.r0;
   GemmParams p1;
   p1.n_recv_slots = has_recv ? a.n_recv_slots : 0;
   p1.groups = a.groups; p1.n_groups = a.n_groups; p1.which = a.which; p1.E = a.E; p1.s_cap = a.s_cap;
   p1.n_tiles_n = (hw1 + bn1 - 1) / bn1; p1.half_width = hw1; p1.b_box = bb1; p1.early_weights = 0;
-  const int bk = a.pair ? Ring<true>::BK : Ring<false>::BK;
+  const int chunks = deep ? 2 : 1;
   p1.halves = halves; p1.b_first = a.w3 < a.w1;
-  p1.num_k_blocks = (a.d + bk - 1) / bk; p1.num_chunks = a.d / kChunk; p1.b_rows_per_expert = a.f; p1.bn = bn1;
+  p1.num_k_blocks = (a.d / kChunk + chunks - 1) / chunks; p1.num_chunks = a.d / kChunk; p1.b_rows_per_expert = a.f; p1.bn = bn1;
   p1.out = (__nv_bfloat16*)a.h; p1.ld_out = a.f; p1.status = a.status; p1.ab_out = (__nv_bfloat16*)a.ab_out;
   const feplb_wm_dyn none;
   p1.dyn = feplb_dyn_table(dyn ? *dyn : none);
@@ -864,16 +862,14 @@ int feplb_launch_expert_ffn(const feplb_gemm_args& a, cudaStream_t st, int64_t* 
   GemmParams p2 = p1;
   p2.n_tiles_n = (hw2 + bn2 - 1) / bn2; p2.half_width = hw2; p2.b_box = bb2; p2.early_weights = 1;
   p2.halves = 1;
-  p2.num_k_blocks = (a.f + bk - 1) / bk; p2.num_chunks = a.f / kChunk; p2.b_rows_per_expert = a.d; p2.bn = bn2;
+  p2.num_k_blocks = (a.f / kChunk + chunks - 1) / chunks; p2.num_chunks = a.f / kChunk; p2.b_rows_per_expert = a.d; p2.bn = bn2;
   p2.out = (__nv_bfloat16*)a.y; p2.ld_out = a.d; p2.ab_out = nullptr;
   p2.stamps = p1.stamps ? p1.stamps + 4 : nullptr;
 
-  cudaError_t e = a.pair ? launch_one<true, true>(tm_x, tm_xs, tm_rx, tm_w1, tm_w3, tm_r1, tm_r3, tm_w13, tm_ho, p1, a.num_sms, st)
-                         : launch_one<true, false>(tm_x, tm_xs, tm_rx, tm_w1, tm_w3, tm_r1, tm_r3, tm_w13, tm_ho, p1, a.num_sms, st);
+  cudaError_t e = launch_one<true>(m1, p1, a.pair, deep, a.num_sms, st);
   ++*n_launch;
   if (e == cudaSuccess) {
-    e = a.pair ? launch_one<false, true>(tm_h, tm_hs, tm_h, tm_w2, tm_w2, tm_r2, tm_r2, tm_w2, tm_yo, p2, a.num_sms, st)
-               : launch_one<false, false>(tm_h, tm_hs, tm_h, tm_w2, tm_w2, tm_r2, tm_r2, tm_w2, tm_yo, p2, a.num_sms, st);
+    e = launch_one<false>(m2, p2, a.pair, deep, a.num_sms, st);
     ++*n_launch;
   }
   if (e != cudaSuccess) {

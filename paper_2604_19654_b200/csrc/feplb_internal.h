@@ -28,6 +28,8 @@
 #define FEPLB_WM_MAX_ROWS_PER_EXPERT 1280       // the weights-on-M form ends here in such launches
 #define FEPLB_SHORT_TILE_WEIGHT (1 << 19)       // below this many elements tiles are short, single-CTA tiles better ...
 #define FEPLB_SHORT_TILE_MIN_ROWS 288           // ... from this many rows per expert
+#define FEPLB_PAIR_DEEP_WEIGHT (2 << 20)        // two-CTA tiles with deep stages: matrices of at least so many elements,
+#define FEPLB_PAIR_DEEP_EXPERTS 25              // or so many experts, or two waves of tiles
 #define FEPLB_PAIR_MIN_ROWS_PER_EXPERT 256     // launches over static and dynamic groups, or all: two-CTA tiles from here
 #define FEPLB_FEW_LARGE_WEIGHT (1 << 20)       // weight matrices of at least so many elements: the form for few rows per expert up to ...
 #define FEPLB_FEW_GUARD_WEIGHT (3 << 17)        // its guard against a nearly empty wave of long units, from so many elements
@@ -115,6 +117,7 @@ struct feplb_gemm_args {
   int E, d, f; int64_t s_cap;
   uint32_t* status;
   int num_sms;
+  int deep;   // pair: stages of 128 elements of K, 128-row last tiles
   int pair;   // 1: clusters of two CTAs on 256-row tiles (cta_group::2); 0: one CTA per 128-row tile
   // receive buffer of migrated experts' weights ([n_recv_slots, f, d] x2 and [n_recv_slots, d, f]); may be null
   const void* recv_w1; const void* recv_w3; const void* recv_w2; int n_recv_slots;

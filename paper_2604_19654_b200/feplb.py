@@ -25,7 +25,7 @@ MASK_GIVEN, MASK_REACTIVE = 0, 1
 FFN_ALL, FFN_STATIC, FFN_DYNAMIC = 0, 1, 2
 FORM_AUTO, FORM_SINGLE, FORM_PAIR, FORM_WEIGHT_M = -1, 0, 1, 2
 PATH_SMALL_FRONT, PATH_HOME_TABLE, PATH_MERGED, PATH_RANGES, PATH_SINGLE, PATH_PAIR, PATH_WEIGHT_M = (1 << i for i in range(7))
-DETAIL_UNITS_32, DETAIL_UNITS_64, DETAIL_UNITS_128 = 32, 64, 128
+DETAIL_DEEP_STAGES, DETAIL_UNITS_32, DETAIL_UNITS_64, DETAIL_UNITS_128 = 1, 32, 64, 128
 HOST_SLOTS = 4            # staging sets of the pipelined host-buffer forward (FEPLB_HOST_SLOTS)
 
 

@@ -71,9 +71,34 @@ def _zeros(T, K, E, d, f):
 @pytest.mark.parametrize("w3_first", [False, True])
 @pytest.mark.parametrize("d,f", [(256, 128), (384, 320), (128, 64)])
 def test_pair_form_tiles_of_128_and_256_rows(d, f, w3_first):
-    """Tiles of at most 128 rows go through the 128-row MMA, 64 rows per CTA; f = 320: K blocks and N tiles half empty."""
-    path = _run([1, 32, 63, 64, 65, 96, 127, 128, 129, 255, 256, 257, 384, 385], d, f, F.FORM_PAIR, w3_first)
+    """Segments around the multiples of 64 and 128 rows in 256-row tiles; f = 320: N tiles half empty."""
+    path = _run([1, 32, 63, 64, 65, 96, 127, 128, 129, 255, 256, 257, 384, 385], d, f, F.FORM_PAIR, w3_first, detail=0)
     assert path & F.PATH_PAIR
+
+
+@pytest.mark.parametrize("w3_first", [False, True])
+@pytest.mark.parametrize("d,f,n_experts", [(384, 320, 25), (1152, 1856, 14)])
+def test_deep_stages_and_tiles_of_128_rows(d, f, n_experts, w3_first):
+    """Tiles of at most 128 rows go through the 128-row MMA, 64 rows per CTA; K blocks and N tiles half empty in either pass;
+    saved pre-activations."""
+    rows = [1, 32, 63, 64, 65, 96, 127, 128, 129, 255, 256, 257, 384, 385]
+    rows += [0] * (n_experts - len(rows))
+    assert _run(rows, d, f, F.FORM_PAIR, w3_first, preact=True, detail=F.DETAIL_DEEP_STAGES) & F.PATH_PAIR
+
+
+@pytest.mark.parametrize("T,E,d,f,deep", [
+    (1024, 16, 2048, 1024, 1), (1024, 16, 2048, 960, 0),          # 2 Mi elements
+    (1600, 25, 1024, 512, 1), (1600, 24, 1024, 512, 0),           # 25 experts
+    (6400, 25, 1024, 256, 0), (6400, 25, 128, 512, 0),            # a short pass
+    (7424, 16, 1024, 512, 1), (7168, 16, 1024, 512, 0),           # 37 row blocks of 4 tiles: two waves of 74 clusters
+])
+def test_rule_of_deep_stages(T, E, d, f, deep):
+    ctx, buf, args, w = _zeros(T, 1, E, d, f)
+    ctx.set_gemm_form(F.FORM_PAIR)
+    ctx.moe_forward(*args, *w, buf)
+    assert ctx.forward_detail() == (F.DETAIL_DEEP_STAGES if deep else 0) and ctx.forward_path() & F.PATH_PAIR
+    ctx.check_status()
+    ctx.close()
 
 
 @pytest.mark.parametrize("form", [F.FORM_PAIR, None])
