@@ -424,7 +424,9 @@ int feplb_set_planner_timeout(feplb_ctx* ctx, int32_t timeout_ms);
  * CTA per 128-row tile), FEPLB_FORM_PAIR (clusters of two CTAs on 256-row tiles) or
  * FEPLB_FORM_WEIGHT_M (weight tiles on the M side, up to 256 rows of a group on the N side; needs
  * f % 128 == 0, d % 256 == 0 and 2*E + R*max_num_dyn <= 1024, else FEPLB_E_INVALID) for every
- * forward launch.
+ * forward launch.  FEPLB_FORM_WEIGHT_M reads W1 and W3 through one tensor map: a launch whose W1 and
+ * W3 are the same memory, or 1 TiB or more apart, runs as FEPLB_FORM_SINGLE or _PAIR instead (by its
+ * rows per expert); feplb_forward_path says which.
  * backward_pair: -1 (default: chosen from the geometry) or a mask, bit 0 = activation-gradient
  * GEMMs in the pair form, bit 1 = weight-gradient GEMMs in the pair form.  Results do not depend
  * on the form beyond fp32 summation order.  Not allowed while a plan is pending. */

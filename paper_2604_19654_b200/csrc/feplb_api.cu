@@ -737,6 +737,7 @@ static int ffn_impl(feplb_ctx* c, const void* x_perm, const void* w1, const void
   a.ab_out = c->d_preact;
   a.recv_w1 = c->d_recv_w1; a.recv_w3 = c->d_recv_w3; a.recv_w2 = c->d_recv_w2; a.n_recv_slots = c->n_recv_slots;
   a.recv_x = c->d_recv_x;
+  // k_ffn_few reads home weights only and one table: not with receive slots, not where a launch picks the planner's table up
   if (c->few && !weights_on_m && !a.n_recv_slots && !(dyn && dyn->seq)) {
     rc = feplb_launch_expert_ffn_few(a, st, &c->launches, c->err, sizeof(c->err), c->few, dyn ? dyn->stamps : nullptr);
     if (rc != FEPLB_E_STATE) {

@@ -10,7 +10,8 @@ from paper_2604_19654_b200 import build as B
 from paper_2604_19654_b200 import feplb as F
 from paper_2604_19654_b200 import workloads as W
 
-from gpu_utils import assert_close
+from gpu_utils import DeviceCase, assert_close, upload_groups
+from test_gpu_parity import _check_forward
 
 pytestmark = pytest.mark.gpu
 
@@ -107,12 +108,65 @@ def test_weights_in_one_buffer(form):
     _run([1, 40, 64, 65, 130], 256, 128, form, same=True)
 
 
+@pytest.mark.parametrize("rows,fallback", [([1, 40, 64, 65, 130], F.PATH_SINGLE), ([300, 257, 256], F.PATH_PAIR)])
+def test_weights_on_m_asked_for_with_weights_in_one_buffer(rows, fallback):
+    forms = F.PATH_SINGLE | F.PATH_PAIR | F.PATH_WEIGHT_M
+    assert _run(rows, 256, 128, F.FORM_WEIGHT_M) & forms == F.PATH_WEIGHT_M
+    assert _run(rows, 256, 128, F.FORM_WEIGHT_M, same=True) & forms == fallback
+
+
 @pytest.mark.parametrize("w3_first", [False, True])
 def test_weights_on_m_units_of_any_width(w3_first):
     """d = 7.5 x 256, f = 13.5 x 128: the second CTA's half of the last weight block lies past the width, the last K block of
     pass 2 is half empty; segments around the multiples of 32 and 256 rows; saved pre-activations."""
     rows = [1, 31, 32, 33, 64, 65, 128, 129, 200, 255, 256, 257, 300]
     assert _run(rows, 1920, 1728, None, w3_first, preact=True) & F.PATH_WEIGHT_M
+
+
+HALF_UNITS = W.get_workload("cfg2").with_(E=8, R=4, K=2, d=1920, f=1728, dyn=2, max_num_dyn=2, tau=1)   # 7.5 and 13.5 weight blocks
+
+
+@pytest.mark.parametrize("split", [0, 1])
+@pytest.mark.parametrize("T", [600, 4100])
+def test_weights_on_m_late_table_at_half_units(T, split):
+    """The planner's table taken up inside the launch where the last weight block is half empty, behind either front."""
+    case = DeviceCase(HALF_UNITS.with_(T=T), mb=1, split=split)
+    case.ctx.set_planner_timing(planner_delay_us=1000)
+    p, _ = _check_forward(case, sample=60)
+    assert len(p.moves) > 0 and any(g[4] for g in p.groups)
+    assert case.ctx.forward_path() & (F.PATH_WEIGHT_M | F.PATH_MERGED) == F.PATH_WEIGHT_M | F.PATH_MERGED
+    case.close()
+
+
+def test_weights_on_m_receive_slots_at_half_units():
+    """Migrated experts' weights from their receive slots, W3 in front of W1 at home: the rows of the relabelled experts, also from
+    home weights of zeros."""
+    w = HALF_UNITS.with_(T=600)
+    weights = W.gen_weights(w)
+    base = DeviceCase(w, mb=1, weights=weights)
+    p0, _ = _check_forward(base, sample=60)
+    case = DeviceCase(w, mb=1, weights=weights, phase2_copy=1)
+    pair = torch.empty(2, *case.d_w1.shape, dtype=torch.bfloat16, device="cuda")
+    pair[0], pair[1] = case.d_w3, case.d_w1
+    case.d_w1, case.d_w3 = pair[1], pair[0]
+    p1, _ = _check_forward(case, sample=60)
+    assert p1.moves == p0.moves and len(p1.moves) > 0
+    assert case.ctx.forward_path() == F.PATH_SMALL_FRONT | F.PATH_WEIGHT_M
+    assert torch.equal(case.buf.out.view(torch.int16), base.buf.out.view(torch.int16))
+    dst, first = p1.moves[0][2], {}
+    for e, src, to, rows in p1.moves:                                  # move i takes the next slot of its destination
+        first.setdefault(to, e)
+    e = first[dst]
+    _, row, rows, _, _ = next(g for g in p1.groups if g[0] == e and g[3] == dst)
+    want = case.buf.y_perm[row:row + rows].clone()
+    pair.zero_()
+    case.buf.y_perm[row:row + rows] = 7.0
+    groups = upload_groups([(e, row, rows, dst, 2 + dst * w.max_num_dyn)])
+    case.ctx.expert_ffn(case.buf.x_perm, case.d_w1, case.d_w3, torch.zeros_like(case.d_w2), groups, 1, case.buf.h_scratch, case.buf.y_perm)
+    case.ctx.check_status()
+    assert torch.equal(case.buf.y_perm[row:row + rows].view(torch.int16), want.view(torch.int16))
+    base.close()
+    case.close()
 
 
 @pytest.mark.parametrize("w3_first", [False, True])
