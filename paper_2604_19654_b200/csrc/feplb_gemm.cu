@@ -241,27 +241,6 @@ __device__ __forceinline__ int put_group(SmemTail* t, int idx, int expert, int r
   return tiles;
 }
 
-// In-place inclusive scan of t->prefix[first+1 .. first+n] (tile counts) by one warp; prefix[first] is the base.
-__device__ __forceinline__ void warp_scan_prefix(SmemTail* t, int first, int n, int lane) {
-  const int per = (n + 31) / 32;
-  const int g0 = min(n, lane * per), g1 = min(n, g0 + per);
-  int sum = 0;
-  for (int g = g0; g < g1; ++g) sum += t->prefix[first + g + 1];
-  int incl = sum;
-#pragma unroll
-  for (int o = 1; o < 32; o <<= 1) {
-    const int y = __shfl_up_sync(0xffffffffu, incl, o);
-    if (lane >= o) incl += y;
-  }
-  int run = t->prefix[first] + incl - sum;
-  __syncwarp();
-  for (int g = g0; g < g1; ++g) {
-    run += t->prefix[first + g + 1];
-    t->prefix[first + g + 1] = run;
-  }
-  __syncwarp();
-}
-
 // NARROW: the last N tile of a row of tiles has fewer columns than the others.  An instantiation of its own, because a
 // width that differs per tile costs the roles more than it saves where it does not: both passes of a large batch in the
 // single form, 64 experts, d = 2048, f = 768, 1536 / 3750 rows per expert on average: 950 / 2187 us with one kernel
@@ -338,7 +317,7 @@ k_grouped_gemm(const __grid_constant__ Maps<DEEP> tm, const GemmParams p) {
         p.dyn, p.n_groups, FEPLB_MAX_GROUPS, p.status, lane,
         [&](int e, int rs) { return tail->g_row_start[e] == rs && tail->prefix[e + 1] == 0; },
         [&](int i, int e, int rs, int rw, int dy) { tail->prefix[i + 1] = put_group<kTileRows>(tail, i, e, rs, rw, dy, true, p); });
-    warp_scan_prefix(tail, 0, n, lane);
+    warp_scan_prefix(tail->prefix, 0, n, lane);
     if (lane == 0) {
       tail->n_entries = n;
       tail->total_mtiles = tail->prefix[n];
@@ -378,7 +357,7 @@ k_grouped_gemm(const __grid_constant__ Maps<DEEP> tm, const GemmParams p) {
         tail->prefix[n_static_entries + i + 1] = put_group<kTileRows>(tail, n_static_entries + i, e, rs, rw, dy, true, p);
       }
       if (!__all_sync(0xffffffffu, good)) return false;
-      warp_scan_prefix(tail, n_static_entries, n_dyn, lane);
+      warp_scan_prefix(tail->prefix, n_static_entries, n_dyn, lane);
       n_entries = n_static_entries + n_dyn;
       total = tail->prefix[n_entries] * p.n_tiles_n;
       if (lane == 0) {
@@ -709,50 +688,18 @@ __global__ void k_wait_selftest(uint32_t* status, unsigned long long limit_ns, i
 
 // ------------------------------------------------------------------------------------------ host
 
-typedef CUresult (*encode_tiled_fn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*,
-                                    const cuuint64_t*, const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave,
-                                    CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
-
-encode_tiled_fn get_encode_fn() {
-  static encode_tiled_fn fn = nullptr;
-  if (!fn) {
-    void* p = nullptr;
-    cudaDriverEntryPointQueryResult q;
-    if (cudaGetDriverEntryPoint("cuTensorMapEncodeTiled", &p, cudaEnableDefault, &q) == cudaSuccess &&
-        q == cudaDriverEntryPointSuccess)
-      fn = reinterpret_cast<encode_tiled_fn>(p);
-  }
-  return fn;
-}
-
-bool encode(CUtensorMap* m, int rank, const void* base, const cuuint64_t* dims, const cuuint64_t* strides, const cuuint32_t* box) {
-  encode_tiled_fn fn = get_encode_fn();
-  const cuuint32_t estr[5] = {1, 1, 1, 1, 1};
-  return fn && fn(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, (cuuint32_t)rank, const_cast<void*>(base), dims, strides, box, estr,
-                  CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-                  CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
-}
 // Row-major bf16 matrix [rows, inner] -> tensor map with a [box_rows, 64] box, 128-byte swizzle.
 bool make_tmap(CUtensorMap* m, const void* base, uint64_t rows, uint64_t inner, uint32_t box_rows) {
   const cuuint64_t dims[2] = {inner, rows}, strides[1] = {inner * 2};
   const cuuint32_t box[2] = {(cuuint32_t)kChunk, box_rows};
-  return encode(m, 2, base, dims, strides, box);
+  return encode_tmap(m, 2, base, dims, strides, box);
 }
-// The same with boxes of two 64-element chunks, chunk after chunk (deep stages).
-bool make_tmap_chunks(CUtensorMap* m, const void* base, uint64_t rows, uint64_t inner, uint32_t box_rows) {
-  const cuuint64_t dims[3] = {(cuuint64_t)kChunk, rows, inner / kChunk}, strides[2] = {inner * 2, kChunk * 2};
-  const cuuint32_t box[3] = {(cuuint32_t)kChunk, box_rows, 2};
-  return encode(m, 3, base, dims, strides, box);
-}
-// 64 rows of W1 and the same 64 of W3, two chunks: {64 columns, rows, W1 and W3, chunks}, beginning at the one in
-// front.  Fails where they are further apart than a map's stride reaches, or the same.
-bool make_tmap_w13(CUtensorMap* m, const void* w1, const void* w3, uint64_t rows, uint64_t inner) {
-  const char *lo = (const char*)(w1 < w3 ? w1 : w3), *hi = (const char*)(w1 < w3 ? w3 : w1);
-  const uint64_t apart = (uint64_t)(hi - lo);
-  if (apart == 0 || apart >= (1ull << 40)) return false;
+// 64 rows of W1 and the same 64 of W3, two chunks: {64 columns, rows, W1 and W3, chunks}.
+bool make_tmap_w13_tile(CUtensorMap* m, const void* w1, const void* w3, uint64_t rows, uint64_t inner) {
+  const uint64_t apart = w13_apart(w1, w3);
   const cuuint64_t dims[4] = {(cuuint64_t)kChunk, rows, 2, inner / kChunk}, strides[3] = {inner * 2, apart, kChunk * 2};
   const cuuint32_t box[4] = {(cuuint32_t)kChunk, 64, 2, 2};
-  return encode(m, 4, lo, dims, strides, box);
+  return apart && encode_tmap(m, 4, w1 < w3 ? w1 : w3, dims, strides, box);
 }
 
 template <bool SWIGLU, bool PAIR, bool NARROW, bool DEEP>
@@ -836,7 +783,7 @@ int feplb_launch_expert_ffn(const feplb_gemm_args& a, cudaStream_t st, int64_t* 
   }
   m2.b1 = m2.w13 = m2.b0;
   m1.w13 = m1.b0;
-  const bool halves = deep && make_tmap_w13(&m1.w13, a.w1, a.w3, w1_rows, d);
+  const bool halves = deep && make_tmap_w13_tile(&m1.w13, a.w1, a.w3, w1_rows, d);
   // receive buffer of migrated experts' weights, addressed by slot like the home weights by expert, and the rows of
   // migrated pieces: pass 1 reads them from the receive region when there is one
   m1.r0 = m1.b0; m1.r1 = m1.b1; m2.r0 = m2.b0; m1.ra = m1.a; m2.ra = m2.a;

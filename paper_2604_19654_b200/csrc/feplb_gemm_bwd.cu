@@ -263,23 +263,9 @@ k_ffn_bwd_gemm(const __grid_constant__ Maps<KIND> maps, const __grid_constant__ 
   tc_fence_before();
   __syncthreads();
   if (warp == 0) {
-    const int per = (p.n_groups + 31) / 32;
-    const int g0 = lane * per, g1 = min(p.n_groups, g0 + per);
-    int sum = 0;
-    for (int g = g0; g < g1; ++g) sum += tail->prefix[g + 1];
-    int incl = sum;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-      const int y = __shfl_up_sync(0xffffffffu, incl, o);
-      if (lane >= o) incl += y;
-    }
-    int run = incl - sum;
-    for (int g = g0; g < g1; ++g) {
-      const int t = tail->prefix[g + 1];
-      run += t;
-      tail->prefix[g + 1] = run;
-    }
     if (lane == 0) tail->prefix[0] = 0;
+    __syncwarp();
+    warp_scan_prefix(tail->prefix, 0, p.n_groups, lane);
   }
   __syncthreads();
   if (PAIR) cluster_sync_all();   // the peer's barriers are initialised before anything signals them
@@ -687,61 +673,29 @@ k_combine_bwd(const uint4* __restrict__ d_out, const uint4* __restrict__ y_perm,
   }
 }
 
-typedef CUresult (*encode_tiled_fn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*,
-                                    const cuuint64_t*, const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave,
-                                    CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
-
-encode_tiled_fn get_encode_fn() {
-  static encode_tiled_fn fn = nullptr;
-  if (!fn) {
-    void* p = nullptr;
-    cudaDriverEntryPointQueryResult q;
-    if (cudaGetDriverEntryPoint("cuTensorMapEncodeTiled", &p, cudaEnableDefault, &q) == cudaSuccess &&
-        q == cudaDriverEntryPointSuccess)
-      fn = reinterpret_cast<encode_tiled_fn>(p);
-  }
-  return fn;
-}
-
 // Row-major bf16 matrix [rows, inner] with a row pitch of ld elements -> [box_rows, 64] boxes, 128-byte swizzle.
 bool make_tmap(CUtensorMap* m, const void* base, uint64_t rows, uint64_t inner, uint64_t ld, uint32_t box_rows) {
-  encode_tiled_fn fn = get_encode_fn();
-  if (!fn) return false;
-  cuuint64_t dims[2] = {inner, rows};
-  cuuint64_t strides[1] = {ld * 2};
-  cuuint32_t box[2] = {(cuuint32_t)BK, box_rows};
-  cuuint32_t estr[2] = {1, 1};
-  return fn(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void*>(base), dims, strides, box, estr,
-            CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-            CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+  const cuuint64_t dims[2] = {inner, rows}, strides[1] = {ld * 2};
+  const cuuint32_t box[2] = {(cuuint32_t)BK, box_rows};
+  return encode_tmap(m, 2, base, dims, strides, box);
 }
 
 // Row-major bf16 [rows, cols] (pitch ld) as the 3-d tensor {64 columns, rows, cols/64 chunks}: a box of
 // 64 x 64 x `chunks` lands in shared memory chunk after chunk, each 64 rows of 128 bytes, 128-byte
 // swizzled: the MN-major operand layout of the weight-gradient kind.
 bool make_tmap_mn(CUtensorMap* m, const void* base, uint64_t rows, uint64_t cols, uint64_t ld, uint32_t chunks) {
-  encode_tiled_fn fn = get_encode_fn();
-  if (!fn) return false;
-  cuuint64_t dims[3] = {64, rows, cols / 64};
-  cuuint64_t strides[2] = {ld * 2, 128};
-  cuuint32_t box[3] = {64, (cuuint32_t)BK, chunks};
-  cuuint32_t estr[3] = {1, 1, 1};
-  return fn(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void*>(base), dims, strides, box, estr,
-            CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-            CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+  const cuuint64_t dims[3] = {64, rows, cols / 64}, strides[2] = {ld * 2, 128};
+  const cuuint32_t box[3] = {64, (cuuint32_t)BK, chunks};
+  return encode_tmap(m, 3, base, dims, strides, box);
 }
 
 // fp32 [E, M, N] as a 3-d map with boxes of 32 x 32 x 1, 128-byte swizzled (the epilogue's staging layout);
 // a box never crosses into the next expert's matrix.
 bool make_tmap_out(CUtensorMap* m, float* base, uint64_t E, uint64_t M, uint64_t N) {
-  encode_tiled_fn fn = get_encode_fn();
-  if (!fn) return false;
-  cuuint64_t dims[3] = {N, M, E};
-  cuuint64_t strides[2] = {N * 4, M * N * 4};
-  cuuint32_t box[3] = {32, 32, 1};
-  cuuint32_t estr[3] = {1, 1, 1};
-  return fn(m, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 3, base, dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
-            CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_NONE, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+  const cuuint64_t dims[3] = {N, M, E}, strides[2] = {N * 4, M * N * 4};
+  const cuuint32_t box[3] = {32, 32, 1};
+  return encode_tmap(m, 3, base, dims, strides, box, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_DATA_TYPE_FLOAT32,
+                     CU_TENSOR_MAP_L2_PROMOTION_NONE);
 }
 
 // Rows of a B half tile for an output n columns wide: the N tile of 2 * 128 or 2 * 64 columns that brings fewer operand

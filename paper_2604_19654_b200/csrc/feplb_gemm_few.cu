@@ -116,16 +116,6 @@ __device__ __forceinline__ void tma_load_5d(uint32_t dst, const CUtensorMap* m, 
       ::"r"(dst), "l"(reinterpret_cast<uint64_t>(m)), "r"(bar), "r"(c0), "r"(c1), "r"(c2), "r"(c3), "r"(c4) : "memory");
 }
 
-// 16 TMEM lanes x 32 fp32 columns in the layout of matrix fragments: registers 4g .. 4g + 3 of a thread are columns
-// 8g + 2 (lane % 4) and the next of row lane / 4, then the same columns of row lane / 4 + 8.
-__device__ __forceinline__ void tmem_ld_frag(uint32_t taddr, uint32_t* r) {
-  asm volatile(
-      "tcgen05.ld.sync.aligned.16x256b.x4.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, [%16];"
-      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]), "=r"(r[9]),
-        "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
-      : "r"(taddr) : "memory");
-}
-
 // 16 or 32 columns (HALVES fragments of 16) x 32 token rows -> rows of global memory: stmatrix transposes into token rows of
 // 64 bytes whose 16-byte pieces are exchanged by bits 1 and 2 of the row number, and 16-byte pieces go out.
 template <int HALVES>
@@ -211,23 +201,7 @@ k_ffn_few(const __grid_constant__ CUtensorMap tm_w, const __grid_constant__ RowM
   }
   tc_fence_before();
   __syncthreads();
-  if (warp == 0) {                                  // inclusive scan of the unit counts
-    const int per = (p.n_groups + 31) / 32;
-    const int g0 = min(p.n_groups, lane * per), g1 = min(p.n_groups, g0 + per);
-    int sum = 0;
-    for (int g = g0; g < g1; ++g) sum += tail->prefix[g + 1];
-    int incl = sum;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-      const int y = __shfl_up_sync(0xffffffffu, incl, o);
-      if (lane >= o) incl += y;
-    }
-    int run = incl - sum;
-    for (int g = g0; g < g1; ++g) {
-      run += tail->prefix[g + 1];
-      tail->prefix[g + 1] = run;
-    }
-  }
+  if (warp == 0) warp_scan_prefix(tail->prefix, 0, p.n_groups, lane);
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem_base = tail->tmem_base;
@@ -381,56 +355,9 @@ k_ffn_few(const __grid_constant__ CUtensorMap tm_w, const __grid_constant__ RowM
 
 // ------------------------------------------------------------------------------------------ host
 
-typedef CUresult (*encode_tiled_fn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*,
-                                    const cuuint64_t*, const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave,
-                                    CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
-
-encode_tiled_fn get_encode_fn() {
-  static encode_tiled_fn fn = nullptr;
-  if (!fn) {
-    void* p = nullptr;
-    cudaDriverEntryPointQueryResult q;
-    if (cudaGetDriverEntryPoint("cuTensorMapEncodeTiled", &p, cudaEnableDefault, &q) == cudaSuccess &&
-        q == cudaDriverEntryPointSuccess)
-      fn = reinterpret_cast<encode_tiled_fn>(p);
-  }
-  return fn;
-}
-
-// Row-major bf16 [rows, inner] as the 3-d tensor {64 columns, rows, inner / 64 chunks}: a box of 64 x box_rows x 2 lands in
-// shared memory chunk after chunk, box_rows rows of 128 bytes each.  A second chunk past the end reads as zeros.
-bool make_tmap(CUtensorMap* m, const void* base, uint64_t rows, uint64_t inner, uint32_t box_rows) {
-  encode_tiled_fn fn = get_encode_fn();
-  if (!fn) return false;
-  cuuint64_t dims[3] = {(cuuint64_t)kChunk, rows, inner / kChunk};
-  cuuint64_t strides[2] = {inner * 2, kChunk * 2};
-  cuuint32_t box[3] = {(cuuint32_t)kChunk, box_rows, 2};
-  cuuint32_t estr[3] = {1, 1, 1};
-  return fn(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void*>(base), dims, strides, box, estr,
-            CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-            CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
-}
-
-// W1 and W3, [rows, inner] each, as one 5-d tensor {64 columns, 16 rows, the two of them, rows / 16, inner / 64 chunks} that
-// begins at the one in front: a box of 64 x 16 x 2 x 4 x 2 brings 64 rows of both, 16 in turn, chunk after chunk.
-// Fails where they are further apart than a map's stride reaches (or the same).
-bool make_tmap_w13(CUtensorMap* m, const void* w1, const void* w3, uint64_t rows, uint64_t inner) {
-  encode_tiled_fn fn = get_encode_fn();
-  const char *lo = (const char*)(w1 < w3 ? w1 : w3), *hi = (const char*)(w1 < w3 ? w3 : w1);
-  const uint64_t apart = (uint64_t)(hi - lo);
-  if (!fn || apart == 0 || apart >= (1ull << 40)) return false;
-  cuuint64_t dims[5] = {(cuuint64_t)kChunk, 16, 2, rows / 16, inner / kChunk};
-  cuuint64_t strides[4] = {inner * 2, apart, inner * 32, kChunk * 2};
-  cuuint32_t box[5] = {(cuuint32_t)kChunk, 16, 2, 4, 2};
-  cuuint32_t estr[5] = {1, 1, 1, 1, 1};
-  return fn(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 5, const_cast<char*>(lo), dims, strides, box, estr,
-            CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-            CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
-}
-
 bool make_row_maps(RowMaps* x, const void* base, uint64_t rows, uint64_t inner, int nmax) {
   for (int i = 0; (nmax >> i) >= 16; ++i)
-    if (!make_tmap(&x->m[i], base, rows, inner, (uint32_t)(nmax >> i))) return false;
+    if (!make_tmap_chunks(&x->m[i], base, rows, inner, (uint32_t)(nmax >> i))) return false;
   return true;
 }
 
@@ -477,7 +404,7 @@ int feplb_launch_expert_ffn_few(const feplb_gemm_args& a, cudaStream_t st, int64
   CUtensorMap w13, w2;
   RowMaps x, h;
   if (!make_tmap_w13(&w13, a.w1, a.w3, (uint64_t)a.E * a.f, (uint64_t)a.d)) return FEPLB_E_STATE;
-  if (!make_tmap(&w2, a.w2, (uint64_t)a.E * a.d, (uint64_t)a.f, kWRows) ||
+  if (!make_tmap_chunks(&w2, a.w2, (uint64_t)a.E * a.d, (uint64_t)a.f, kWRows) ||
       !make_row_maps(&x, a.x_perm, (uint64_t)a.s_cap, (uint64_t)a.d, nmax) ||
       !make_row_maps(&h, a.h, (uint64_t)a.s_cap, (uint64_t)a.f, nmax)) {
     snprintf(err, errn, "cuTensorMapEncodeTiled failed (driver entry point missing or bad pointer/shape)");

@@ -161,37 +161,6 @@ __device__ __forceinline__ int put_entry(Tail* t, int idx, int expert, int row_s
   return units;
 }
 
-// In-place inclusive scan of t->prefix[first+1 .. first+n] (unit counts) by one warp; prefix[first] is the base.
-__device__ __forceinline__ void warp_scan_prefix(Tail* t, int first, int n, int lane) {
-  const int per = (n + 31) / 32;
-  const int g0 = min(n, lane * per), g1 = min(n, g0 + per);
-  int sum = 0;
-  for (int g = g0; g < g1; ++g) sum += t->prefix[first + g + 1];
-  int incl = sum;
-#pragma unroll
-  for (int o = 1; o < 32; o <<= 1) {
-    const int y = __shfl_up_sync(0xffffffffu, incl, o);
-    if (lane >= o) incl += y;
-  }
-  int run = t->prefix[first] + incl - sum;
-  __syncwarp();
-  for (int g = g0; g < g1; ++g) {
-    run += t->prefix[first + g + 1];
-    t->prefix[first + g + 1] = run;
-  }
-  __syncwarp();
-}
-
-// 16 TMEM lanes x 32 fp32 columns in the layout of matrix fragments: registers 4g .. 4g + 3 of a thread are columns
-// 8g + 2 (lane % 4) and the next of row lane / 4, then the same columns of row lane / 4 + 8.
-__device__ __forceinline__ void tmem_ld_frag(uint32_t taddr, uint32_t* r) {
-  asm volatile(
-      "tcgen05.ld.sync.aligned.16x256b.x4.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, [%16];"
-      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]), "=r"(r[9]),
-        "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
-      : "r"(taddr) : "memory");
-}
-
 // The warp's staging area may still be read by the TMA store of its previous chunk.
 __device__ __forceinline__ void staging_ready(int lane) {
   if (lane == 0) asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
@@ -305,7 +274,7 @@ k_ffn_wm(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__ CUten
         p.dyn, p.n_groups, kMaxEntries, p.status, lane,
         [&](int e, int rs) { return tail->row_start[e] == rs && tail->prefix[e + 1] == 0; },
         [&](int i, int e, int rs, int rw, int dy) { tail->prefix[i + 1] = put_entry(tail, i, e, rs, rw, dy, true, p); });
-    warp_scan_prefix(tail, 0, n, lane);
+    warp_scan_prefix(tail->prefix, 0, n, lane);
     if (lane == 0) {
       tail->n_entries = n;
       tail->total_units = tail->prefix[n];
@@ -346,7 +315,7 @@ k_ffn_wm(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__ CUten
         tail->prefix[n_static_entries + i + 1] = put_entry(tail, n_static_entries + i, e, rs, rw, dy, true, p);
       }
       if (!__all_sync(0xffffffffu, good)) return false;
-      warp_scan_prefix(tail, n_static_entries, n_dyn, lane);
+      warp_scan_prefix(tail->prefix, n_static_entries, n_dyn, lane);
       n_entries = n_static_entries + n_dyn;
       total = tail->prefix[n_entries];
       if (lane == 0) {
@@ -588,67 +557,16 @@ k_ffn_wm(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__ CUten
 
 // ------------------------------------------------------------------------------------------ host
 
-typedef CUresult (*encode_tiled_fn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*,
-                                    const cuuint64_t*, const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave,
-                                    CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
-
-encode_tiled_fn get_encode_fn() {
-  static encode_tiled_fn fn = nullptr;
-  if (!fn) {
-    void* p = nullptr;
-    cudaDriverEntryPointQueryResult q;
-    if (cudaGetDriverEntryPoint("cuTensorMapEncodeTiled", &p, cudaEnableDefault, &q) == cudaSuccess &&
-        q == cudaDriverEntryPointSuccess)
-      fn = reinterpret_cast<encode_tiled_fn>(p);
-  }
-  return fn;
-}
-
-// Row-major bf16 matrix [rows, inner] as {64 columns, rows, inner / 64 chunks} with boxes of box_rows rows x kChunks chunks,
-// 128-byte swizzle.  A chunk past the end reads as zeros.
-bool make_tmap(CUtensorMap* m, const void* base, uint64_t rows, uint64_t inner, uint32_t box_rows) {
-  encode_tiled_fn fn = get_encode_fn();
-  if (!fn) return false;
-  cuuint64_t dims[3] = {(cuuint64_t)kChunk, rows, inner / kChunk};
-  cuuint64_t strides[2] = {inner * 2, kChunk * 2};
-  cuuint32_t box[3] = {(cuuint32_t)kChunk, box_rows, (cuuint32_t)kChunks};
-  cuuint32_t estr[3] = {1, 1, 1};
-  return fn(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void*>(base), dims, strides, box, estr,
-            CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-            CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
-}
 // The output, 32 rows x 16 (pass 1) or 32 columns per box, swizzled by the box's width.
 bool make_tmap_out(CUtensorMap* m, void* base, uint64_t rows, uint64_t inner, uint32_t cols) {
-  encode_tiled_fn fn = get_encode_fn();
-  if (!fn) return false;
-  cuuint64_t dims[2] = {inner, rows};
-  cuuint64_t strides[1] = {inner * 2};
-  cuuint32_t box[2] = {cols, 32};
-  cuuint32_t estr[2] = {1, 1};
-  return fn(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, base, dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
-            cols == 16 ? CU_TENSOR_MAP_SWIZZLE_32B : CU_TENSOR_MAP_SWIZZLE_64B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-            CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
-}
-// W1 and W3, [rows, inner] each, as {64 columns, 16 rows, the two of them, rows / 16, inner / 64 chunks}, beginning at the one in
-// front: a box brings 64 rows of both, 16 in turn.  Fails where they are further apart than a map's stride
-// reaches, or the same.
-bool make_tmap_w13(CUtensorMap* m, const void* w1, const void* w3, uint64_t rows, uint64_t inner) {
-  encode_tiled_fn fn = get_encode_fn();
-  const char *lo = (const char*)(w1 < w3 ? w1 : w3), *hi = (const char*)(w1 < w3 ? w3 : w1);
-  const uint64_t apart = (uint64_t)(hi - lo);
-  if (!fn || apart == 0 || apart >= (1ull << 40)) return false;
-  cuuint64_t dims[5] = {(cuuint64_t)kChunk, 16, 2, rows / 16, inner / kChunk};
-  cuuint64_t strides[4] = {inner * 2, apart, inner * 32, kChunk * 2};
-  cuuint32_t box[5] = {(cuuint32_t)kChunk, 16, 2, 4, (cuuint32_t)kChunks};
-  cuuint32_t estr[5] = {1, 1, 1, 1, 1};
-  return fn(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 5, const_cast<char*>(lo), dims, strides, box, estr,
-            CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-            CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+  const cuuint64_t dims[2] = {inner, rows}, strides[1] = {inner * 2};
+  const cuuint32_t box[2] = {cols, 32};
+  return encode_tmap(m, 2, base, dims, strides, box, cols == 16 ? CU_TENSOR_MAP_SWIZZLE_32B : CU_TENSOR_MAP_SWIZZLE_64B);
 }
 
 bool make_bmaps(BMaps* b, const void* base, uint64_t rows, uint64_t inner) {
   for (int i = 0; i < kBoxes; ++i)
-    if (!make_tmap(&b->m[i], base, rows, inner, (uint32_t)((kNMax / 2) >> i))) return false;   // rows past the tensor read as zeros
+    if (!make_tmap_chunks(&b->m[i], base, rows, inner, (uint32_t)((kNMax / 2) >> i))) return false;   // rows past the tensor read as zeros
   return true;
 }
 
@@ -701,7 +619,7 @@ int feplb_launch_expert_ffn_wm(const feplb_gemm_args& a, const feplb_wm_dyn& dyn
   CUtensorMap tm_w13, tm_w2, tm_h, tm_y;
   BMaps bx, bh;
   if (!make_tmap_w13(&tm_w13, a.w1, a.w3, (uint64_t)a.E * a.f, (uint64_t)a.d)) return FEPLB_E_STATE;
-  if (!make_tmap(&tm_w2, a.w2, (uint64_t)a.E * a.d, (uint64_t)a.f, WM) ||
+  if (!make_tmap_chunks(&tm_w2, a.w2, (uint64_t)a.E * a.d, (uint64_t)a.f, WM) ||
       !make_tmap_out(&tm_h, a.h, (uint64_t)a.s_cap, (uint64_t)a.f, 16) ||
       !make_tmap_out(&tm_y, a.y, (uint64_t)a.s_cap, (uint64_t)a.d, 32) ||
       !make_bmaps(&bx, a.x_perm, (uint64_t)a.s_cap, (uint64_t)a.d) ||
@@ -712,7 +630,7 @@ int feplb_launch_expert_ffn_wm(const feplb_gemm_args& a, const feplb_wm_dyn& dyn
   CUtensorMap tm_r13 = tm_w13, tm_r2 = tm_w2;
   const bool has_recv = a.recv_w1 && a.recv_w3 && a.recv_w2 && a.n_recv_slots > 0;
   if (has_recv && !make_tmap_w13(&tm_r13, a.recv_w1, a.recv_w3, (uint64_t)a.n_recv_slots * a.f, (uint64_t)a.d)) return FEPLB_E_STATE;
-  if (has_recv && !make_tmap(&tm_r2, a.recv_w2, (uint64_t)a.n_recv_slots * a.d, (uint64_t)a.f, WM)) {
+  if (has_recv && !make_tmap_chunks(&tm_r2, a.recv_w2, (uint64_t)a.n_recv_slots * a.d, (uint64_t)a.f, WM)) {
     snprintf(err, errn, "cuTensorMapEncodeTiled failed for the receive buffer");
     return FEPLB_E_CUDA;
   }

@@ -1,6 +1,6 @@
 // Inline-PTX building blocks shared by the tensor-core kernels of libfeplb (sm_100a): mbarriers
 // with bounded waits, TMA tile loads, TMEM allocation, tcgen05.mma / commit / ld, cluster-of-two
-// helpers, shared-memory and instruction descriptors.
+// helpers, shared-memory and instruction descriptors; and the tensor maps that several of them use.
 #ifndef FEPLB_TC_CUH_
 #define FEPLB_TC_CUH_
 
@@ -190,11 +190,94 @@ __device__ __forceinline__ uint32_t make_idesc(int m, int n) {
   return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(n >> 3) << 17) | ((uint32_t)(m >> 4) << 24);
 }
 
+// 16 TMEM lanes x 32 fp32 columns in the layout of matrix fragments: registers 4g .. 4g + 3 of a thread are columns
+// 8g + 2 (lane % 4) and the next of row lane / 4, then the same columns of row lane / 4 + 8.
+__device__ __forceinline__ void tmem_ld_frag(uint32_t taddr, uint32_t* r) {
+  asm volatile(
+      "tcgen05.ld.sync.aligned.16x256b.x4.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, [%16];"
+      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]), "=r"(r[9]),
+        "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
+      : "r"(taddr) : "memory");
+}
+
+// In-place inclusive scan of prefix[first+1 .. first+n] (counts) by one warp; prefix[first] is the base.
+__device__ __forceinline__ void warp_scan_prefix(int* prefix, int first, int n, int lane) {
+  const int per = (n + 31) / 32;
+  const int g0 = min(n, lane * per), g1 = min(n, g0 + per);
+  int sum = 0;
+  for (int g = g0; g < g1; ++g) sum += prefix[first + g + 1];
+  int incl = sum;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const int y = __shfl_up_sync(0xffffffffu, incl, o);
+    if (lane >= o) incl += y;
+  }
+  int run = prefix[first] + incl - sum;
+  __syncwarp();
+  for (int g = g0; g < g1; ++g) {
+    run += prefix[first + g + 1];
+    prefix[first + g + 1] = run;
+  }
+  __syncwarp();
+}
+
 __device__ __forceinline__ uint32_t pack_bf16x2(float lo, float hi) {
   __nv_bfloat162 h = __floats2bfloat162_rn(lo, hi);
   return *reinterpret_cast<uint32_t*>(&h);
 }
 __device__ __forceinline__ float silu_f(float a) { return __fdividef(a, 1.f + __expf(-a)); }
+
+// ------------------------------------------------------------------------------------------ tensor maps (host)
+
+typedef CUresult (*encode_tiled_fn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*,
+                                    const cuuint64_t*, const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave,
+                                    CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
+
+inline encode_tiled_fn get_encode_fn() {
+  static encode_tiled_fn fn = nullptr;
+  if (!fn) {
+    void* p = nullptr;
+    cudaDriverEntryPointQueryResult q;
+    if (cudaGetDriverEntryPoint("cuTensorMapEncodeTiled", &p, cudaEnableDefault, &q) == cudaSuccess &&
+        q == cudaDriverEntryPointSuccess)
+      fn = reinterpret_cast<encode_tiled_fn>(p);
+  }
+  return fn;
+}
+
+// A map of the given rank (elements, strides in bytes); boxes past the end read as zeros.
+inline bool encode_tmap(CUtensorMap* m, int rank, const void* base, const cuuint64_t* dims, const cuuint64_t* strides, const cuuint32_t* box,
+                        CUtensorMapSwizzle swizzle = CU_TENSOR_MAP_SWIZZLE_128B, CUtensorMapDataType type = CU_TENSOR_MAP_DATA_TYPE_BFLOAT16,
+                        CUtensorMapL2promotion l2 = CU_TENSOR_MAP_L2_PROMOTION_L2_256B) {
+  const encode_tiled_fn fn = get_encode_fn();
+  const cuuint32_t estr[5] = {1, 1, 1, 1, 1};
+  return fn && fn(m, type, (cuuint32_t)rank, const_cast<void*>(base), dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE, swizzle, l2,
+                  CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+
+// Row-major bf16 [rows, inner] as the 3-d tensor {64 columns, rows, inner / 64 chunks}: a box of 64 x box_rows x 2 lands in
+// shared memory chunk after chunk, box_rows rows of 128 bytes each.
+inline bool make_tmap_chunks(CUtensorMap* m, const void* base, uint64_t rows, uint64_t inner, uint32_t box_rows) {
+  const cuuint64_t dims[3] = {64, rows, inner / 64}, strides[2] = {inner * 2, 128};
+  const cuuint32_t box[3] = {64, box_rows, 2};
+  return encode_tmap(m, 3, base, dims, strides, box);
+}
+
+// Distance of W1 and W3 where one map can cover both (beginning at the one in front), else 0: the same, or further apart
+// than a map's stride reaches.
+inline uint64_t w13_apart(const void* w1, const void* w3) {
+  const uint64_t apart = w1 < w3 ? (uint64_t)((const char*)w3 - (const char*)w1) : (uint64_t)((const char*)w1 - (const char*)w3);
+  return apart < (1ull << 40) ? apart : 0;
+}
+
+// W1 and W3, [rows, inner] each, as {64 columns, 16 rows, the two of them, rows / 16, inner / 64 chunks}: a box of 64 x 16 x 2 x
+// 4 x 2 brings 64 rows of both, 16 in turn, chunk after chunk.
+inline bool make_tmap_w13(CUtensorMap* m, const void* w1, const void* w3, uint64_t rows, uint64_t inner) {
+  const uint64_t apart = w13_apart(w1, w3);
+  const cuuint64_t dims[5] = {64, 16, 2, rows / 16, inner / 64}, strides[4] = {inner * 2, apart, inner * 32, 128};
+  const cuuint32_t box[5] = {64, 16, 2, 4, 2};
+  return apart && encode_tmap(m, 5, w1 < w3 ? w1 : w3, dims, strides, box);
+}
 
 }  // namespace
 
