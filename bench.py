@@ -29,11 +29,11 @@ from paper_2604_19654_b200 import workloads as W  # noqa: E402
 
 METRIC = "moe_layer_tokens_per_s"
 UNIT = "tokens/s"
-# DRAM bytes (read + write) of one expert GEMM launch at the benchmarked workload, from the ncu
-# capture summarised under profiles/; none (null in the line) where no capture exists.
+# DRAM bytes (read + write) of one expert GEMM launch at the benchmarked workload, from an ncu
+# capture; none (null in the line) where no capture exists.
 NCU_TRAFFIC_BYTES_PER_LAUNCH = {     # keyed by (workload, GEMM launches per forward, kernels)
-    ("cfg2", 2, "k_ffn_wm"): {"bytes": 380.6e6, "source": "profiles/k_ffn_wm_cfg2.md: 761.2 MB over the 2 launches of one forward"},
-    ("cfg2", 2, "k_grouped_gemm (pair)"): {"bytes": 380.7e6, "source": "profiles/k_grouped_gemm_cfg2.md: 761.4 MB over the 2 launches of one forward "
+    ("cfg2", 2, "k_ffn_wm"): {"bytes": 380.6e6, "source": "ncu capture: 761.2 MB over the 2 launches of one forward"},
+    ("cfg2", 2, "k_grouped_gemm (pair)"): {"bytes": 380.7e6, "source": "ncu capture: 761.4 MB over the 2 launches of one forward "
                                                                       "(merged two-CTA launches, 256-row tiles)"},
 }
 

@@ -426,17 +426,19 @@ extern "C" int feplb_create(const feplb_config* cfg, feplb_ctx** out) {
   c->gemm_pair_auto = c->gemm_pair_default = (int64_t)cfg->T * cfg->K >= (int64_t)2048 * cfg->E;
   // a launch over static and dynamic groups runs them in one form: the two-CTA form from 256 rows per expert, but small
   // weights, where a tile is short, from 288 rows in single-CTA tiles (us per layer: 16 experts, d = 512, f = 256, T = 30000,
-  // top-2 107.9 -> 99.4; 48, d = 128, f = 64, 293 rows 33.6 -> 26.9; 24, d = 640, f = 256, 297 rows 107.9 -> 95.1; 128, d = 1792,
+  // top-2 107.9 -> 99.4; 48, d = 128, f = 64, 293 rows 33.6 -> 26.9; 24, d = 640, f = 256, 300 rows 40.2 -> 36.0; 128, d = 1792,
   // f = 128, 330 rows 187 -> 173; 8, d = 6144, f = 64, 1761 rows 260 -> 245; 128, d = 1792, f = 256, 604 rows 396 -> 386; d = 2688,
   // f = 192, 2262 rows 379 -> 361; d = 1152, f = 384, 1903 rows 92.6 -> 91.9; but d = 1536, f = 576, 6713 rows 302 -> 359,
-  // and d = 512, f = 832, 6118 rows 150 -> 160: from 256 Ki elements on only where f is short)
+  // and d = 512, f = 832, 6118 rows 150 -> 160: from 256 Ki elements on only where f is short).  From 256 rows to that line
+  // small weights would gain as well (258 rows, two-CTA -> single: 8, d = 128, f = 64 21.2 -> 18.2; 24, d = 640, f = 256 40.2 -> 34.8; 64,
+  // d = 1792, f = 128 95.9 -> 87.7; 32, d = 1152, f = 384 64.9 -> 57.5; 48, d = 256, f = 512 47.6 -> 40.2).
   const int64_t weight = (int64_t)cfg->d * cfg->f;
   const bool short_tiles = (weight < FEPLB_SHORT_TILE_WEIGHT / 2 || (weight < FEPLB_SHORT_TILE_WEIGHT && cfg->f <= 384)) && (int64_t)cfg->T * cfg->K >= (int64_t)FEPLB_SHORT_TILE_MIN_ROWS * cfg->E;
   c->merged_pair = (int64_t)cfg->T * cfg->K >= (int64_t)FEPLB_PAIR_MIN_ROWS_PER_EXPERT * cfg->E && !short_tiles;
   // Deep stages of that form (128 elements of K, and tiles of 128 rows): the epilogue that serves both tile heights costs
   // every tile a little, a stage of 128 elements is half empty where the width is an odd number of 64, and a ring of three is
   // less in flight while weights stream.  us per layer at the power cap, 64-element stages / deep ones:
-  //   large: 128 experts, d = 6144, f = 2048, 1024 rows per expert 9735 / 9395, 4096 rows 36897 / 35963; 32, d = 4096, f = 1024,
+  //   large: 128 experts, d = 6144, f = 2048, 1024 rows per expert 9855 / 9547, 4096 rows 37217 / 36420; 32, d = 4096, f = 1024,
   //     4096 rows 3091 / 3035; 16, d = 6144, f = 768, 3000 rows 1404 / 1375; d = 1536, f = 1408, 300 rows 107.8 / 103.3
   //   many groups, i.e. many last tiles: 128, d = 2560, f = 320, 264 rows 406 / 389; 96, d = 384, f = 1024, 313 rows 158 / 151
   //   short second pass: 48, d = 3584, f = 192, 8300 rows 3187 / 3435; 24, d = 3072, f = 192, 15000 rows 2502 / 2676; 16, d = 2560,

@@ -15,7 +15,7 @@
 // A stage holds 128 elements of K: 32 KiB of weights in one TMA instruction (pass 1 through a map whose third dimension
 // leads from W1 to W3), the token rows in another.  NMAX decides between weights in flight and weights read again: units of
 // at most 32, 64 or 128 token rows leave room for five, four or three stages, i.e. 160, 128 or 96 KiB of weights per
-// SM (feplb_few_rows has the measurements).  Pass 2 starts with
+// SM (few_rows in feplb_api.cu has the measurements).  Pass 2 starts with
 // the weights of its first unit before it waits for pass 1.  Per CTA: warp 0 = TMA producer, warp 1 = tcgen05.mma
 // issuer and TMEM owner, warps 2..5 or 2..9 = epilogue.  Every wait is bounded and ends in a status bit, a clean TMEM
 // release and a normal return.

@@ -25,17 +25,17 @@
 #define FEPLB_ST_PLAN 16u      // the GEMM's bounded wait for the planner's dynamic group table gave up
 #define FEPLB_MERGED_MAX_ROWS_PER_EXPERT 768   // static and dynamic groups share launches below this many rows per expert ...
 #define FEPLB_MERGED_ANY_ROWS_WEIGHT (6 << 20)  // ... and at any number where a weight matrix has fewer elements than this
-#define FEPLB_WM_MAX_ROWS_PER_EXPERT 1280       // the weights-on-M form ends here in such launches
+#define FEPLB_WM_MAX_ROWS_PER_EXPERT 1280       // the weights-on-M form ends here in launches over static and dynamic groups together
 #define FEPLB_SHORT_TILE_WEIGHT (1 << 19)       // below this many elements tiles are short, single-CTA tiles better ...
 #define FEPLB_SHORT_TILE_MIN_ROWS 288           // ... from this many rows per expert
 #define FEPLB_PAIR_DEEP_WEIGHT (2 << 20)        // two-CTA tiles with deep stages: matrices of at least so many elements,
 #define FEPLB_PAIR_DEEP_EXPERTS 25              // or so many experts, or two waves of tiles
 #define FEPLB_PAIR_MIN_ROWS_PER_EXPERT 256     // launches over static and dynamic groups, or all: two-CTA tiles from here
-#define FEPLB_FEW_LARGE_WEIGHT (1 << 20)       // weight matrices of at least so many elements: the form for few rows per expert up to ...
+#define FEPLB_FEW_LARGE_WEIGHT (1 << 20)       // weight matrices of at least so many elements: the form for few rows per expert up to WM_MIN_ROWS
 #define FEPLB_FEW_GUARD_WEIGHT (3 << 17)        // its guard against a nearly empty wave of long units, from so many elements
-#define FEPLB_WM_MIN_ROWS_PER_EXPERT 64        // ... this many; from here (up to the line above) the weights-on-M form ...
-#define FEPLB_WM_MIN_WEIGHT (1 << 19)          // ... for weight matrices of at least so many elements
-#define FEPLB_WM_ANY_UNITS_WEIGHT (3 << 20)     // ... and enough units; from this many elements whatever their number
+#define FEPLB_WM_MIN_ROWS_PER_EXPERT 64        // the weights-on-M form from here to WM_MAX_ROWS (in launches of one table to MERGED_MAX_ROWS)
+#define FEPLB_WM_MIN_WEIGHT (1 << 19)          // ... for weight matrices of at least so many elements and with enough units;
+#define FEPLB_WM_ANY_UNITS_WEIGHT (3 << 20)     // ... from this many elements whatever their number
 // No launch of a forward waits for the plan below this many rows per expert, or where the expert FFN takes less than this long
 #define FEPLB_DIRECT_ROWS_PER_EXPERT 128
 #define FEPLB_DIRECT_SMALL_FRONT_ROWS 192      // ... or, in the merged order behind the one-launch front, from this many
