@@ -444,13 +444,15 @@ extern "C" int feplb_create(const feplb_config* cfg, feplb_ctx** out) {
   //   short second pass: 48, d = 3584, f = 192, 8300 rows 3187 / 3435; 24, d = 3072, f = 192, 15000 rows 2502 / 2676; 16, d = 2560,
   //     f = 256, 1294 rows 199.5 / 205.0; 16, d = 4736, f = 256, 269 rows 85.5 / 87.9; short first pass: 96, d = 128, f = 512, 286
   //     rows 58.3 / 61.7
+  //   ... and few groups: 8, d = 512, f = 832, 6118 rows 169.5 / 173.6; 16, d = 512, f = 1024, 1754 rows 122.5 / 124.6; 8, d = 512, f =
+  //     704, 2088 rows 63.5 / 64.9; d = 640 level
   //   less than two waves of tiles: 16, d = 1536, f = 640, 290 rows 55.2 / 57.9; 16, d = 3328, f = 320, 306 rows 89.4 / 90.5; 16, d =
   //     512, f = 640, 441 rows 41.9 / 42.9; 16, d = 1664, f = 448, 304 rows 59.2 / 61.5
   {
     const int64_t m_tiles = (int64_t)cfg->T * cfg->K / 256 + cfg->E / 2, clusters = c->num_sms / 2;
     const int64_t blocks = std::min((cfg->f + 127) / 128, (cfg->d + 255) / 256);     // N tiles of the narrower pass
     c->pair_deep = cfg->f > 256 && cfg->d >= 256 &&
-                   (weight >= FEPLB_PAIR_DEEP_WEIGHT || cfg->E >= FEPLB_PAIR_DEEP_EXPERTS || m_tiles * blocks >= 2 * clusters);
+                   (weight >= FEPLB_PAIR_DEEP_WEIGHT || cfg->E >= FEPLB_PAIR_DEEP_EXPERTS || (cfg->d >= 768 && m_tiles * blocks >= 2 * clusters));
   }
   // backward GEMMs: the pair form pays once an expert's segment spans several 256-row tiles
   // (measured: -7.5 % backward time at 1024 rows per expert, slower at 384)

@@ -92,6 +92,7 @@ def test_deep_stages_and_tiles_of_128_rows(d, f, n_experts, w3_first):
     (1600, 25, 1024, 512, 1), (1600, 24, 1024, 512, 0),           # 25 experts
     (6400, 25, 1024, 256, 0), (6400, 25, 128, 512, 0),            # a short pass
     (7424, 16, 1024, 512, 1), (7168, 16, 1024, 512, 0),           # 37 row blocks of 4 tiles: two waves of 74 clusters
+    (24472, 8, 768, 832, 1), (24472, 8, 640, 832, 0),             # which a short first pass does without
 ])
 def test_rule_of_deep_stages(T, E, d, f, deep):
     ctx, buf, args, w = _zeros(T, 1, E, d, f)
